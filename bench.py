@@ -107,7 +107,8 @@ ROW_KERNEL_SOURCES = ("lbm_fast.cu", "lbm_lattice.cuh", "lbm_internal.h", "lbm_d
 KERNEL_NAMES = {0: "k_stream_collide (generic tile kernel)",
                 1: "k_stream_collide_rows (row kernel, per-thread loads)",
                 2: "k_stream_collide_rows (row kernel, shared-memory staging)",
-                3: "k_stream_collide_ws (row kernel, loader and collider threads)"}
+                3: "k_stream_collide_ws (row kernel, loader and collider threads)",
+                4: "k_flat_rho + k_flat_collide (density and collision passes)"}
 
 
 def row_kernel_sha1():

@@ -151,7 +151,9 @@ void lbm_opts_default(lbm_opts* opts);
  * ghost densities are rho_b^A = rho_lo and rho_b^B = rho_hi (density ratio 1,
  * Sec. 3).  Device memory: two population buffers of
  * 38 (box[2]+2)(box[1]+2) pitch elements (float64 / float32), pitch >=
- * box[0] + 2, or 88 (box[2]+2)(box[1]+2) pitch bytes (16-bit deviations).
+ * box[0] + 2, or 88 (box[2]+2)(box[1]+2) pitch bytes (16-bit deviations);
+ * with float64 storage also 16 (box[2]+2)(box[1]+2)(box[0]+2) bytes of
+ * densities where they fit.
  * On success *out receives the context; on failure *out is NULL.
  */
 int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[2], double G,
@@ -291,7 +293,9 @@ int lbm_launch_shape(lbm_ctx* ctx, int32_t* tile_y, int32_t* z_chunk, int32_t* c
 /* The stream-collide kernel in use: *variant = 0 the generic tile kernel
  * (k_stream_collide), or the row-tiled cluster kernel's variant as in
  * lbm_opts.row_variant (1 per-thread loads and 2 shared-memory staging, both
- * k_stream_collide_rows; 3 loader and collider threads, k_stream_collide_ws).
+ * k_stream_collide_rows; 3 loader and collider threads, k_stream_collide_ws),
+ * or 4 the density and collision passes (k_flat_rho, k_flat_collide) that
+ * float64 storage takes unless opts->tile_y or z_chunk is set.
  * LBM_EINVAL for a NULL context or pointer. */
 int lbm_launch_variant(lbm_ctx* ctx, int32_t* variant);
 

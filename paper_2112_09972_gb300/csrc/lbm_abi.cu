@@ -40,6 +40,7 @@ struct lbm_ctx {
     std::vector<double> kt, kA;
     // per-CTA droplet moments of the current state (frame origin of the next step)
     CentreParts centre;
+    void* rho;  // density array of the two-pass kernels (NULL otherwise)
     // reduction scratch
     double* d_partials;
     int red_blocks;
@@ -275,13 +276,23 @@ int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[
     c->elem = elem_bytes_of(c->prec);
     c->L = make_layout(box[0], box[1], box[2], c->prec);
     c->shape = choose_shape(c->L, c->prec, o.bc == LBM_BC_PERIODIC_TEST, c->model.mrt, o.tile_y, o.z_chunk,
-                            o.row_variant, c->num_sms);
+                            o.row_variant, c->num_sms, true);
+    if (c->shape.flat && cudaMalloc(&c->rho, (size_t)flat_rho_bytes(c->L)) != cudaSuccess) {
+        cudaGetLastError();  // no room for the density array: the tile kernel needs none
+        c->rho = nullptr;
+        c->shape = choose_shape(c->L, c->prec, o.bc == LBM_BC_PERIODIC_TEST, c->model.mrt, o.tile_y, o.z_chunk,
+                                o.row_variant, c->num_sms, false);
+    }
     c->cur = 0;
     c->stream = (cudaStream_t)o.cuda_stream;
     c->own_stream = false;
     int st = LBM_OK;
     if (!c->stream) {
-        if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) { delete c; return LBM_ECUDA; }
+        if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaFree(c->rho);
+            delete c;
+            return LBM_ECUDA;
+        }
         c->own_stream = true;
     }
     c->red_blocks = std::max(moments_blocks(c->L, c->num_sms), 1);
@@ -307,6 +318,7 @@ int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[0], 0, bytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, bytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
+    if (e == cudaSuccess && c->rho) e = launch_flat_fill(c->rho, c->L, c->model, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         st = cuda_status(e);
@@ -327,6 +339,7 @@ void lbm_destroy(lbm_ctx* c) {
     cudaFree(c->d_err);
     cudaFree(c->d_partials);
     cudaFree(c->centre.p);
+    cudaFree(c->rho);
     cudaFree(c->d_result);
     if (c->h_result) cudaFreeHost(c->h_result);
     if (c->h_err) cudaFreeHost(c->h_err);
@@ -384,7 +397,8 @@ int lbm_step(lbm_ctx* c, int64_t n) {
             cudaEventCreate(&b);
             cudaEventRecord(a, c->stream);
         }
-        LBM_TRY(launch_stream_collide(c->prec, src, dst, c->L, c->model, c->shape, A, c->centre, c->d_err, c->stream));
+        LBM_TRY(launch_stream_collide(c->prec, src, dst, c->L, c->model, c->shape, A, c->rho, c->centre, c->d_err,
+                                      c->stream));
         if (timed) {
             cudaEventRecord(b, c->stream);
             c->ev[0].push_back(a);
@@ -696,6 +710,7 @@ int lbm_load(lbm_ctx* c, const char* path) {
     c->model.tau[0] = h.tau[0]; c->model.tau[1] = h.tau[1];
     c->model.G = h.G;
     c->model.rho_b[0] = h.rho_b[0]; c->model.rho_b[1] = h.rho_b[1];
+    if (c->rho) LBM_TRY(launch_flat_fill(c->rho, c->L, c->model, c->stream));  // the ghost densities may differ
     c->kt.swap(kt);
     c->kA.swap(kA);
     if (is_dev(c->prec)) {
@@ -760,7 +775,8 @@ int lbm_launch_shape(lbm_ctx* c, int32_t* tile_y, int32_t* z_chunk, int32_t* cta
 
 int lbm_launch_variant(lbm_ctx* c, int32_t* variant) {
     if (!c || !variant) return LBM_EINVAL;
-    if (!c->shape.rows) *variant = 0;
+    if (c->shape.flat) *variant = 4;
+    else if (!c->shape.rows) *variant = 0;
     else *variant = c->shape.variant == kRowStaged ? 2 : (c->shape.variant == kRowWs ? 3 : 1);
     return LBM_OK;
 }

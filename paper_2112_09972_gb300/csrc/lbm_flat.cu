@@ -1,0 +1,270 @@
+// Two-pass stream-collide step for float64 storage: a density pass and a
+// collision pass, each with one thread per node and no march (Sec. 2, Eqs.
+// 6-10 of Milan et al., arXiv:2112.09972).
+//
+//   k_flat_rho     -- post-streaming densities of every node (Eq. 6) into a
+//                     padded array [Lz + 2][Ly + 2][Lx + 2] of {rho_A, rho_B};
+//                     its halo holds the ghost densities (ghost boundary,
+//                     written once) or the periodic images
+//   k_flat_collide -- pulls the populations, reads the node's and its
+//                     neighbours' densities, Shan-Chen force (Eq. 7),
+//                     velocity shift, BGK or MRT collision, store, and the
+//                     droplet's centre of mass
+//
+// What bounds it.  This GPU's FP64 pipe issues one warp instruction per 16
+// cycles and SM, so a float64 node update is bound by its FP64 instructions,
+// not by memory: at 128^3 the 608 bytes of a node take 94 ns per 512 nodes of
+// copy bandwidth and 300 FP64 instructions five times that.  The marched tile
+// kernel sums every density about twice (the tile's halo, and the planes
+// before and after each z chunk) and evaluates each equilibrium on its own,
+// 560 instructions per node.  Here each density is summed once (the second
+// read of the populations costs bandwidth that is idle), opposite
+// directions share their equilibria, and the launch covers the chip for any
+// box: one node per thread instead of a z march per tile.  Measured per step
+// against the tile kernel: 32^3 44.8 us (178), 64^3 207 us (365), 128^3 1557 us
+// (3174), 37 x 29 x 23 37 us (160); float64 storage therefore takes these
+// kernels at every size.
+#include <cuda_runtime.h>
+
+#include "lbm_internal.h"
+#include "lbm_lattice.cuh"
+#include "lbm_pdl.cuh"
+#include "lbm_tile.cuh"
+
+namespace lbmgb {
+namespace {
+
+constexpr int kFlatThreads = 64;  // two warps: CTAs spread evenly over the SMs, whose FP64 pipes are the bound
+
+// The padded density array: node (x, y, z) at ((z + 1) ny + y + 1) nx + x + 1.
+struct RhoGeo {
+    int nx, ny;
+    __host__ __device__ long long at(int x, int y, int z) const {
+        return ((long long)(z + 1) * ny + y + 1) * nx + x + 1;
+    }
+};
+RhoGeo rho_geo(const Layout& L) { return {L.Lx + 2, L.Ly + 2}; }
+
+struct FlatModel {
+    double inv_tau[2], omit[2];  // 1 / tau, 1 - 1 / tau
+    double sh[2];                // -G tau / 36: the velocity shift per unit of the other component's force sum
+    double mrt[5];
+};
+
+FlatModel flat_model(const Model& m) {
+    FlatModel r;
+    for (int s = 0; s < 2; ++s) {
+        r.inv_tau[s] = 1.0 / m.tau[s];
+        r.omit[s] = 1.0 - 1.0 / m.tau[s];
+        r.sh[s] = -m.G * m.tau[s] / 36.0;
+    }
+    for (int k = 0; k < 5; ++k) r.mrt[k] = m.mrt_rates[k];
+    return r;
+}
+
+__global__ void k_flat_fill(double2* __restrict__ rho, long long n, double a, double b) {
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) rho[k] = make_double2(a, b);
+}
+
+template <bool PER>
+__global__ void __launch_bounds__(kFlatThreads) k_flat_rho(const double* __restrict__ src, Layout L,
+                                                           double2* __restrict__ rho, RhoGeo g, int zchunk) {
+    pdl_wait();
+    pdl_trigger();
+    const int p = blockIdx.x * kFlatThreads + threadIdx.x;
+    if (p >= L.Lx * L.Ly) return;
+    const int y = p / L.Lx, x = p - y * L.Lx;
+    const Puller<double, double, PER> P{src, L};
+    const int z1 = min(((int)blockIdx.y + 1) * zchunk, L.Lz);
+    for (int z = blockIdx.y * zchunk; z < z1; ++z) {
+        double f[2][19];
+        P.pull(x, y, z, f);
+        const double2 r = make_double2(sum19<double>(f[0]), sum19<double>(f[1]));
+        rho[g.at(x, y, z)] = r;
+        if (PER) {  // the images in the halo (the force reads no corner)
+            const int ix = x == 0 ? L.Lx : (x == L.Lx - 1 ? -1 : x);
+            const int iy = y == 0 ? L.Ly : (y == L.Ly - 1 ? -1 : y);
+            const int iz = z == 0 ? L.Lz : (z == L.Lz - 1 ? -1 : z);
+            if (ix != x) rho[g.at(ix, y, z)] = r;
+            if (iy != y) rho[g.at(x, iy, z)] = r;
+            if (iz != z) rho[g.at(x, y, iz)] = r;
+            if (ix != x && iy != y) rho[g.at(ix, iy, z)] = r;
+            if (ix != x && iz != z) rho[g.at(ix, y, iz)] = r;
+            if (iy != y && iz != z) rho[g.at(x, iy, iz)] = r;
+        }
+    }
+}
+
+__device__ __forceinline__ bool finite64(double v) {  // on the integer pipe
+    return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+}
+
+// Collision of one node from its pulled populations f and the density array
+// (r: the node's entry; rows sy, planes sz apart), stored to dst.
+template <bool MRT>
+__device__ __forceinline__ void flat_node(const double2* __restrict__ r, int sy, int sz, const FlatModel& m,
+                                          const double (&f)[2][19], double* __restrict__ o, long long pitch,
+                                          double2& rho) {
+    // momentum (Eq. 6) of both components, opposite pairs differenced first,
+    // combined with the weights of the common velocity
+    double j[2][3];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        double jx = 0.0, jy = 0.0, jz = 0.0;
+#pragma unroll
+        for (int i = 1; i < 19; i += 2) {
+            const double d = f[s][i] - f[s][i + 1];
+            if (cx_(i)) jx = cx_(i) > 0 ? jx + d : jx - d;
+            if (cy_(i)) jy = cy_(i) > 0 ? jy + d : jy - d;
+            if (cz_(i)) jz = cz_(i) > 0 ? jz + d : jz - d;
+        }
+        j[s][0] = jx; j[s][1] = jy; j[s][2] = jz;
+    }
+    // Shan-Chen force sums (Eq. 7) in units of the edge weight 1/36
+    double acc[2][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
+#pragma unroll
+    for (int i = 1; i < 19; i += 2) {
+        const int off = cz_(i) * sz + cy_(i) * sy + cx_(i);
+        const double2 a = r[off], b = r[-off];
+        const double dA = i < 7 ? 2.0 * (a.x - b.x) : a.x - b.x, dB = i < 7 ? 2.0 * (a.y - b.y) : a.y - b.y;
+        if (cx_(i)) { acc[0][0] += cx_(i) > 0 ? dA : -dA; acc[1][0] += cx_(i) > 0 ? dB : -dB; }
+        if (cy_(i)) { acc[0][1] += cy_(i) > 0 ? dA : -dA; acc[1][1] += cy_(i) > 0 ? dB : -dB; }
+        if (cz_(i)) { acc[0][2] += cz_(i) > 0 ? dA : -dA; acc[1][2] += cz_(i) > 0 ? dB : -dB; }
+    }
+    rho = *r;
+    const double rden = 1.0 / (rho.x * m.inv_tau[0] + rho.y * m.inv_tau[1]);
+    double up[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) up[a] = (j[0][a] * m.inv_tau[0] + j[1][a] * m.inv_tau[1]) * rden;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const double rs = s ? rho.y : rho.x;
+        const double ux = fma(m.sh[s], acc[1 - s][0], up[0]);
+        const double uy = fma(m.sh[s], acc[1 - s][1], up[1]);
+        const double uz = fma(m.sh[s], acc[1 - s][2], up[2]);
+        double* os = o + (long long)(19 * s) * pitch;
+        if constexpr (MRT) {
+            const double u2x = 1.5 * (ux * ux + uy * uy + uz * uz);
+            double dv[19], out[19];
+#pragma unroll
+            for (int i = 0; i < 19; ++i) dv[i] = f[s][i] - feq<double>(i, rs, ux, uy, uz, u2x);
+            mrt_relax<double>(f[s], dv, m.inv_tau[s], m.mrt, out);
+#pragma unroll
+            for (int i = 0; i < 19; ++i) os[i * pitch] = out[i];
+        } else {
+            // with v = 1.5 u and c = c_i . v, the even and odd parts of
+            // f_eq / tau of a pair are e base + c (2 e c) and 2 e c
+            const double base = fma(-1.5, ux * ux + uy * uy + uz * uz, 1.0);
+            const double ir = m.inv_tau[s] * rs;
+            const double vx = 1.5 * ux, vy = 1.5 * uy, vz = 1.5 * uz;
+            const double e2A = ir * (1.0 / 9.0), e2E = ir * (1.0 / 18.0);  // 2 e of axis and edge directions
+            const double ib = ir * base;
+            const double ebA = ib * (1.0 / 18.0), ebE = ib * (1.0 / 36.0);
+            const double om = m.omit[s];
+#pragma unroll
+            for (int i = 1; i < 19; i += 2) {
+                const double c = cx_(i) * vx + cy_(i) * vy + cz_(i) * vz;
+                const double od = (i < 7 ? e2A : e2E) * c;
+                const double ev = fma(c, od, i < 7 ? ebA : ebE);
+                os[i * pitch] = fma(om, f[s][i], ev + od);
+                os[(i + 1) * pitch] = fma(om, f[s][i + 1], ev - od);
+            }
+            os[0] = fma(om, f[s][0], ib * (1.0 / 3.0));
+        }
+    }
+}
+
+template <bool PER, bool MRT>
+__global__ void __launch_bounds__(kFlatThreads, 6)
+    k_flat_collide(const double* __restrict__ src, double* __restrict__ dst, Layout L, FlatModel m,
+                   const double2* __restrict__ rho, RhoGeo g, int zchunk, CentreParts cp, int* __restrict__ d_err) {
+    __shared__ double scratch[4 * (kFlatThreads / 32)];
+    pdl_wait();
+    const int p = blockIdx.x * kFlatThreads + threadIdx.x;
+    const int y = p / L.Lx, x = p - y * L.Lx;
+    const Puller<double, double, PER> P{src, L};
+    double cm[4] = {0.0, 0.0, 0.0, 0.0};
+    bool drop = false, bad = false;
+    if (p < L.Lx * L.Ly) {
+        const double px = x - 0.5 * (L.Lx - 1), py = y - 0.5 * (L.Ly - 1);
+        const int z1 = min(((int)blockIdx.y + 1) * zchunk, L.Lz);
+        for (int z = blockIdx.y * zchunk; z < z1; ++z) {
+            double f[2][19];
+            P.pull(x, y, z, f);
+            double2 r;
+            flat_node<MRT>(rho + g.at(x, y, z), g.nx, g.nx * g.ny, m, f, dst + L.at(0, 0, x, y, z), L.pitch, r);
+            bad |= !(finite64(r.x) && finite64(r.y));
+            // w = max(phi, 0): the division only where phi is not negative
+            const double d = r.x - r.y, t = r.x + r.y;
+            if ((__double2hiint(d) ^ __double2hiint(t)) >= 0) {
+                const double w = fmax(d / t, 0.0);
+                cm[0] += w;
+                cm[1] = fma(w, px, cm[1]);
+                cm[2] = fma(w, py, cm[2]);
+                cm[3] = fma(w, z - 0.5 * (L.Lz - 1), cm[3]);
+                drop = true;
+            }
+        }
+    }
+    pdl_trigger();
+    if (bad) atomicOr(d_err, 1);
+    // the droplet's centre of mass: partials in CTA order, as centre_epilogue,
+    // whose FP64 shuffles a CTA without droplet nodes does without
+    const unsigned cta = blockIdx.y * gridDim.x + blockIdx.x, total = gridDim.x * gridDim.y;
+    const bool any = __syncthreads_or(drop) != 0;
+    centre_reduce_last<kFlatThreads>(cm, any, cp.p, cta, total, cp.counter, cp.sum, cp.frame, scratch);
+}
+
+}  // namespace
+
+long long flat_rho_bytes(const Layout& L) {
+    return (long long)sizeof(double2) * (L.Lx + 2) * (L.Ly + 2) * (L.Lz + 2);
+}
+
+// One node per thread; the z extent is cut so that the launch has at most
+// about 16 CTAs per SM, which bounds the centre-of-mass partials the last CTA
+// sums (small boxes: one plane per CTA).
+Shape flat_shape(const Layout& L, int num_sms) {
+    Shape sh = {};
+    const long long per_plane = ((long long)L.Lx * L.Ly + kFlatThreads - 1) / kFlatThreads;
+    const long long want = 16LL * (num_sms > 0 ? num_sms : 152);
+    long long zc = (per_plane * L.Lz + want - 1) / want;
+    if (zc < 1) zc = 1;
+    while ((L.Lz + zc - 1) / zc > 65535) ++zc;
+    sh.flat = 1;
+    sh.tx = L.Lx;
+    sh.ty = L.Lx >= kFlatThreads ? 1 : kFlatThreads / L.Lx;
+    sh.zchunk = (int)zc;
+    sh.grid = dim3((unsigned)per_plane, (unsigned)((L.Lz + zc - 1) / zc), 1);
+    sh.threads = kFlatThreads;
+    return sh;
+}
+
+cudaError_t launch_flat_fill(void* rho, const Layout& L, const Model& m, cudaStream_t s) {
+    const long long n = flat_rho_bytes(L) / (long long)sizeof(double2);
+    k_flat_fill<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((double2*)rho, n, m.rho_b[0], m.rho_b[1]);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_flat(const void* src, void* dst, void* rho, const Layout& L, const Model& m, const Shape& sh,
+                        CentreParts cp, int* d_err, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = sh.grid;
+    cfg.blockDim = dim3(kFlatThreads, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1] = {pdl_attribute()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const RhoGeo g = rho_geo(L);
+    const FlatModel fm = flat_model(m);
+    const double* f = (const double*)src;
+    double2* r = (double2*)rho;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, m.periodic ? k_flat_rho<true> : k_flat_rho<false>, f, L, r, g, sh.zchunk);
+    if (e != cudaSuccess) return e;
+    auto k = m.periodic ? (m.mrt ? k_flat_collide<true, true> : k_flat_collide<true, false>)
+                        : (m.mrt ? k_flat_collide<false, true> : k_flat_collide<false, false>);
+    return cudaLaunchKernelEx(&cfg, k, f, (double*)dst, L, fm, (const double2*)r, g, sh.zchunk, cp, d_err);
+}
+
+}  // namespace lbmgb

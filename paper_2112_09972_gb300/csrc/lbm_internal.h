@@ -103,6 +103,7 @@ struct Grad {
 // Launch shape of the stream-collide kernel.
 struct Shape {
     int rows;       // 1: the row-tiled cluster kernel (lbm_fast.cu), 0: the generic tile kernel
+    int flat;       // 1: the two-pass kernels (lbm_flat.cu), which need a density array
     int tx, ty;     // tile of the x-y plane per CTA
     int zchunk;     // z planes marched per CTA
     int variant;    // row kernel: kRowDirect, kRowStaged or kRowWs
@@ -124,18 +125,29 @@ enum { kRowDirect = 0, kRowStaged = 1, kRowWs = 2 };
 // variant_req: the row_variant of lbm_opts (1 direct loads, 2 staged,
 // 3 warp-specialised, 0 automatic); mrt: the MRT collision (the row kernel's
 // direct variant for float32 storage, the generic kernel otherwise)
+// allow_flat: the two-pass kernels may be chosen
 Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req, int zchunk_req, int variant_req,
-                   int num_sms);
+                   int num_sms, bool allow_flat);
 cudaError_t launch_init(int prec, void* f, const Layout& L, double R, double xi, double rho_hi, double rho_lo,
                         Grad A0, cudaStream_t s);
 cudaError_t launch_ghost(int prec, void* f, const Layout& L, const Model& m, Grad A, CentreParts cp, int* d_err,
                          cudaStream_t s);
 // A: the boundary gradient of this step (the kernels read the ghost shell
 // written by launch_ghost; A is passed for kernels that may compute it).
+// rho: the density array of the two-pass kernels (sh.flat).
 cudaError_t launch_stream_collide(int prec, const void* src, void* dst, const Layout& L, const Model& m,
-                                  const Shape& sh, const Grad& A, CentreParts cp, int* d_err, cudaStream_t s);
+                                  const Shape& sh, const Grad& A, void* rho, CentreParts cp, int* d_err,
+                                  cudaStream_t s);
 // Centre-of-mass partials of the stored populations f (cp.n CTAs, grid-stride).
 cudaError_t launch_centre(int prec, const void* f, const Layout& L, CentreParts cp, cudaStream_t s);
+
+// ---- two-pass kernels (lbm_flat.cu): fp64, any box and boundary mode ----
+Shape flat_shape(const Layout& L, int num_sms);
+long long flat_rho_bytes(const Layout& L);
+// Fill the density array with the ghost densities (its halo keeps them).
+cudaError_t launch_flat_fill(void* rho, const Layout& L, const Model& m, cudaStream_t s);
+cudaError_t launch_flat(const void* src, void* dst, void* rho, const Layout& L, const Model& m, const Shape& sh,
+                        CentreParts cp, int* d_err, cudaStream_t s);
 
 // ---- row-tiled cluster kernel (lbm_fast.cu): fp32 or 16-bit deviations, ghost boundary,
 //      Lx in {32, 64, 128, 256}, Ly % 8 == 0 ----

@@ -259,9 +259,13 @@ Layout make_layout(int Lx, int Ly, int Lz, int prec) {
 }
 
 Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req, int zchunk_req, int variant_req,
-                   int num_sms) {
+                   int num_sms, bool allow_flat) {
+    // float64: the two-pass kernels at every size (measured against the tile
+    // kernel in lbm_flat.cu), unless a launch shape is asked for
+    if (allow_flat && prec == kFP64 && ty_req <= 0 && zchunk_req <= 0) return flat_shape(L, num_sms);
     Shape sh;
     sh.rows = 0;
+    sh.flat = 0;
     sh.variant = kRowDirect;
     if (ty_req <= 0 && (!mrt || prec == kFP32) && rows_kernel_applies(L, prec, periodic)) {
         // One CTA per row.  MRT rows: direct loads only.  Automatic choice,
@@ -355,8 +359,9 @@ cudaError_t launch_ghost(int prec, void* f, const Layout& L, const Model& m, Gra
                          cudaStream_t s) {
     const int fast = (L.Lx > 2 * (L.Ly + 2) ? L.Lx : 2 * (L.Ly + 2));  // x faces: two threads per node
     const int slow = (L.Lz + 2 > L.Ly ? L.Lz + 2 : L.Ly);
-    const dim3 block(32, 8, 1);
-    const dim3 grid((fast + 31) / 32, (slow + 7) / 8, 6);
+    // float64: small CTAs, which spread the work over the SMs' FP64 pipes
+    const dim3 block(32, prec == kFP64 ? 2 : 8, 1);
+    const dim3 grid((fast + 31) / 32, (slow + block.y - 1) / block.y, 6);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -382,7 +387,9 @@ cudaError_t launch_centre(int prec, const void* f, const Layout& L, CentreParts 
 }
 
 cudaError_t launch_stream_collide(int prec, const void* src, void* dst, const Layout& L, const Model& m,
-                                  const Shape& sh, const Grad& A, CentreParts cp, int* d_err, cudaStream_t s) {
+                                  const Shape& sh, const Grad& A, void* rho, CentreParts cp, int* d_err,
+                                  cudaStream_t s) {
+    if (sh.flat) return launch_flat(src, dst, rho, L, m, sh, cp, d_err, s);
     if (sh.rows) return launch_stream_collide_rows(prec, sh.variant, src, dst, L, m, A, sh.zchunk, cp, d_err, s);
     if (prec == kFP64) return stream_collide_t<double, double, kMaxThreadsF64>(src, dst, L, m, sh, cp, d_err, s);
     if (prec == kFP32) return stream_collide_t<float, float, kMaxThreadsF32>(src, dst, L, m, sh, cp, d_err, s);

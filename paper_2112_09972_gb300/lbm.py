@@ -350,7 +350,7 @@ class DropletLBM:
         return ty.value, zc.value, ctas.value
 
     def launch_variant(self):
-        """0: the generic tile kernel; 1, 2, 3: the row kernel's variant (lbm_opts.row_variant)."""
+        """0: the generic tile kernel; 1, 2, 3: the row kernel's variant (lbm_opts.row_variant); 4: the two-pass kernels."""
         v = ctypes.c_int32()
         _check(self._lib.lbm_launch_variant(self._h, ctypes.byref(v)), "lbm_launch_variant")
         return v.value
