@@ -233,8 +233,8 @@ int lbm_checksums(lbm_ctx* ctx, double mass[2], double mom[3]);
  * components with at least min_nodes nodes and sizes[0 .. max_sizes-1] their
  * node counts, largest first (0 past the last).  A droplet that broke up
  * has count >= 2.  Periodic images connect in the periodic test mode.
- * Synchronises; allocates 16 bytes per node of scratch for the call
- * (LBM_ETIMEOUT if the labelling did not settle within its sweep bound).
+ * Synchronises; its scratch is the buffer of the next step's state
+ * (LBM_ETIMEOUT if a walk of the labelling exceeded its bound).
  */
 int lbm_components(lbm_ctx* ctx, double threshold, int64_t min_nodes, int32_t* count, int64_t* sizes,
                    int32_t max_sizes);
@@ -246,8 +246,8 @@ int lbm_components(lbm_ctx* ctx, double threshold, int64_t min_nodes, int32_t* c
  * sets of phi between its extremes (co-area formula): Omega = sum |grad phi| /
  * (phi_max - phi_min), central differences at interior nodes; the volume
  * V = sum (phi - phi_min) / (phi_max - phi_min); Omega_0 = (36 pi V^2)^(1/3).
- * area and volume (may be NULL) receive Omega and V.  Synchronises;
- * allocates 8 bytes per node of scratch for the call.
+ * area and volume (may be NULL) receive Omega and V.  Synchronises; its
+ * scratch is the buffer of the next step's state.
  */
 int lbm_surface_deformation(lbm_ctx* ctx, double* D_lbm, double* area, double* volume);
 

@@ -445,13 +445,11 @@ int lbm_get_fields(lbm_ctx* c, double* rho_A, double* rho_B, double* u) {
     int st = set_device(c);
     if (st || (st = lazy_init(c))) return st;
     const size_t N = (size_t)c->box[0] * c->box[1] * c->box[2];
-    double* d = nullptr;
-    LBM_TRY(cudaMallocAsync(&d, sizeof(double) * 5 * N, c->stream));
+    double* d = (double*)c->f[1 - c->cur];  // scratch in the buffer of the next step's state (40 of its 88 .. 304 B per node)
     cudaError_t e = launch_fields(c->prec, c->f[c->cur], c->L, c->model, d, d + N, d + 2 * N, c->stream);
     if (e == cudaSuccess && rho_A) e = cudaMemcpyAsync(rho_A, d, sizeof(double) * N, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess && rho_B) e = cudaMemcpyAsync(rho_B, d + N, sizeof(double) * N, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess && u) e = cudaMemcpyAsync(u, d + 2 * N, sizeof(double) * 3 * N, cudaMemcpyDeviceToHost, c->stream);
-    cudaFreeAsync(d, c->stream);
     if (e != cudaSuccess) return cuda_status(e);
     return sync_and_check(c);
 }
@@ -511,52 +509,39 @@ int lbm_components(lbm_ctx* c, double threshold, int64_t min_nodes, int32_t* cou
     if (st || (st = lazy_init(c))) return st;
     const long long N = (long long)c->box[0] * c->box[1] * c->box[2];
     if (N > INT32_MAX) return LBM_EINVAL;
-    // scratch: labels and sizes (N ints each), the change flag and root counter,
-    // and the root sizes (N 64-bit)
-    char* d = nullptr;
-    const size_t bytes = sizeof(int) * (2 * N + 2) + sizeof(long long) * N + 16;
-    LBM_TRY(cudaMallocAsync((void**)&d, bytes, c->stream));
-    int* label = (int*)d;
+    // scratch in the buffer of the next step's state: labels and sizes (N ints
+    // each), the component sizes (N 64-bit), two flags
+    long long* out = (long long*)c->f[1 - c->cur];
+    int* label = (int*)(out + N);
     int* size = label + N;
-    int* flags = size + N;  // [0] changed, [1] root count
-    long long* out = (long long*)(((uintptr_t)(flags + 2) + 15) & ~(uintptr_t)15);
-    int h_flags[2] = {0, 0};
-    cudaError_t e = cudaMemsetAsync(size, 0, sizeof(int) * (N + 2), c->stream);
-    if (e == cudaSuccess) e = launch_cc_init(c->prec, c->f[c->cur], c->L, threshold, label, c->stream);
-    // propagation sweeps until no label changes; bounded (a component's
-    // labels settle within its node count of sweeps)
-    const long long max_sweeps = std::min<long long>(N + 8, 1LL << 22);
-    bool converged = false;
-    for (long long it = 0; e == cudaSuccess && it < max_sweeps; it += 4) {
-        e = cudaMemsetAsync(flags, 0, sizeof(int), c->stream);
-        for (int q = 0; q < 4 && e == cudaSuccess; ++q) e = launch_cc_sweep(c->L, c->model.periodic, label, flags, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h_flags, flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        if (e == cudaSuccess && h_flags[0] == 0) {
-            converged = true;
-            break;
-        }
-    }
-    std::vector<long long> roots;
-    if (e == cudaSuccess && converged) e = launch_cc_sizes(c->L, label, size, flags + 1, out, (int)N, c->stream);
-    if (e == cudaSuccess && converged) e = cudaMemcpyAsync(h_flags, flags, sizeof(int) * 2, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess && converged) e = cudaStreamSynchronize(c->stream);
-    if (e == cudaSuccess && converged) {
-        try { roots.resize((size_t)h_flags[1]); } catch (...) { e = cudaErrorMemoryAllocation; }
-        if (e == cudaSuccess && !roots.empty())
-            e = cudaMemcpyAsync(roots.data(), out, sizeof(long long) * roots.size(), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    }
-    cudaFreeAsync(d, c->stream);
-    if (e != cudaSuccess) return cuda_status(e);
-    if (!converged) return LBM_ETIMEOUT;
+    int* flags = size + N;  // [0] a walk gave up, [1] component count
+    constexpr int kFirst = 24;  // sizes read back with the count
+    long long* h = (long long*)c->h_result;
+    LBM_TRY(launch_cc(c->prec, c->f[c->cur], c->L, c->model.periodic, threshold, label, size, flags, out, (int)N,
+                      c->stream));
+    LBM_TRY(cudaMemcpyAsync(h, flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    LBM_TRY(cudaMemcpyAsync(h + 1, out, sizeof(long long) * kFirst, cudaMemcpyDeviceToHost, c->stream));
+    if ((st = sync_and_check(c))) return st;
+    int h_flags[2];
+    memcpy(h_flags, h, sizeof(h_flags));
+    if (h_flags[0]) return LBM_ETIMEOUT;
     std::vector<long long> kept;
-    for (long long v : roots)
-        if (v >= min_nodes) kept.push_back(v);
+    try {
+        kept.assign(h + 1, h + 1 + std::min(h_flags[1], kFirst));
+        if (h_flags[1] > kFirst) {
+            kept.resize((size_t)h_flags[1]);
+            LBM_TRY(cudaMemcpyAsync(kept.data(), out, sizeof(long long) * kept.size(), cudaMemcpyDeviceToHost,
+                                    c->stream));
+            LBM_TRY(cudaStreamSynchronize(c->stream));
+        }
+    } catch (...) {
+        return LBM_ENOMEM;
+    }
+    kept.erase(std::remove_if(kept.begin(), kept.end(), [&](long long v) { return v < min_nodes; }), kept.end());
     std::sort(kept.begin(), kept.end(), [](long long a, long long b) { return a > b; });
     *count = (int32_t)kept.size();
     for (int32_t k = 0; k < max_sizes; ++k) sizes[k] = k < (int32_t)kept.size() ? kept[k] : 0;
-    return sync_and_check(c);
+    return LBM_OK;
 }
 
 int lbm_surface_deformation(lbm_ctx* c, double* D_lbm, double* area, double* volume) {
@@ -564,13 +549,11 @@ int lbm_surface_deformation(lbm_ctx* c, double* D_lbm, double* area, double* vol
     int st = set_device(c);
     if (st || (st = lazy_init(c))) return st;
     const long long N = (long long)c->box[0] * c->box[1] * c->box[2];
-    double* phi = nullptr;
-    LBM_TRY(cudaMallocAsync(&phi, sizeof(double) * N, c->stream));
+    double* phi = (double*)c->f[1 - c->cur];  // scratch in the buffer of the next step's state
     cudaError_t e = launch_surface_stats(c->prec, c->f[c->cur], c->L, phi, c->d_partials, c->red_blocks, c->d_result,
                                          c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->h_result, c->d_result, sizeof(double) * 4, cudaMemcpyDeviceToHost, c->stream);
-    cudaFreeAsync(phi, c->stream);
     if (e != cudaSuccess) return cuda_status(e);
     if ((st = sync_and_check(c))) return st;
     const double sum = c->h_result[0], lo = c->h_result[1], hi = c->h_result[2], grad = c->h_result[3];

@@ -98,40 +98,78 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float v) {
     lo += e;
 }
 
-// Component densities of fluid node (x, y, z): the sum of its populations,
-// or rho* of deviation storage (the same value up to float32 rounding).
+// Component densities of fluid node (x, y, z) as unevaluated pairs hi + lo:
+// the sum of its populations, or rho* of deviation storage (the same value up
+// to float32 rounding).  Float32 storage sums in float32 (Knuth's TwoSum per
+// addition, its rounding errors gathered in lo), so that the 36 additions run
+// on the float32 pipe (this GPU's FP64 pipe runs at 1/64 of its rate); hi +
+// lo agrees with a float64 sum to about 1e-14 relative.
+template <typename S>
+struct RhoPair {
+    using T = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
+    T ah, al, bh, bl;
+    __device__ __forceinline__ double a() const {
+        if constexpr (std::is_same<S, float>::value) return (double)ah + (double)al;
+        else return ah;
+    }
+    __device__ __forceinline__ double b() const {
+        if constexpr (std::is_same<S, float>::value) return (double)bh + (double)bl;
+        else return bh;
+    }
+    // false only when phi = (a - b) / (a + b) is certainly not above zero:
+    // a - b below and a + b above what their evaluation here can be off by
+    __device__ __forceinline__ bool droplet() const {
+        if constexpr (std::is_same<S, double>::value)  // the signs, read on the integer pipe
+            return (__double2hiint(ah - bh) ^ __double2hiint(ah + bh)) >= 0;
+        const T d = (ah - bh) + (al - bl), t = (ah + bh) + (al + bl);
+        const T m = T(1e-6) * ((fabs(ah) + fabs(bh)) + (fabs(al) + fabs(bl)));
+        return !(d < -m && t > m);
+    }
+};
+template <typename S>
+__device__ __forceinline__ RhoPair<S> node_rho_pair(const S* __restrict__ f, const Layout& L, int x, int y, int z) {
+    RhoPair<S> r;
+    r.al = r.bl = 0;
+    if constexpr (is_dev_t<S>::value) {
+        const float4 o = reinterpret_cast<const float4*>(f)[L.dev_node(x, y, z)];
+        r.ah = o.x;
+        r.bh = o.y;
+    } else {
+        const long long b = L.at(0, 0, x, y, z);
+        r.ah = f[b];
+        r.bh = f[b + 19LL * L.pitch];
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            const S va = f[b + (long long)i * L.pitch], vb = f[b + (long long)(19 + i) * L.pitch];
+            if constexpr (std::is_same<S, float>::value) {
+                two_sum_acc(r.ah, r.al, va);
+                two_sum_acc(r.bh, r.bl, vb);
+            } else {
+                r.ah += va;
+                r.bh += vb;
+            }
+        }
+    }
+    return r;
+}
 template <typename S>
 __device__ __forceinline__ void node_rho(const S* __restrict__ f, const Layout& L, int x, int y, int z, double& ra,
                                          double& rb) {
-    if constexpr (is_dev_t<S>::value) {
-        const float4 o = reinterpret_cast<const float4*>(f)[L.dev_node(x, y, z)];
-        ra = o.x;
-        rb = o.y;
-    } else if constexpr (std::is_same<S, float>::value) {
-        // float32 storage: each density as an unevaluated pair hi + lo of
-        // float32 sums (Knuth's TwoSum per addition, its rounding errors
-        // gathered in lo), so that the 36 additions run on the float32 pipe
-        // (this GPU's FP64 pipe runs at 1/64 of its rate); hi + lo agrees
-        // with a float64 sum to about 1e-14 relative.
-        const long long b = L.at(0, 0, x, y, z);
-        float ah = f[b], al = 0.f, bh = f[b + 19LL * L.pitch], bl = 0.f;
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            two_sum_acc(ah, al, f[b + (long long)i * L.pitch]);
-            two_sum_acc(bh, bl, f[b + (long long)(19 + i) * L.pitch]);
-        }
-        ra = (double)ah + (double)al;
-        rb = (double)bh + (double)bl;
-    } else {
-        const long long b = L.at(0, 0, x, y, z);
-        ra = 0.0;
-        rb = 0.0;
-#pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            ra += (double)f[b + (long long)i * L.pitch];
-            rb += (double)f[b + (long long)(19 + i) * L.pitch];
-        }
-    }
+    const RhoPair<S> r = node_rho_pair(f, L, x, y, z);
+    ra = r.a();
+    rb = r.b();
+}
+
+// n / d to float64 rounding or one unit more: a float32 quotient carried to
+// float64 by two Newton steps (4 FP64 instructions instead of a divide's
+// dozen); the plain divide outside float32's range.
+__device__ __forceinline__ double div64(double n, double d) {
+    const float df = (float)d;
+    if (!(fabsf(df) > 1e-30f && fabsf(df) < 1e30f)) return n / d;
+    const double y = (double)__frcp_rn(df);
+    double q = n * y;
+    q = fma(fma(-q, d, n), y, q);
+    return fma(fma(-q, d, n), y, q);
 }
 
 // Block-wide sum of K doubles per thread; thread 0 writes them to out[0..K).
@@ -161,41 +199,109 @@ __device__ void block_sum(double (&v)[K], double* out) {
     }
 }
 
+// How k_moments and k_grad_phi walk the box: a warp takes 32 consecutive
+// nodes of an x-y plane (flattened, so that no width leaves lanes idle) and
+// marches one of `zparts` parts of the z extent; units of work are numbered
+// segment first.
+struct Columns {
+    int segs, zparts, zlen;
+};
+Columns columns(const Layout& L, long long warps) {
+    Columns c;
+    c.segs = (int)(((long long)L.Lx * L.Ly + 31) / 32);
+    long long zp = warps / c.segs;
+    zp = zp < 1 ? 1 : (zp > L.Lz ? L.Lz : zp);
+    c.zlen = (int)((L.Lz + zp - 1) / zp);
+    c.zparts = (L.Lz + c.zlen - 1) / c.zlen;
+    return c;
+}
+
+// Ten moments of w = max(phi, 0).  Few nodes have phi > 0 (a droplet of R =
+// L / 8 fills 0.8 % of its box), so only those run FP64 instructions: a
+// lane's x and y stay fixed along its march, its three sums {w, w z, w z^2}
+// give all ten moments at the end, and warps and CTAs without a droplet node
+// skip the FP64 reductions.  128^3 float32 on GB300: 180 us with ten FP64
+// sums per node and the reductions in every warp, bound by the FP64 pipe.
 template <typename S>
-__global__ void __launch_bounds__(kRedThreads) k_moments(const S* __restrict__ f, Layout L, double* __restrict__ partials) {
+__global__ void __launch_bounds__(kRedThreads, 4) k_moments(const S* __restrict__ f, Layout L, Columns c,
+                                                         double* __restrict__ partials) {
+    __shared__ double part[kRedThreads / 32][10];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double cx = 0.5 * (L.Lx - 1), cy = 0.5 * (L.Ly - 1), cz = 0.5 * (L.Lz - 1);
     double m[10];
 #pragma unroll
     for (int k = 0; k < 10; ++k) m[k] = 0.0;
-    const long long N = (long long)L.Lx * L.Ly * L.Lz;
-    const double cx = 0.5 * (L.Lx - 1), cy = 0.5 * (L.Ly - 1), cz = 0.5 * (L.Lz - 1);
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % L.Lx), y = (int)((n / L.Lx) % L.Ly), z = (int)(n / ((long long)L.Lx * L.Ly));
-        double ra, rb;
-        node_rho(f, L, x, y, z, ra, rb);
-        const double phi = (ra - rb) / (ra + rb);
-        const double w = phi > 0.0 ? phi : 0.0;
-        const double px = x - cx, py = y - cy, pz = z - cz;
-        m[0] += w;
-        m[1] += w * px; m[2] += w * py; m[3] += w * pz;
-        m[4] += w * px * px; m[5] += w * px * py; m[6] += w * px * pz;
-        m[7] += w * py * py; m[8] += w * py * pz; m[9] += w * pz * pz;
+    bool some = false;
+    const long long units = (long long)c.segs * c.zparts;
+    const long long stride = (long long)gridDim.x * (kRedThreads / 32);
+    for (long long u = (long long)blockIdx.x * (kRedThreads / 32) + warp; u < units; u += stride) {
+        const int zp = (int)(u / c.segs), p = (int)(u - (long long)zp * c.segs) * 32 + lane;
+        const bool on = p < L.Lx * L.Ly;
+        const int y = on ? p / L.Lx : 0, x = on ? p - y * L.Lx : 0;
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+        bool drop = false;
+        const int z1 = min((zp + 1) * c.zlen, L.Lz);
+        for (int z = zp * c.zlen; z < z1; ++z) {
+            if (!on) continue;
+            const RhoPair<S> r = node_rho_pair(f, L, x, y, z);
+            if (!r.droplet()) continue;
+            const double ra = r.a(), rb = r.b();
+            const double phi = (ra - rb) / (ra + rb);
+            if (phi > 0.0) {
+                const double pz = z - cz, wz = phi * pz;
+                s0 += phi;
+                s1 += wz;
+                s2 = fma(wz, pz, s2);
+                drop = true;
+            }
+        }
+        if (__any_sync(0xffffffffu, drop)) {
+            const double px = x - cx, py = y - cy, sx = s0 * px, sy = s0 * py;
+            m[0] += s0;
+            m[1] += sx; m[2] += sy; m[3] += s1;
+            m[4] = fma(sx, px, m[4]); m[5] = fma(sx, py, m[5]); m[6] = fma(s1, px, m[6]);
+            m[7] = fma(sy, py, m[7]); m[8] = fma(s1, py, m[8]); m[9] += s2;
+            some = true;
+        }
     }
-    block_sum<10>(m, partials + 10LL * blockIdx.x);
+    if (some) {
+#pragma unroll
+        for (int k = 0; k < 10; ++k) {
+            double a = m[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+            if (lane == 0) part[warp][k] = a;
+        }
+    } else if (lane < 10) {
+        part[warp][lane] = 0.0;
+    }
+    const int any = __syncthreads_or(some);
+    if (threadIdx.x < 10) {
+        double a = part[0][threadIdx.x];
+        if (any)
+            for (int w = 1; w < kRedThreads / 32; ++w) a += part[w][threadIdx.x];
+        partials[10LL * blockIdx.x + threadIdx.x] = a;
+    }
 }
 
-// Sum the per-block partials in block order, then derive D and the axes.
-__global__ void k_moments_final(const double* __restrict__ partials, int nblocks, double* __restrict__ result) {
-    const int lane = threadIdx.x;  // 32 threads
+// Sum the per-block partials in a fixed order (warp k sums moment k), then
+// derive D and the axes (one thread).
+constexpr int kMomentsFinalThreads = 320;
+__global__ void __launch_bounds__(kMomentsFinalThreads) k_moments_final(const double* __restrict__ partials,
+                                                                        int nblocks, double* __restrict__ result) {
+    __shared__ double sum[10];
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    double a = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < nblocks; b += 32) a += partials[10LL * b + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if (lane == 0) sum[k] = a;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     double m[10];
 #pragma unroll
-    for (int k = 0; k < 10; ++k) {
-        double a = 0.0;
-        for (int b = lane; b < nblocks; b += 32) a += partials[10LL * b + k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        m[k] = a;
-    }
-    if (lane != 0) return;
+    for (int q = 0; q < 10; ++q) m[q] = sum[q];
     deformation_from_moments(m, result);
 }
 
@@ -213,7 +319,9 @@ __global__ void k_fields(const S* __restrict__ f, Layout L, DevRef dr, double* _
         for (int i = 0; i < 19; ++i) {
             const double v = population(f, L, dr, s, i, x, y, z);
             r[s] += v;
-            j[0] += qx(i) * v; j[1] += qy(i) * v; j[2] += qz(i) * v;
+            if (qx(i)) j[0] += qx(i) * v;
+            if (qy(i)) j[1] += qy(i) * v;
+            if (qz(i)) j[2] += qz(i) * v;
         }
     if (ra_out) ra_out[n] = r[0];
     if (rb_out) rb_out[n] = r[1];
@@ -238,7 +346,9 @@ __global__ void __launch_bounds__(kRedThreads) k_checksums(const S* __restrict__
             for (int i = 0; i < 19; ++i) {
                 const double q = population(f, L, dr, s, i, x, y, z);
                 v[s] += q;
-                v[2] += qx(i) * q; v[3] += qy(i) * q; v[4] += qz(i) * q;
+                if (qx(i)) v[2] += qx(i) * q;
+                if (qy(i)) v[3] += qy(i) * q;
+                if (qz(i)) v[4] += qz(i) * q;
             }
     }
     block_sum<5>(v, partials + 5LL * blockIdx.x);
@@ -328,75 +438,132 @@ __global__ void k_unpack(S* __restrict__ f, Layout L, const double* __restrict__
 
 // ---- connected components of the droplet phase (breakup detection) ----
 
-// label[n] = n where phi > threshold (phi = (rho_A - rho_B) / (rho_A + rho_B)), -1 elsewhere;
-// n = (z Ly + y) Lx + x.
+// The labels are a union-find forest in memory: label[n] <= n is the parent
+// of node n (itself for a root), -1 outside the phase, and roots end as the
+// smallest node index of their component.  Three launches, whatever the
+// components' shapes, and no host round trip between them; the sweeps of
+// minimum-label propagation that this replaced were launched four at a time
+// with a read-back after each four.
+
+// label[n] = the start of the run of phase nodes along x that n belongs to
+// (within the 32 nodes of its warp), -1 where phi <= threshold; n = (z Ly + y)
+// Lx + x.  Also zeroes the sizes and the root counter.
 template <typename S>
-__global__ void k_cc_init(const S* __restrict__ f, Layout L, double threshold, int* __restrict__ label) {
+__global__ void k_cc_init(const S* __restrict__ f, Layout L, double threshold, int* __restrict__ label,
+                          int* __restrict__ size, int* __restrict__ flags) {
     const long long N = (long long)L.Lx * L.Ly * L.Lz;
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const int x = (int)(n % L.Lx), y = (int)((n / L.Lx) % L.Ly), z = (int)(n / ((long long)L.Lx * L.Ly));
-    double ra, rb;
-    node_rho(f, L, x, y, z, ra, rb);
-    label[n] = (ra - rb) / (ra + rb) > threshold ? (int)n : -1;
-}
-
-// One sweep of minimum-label propagation over the 6 face neighbours (wrapping
-// in the periodic mode), with pointer jumping; sets *changed when a label
-// decreased.  Labels only decrease and stay labels of the same component, so
-// repeated sweeps converge to the smallest index of each component.
-__global__ void k_cc_sweep(Layout L, int periodic, int* __restrict__ label, int* __restrict__ changed) {
-    const long long N = (long long)L.Lx * L.Ly * L.Lz;
-    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const int own = label[n];
-    if (own < 0) return;
-    const int x = (int)(n % L.Lx), y = (int)((n / L.Lx) % L.Ly), z = (int)(n / ((long long)L.Lx * L.Ly));
-    int m = own;
-    const int dx[6] = {1, -1, 0, 0, 0, 0}, dy[6] = {0, 0, 1, -1, 0, 0}, dz[6] = {0, 0, 0, 0, 1, -1};
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        int xn = x + dx[q], yn = y + dy[q], zn = z + dz[q];
-        if (periodic) {
-            xn = (xn + L.Lx) % L.Lx; yn = (yn + L.Ly) % L.Ly; zn = (zn + L.Lz) % L.Lz;
-        } else if (xn < 0 || xn >= L.Lx || yn < 0 || yn >= L.Ly || zn < 0 || zn >= L.Lz) {
-            continue;
+    if (n < 2) flags[n] = 0;
+    bool in = false;
+    int x = 0;
+    if (n < N) {
+        const int row = (int)n / L.Lx, y = row % L.Ly, z = row / L.Ly;
+        x = (int)n - row * L.Lx;
+        const RhoPair<S> r = node_rho_pair(f, L, x, y, z);
+        // phi > threshold >= 0 needs phi > 0: no FP64 outside the droplet
+        if (threshold < 0.0 || r.droplet()) {
+            const double ra = r.a(), rb = r.b();
+            in = (ra - rb) / (ra + rb) > threshold;
         }
-        const int v = label[((long long)zn * L.Ly + yn) * L.Lx + xn];
-        if (v >= 0 && v < m) m = v;
     }
-    const int jump = label[m];  // the label of the smallest label seen (pointer jumping)
-    if (jump >= 0 && jump < m) m = jump;
-    if (m < own) {
-        label[n] = m;
-        *changed = 1;
+    const int lane = threadIdx.x & 31;
+    const unsigned ins = __ballot_sync(0xffffffffu, in);
+    const bool first = in && (lane == 0 || x == 0 || !((ins >> (lane - 1)) & 1u));
+    const unsigned starts = __ballot_sync(0xffffffffu, first);
+    if (n >= N) return;
+    const int start = 31 - __clz((int)(starts & (0xffffffffu >> (31 - lane))));
+    label[n] = in ? (int)n - (lane - start) : -1;
+    size[n] = 0;
+}
+
+// Root of node a's tree.  Parents are smaller than their children, so the
+// walk ends; `steps` bounds it all the same.
+__device__ __forceinline__ int cc_find(const int* label, int a, long long& steps) {
+    int p = __ldcg(label + a);
+    while (p != a && --steps > 0) {
+        a = p;
+        p = __ldcg(label + a);
+    }
+    return a;
+}
+
+// Join the trees of nodes a and b: the larger root's parent becomes the
+// smaller root.  A root that another thread has attached meanwhile yields its
+// new parent, which is joined instead (parents only decrease).
+__device__ __forceinline__ void cc_join(int* label, int a, int b, long long& steps) {
+    while (steps > 0) {
+        a = cc_find(label, a, steps);
+        b = cc_find(label, b, steps);
+        if (a == b) return;
+        const int hi = a > b ? a : b, lo = a > b ? b : a;
+        const int old = atomicMin(label + hi, lo);
+        if (old == hi) return;
+        a = old;
+        b = lo;
+        --steps;
     }
 }
 
-// Component sizes: size[label[n]] += 1; then roots (label[n] == n) append
-// (root, size) to out with an atomic counter.
-__global__ void k_cc_sizes(Layout L, const int* __restrict__ label, int* __restrict__ size) {
+// Joins every phase node with its phase neighbours at x + 1 (where the runs
+// of k_cc_init end), y + 1 and z + 1, wrapping in the periodic mode.  A y or z
+// edge is left out where the nodes at x - 1 have one too (both pairs are
+// joined along x).  flags[0] is set if a walk exceeded its bound.
+__global__ void k_cc_join(Layout L, int periodic, int* __restrict__ label, int* __restrict__ flags) {
     const long long N = (long long)L.Lx * L.Ly * L.Lz;
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const int v = label[n];
-    if (v >= 0) atomicAdd(size + v, 1);
+    if (n >= N || __ldcg(label + n) < 0) return;
+    const int row = (int)n / L.Lx, y = row % L.Ly, z = row / L.Ly, x = (int)n - row * L.Lx;
+    long long steps = 64 * (N + 8);
+    const bool left = x > 0 && __ldcg(label + n - 1) >= 0;
+    auto edge = [&](long long nb, bool skippable) {
+        if (__ldcg(label + nb) < 0) return;
+        if (skippable && left && __ldcg(label + nb - 1) >= 0) return;
+        cc_join(label, (int)n, (int)nb, steps);
+    };
+    const long long sy = L.Lx, sz = (long long)L.Lx * L.Ly;
+    if (x + 1 < L.Lx) {
+        if ((n & 31) == 31) edge(n + 1, false);
+    } else if (periodic) {
+        edge(n - x, false);
+    }
+    if (y + 1 < L.Ly) edge(n + sy, true);
+    else if (periodic) edge(n - (long long)y * sy, true);
+    if (z + 1 < L.Lz) edge(n + sz, true);
+    else if (periodic) edge(n - (long long)z * sz, true);
+    if (steps <= 0) flags[0] = 1;
 }
 
+// Component sizes: size[root] += 1 for every phase node, one atomic per
+// distinct root of a warp.
+__global__ void k_cc_sizes(Layout L, const int* __restrict__ label, int* __restrict__ size, int* __restrict__ flags) {
+    const long long N = (long long)L.Lx * L.Ly * L.Lz;
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = n < N && label[n] >= 0;
+    const unsigned mask = __ballot_sync(0xffffffffu, in);
+    if (!in) return;
+    long long steps = N + 8;
+    const int root = cc_find(label, (int)n, steps);
+    if (steps <= 0) flags[0] = 1;
+    const unsigned same = __match_any_sync(mask, root);
+    if ((int)(threadIdx.x & 31) == __ffs((int)same) - 1) atomicAdd(size + root, __popc(same));
+}
+
+// The roots' sizes, in no particular order; flags[1] counts them.
 __global__ void k_cc_roots(Layout L, const int* __restrict__ label, const int* __restrict__ size,
-                           int* __restrict__ count, long long* __restrict__ out, int cap) {
+                           int* __restrict__ flags, long long* __restrict__ out, int cap) {
     const long long N = (long long)L.Lx * L.Ly * L.Lz;
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= N) return;
     if (label[n] != (int)n) return;
-    const int k = atomicAdd(count, 1);
+    const int k = atomicAdd(flags + 1, 1);
     if (k < cap) out[k] = size[n];
 }
 
 // ---- surface-area deformation (Eq. 17) and mass reinjection ----
 
 // phi of every fluid node into phi[n] (n = (z Ly + y) Lx + x) and per-block
-// {sum phi, min phi, max phi}.
+// {sum phi, min phi, max phi}.  Bound by the FP64 pipe after the float32
+// density sums: the quotient is div64.
 template <typename S>
 __global__ void __launch_bounds__(kRedThreads) k_phi(const S* __restrict__ f, Layout L, double* __restrict__ phi,
                                                      double* __restrict__ partials) {
@@ -404,10 +571,10 @@ __global__ void __launch_bounds__(kRedThreads) k_phi(const S* __restrict__ f, La
     const long long N = (long long)L.Lx * L.Ly * L.Lz;
     double sum = 0.0, lo = 1e300, hi = -1e300;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % L.Lx), y = (int)((n / L.Lx) % L.Ly), z = (int)(n / ((long long)L.Lx * L.Ly));
+        const int row = (int)(n / L.Lx), y = row % L.Ly, z = row / L.Ly, x = (int)(n - (long long)row * L.Lx);
         double ra, rb;
         node_rho(f, L, x, y, z, ra, rb);
-        const double p = (ra - rb) / (ra + rb);
+        const double p = div64(ra - rb, ra + rb);
         phi[n] = p;
         sum += p;
         lo = fmin(lo, p);
@@ -432,37 +599,74 @@ __global__ void __launch_bounds__(kRedThreads) k_phi(const S* __restrict__ f, La
     }
 }
 
-// Per-block sum of |grad phi| (central differences) over interior nodes into partials[4 b + 3].
-__global__ void __launch_bounds__(kRedThreads) k_grad_phi(Layout L, const double* __restrict__ phi,
+// sqrt(s) to float64 rounding or one unit more, from a float32 reciprocal
+// square root (6 FP64 instructions instead of about 20).
+__device__ __forceinline__ double sqrt64(double s) {
+    const float sf = (float)s;
+    if (!(sf > 1e-30f && sf < 1e30f)) return sqrt(s);
+    const float yf = rsqrtf(sf);
+    const double h = (double)(0.5f * yf);
+    double r = s * (double)yf;
+    r = fma(fma(-r, r, s), h, r);
+    return fma(fma(-r, r, s), h, r);
+}
+
+// Per-block sum of |grad phi| (central differences) over interior nodes into
+// partials[4 b + 3]; a lane marches in z (Columns) and keeps the two planes
+// beside it in registers.
+__global__ void __launch_bounds__(kRedThreads) k_grad_phi(Layout L, Columns c, const double* __restrict__ phi,
                                                           double* __restrict__ partials) {
     double v[1] = {0.0};
-    const long long N = (long long)L.Lx * L.Ly * L.Lz;
-    const long long sx = 1, sy = L.Lx, sz = (long long)L.Lx * L.Ly;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % L.Lx), y = (int)((n / L.Lx) % L.Ly), z = (int)(n / ((long long)L.Lx * L.Ly));
-        if (x < 1 || x > L.Lx - 2 || y < 1 || y > L.Ly - 2 || z < 1 || z > L.Lz - 2) continue;
-        const double gx = 0.5 * (phi[n + sx] - phi[n - sx]);
-        const double gy = 0.5 * (phi[n + sy] - phi[n - sy]);
-        const double gz = 0.5 * (phi[n + sz] - phi[n - sz]);
-        v[0] += sqrt(gx * gx + gy * gy + gz * gz);
+    const long long sy = L.Lx, sz = (long long)L.Lx * L.Ly;
+    const long long units = (long long)c.segs * c.zparts;
+    const long long stride = (long long)gridDim.x * (kRedThreads / 32);
+    for (long long u = (long long)blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5); u < units; u += stride) {
+        const int zp = (int)(u / c.segs), p = (int)(u - (long long)zp * c.segs) * 32 + (threadIdx.x & 31);
+        const int y = p / L.Lx, x = p - y * L.Lx;
+        if (x < 1 || x > L.Lx - 2 || y < 1 || y > L.Ly - 2) continue;
+        const int z0 = max(zp * c.zlen, 1), z1 = min((zp + 1) * c.zlen, L.Lz - 1);
+        if (z0 >= z1) continue;
+        const double* q = phi + (long long)z0 * sz + p;
+        double below = q[-sz], here = q[0];
+        for (int z = z0; z < z1; ++z, q += sz) {
+            const double above = q[sz];
+            const double gx = q[1] - q[-1], gy = q[sy] - q[-sy], gz = above - below;
+            v[0] += sqrt64(fma(gx, gx, fma(gy, gy, gz * gz)));
+            below = here;
+            here = above;
+        }
     }
+    v[0] *= 0.5;
     double out[1];
     block_sum<1>(v, out);
     if (threadIdx.x == 0) partials[4LL * blockIdx.x + 3] = out[0];
 }
 
-// Block order reduction of the partials: {sum phi, min, max, sum |grad phi|}.
-__global__ void k_phi_final(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Reduction of the partials in a fixed order: {sum phi, min, max, sum |grad phi|}.
+__global__ void __launch_bounds__(kRedThreads) k_phi_final(const double* __restrict__ partials, int nblocks,
+                                                           double* __restrict__ out) {
+    __shared__ double red[4][kRedThreads];
     double sum = 0.0, lo = 1e300, hi = -1e300, g = 0.0;
-    for (int b = 0; b < nblocks; ++b) {
+    for (int b = threadIdx.x; b < nblocks; b += kRedThreads) {
         const double* p = partials + 4LL * b;
         sum += p[0];
         lo = fmin(lo, p[1]);
         hi = fmax(hi, p[2]);
         g += p[3];
     }
-    out[0] = sum; out[1] = lo; out[2] = hi; out[3] = g;
+    const int t = threadIdx.x;
+    red[0][t] = sum; red[1][t] = lo; red[2][t] = hi; red[3][t] = g;
+    for (int h = kRedThreads / 2; h > 0; h >>= 1) {
+        __syncthreads();
+        if (t < h) {
+            red[0][t] += red[0][t + h];
+            red[1][t] = fmin(red[1][t], red[1][t + h]);
+            red[2][t] = fmax(red[2][t], red[2][t + h]);
+            red[3][t] += red[3][t + h];
+        }
+    }
+    if (t == 0)
+        for (int q = 0; q < 4; ++q) out[q] = red[q][0];
 }
 
 // Per-block {mass of A where phi > 0, mass of A elsewhere}.
@@ -480,11 +684,14 @@ __global__ void __launch_bounds__(kRedThreads) k_mass_split(const S* __restrict_
     block_sum<2>(v, partials + 2LL * blockIdx.x);
 }
 
-__global__ void k_mass_final(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double a = 0.0, b = 0.0;
-    for (int k = 0; k < nblocks; ++k) { a += partials[2LL * k]; b += partials[2LL * k + 1]; }
-    out[0] = a; out[1] = b;
+__global__ void __launch_bounds__(kRedThreads) k_mass_final(const double* __restrict__ partials, int nblocks,
+                                                            double* __restrict__ out) {
+    double v[2] = {0.0, 0.0};
+    for (int k = threadIdx.x; k < nblocks; k += kRedThreads) {
+        v[0] += partials[2LL * k];
+        v[1] += partials[2LL * k + 1];
+    }
+    block_sum<2>(v, out);
 }
 
 // f_A,i *= k at the nodes where phi > 0 (phi of the populations before scaling).
@@ -515,11 +722,13 @@ int moments_blocks(const Layout& L, int num_sms) {
 
 cudaError_t launch_moments(int prec, const void* f, const Layout& L, double* partials, int nblocks, double* result,
                            cudaStream_t s) {
-    if (prec == kFP64) k_moments<double><<<nblocks, kRedThreads, 0, s>>>((const double*)f, L, partials);
-    else if (prec == kFP32) k_moments<float><<<nblocks, kRedThreads, 0, s>>>((const float*)f, L, partials);
-    else if (prec == kFP16Dev) k_moments<Dev<__half>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__half>*)f, L, partials);
-    else k_moments<Dev<__nv_bfloat16>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__nv_bfloat16>*)f, L, partials);
-    k_moments_final<<<1, 32, 0, s>>>(partials, nblocks, result);
+    const Columns c = columns(L, (long long)nblocks * (kRedThreads / 32));
+    if (prec == kFP64) k_moments<double><<<nblocks, kRedThreads, 0, s>>>((const double*)f, L, c, partials);
+    else if (prec == kFP32) k_moments<float><<<nblocks, kRedThreads, 0, s>>>((const float*)f, L, c, partials);
+    else if (prec == kFP16Dev)
+        k_moments<Dev<__half>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__half>*)f, L, c, partials);
+    else k_moments<Dev<__nv_bfloat16>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__nv_bfloat16>*)f, L, c, partials);
+    k_moments_final<<<1, kMomentsFinalThreads, 0, s>>>(partials, nblocks, result);
     return cudaGetLastError();
 }
 
@@ -581,28 +790,20 @@ cudaError_t launch_unpack(int prec, void* f, const Layout& L, const Model& m, co
 
 namespace lbmgb {
 
-cudaError_t launch_cc_init(int prec, const void* f, const Layout& L, double threshold, int* label, cudaStream_t s) {
+cudaError_t launch_cc(int prec, const void* f, const Layout& L, int periodic, double threshold, int* label, int* size,
+                      int* flags, long long* out, int cap, cudaStream_t s) {
     const long long N = (long long)L.Lx * L.Ly * L.Lz;
     const unsigned blocks = (unsigned)((N + 255) / 256);
-    if (prec == kFP64) k_cc_init<double><<<blocks, 256, 0, s>>>((const double*)f, L, threshold, label);
-    else if (prec == kFP32) k_cc_init<float><<<blocks, 256, 0, s>>>((const float*)f, L, threshold, label);
-    else if (prec == kFP16Dev) k_cc_init<Dev<__half>><<<blocks, 256, 0, s>>>((const Dev<__half>*)f, L, threshold, label);
-    else k_cc_init<Dev<__nv_bfloat16>><<<blocks, 256, 0, s>>>((const Dev<__nv_bfloat16>*)f, L, threshold, label);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cc_sweep(const Layout& L, int periodic, int* label, int* changed, cudaStream_t s) {
-    const long long N = (long long)L.Lx * L.Ly * L.Lz;
-    k_cc_sweep<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(L, periodic, label, changed);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cc_sizes(const Layout& L, const int* label, int* size, int* count, long long* out, int cap,
-                            cudaStream_t s) {
-    const long long N = (long long)L.Lx * L.Ly * L.Lz;
-    const unsigned blocks = (unsigned)((N + 255) / 256);
-    k_cc_sizes<<<blocks, 256, 0, s>>>(L, label, size);
-    k_cc_roots<<<blocks, 256, 0, s>>>(L, label, size, count, out, cap);
+    if (prec == kFP64) k_cc_init<double><<<blocks, 256, 0, s>>>((const double*)f, L, threshold, label, size, flags);
+    else if (prec == kFP32) k_cc_init<float><<<blocks, 256, 0, s>>>((const float*)f, L, threshold, label, size, flags);
+    else if (prec == kFP16Dev)
+        k_cc_init<Dev<__half>><<<blocks, 256, 0, s>>>((const Dev<__half>*)f, L, threshold, label, size, flags);
+    else
+        k_cc_init<Dev<__nv_bfloat16>>
+            <<<blocks, 256, 0, s>>>((const Dev<__nv_bfloat16>*)f, L, threshold, label, size, flags);
+    k_cc_join<<<blocks, 256, 0, s>>>(L, periodic, label, flags);
+    k_cc_sizes<<<blocks, 256, 0, s>>>(L, label, size, flags);
+    k_cc_roots<<<blocks, 256, 0, s>>>(L, label, size, flags, out, cap);
     return cudaGetLastError();
 }
 
@@ -618,8 +819,9 @@ cudaError_t launch_surface_stats(int prec, const void* f, const Layout& L, doubl
     else if (prec == kFP32) k_phi<float><<<nblocks, kRedThreads, 0, s>>>((const float*)f, L, phi, partials);
     else if (prec == kFP16Dev) k_phi<Dev<__half>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__half>*)f, L, phi, partials);
     else k_phi<Dev<__nv_bfloat16>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__nv_bfloat16>*)f, L, phi, partials);
-    k_grad_phi<<<nblocks, kRedThreads, 0, s>>>(L, phi, partials);
-    k_phi_final<<<1, 32, 0, s>>>(partials, nblocks, out);
+    const Columns c = columns(L, (long long)nblocks * (kRedThreads / 32));
+    k_grad_phi<<<nblocks, kRedThreads, 0, s>>>(L, c, phi, partials);
+    k_phi_final<<<1, kRedThreads, 0, s>>>(partials, nblocks, out);
     return cudaGetLastError();
 }
 
@@ -629,7 +831,7 @@ cudaError_t launch_mass_split(int prec, const void* f, const Layout& L, double* 
     if (prec == kFP64) k_mass_split<double><<<nblocks, kRedThreads, 0, s>>>((const double*)f, L, partials);
     else if (prec == kFP32) k_mass_split<float><<<nblocks, kRedThreads, 0, s>>>((const float*)f, L, partials);
     else return cudaErrorInvalidValue;
-    k_mass_final<<<1, 32, 0, s>>>(partials, nblocks, out);
+    k_mass_final<<<1, kRedThreads, 0, s>>>(partials, nblocks, out);
     return cudaGetLastError();
 }
 
