@@ -848,21 +848,44 @@ __device__ __forceinline__ void collide_node(const float2* rzm, const float2* rz
             if constexpr (MRT) {
                 // MRT: relax the moments of the deviation from equilibrium
                 // (d'Humieres basis; momentum and stress at 1/tau)
-                const float u2x = 1.5f * (ux * ux + uy * uy + uz * uz);
-                float dv[19], o[19];
-#pragma unroll
-                for (int i = 0; i < 19; ++i) dv[i] = f[s][i] - feq<float>(i, r, ux, uy, uz, u2x);
-                mrt_relax<float>(f[s], dv, m.inv_tau[s], m.mrt, o);
+                // as BGK plus the free moments' part (mrt_free); the
+                // equilibria are evaluated twice rather than held
+                const float base = 1.f - 1.5f * (ux * ux + uy * uy + uz * uz);
+                const float e1 = r * wgt<float>(1), e2 = r * wgt<float>(7), it = m.inv_tau[s];
+                float g[7] = {f[s][0] - (r * wgt<float>(0)) * base, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                float o[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                auto deviations = [&](auto I, float& dp, float& dm) {
+                    constexpr int i = decltype(I)::value;
+                    const float cu = (float)cx_(i) * ux + (float)cy_(i) * uy + (float)cz_(i) * uz;
+                    const float e = i < 7 ? e1 : e2;
+                    const float ev = e * fmaf(4.5f * cu, cu, base);
+                    const float od = (3.f * e) * cu;
+                    dp = f[s][i] - (ev + od);
+                    dm = f[s][i + 1] - (ev - od);
+                };
                 sfor<9>([&](auto K) {
                     constexpr int i = 2 * decltype(K)::value + 1;
+                    float dp, dm;
+                    deviations(std::integral_constant<int, i>{}, dp, dm);
+                    mrt_gather<float>(i, dp, dm, g, o);
+                });
+                float ce[7], co[9];
+                mrt_free<float>(g, o, it, m.mrt, ce, co);
+                sfor<9>([&](auto K) {
+                    constexpr int i = 2 * decltype(K)::value + 1;
+                    float dp, dm;
+                    deviations(std::integral_constant<int, i>{}, dp, dm);
+                    const float e = ce[mrt_group(i)], d = mrt_odd<float>(i, co);
+                    const float oa = fmaf(-it, dp, f[s][i]) - (e + d);
+                    const float ob = fmaf(-it, dm, f[s][i + 1]) - (e - d);
                     if (s == 0) {
-                        IO::template store<0, i>(out, o[i]);
-                        IO::template store<0, i + 1>(out, o[i + 1]);
+                        IO::template store<0, i>(out, oa);
+                        IO::template store<0, i + 1>(out, ob);
                     } else {
-                        IO::template store<1, i>(out, o[i]);
-                        IO::template store<1, i + 1>(out, o[i + 1]);
+                        IO::template store<1, i>(out, oa);
+                        IO::template store<1, i + 1>(out, ob);
                     }
-                    others += o[i] + o[i + 1];
+                    others += oa + ob;
                 });
             } else {
                 const float base = 1.f - 1.5f * (ux * ux + uy * uy + uz * uz);
@@ -1644,9 +1667,12 @@ cudaError_t ws_for(bool query, const void* src, void* dst, const Layout& L, cons
 template <int TX, typename S>
 cudaError_t rows_variant(int variant, bool query, const void* src, void* dst, const Layout& L, const Model& m,
                          int zchunk, CentreParts cp, int* d_err, cudaStream_t s, int* resident) {
-    if (m.mrt) {  // MRT: float32 storage, direct loads only
-        if constexpr (std::is_same<S, float>::value)
+    if (m.mrt) {  // MRT: float32 storage, direct or staged
+        if constexpr (std::is_same<S, float>::value) {
+            if (variant == kRowStaged)
+                return rows_for<TX, S, true, true>(query, src, dst, L, m, zchunk, cp, d_err, s, resident);
             return rows_for<TX, S, false, true>(query, src, dst, L, m, zchunk, cp, d_err, s, resident);
+        }
         return cudaErrorInvalidValue;
     }
     if (variant == kRowWs) return ws_for<TX, kRowCluster, S>(query, src, dst, L, m, zchunk, cp, d_err, s, resident);
