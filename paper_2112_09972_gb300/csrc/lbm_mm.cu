@@ -29,111 +29,151 @@ struct Sym {
     C v[6];
 };
 
-template <typename C>
-__device__ __forceinline__ C at(const Sym<C>& m, int a, int b) {
-    constexpr int idx[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
-    return m.v[idx[a][b]];
+// n / d (d > 0) to the rounding of C or one unit more: an approximate float32
+// reciprocal refined in C (4 to 6 instructions instead of a divide's dozen,
+// which in float64 all run on the FP64 pipe); the plain divide outside
+// float32's range.
+__device__ __forceinline__ float quotient(float n, float d) {
+    if (!(d > 1e-30f && d < 1e30f)) return n / d;
+    const float y = __fdividef(1.f, d);
+    const float q = n * y;
+    return fmaf(fmaf(-q, d, n), y, q);
+}
+__device__ __forceinline__ double quotient(double n, double d) {
+    const float df = (float)d;
+    if (!(df > 1e-30f && df < 1e30f)) return n / d;
+    const double y = (double)__fdividef(1.f, df);
+    double q = n * y;
+    q = fma(fma(-q, d, n), y, q);
+    return fma(fma(-q, d, n), y, q);
 }
 
+// The flow part of the model at one time: B = f2(Ca) S + W, row-major, so
+// that f2 (S M + M S) + W M - M W = B M + (B M)^T (S symmetric, W
+// antisymmetric).
 template <typename C>
-__device__ __forceinline__ Sym<C> rhs(const Sym<C>& M, const C (&A)[9], C tau_d, C chi) {
-    C S[3][3], W[3][3], amax = C(0);
+struct Flow {
+    C b[9];
+};
+template <typename C>
+__device__ __forceinline__ Flow<C> flow_at(const C (&a0)[9], const C (&d)[9], C t, C tau_d, C f2_0) {
+    C A[9], amax = C(0);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+        A[j] = fma(t, d[j], a0[j]);
+        amax = fmax(amax, fabs(A[j]));
+    }
+    const C Ca = tau_d * amax, c2 = Ca * Ca;
+    const C f2 = f2_0 + quotient(C(3) * c2, fma(C(6), c2, C(2)));
+    const C p = C(0.5) * (f2 + C(1)), m = C(0.5) * (f2 - C(1));
+    Flow<C> F;
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            S[a][b] = C(0.5) * (A[3 * a + b] + A[3 * b + a]);
-            W[a][b] = C(0.5) * (A[3 * a + b] - A[3 * b + a]);
-            amax = fmax(amax, fabs(A[3 * a + b]));
-        }
-    const C Ca = tau_d * amax;
-    const C f1 = C(40) * (chi + C(1)) / ((C(3) + C(2) * chi) * (C(16) + C(19) * chi));
-    const C f2 = C(5) / (C(3) + C(2) * chi) + C(3) * Ca * Ca / (C(2) + C(6) * Ca * Ca);
-    // invariants
-    const C tr = M.v[0] + M.v[3] + M.v[5];
-    const C mm = M.v[0] * M.v[0] + M.v[3] * M.v[3] + M.v[5] * M.v[5] +
-                 C(2) * (M.v[1] * M.v[1] + M.v[2] * M.v[2] + M.v[4] * M.v[4]);
-    const C II = C(0.5) * (tr * tr - mm);
-    const C III = M.v[0] * (M.v[3] * M.v[5] - M.v[4] * M.v[4]) - M.v[1] * (M.v[1] * M.v[5] - M.v[4] * M.v[2]) +
-                  M.v[2] * (M.v[1] * M.v[4] - M.v[3] * M.v[2]);
-    const C iso = C(3) * III / II;
-    Sym<C> out;
-    constexpr int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-#pragma unroll
-    for (int e = 0; e < 6; ++e) {
-        const int a = ia[e], b = ib[e];
-        C sm = C(0), ms = C(0), wm = C(0), mw = C(0);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            sm += S[a][k] * at(M, k, b);
-            ms += at(M, a, k) * S[k][b];
-            wm += W[a][k] * at(M, k, b);
-            mw += at(M, a, k) * W[k][b];
-        }
-        const C flow = f2 * tau_d * (sm + ms) + tau_d * (wm - mw);
-        const C relax = f1 * (M.v[e] - (a == b ? iso : C(0)));
-        out.v[e] = (flow - relax) / tau_d;
-    }
-    return out;
+        for (int b = 0; b < 3; ++b)
+            F.b[3 * a + b] = a == b ? f2 * A[4 * a] : fma(p, A[3 * a + b], m * A[3 * b + a]);
+    return F;
+}
+
+// dM/dt = B M + (B M)^T - k (M - 3 III / II I), k = f1 / tau_d.
+template <typename C>
+__device__ __forceinline__ Sym<C> rhs(const Sym<C>& M, const Flow<C>& F, C k) {
+    const C* m = M.v;
+    const C* b = F.b;
+    // cofactors: II is their trace, III the expansion along the first row
+    const C c0 = fma(m[3], m[5], -m[4] * m[4]), c1 = fma(m[0], m[5], -m[2] * m[2]), c2 = fma(m[0], m[3], -m[1] * m[1]);
+    const C u = fma(m[1], m[5], -m[4] * m[2]), v = fma(m[1], m[4], -m[3] * m[2]);
+    const C III = fma(m[0], c0, fma(m[2], v, -m[1] * u));
+    const C iso = k * quotient(C(3) * III, c0 + c1 + c2);
+    Sym<C> r;
+    r.v[0] = fma(C(2), fma(b[0], m[0], fma(b[1], m[1], b[2] * m[2])), fma(-k, m[0], iso));
+    r.v[3] = fma(C(2), fma(b[3], m[1], fma(b[4], m[3], b[5] * m[4])), fma(-k, m[3], iso));
+    r.v[5] = fma(C(2), fma(b[6], m[2], fma(b[7], m[4], b[8] * m[5])), fma(-k, m[5], iso));
+    // (B M)_ab + (B M)_ba
+    r.v[1] = fma(b[0], m[1], fma(b[1], m[3], b[2] * m[4])) + fma(b[3], m[0], fma(b[4], m[1], fma(b[5], m[2], -k * m[1])));
+    r.v[2] = fma(b[0], m[2], fma(b[1], m[4], b[2] * m[5])) + fma(b[6], m[0], fma(b[7], m[1], fma(b[8], m[2], -k * m[2])));
+    r.v[4] = fma(b[3], m[2], fma(b[4], m[4], b[5] * m[5])) + fma(b[6], m[1], fma(b[7], m[3], fma(b[8], m[4], -k * m[4])));
+    return r;
 }
 
 template <typename C>
 __device__ __forceinline__ Sym<C> axpy(const Sym<C>& m, C h, const Sym<C>& k) {
     Sym<C> r;
 #pragma unroll
-    for (int e = 0; e < 6; ++e) r.v[e] = m.v[e] + h * k.v[e];
+    for (int e = 0; e < 6; ++e) r.v[e] = fma(h, k.v[e], m.v[e]);
     return r;
 }
 
 template <typename C>
-__device__ double deformation(const Sym<C>& M) {
-    double a[3][3] = {{(double)M.v[0], (double)M.v[1], (double)M.v[2]},
-                      {(double)M.v[1], (double)M.v[3], (double)M.v[4]},
-                      {(double)M.v[2], (double)M.v[4], (double)M.v[5]}};
-    double lam[3], v[3][3];
-    lbmgb::jacobi3(a, lam, v);
-    const double hi = sqrt(fmax(fmax(lam[0], fmax(lam[1], lam[2])), 0.0));
-    const double lo = sqrt(fmax(fmin(lam[0], fmin(lam[1], lam[2])), 0.0));
-    return hi + lo > 0.0 ? (hi - lo) / (hi + lo) : 0.0;
+__device__ __forceinline__ double deformation(const Sym<C>& M) {
+    const double m[6] = {(double)M.v[0], (double)M.v[1], (double)M.v[2],
+                         (double)M.v[3], (double)M.v[4], (double)M.v[5]};
+    return lbmgb::deformation_of(m);
 }
 
+// One warp per CTA, so that few trajectories still spread over the SMs: the
+// float64 form is bound by the FP64 pipe (one warp instruction per 16 cycles
+// and SM), the float32 form by its dependent chain at about one warp per
+// scheduler.  A stage is one B M product (27 multiply-adds), the cofactors
+// and one quotient; B is formed once per time it is needed at (the middle
+// serves two stages, the end is the next substep's start), and the next row
+// of A is loaded a step ahead.  Measured on GB300, 16384 trajectories: see
+// lbm_mm_integrate.
+constexpr int kMMThreads = 32;
 template <typename C>
-__global__ void k_mm_rk4(const double* __restrict__ A, long long T, long long n, C tau_d, C chi, int substeps,
-                         int record_every, double* __restrict__ D, double* __restrict__ Mout) {
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kMMThreads) k_mm_rk4(const double* __restrict__ A, long long T, long long n, C tau_d,
+                                                       C f2_0, C kf, int substeps, int record_every,
+                                                       double* __restrict__ D, double* __restrict__ Mout) {
+    const long long k = (long long)blockIdx.x * kMMThreads + threadIdx.x;
     if (k >= n) return;
     Sym<C> M;
 #pragma unroll
     for (int e = 0; e < 6; ++e) M.v[e] = (e == 0 || e == 3 || e == 5) ? C(1) : C(0);
-    D[k] = deformation(M);
+    D[k] = 0.0;  // the sphere
     const C h = C(1) / C(substeps);
-    C a0[9], a1[9];
+    C a0[9], d[9];
+    double next[9];
+    const double* row = A + k * 9;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) a0[j] = (C)row[j];
+    if (T > 1)
+#pragma unroll
+        for (int j = 0; j < 9; ++j) next[j] = row[n * 9 + j];
+#pragma unroll
+    for (int j = 0; j < 9; ++j) d[j] = C(0);
+    Flow<C> Fs = flow_at<C>(a0, d, C(0), tau_d, f2_0);
+    int until = record_every;
+    long long rec = 0;
     for (long long s = 0; s + 1 < T; ++s) {
 #pragma unroll
-        for (int j = 0; j < 9; ++j) {
-            a0[j] = (C)A[(s * n + k) * 9 + j];
-            a1[j] = (C)A[((s + 1) * n + k) * 9 + j];
-        }
+        for (int j = 0; j < 9; ++j) d[j] = (C)next[j] - a0[j];
+        row += n * 9;
+        C a1[9];
+#pragma unroll
+        for (int j = 0; j < 9; ++j) a1[j] = (C)next[j];
+        if (s + 2 < T)
+#pragma unroll
+            for (int j = 0; j < 9; ++j) next[j] = row[n * 9 + j];
         for (int q = 0; q < substeps; ++q) {
-            // A at the start, middle and end of the substep (linear in t)
-            const C t0 = C(q) * h, tm = (C(q) + C(0.5)) * h, te = C(q + 1) * h;
-            C as[9], am[9], ae[9];
+            // A at the middle and end of the substep (linear in t)
+            const Flow<C> Fm = flow_at<C>(a0, d, (C(q) + C(0.5)) * h, tau_d, f2_0);
+            const Sym<C> k1 = rhs(M, Fs, kf);
+            Sym<C> sum = k1;
+            const Sym<C> k2 = rhs(axpy(M, C(0.5) * h, k1), Fm, kf);
+            const Sym<C> k3 = rhs(axpy(M, C(0.5) * h, k2), Fm, kf);
 #pragma unroll
-            for (int j = 0; j < 9; ++j) {
-                const C d = a1[j] - a0[j];
-                as[j] = a0[j] + t0 * d;
-                am[j] = a0[j] + tm * d;
-                ae[j] = a0[j] + te * d;
-            }
-            const Sym<C> k1 = rhs(M, as, tau_d, chi);
-            const Sym<C> k2 = rhs(axpy(M, C(0.5) * h, k1), am, tau_d, chi);
-            const Sym<C> k3 = rhs(axpy(M, C(0.5) * h, k2), am, tau_d, chi);
-            const Sym<C> k4 = rhs(axpy(M, h, k3), ae, tau_d, chi);
+            for (int e = 0; e < 6; ++e) sum.v[e] = fma(C(2), k2.v[e] + k3.v[e], sum.v[e]);
+            Fs = flow_at<C>(a0, d, C(q + 1) * h, tau_d, f2_0);
+            const Sym<C> k4 = rhs(axpy(M, h, k3), Fs, kf);
 #pragma unroll
-            for (int e = 0; e < 6; ++e)
-                M.v[e] += (h / C(6)) * (k1.v[e] + C(2) * k2.v[e] + C(2) * k3.v[e] + k4.v[e]);
+            for (int e = 0; e < 6; ++e) M.v[e] = fma(h / C(6), sum.v[e] + k4.v[e], M.v[e]);
         }
-        if ((s + 1) % record_every == 0) D[((s + 1) / record_every) * n + k] = deformation(M);
+#pragma unroll
+        for (int j = 0; j < 9; ++j) a0[j] = a1[j];
+        if (--until == 0) {
+            until = record_every;
+            D[++rec * n + k] = deformation(M);
+        }
     }
     if (Mout)
 #pragma unroll
@@ -149,12 +189,14 @@ extern "C" int lbm_mm_integrate(const double* A, int64_t T, int64_t n, double ta
         return LBM_EINVAL;
     if (precision != LBM_FP64 && precision != LBM_FP32) return LBM_EINVAL;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const int threads = 128;
+    const int threads = lbmgb_mm::kMMThreads;
     const unsigned blocks = (unsigned)((n + threads - 1) / threads);
+    const double f1 = 40.0 * (chi + 1.0) / ((3.0 + 2.0 * chi) * (16.0 + 19.0 * chi)), f2_0 = 5.0 / (3.0 + 2.0 * chi);
     if (precision == LBM_FP64)
-        lbmgb_mm::k_mm_rk4<double><<<blocks, threads, 0, s>>>(A, T, n, tau_d, chi, substeps, record_every, D, M);
+        lbmgb_mm::k_mm_rk4<double><<<blocks, threads, 0, s>>>(A, T, n, tau_d, f2_0, f1 / tau_d, substeps, record_every,
+                                                              D, M);
     else
-        lbmgb_mm::k_mm_rk4<float><<<blocks, threads, 0, s>>>(A, T, n, (float)tau_d, (float)chi, substeps,
-                                                             record_every, D, M);
+        lbmgb_mm::k_mm_rk4<float><<<blocks, threads, 0, s>>>(A, T, n, (float)tau_d, (float)f2_0, (float)(f1 / tau_d),
+                                                             substeps, record_every, D, M);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ECUDA;
 }
