@@ -540,6 +540,326 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
 }
 
+// ---------------------------------------------------------------------------
+// The whole forward pass of 128-row tiles in one persistent kernel: input
+// normalisation, every layer's product on the tensor cores, bias and ReLU,
+// output scaling.  The hidden activations of a tile stay in shared memory and
+// its accumulators in tensor memory, so global memory sees the float32 input
+// once and the outputs once; the weights come from L2 for every tile.
+//
+// What bounds it: reading x (d0 x 512 bytes a tile) and the weights through
+// the SM's L2 port, about 7 us a tile at d0 = 576 and widths of 256, against
+// 5 us of tensor-core time.  Layer by layer, each product wrote and read its
+// activations through memory and was a launch of its own, as were the input
+// normalisation and the output scaling.
+//
+// Roles (14 warps):
+//   warps 0-3   the epilogues: a warp reads its 32 rows of an accumulator
+//               (tcgen05.ld), adds the bias, applies ReLU, rounds to bfloat16
+//               and writes the next layer's A operand (128-byte swizzle);
+//               after the last layer it scales and stores the outputs
+//   warps 4-11  read x two 64-column chunks ahead into registers, normalise,
+//               round to bfloat16 and fill the ring of first-layer A chunks
+//   warp 12     loads the weight chunks by TMA, in the order of their use
+//   warp 13     issues the products.  The first layer of the next tile
+//               accumulates in its own half of tensor memory, cut into
+//               pieces that run between the hidden layers of this tile, so
+//               that the tensor core has work while the epilogues run
+// The products take the same K steps in the same order as k_gemm_tc's, with
+// the same rounding points, so the outputs are the same bits.  Waits are
+// bounded as in k_gemm_tc.
+constexpr int kFwEpiWarps = 4, kFwLoadWarps = 8;
+constexpr int kFwThreads = 32 * (kFwEpiWarps + kFwLoadWarps + 2);
+constexpr int kFwMaxLayers = 6, kFwMaxWidth = 256;
+constexpr int kFwWStages = 4, kFwXStages = 2;
+constexpr unsigned kFwWBytes = kFwMaxWidth * TC_K * 2;  // 32 KB: one K chunk of a layer's weights
+constexpr unsigned kFwChunk = TC_M * TC_K * 2;          // 16 KB: one K chunk of an A operand
+constexpr unsigned kFwX0 = kFwWStages * kFwWBytes, kFwH0 = kFwX0 + kFwXStages * kFwChunk;
+constexpr unsigned kFwBar0 = kFwH0 + (kFwMaxWidth / TC_K) * kFwChunk;
+constexpr int kFwBars = 2 * kFwWStages + 2 * kFwXStages + 2 + 1 + 1;  // W and X full, empty; acc full; epilogue; drain
+constexpr unsigned kFwSmem = 1024 + kFwBar0 + 8 * kFwBars + 16;
+constexpr unsigned kFwCols = 512;
+
+struct FwArgs {
+    CUtensorMap w[kFwMaxLayers];  // [dp_l, d_{l-1}], boxes of 64 x dp_l
+    const float* bias[kFwMaxLayers];
+    int width[kFwMaxLayers];  // dp_l
+    int layers, d0, dL;
+    const float *x, *x_mean, *x_scale, *y_mean, *y_scale;
+    float* y;
+    int tiles;
+    int* err;
+};
+
+// 32 columns of this warp's 32 TMEM lanes; the registers are valid after fw_wait_ld.
+__device__ __forceinline__ void fw_ld32(unsigned addr, unsigned (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+        "%13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, "
+        "[%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+          "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
+          "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
+          "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);  // .x at the lower address
+    return *reinterpret_cast<const unsigned*>(&h);
+}
+__device__ __forceinline__ void st_shared16(unsigned addr, unsigned a, unsigned b, unsigned c, unsigned d) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void st_shared8(unsigned addr, unsigned a, unsigned b) {
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+// Generic-proxy writes to shared memory before the tensor core's reads.
+__device__ __forceinline__ void fw_fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+__global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_constant__ FwArgs a) {
+    extern __shared__ __align__(1024) unsigned char fw_smem_raw[];
+    __shared__ int stop_flag;
+    const unsigned raw = tc_smem(fw_smem_raw);
+    const unsigned base = (raw + 1023u) & ~1023u;
+    const unsigned bar0 = base + kFwBar0;
+    unsigned* tmem_slot = reinterpret_cast<unsigned*>(fw_smem_raw + (bar0 + 8u * kFwBars - raw));
+    auto wfull = [&](unsigned s) { return bar0 + 8u * s; };
+    auto wempty = [&](unsigned s) { return bar0 + 8u * (kFwWStages + s); };
+    auto xfull = [&](unsigned s) { return bar0 + 8u * (2 * kFwWStages + s); };
+    auto xempty = [&](unsigned s) { return bar0 + 8u * (2 * kFwWStages + kFwXStages + s); };
+    auto accfull = [&](unsigned b) { return bar0 + 8u * (2 * kFwWStages + 2 * kFwXStages + b); };
+    const unsigned epi_bar = bar0 + 8u * (2 * kFwWStages + 2 * kFwXStages + 2), drain_bar = epi_bar + 8u;
+    volatile int* stop = &stop_flag;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+
+    if (t == 0) {
+        stop_flag = 0;
+        for (unsigned s = 0; s < kFwWStages; ++s) {
+            tc_mbar_init(wfull(s), 1);
+            tc_mbar_init(wempty(s), 1);
+        }
+        for (unsigned s = 0; s < kFwXStages; ++s) {
+            tc_mbar_init(xfull(s), kFwLoadWarps);
+            tc_mbar_init(xempty(s), 1);
+        }
+        tc_mbar_init(accfull(0), 1);
+        tc_mbar_init(accfull(1), 1);
+        tc_mbar_init(epi_bar, kFwEpiWarps);
+        tc_mbar_init(drain_bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 13) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(tmem_slot)),
+                     "n"(kFwCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const unsigned tmem = *tmem_slot;
+
+    const int mine = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // tiles of this CTA
+    const int L = a.layers, nk0 = a.d0 / TC_K;
+    auto give_up = [&]() {
+        *stop = 1;
+        atomicOr(a.err, 1);
+    };
+    unsigned issued = 0;  // warp 12, lane 0: weight chunks loaded
+
+    if (warp < kFwEpiWarps) {
+        const int row = warp * 32 + lane;
+        const unsigned swz = (unsigned)(row & 7), hrow = base + kFwH0 + (unsigned)row * 128u;
+        const unsigned lanes = tmem + ((unsigned)(warp * 32) << 16);
+        unsigned hidden = 0;  // accumulations in the second half so far
+        for (int j = 0; j < mine; ++j) {
+            const long long m = (long long)(blockIdx.x + j * gridDim.x) * TC_M + row;
+            for (int l = 0; l < L; ++l) {
+                int ok = 1;
+                if (lane == 0) {
+                    ok = l == 0 ? tc_wait(accfull(0), (unsigned)j & 1u, stop) : tc_wait(accfull(1), hidden & 1u, stop);
+                    if (!ok) give_up();
+                }
+                if (l > 0) ++hidden;
+                if (!__shfl_sync(0xffffffffu, ok, 0)) goto done;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const unsigned acc = lanes + (l == 0 ? 0u : 256u);
+                const float* bias = a.bias[l];
+                if (l + 1 < L) {
+#pragma unroll 1
+                    for (int n = 0; n < a.width[l]; n += 32) {
+                        unsigned v[32];
+                        fw_ld32(acc + (unsigned)n, v);
+                        const unsigned dst = hrow + (unsigned)(n / TC_K) * kFwChunk;
+                        const unsigned c0 = (unsigned)(n % TC_K) / 8u;  // 16-byte column of the 128-byte row
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float4 b0 = __ldg(reinterpret_cast<const float4*>(bias + n) + 2 * q);
+                            const float4 b1 = __ldg(reinterpret_cast<const float4*>(bias + n) + 2 * q + 1);
+                            const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                            float f[8];
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) f[e] = fmaxf(__uint_as_float(v[8 * q + e]) + bb[e], 0.f);
+                            st_shared16(dst + (((c0 + q) ^ swz) << 4), pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]),
+                                        pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+                        }
+                    }
+                    fw_fence_async();
+                } else {
+                    unsigned v[32];
+                    fw_ld32(acc, v);
+                    float* out = a.y + m * a.dL;
+#pragma unroll
+                    for (int c = 0; c < 32; ++c)
+                        if (c < a.dL) {
+                            const float yh = __uint_as_float(v[c]) + __ldg(bias + c);
+                            out[c] = yh / __ldg(a.y_scale + c) + __ldg(a.y_mean + c);
+                        }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) tc_arrive(epi_bar);
+            }
+        }
+    } else if (warp < kFwEpiWarps + kFwLoadWarps) {
+        // chunk q of this CTA: 64 columns of a tile; a thread takes 4 columns of 8 rows
+        const int lt = t - 32 * kFwEpiWarps, g = lt & 15, r0 = lt >> 4;
+        const int total = mine * nk0;
+        auto load = [&](int q, float4 (&v)[8]) {
+            if (q >= total) return;
+            const int j = q / nk0, c = q - j * nk0;
+            const float* p = a.x + ((long long)(blockIdx.x + j * gridDim.x) * TC_M + r0) * a.d0 + c * TC_K + 4 * g;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = __ldcs(reinterpret_cast<const float4*>(p + (long long)(16 * i) * a.d0));
+        };
+        auto put = [&](int q, const float4 (&v)[8]) -> bool {
+            const unsigned s = (unsigned)q % kFwXStages, round = (unsigned)q / kFwXStages;
+            int ok = 1;
+            if (round > 0) {
+                if (lane == 0) {
+                    ok = tc_wait(xempty(s), (round - 1u) & 1u, stop);
+                    if (!ok) give_up();
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+            }
+            if (!ok) return false;
+            const int c = (q % nk0) * TC_K + 4 * g;
+            const float4 mu = __ldg(reinterpret_cast<const float4*>(a.x_mean + c));
+            const float4 sc = __ldg(reinterpret_cast<const float4*>(a.x_scale + c));
+            const unsigned dst = base + kFwX0 + s * kFwChunk;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const unsigned r = (unsigned)(r0 + 16 * i);
+                st_shared8(dst + r * 128u + ((((unsigned)g >> 1) ^ (r & 7u)) << 4) + 8u * ((unsigned)g & 1u),
+                           pack_bf16((v[i].x - mu.x) * sc.x, (v[i].y - mu.y) * sc.y),
+                           pack_bf16((v[i].z - mu.z) * sc.z, (v[i].w - mu.w) * sc.w));
+            }
+            fw_fence_async();
+            __syncwarp();
+            if (lane == 0) tc_arrive(xfull(s));
+            return true;
+        };
+        float4 va[8], vb[8];
+        load(0, va);
+        load(1, vb);
+        for (int q = 0; q < total; q += 2) {
+            if (!put(q, va)) break;
+            load(q + 2, va);
+            if (q + 1 < total && !put(q + 1, vb)) break;
+            load(q + 3, vb);
+        }
+    } else if (lane == 0) {
+        // the weight chunks and the products follow one schedule: the first
+        // layer of the first tile; then per tile each hidden layer, followed
+        // by its share of the next tile's first layer
+        const bool loader = warp == 12;
+        unsigned wit = 0, xit = 0, epi = 0, epis_due = 0;
+        bool ok = true;
+        auto chunk = [&](int l, int kt) {  // one K chunk of layer l
+            const unsigned s = wit % kFwWStages, round = wit / kFwWStages;
+            ++wit;
+            if (loader) {
+                if (round > 0 && !tc_wait(wempty(s), (round - 1u) & 1u, stop)) {
+                    ok = false;
+                    return;
+                }
+                tc_expect_tx(wfull(s), (unsigned)a.width[l] * TC_K * 2u);
+                tc_tma_load(base + s * kFwWBytes, &a.w[l], kt * TC_K, 0, wfull(s));
+                ++issued;
+                return;
+            }
+            unsigned a_s = base + kFwH0 + (unsigned)kt * kFwChunk, xs = 0;
+            if (l == 0) {
+                xs = xit % kFwXStages;
+                if (!tc_wait(xfull(xs), (xit / kFwXStages) & 1u, stop)) {
+                    ok = false;
+                    return;
+                }
+                ++xit;
+                a_s = base + kFwX0 + xs * kFwChunk;
+            }
+            if (!tc_wait(wfull(s), round & 1u, stop)) {
+                ok = false;
+                return;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const unsigned acc = tmem + (l == 0 ? 0u : 256u), idesc = tc_idesc(TC_M, a.width[l]);
+#pragma unroll
+            for (int kk = 0; kk < TC_K / 16; ++kk) {
+                const unsigned long long ad = tc_desc_sw128(a_s + 32u * kk);
+                const unsigned long long bd = tc_desc_sw128(base + s * kFwWBytes + 32u * kk);
+                const unsigned accumulate = (kt > 0 || kk > 0) ? 1u : 0u;
+                asm volatile(
+                    "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(acc),
+                    "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate)
+                    : "memory");
+            }
+            tc_commit(wempty(s));
+            if (l == 0) tc_commit(xempty(xs));
+        };
+        for (int kt = 0; ok && kt < nk0; ++kt) chunk(0, kt);
+        if (ok && !loader) tc_commit(accfull(0));
+        for (int j = 0; ok && j < mine; ++j) {
+            for (int l = 1; ok && l < L; ++l) {
+                if (!loader) {
+                    // the epilogue of the layer before (and, at l = 1, of the
+                    // tile before): every phase is waited for in turn
+                    epis_due = (unsigned)(j * L + l);
+                    for (; ok && epi < epis_due; ++epi) ok = tc_wait(epi_bar, epi & 1u, stop);
+                    if (!ok) break;
+                }
+                for (int kt = 0; ok && kt < a.width[l - 1] / TC_K; ++kt) chunk(l, kt);
+                if (ok && !loader) tc_commit(accfull(1));
+                if (j + 1 < mine) {
+                    for (int kt = (l - 1) * nk0 / (L - 1); ok && kt < l * nk0 / (L - 1); ++kt) chunk(0, kt);
+                    if (ok && !loader && l == L - 1) tc_commit(accfull(0));
+                }
+            }
+        }
+        if (!ok) give_up();
+        if (!loader) tc_commit(drain_bar);  // completes when every product issued above has
+    }
+done:
+    __syncthreads();
+    if (warp == 12 && lane == 0 && *stop) {
+        for (unsigned s = 0; s < kFwWStages; ++s) {  // copies issued but perhaps not consumed: the last one of each stage
+            if (issued <= s) continue;
+            const unsigned last = issued - 1u - ((issued - 1u - s) % kFwWStages);
+            tc_wait(wfull(s), (last / kFwWStages) & 1u, nullptr);
+        }
+    }
+    if (warp == 13 && lane == 0 && !tc_wait(drain_bar, 0u, nullptr)) atomicOr(a.err, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 13) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kFwCols) : "memory");
+    }
+}
+
 namespace {
 
 // Normalised input in bfloat16: xb[r, c] = (x[r, c] - mean[c]) scale[c].
@@ -719,13 +1039,8 @@ __global__ void k_deform_from_m(const float* __restrict__ m6, long long n, doubl
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const float* q = m6 + 6 * r;
-    double a[3][3] = {{q[0], q[1], q[2]}, {q[1], q[3], q[4]}, {q[2], q[4], q[5]}};
-    double lam[3], v[3][3];
-    lbmgb::jacobi3(a, lam, v);
-    double hi = fmax(lam[0], fmax(lam[1], lam[2])), lo = fmin(lam[0], fmin(lam[1], lam[2]));
-    hi = sqrt(fmax(hi, 0.0));
-    lo = sqrt(fmax(lo, 0.0));
-    D[r] = hi + lo > 0.0 ? (hi - lo) / (hi + lo) : 0.0;
+    const double m[6] = {q[0], q[1], q[2], q[3], q[4], q[5]};
+    D[r] = lbmgb::deformation_of(m);
 }
 
 }  // namespace
@@ -762,6 +1077,8 @@ struct lbm_mlp {
     int sms;                     // multiprocessors of the device
     float* ws;                   // split-K partials, kMaxSplit x the largest weight matrix
     float* cs_parts;             // column-sum partials, kColSlices x the widest layer
+    bool fused;                  // k_mlp_forward takes this network's shapes
+    FwArgs fw;                   // its weights' tensor maps and constants (rows and pointers set per call)
 };
 
 namespace {
@@ -923,6 +1240,57 @@ cudaError_t forward(lbm_mlp* c, const float* x, int n) {
     return e;
 }
 
+// k_mlp_forward's constants: input width a multiple of 64, two layers or more,
+// hidden widths multiples of 64 up to 256.
+void fused_setup(lbm_mlp* c) {
+    c->fused = false;
+    if (c->L < 2 || c->L > kFwMaxLayers || c->d[0] % TC_K) return;
+    for (int l = 1; l < c->L; ++l)
+        if (c->d[l] % TC_K || c->d[l] > kFwMaxWidth) return;
+    FwArgs& a = c->fw;
+    memset(&a, 0, sizeof(a));
+    for (int l = 1; l <= c->L; ++l) {
+        if (!tc_map(&a.w[l - 1], c->Wb[l], c->dp[l], c->d[l - 1], c->d[l - 1], c->dp[l])) return;
+        a.bias[l - 1] = c->p + c->offb[l];
+        a.width[l - 1] = c->dp[l];
+        if (!aligned16(a.bias[l - 1])) return;
+    }
+    a.layers = c->L;
+    a.d0 = c->d[0];
+    a.dL = c->d[c->L];
+    a.x_mean = c->x_mean;
+    a.x_scale = c->x_scale;
+    a.y_mean = c->y_mean;
+    a.y_scale = c->y_scale;
+    a.err = c->d_err;
+    c->fused = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwSmem) ==
+               cudaSuccess;
+    if (!c->fused) cudaGetLastError();
+}
+
+// The leading rows of a forward pass that k_mlp_forward takes: those of the
+// chunks of max_batch rows whose products would all run on k_gemm_tc (whole
+// 128-row tiles), so that every row keeps its arithmetic.
+int64_t fused_rows(const lbm_mlp* c, const float* x, int64_t n) {
+    if (!c->fused || c->tensor_path != 0 || !aligned16(x) || c->max_batch % TC_M) return 0;
+    const int64_t tail = n % c->max_batch;
+    return tail % TC_M ? n - tail : n;
+}
+
+cudaError_t fused_forward(lbm_mlp* c, const float* x, float* y, int64_t rows) {
+    constexpr int64_t kMaxTiles = 1 << 24;
+    for (int64_t t0 = 0; t0 < rows / TC_M; t0 += kMaxTiles) {
+        FwArgs a = c->fw;
+        a.tiles = (int)std::min<int64_t>(kMaxTiles, rows / TC_M - t0);
+        a.x = x + t0 * TC_M * c->d[0];
+        a.y = y + t0 * TC_M * c->d[c->L];
+        k_mlp_forward<<<std::min(a.tiles, c->sms), kFwThreads, kFwSmem, c->stream>>>(a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // Loss and parameter gradients of n samples (targets t on the device, float32 [n, dL]).
 cudaError_t backward(lbm_mlp* c, const float* t, int n) {
     const int L = c->L, dL = c->d[L], dLp = c->dp[L];
@@ -1064,6 +1432,7 @@ int lbm_mlp_create(lbm_mlp** out, int32_t nlayers, const int32_t* sizes, int32_t
         lbm_mlp_destroy(c);
         return st;
     }
+    fused_setup(c);
     *out = c;
     return LBM_OK;
 }
@@ -1165,7 +1534,9 @@ int lbm_mlp_forward(lbm_mlp* c, const float* x, float* y, int64_t n) {
     if (!c || n < 0 || (n > 0 && (!x || !y))) return LBM_EINVAL;
     cudaSetDevice(c->device);
     const int d0 = c->d[0], dL = c->d[c->L];
-    for (int64_t s = 0; s < n; s += c->max_batch) {
+    const int64_t rows = fused_rows(c, x, n);
+    MLP_TRY(fused_forward(c, x, y, rows));
+    for (int64_t s = rows; s < n; s += c->max_batch) {
         const int k = (int)std::min<int64_t>(c->max_batch, n - s);
         MLP_TRY(forward(c, x + s * d0, k));
         k_output<<<blocks_for((long long)k * dL, 256), 256, 0, c->stream>>>(c->yhat, 32, k, dL, c->y_mean, c->y_scale,
