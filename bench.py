@@ -100,7 +100,7 @@ def measured_peaks():
 
 # Sources that define the row kernel and its launch shape: a committed DRAM
 # traffic figure holds only while these are unchanged.
-ROW_KERNEL_SOURCES = ("lbm_fast.cu", "lbm_lattice.cuh", "lbm_internal.h", "lbm_dev.cuh", "lbm_step.cu", "lbm_centre.cuh")
+ROW_KERNEL_SOURCES = ("lbm_fast.cu", "lbm_node.cuh", "lbm_lattice.cuh", "lbm_internal.h", "lbm_dev.cuh", "lbm_step.cu", "lbm_centre.cuh")
 
 
 # The stream-collide kernel a context runs, by lbm_launch_variant.
@@ -108,7 +108,7 @@ KERNEL_NAMES = {0: "k_stream_collide (generic tile kernel)",
                 1: "k_stream_collide_rows (row kernel, per-thread loads)",
                 2: "k_stream_collide_rows (row kernel, shared-memory staging)",
                 3: "k_stream_collide_ws (row kernel, loader and collider threads)",
-                4: "k_flat_rho + k_flat_collide (density and collision passes)"}
+                4: "two-pass kernels (density and collision pass)"}
 
 
 def row_kernel_sha1():

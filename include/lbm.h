@@ -152,8 +152,8 @@ void lbm_opts_default(lbm_opts* opts);
  * Sec. 3).  Device memory: two population buffers of
  * 38 (box[2]+2)(box[1]+2) pitch elements (float64 / float32), pitch >=
  * box[0] + 2, or 88 (box[2]+2)(box[1]+2) pitch bytes (16-bit deviations);
- * with float64 storage also 16 (box[2]+2)(box[1]+2)(box[0]+2) bytes of
- * densities where they fit.
+ * where a two-pass kernel runs (lbm_launch_variant 4) also 16 (float64) or 8
+ * (box[2]+2)(box[1]+2)(box[0]+2) bytes of densities where they fit.
  * On success *out receives the context; on failure *out is NULL.
  */
 int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[2], double G,
@@ -294,8 +294,11 @@ int lbm_launch_shape(lbm_ctx* ctx, int32_t* tile_y, int32_t* z_chunk, int32_t* c
  * (k_stream_collide), or the row-tiled cluster kernel's variant as in
  * lbm_opts.row_variant (1 per-thread loads and 2 shared-memory staging, both
  * k_stream_collide_rows; 3 loader and collider threads, k_stream_collide_ws),
- * or 4 the density and collision passes (k_flat_rho, k_flat_collide) that
- * float64 storage takes unless opts->tile_y or z_chunk is set.
+ * or 4 a density and a collision pass without a march, which these take
+ * unless opts->tile_y, z_chunk or (second) row_variant is set: float64 storage
+ * (k_flat_rho, k_flat_collide); boxes of a row-tiled shape up to 393216 nodes
+ * (k_row_rho, k_row_collide; the cluster kernel's states bit for bit); float32
+ * boxes of other shapes with the ghost boundary (k_any_rho, k_any_collide).
  * LBM_EINVAL for a NULL context or pointer. */
 int lbm_launch_variant(lbm_ctx* ctx, int32_t* variant);
 

@@ -132,6 +132,15 @@ int lazy_init(lbm_ctx* c) {
     return LBM_OK;
 }
 
+// The density array of the two-pass kernels.
+size_t rho_bytes(const lbm_ctx* c) {
+    return (size_t)(c->shape.flat == kFlat64 ? flat_rho_bytes(c->L) : flat32_rho_bytes(c->L));
+}
+cudaError_t fill_rho(lbm_ctx* c) {
+    return c->shape.flat == kFlat64 ? launch_flat_fill(c->rho, c->L, c->model, c->stream)
+                                    : launch_flat32_fill(c->rho, c->L, c->model, c->stream);
+}
+
 int set_device(lbm_ctx* c) { return cuda_status(cudaSetDevice(c->device)); }
 
 bool finite_all(const double* a, int n) {
@@ -277,7 +286,7 @@ int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[
     c->L = make_layout(box[0], box[1], box[2], c->prec);
     c->shape = choose_shape(c->L, c->prec, o.bc == LBM_BC_PERIODIC_TEST, c->model.mrt, o.tile_y, o.z_chunk,
                             o.row_variant, c->num_sms, true);
-    if (c->shape.flat && cudaMalloc(&c->rho, (size_t)flat_rho_bytes(c->L)) != cudaSuccess) {
+    if (c->shape.flat && cudaMalloc(&c->rho, rho_bytes(c)) != cudaSuccess) {
         cudaGetLastError();  // no room for the density array: the tile kernel needs none
         c->rho = nullptr;
         c->shape = choose_shape(c->L, c->prec, o.bc == LBM_BC_PERIODIC_TEST, c->model.mrt, o.tile_y, o.z_chunk,
@@ -318,7 +327,7 @@ int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[0], 0, bytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, bytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
-    if (e == cudaSuccess && c->rho) e = launch_flat_fill(c->rho, c->L, c->model, c->stream);
+    if (e == cudaSuccess && c->rho) e = fill_rho(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         st = cuda_status(e);
@@ -693,7 +702,7 @@ int lbm_load(lbm_ctx* c, const char* path) {
     c->model.tau[0] = h.tau[0]; c->model.tau[1] = h.tau[1];
     c->model.G = h.G;
     c->model.rho_b[0] = h.rho_b[0]; c->model.rho_b[1] = h.rho_b[1];
-    if (c->rho) LBM_TRY(launch_flat_fill(c->rho, c->L, c->model, c->stream));  // the ghost densities may differ
+    if (c->rho) LBM_TRY(fill_rho(c));  // the ghost densities may differ
     c->kt.swap(kt);
     c->kA.swap(kA);
     if (is_dev(c->prec)) {

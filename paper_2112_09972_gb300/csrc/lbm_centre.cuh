@@ -81,50 +81,56 @@ __device__ void centre_epilogue(C (&cm)[4], CentreParts cp, C* scratch) {
     centre_reduce(cm, reinterpret_cast<C*>(cp.p), cta, total, cp.counter, cp.sum, cp.frame, scratch);
 }
 
-// centre_reduce in float64 for kernels whose CTAs mostly hold no droplet node:
-// a CTA with any = false (uniform) writes zero partials without the FP64
-// shuffles, and every thread of the last CTA takes part in the final sum.
-template <int NT>
-__device__ void centre_reduce_last(double (&cm)[4], bool any, double* parts, unsigned slot, unsigned total,
-                                   unsigned* counter, double* sum8, float* frame, double* scratch) {
+// centre_reduce for kernels whose CTAs mostly hold no droplet node: a CTA with
+// any = false (uniform) writes zero partials without the shuffles (float64
+// ones run on the slow FP64 pipe), and every thread of the last CTA takes part
+// in the final sum.
+template <int NT, typename C>
+__device__ void centre_reduce_last(C (&cm)[4], bool any, C* parts, unsigned slot, unsigned total, unsigned* counter,
+                                   double* sum8, float* frame, C* scratch) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     __shared__ unsigned last;
-    auto warp_sums = [&](const double (&v)[4]) {
+    auto warp_sums = [&](const C (&v)[4]) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            double a = v[q];
+            C a = v[q];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
             if (lane == 0) scratch[4 * warp + q] = a;
         }
     };
     auto total_of = [&](int q) {
-        double a = scratch[q];
+        C a = scratch[q];
         for (int w = 1; w < NT / 32; ++w) a += scratch[4 * w + q];
         return a;
     };
     if (any) warp_sums(cm);
     __syncthreads();
     if (t == 0) {
-        for (int q = 0; q < 4; ++q) parts[4LL * slot + q] = any ? total_of(q) : 0.0;
+        for (int q = 0; q < 4; ++q) parts[4LL * slot + q] = any ? total_of(q) : C(0);
         __threadfence();
         last = atomicAdd(counter, 1u) == total - 1 ? 1u : 0u;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double s4[4] = {0.0, 0.0, 0.0, 0.0};
+    C s4[4] = {C(0), C(0), C(0), C(0)};
+#pragma unroll 4
     for (unsigned b = t; b < total; b += NT)
 #pragma unroll
         for (int q = 0; q < 4; ++q) s4[q] += __ldcg(parts + 4LL * b + q);
     warp_sums(s4);
     __syncthreads();
     if (t == 0) {
-        for (int q = 0; q < 4; ++q) sum8[q] = total_of(q);
-        const bool have = sum8[0] > 0.0;
+        C sum[4];
+        for (int q = 0; q < 4; ++q) {
+            sum[q] = total_of(q);
+            sum8[q] = (double)sum[q];
+        }
+        const bool have = sum[0] > C(0);
         for (int q = 0; q < 3; ++q) {
-            const double xc = have ? sum8[1 + q] / sum8[0] : 0.0;
-            sum8[4 + q] = xc;
+            const C xc = have ? sum[1 + q] / sum[0] : C(0);
+            sum8[4 + q] = (double)xc;
             frame[q] = (float)xc;
         }
         *counter = 0u;

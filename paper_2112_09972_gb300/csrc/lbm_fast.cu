@@ -58,9 +58,8 @@
 #include <utility>
 
 #include "lbm_centre.cuh"
-#include "lbm_dev.cuh"
 #include "lbm_internal.h"
-#include "lbm_lattice.cuh"
+#include "lbm_node.cuh"
 #include "lbm_pdl.cuh"
 
 namespace cg = cooperative_groups;
@@ -90,37 +89,6 @@ namespace cg = cooperative_groups;
 
 namespace lbmgb {
 namespace {
-
-struct FastModel {
-    float inv_tau[2], tau[2], G, rho_b[2];
-    float omit[2];  // 1 - 1/tau
-    float sh[2];    // -G tau: the velocity shift tau_s F^s / rho_s per unit of the other component's force sum
-    float mrt[5];   // MRT free rates (s_e, s_eps, s_q, s_pi, s_m) when the kernel relaxes moments
-};
-
-FastModel fast_model(const Model& m) {
-    FastModel fm;
-    for (int q = 0; q < 2; ++q) {
-        fm.inv_tau[q] = (float)(1.0 / m.tau[q]);
-        fm.tau[q] = (float)m.tau[q];
-        fm.rho_b[q] = (float)m.rho_b[q];
-        fm.omit[q] = (float)(1.0 - 1.0 / m.tau[q]);
-        fm.sh[q] = (float)(-m.G * m.tau[q]);
-    }
-    fm.G = (float)m.G;
-    for (int k = 0; k < 5; ++k) fm.mrt[k] = (float)m.mrt_rates[k];
-    return fm;
-}
-
-// Compile-time loop: f(std::integral_constant<int, 0>) ... f(..., N - 1).
-template <typename F, int... I>
-__device__ __forceinline__ void sfor_(F& f, std::integer_sequence<int, I...>) {
-    (f(std::integral_constant<int, I>{}), ...);
-}
-template <int N, typename F>
-__device__ __forceinline__ void sfor(F&& f) {
-    sfor_(f, std::make_integer_sequence<int, N>{});
-}
 
 // Shared-memory, cluster-address and mbarrier helpers (inline PTX).
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -213,269 +181,6 @@ __device__ __forceinline__ void cp_async16(unsigned dst, const void* src, unsign
                  : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Global loads and stores at a pointer plus an immediate byte offset.  The
-// first read of a plane keeps its lines in L2 (evict_last policy) for the
-// second read one plane later, which marks them last-use; the written state
-// is streamed out.  The populations read are never written by the kernel, so
-// the loads may be scheduled freely.
-template <int OFF>
-__device__ __forceinline__ float ld_keep(const void* p, unsigned long long pol) {
-    float v;
-    asm("ld.global.nc.L2::cache_hint.f32 %0, [%1+%3], %2;" : "=f"(v) : "l"(p), "l"(pol), "n"(OFF));
-    return v;
-}
-template <int OFF>
-__device__ __forceinline__ float ld_last(const void* p) {
-    float v;
-    asm("ld.global.lu.f32 %0, [%1+%2];" : "=f"(v) : "l"(p), "n"(OFF));
-    return v;
-}
-template <int OFF>
-__device__ __forceinline__ unsigned ld_keep_u32(const void* p, unsigned long long pol) {
-    unsigned v;
-    asm("ld.global.nc.L2::cache_hint.b32 %0, [%1+%3], %2;" : "=r"(v) : "l"(p), "l"(pol), "n"(OFF));
-    return v;
-}
-template <int OFF>
-__device__ __forceinline__ unsigned ld_last_u32(const void* p) {
-    unsigned v;
-    asm("ld.global.lu.b32 %0, [%1+%2];" : "=r"(v) : "l"(p), "n"(OFF));
-    return v;
-}
-__device__ __forceinline__ float4 ld_keep_f4(const void* p, unsigned long long pol) {
-    float4 v;
-    asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
-        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-        : "l"(p), "l"(pol));
-    return v;
-}
-__device__ __forceinline__ float4 ld_last_f4(const void* p) {
-    float4 v;
-    asm("ld.global.lu.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-    return v;
-}
-template <int OFF>
-__device__ __forceinline__ void st_cs(void* p, float v) {
-    asm volatile("st.global.cs.f32 [%0+%2], %1;" ::"l"(p), "f"(v), "n"(OFF));
-}
-template <int OFF>
-__device__ __forceinline__ void st_cs_u32(void* p, unsigned v) {
-    asm volatile("st.global.cs.b32 [%0+%2], %1;" ::"l"(p), "r"(v), "n"(OFF));
-}
-__device__ __forceinline__ void st_cs_f4(void* p, float4 v) {
-    asm volatile("st.global.cs.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
-}
-
-// Compile-time geometry of the row-interleaved layout for row width TX (the
-// values make_layout computes): entries before x = 0, entries per population
-// row and layout units per row block (elements of 4 bytes for float32, units
-// of 2 bytes for deviations).
-template <int TX, typename ST>
-struct RowGeo;
-template <int TX>
-struct RowGeo<TX, float> {
-    static constexpr int X0 = 8, PITCH = TX + 16, ROW = 38 * PITCH;
-};
-template <int TX, typename T>
-struct RowGeo<TX, Dev<T>> {
-    static constexpr int X0 = 16, PITCH = TX + 32, ROW = 44 * PITCH;
-};
-
-// Storage-specific reads and writes of the row kernels.  A node's accesses
-// go through its pointer `base` (the node in plane -1) and, per plane p, the
-// three pointers P3 of planes p - 1, p, p + 1.
-template <int TX, typename ST>
-struct RowIO;
-
-template <int TX>
-struct RowIO<TX, float> {
-    using G = RowGeo<TX, float>;
-    struct P3 {
-        const char* m;
-        const char* o;
-        const char* p;
-    };
-    using Out = float*;  // element (s = 0, i = 0) of the node in the written plane
-    // element (s = 0, i = 0) of node (x, y) in plane -1
-    static __device__ __forceinline__ const char* base(const float* src, int x, int y) {
-        return reinterpret_cast<const char*>(src + (long long)(y + 1) * G::ROW + G::X0 + x);
-    }
-    // the same node, component s (the halo threads sum one component each)
-    static __device__ __forceinline__ const char* base_c(const float* src, int x, int y, int s) {
-        return base(src, x, y) + 4 * s * 19 * G::PITCH;
-    }
-    static __device__ __forceinline__ P3 planes(const char* b, const Layout& L, int p) {
-        const long long pl = 4 * L.plane;
-        const char* o = b + (long long)(p + 1) * pl;
-        return {o - pl, o, o + pl};
-    }
-    static __device__ __forceinline__ Out out(float* dst, const Layout& L, int x, int y, int z) {
-        return dst + (long long)(z + 1) * L.plane + (long long)(y + 1) * G::ROW + G::X0 + x;
-    }
-    // byte offset of population (s, i) pulled into the node (it comes from
-    // x - c_i, which lies in plane p - c_iz: the pointer src_plane picks)
-    template <int S, int I>
-    static constexpr int poff() {
-        return 4 * ((S * 19 + I) * G::PITCH - cy_(I) * G::ROW - cx_(I));
-    }
-    template <int I>
-    static __device__ __forceinline__ const char* src_plane(const P3& q) {
-        return cz_(I) > 0 ? q.m : (cz_(I) < 0 ? q.p : q.o);
-    }
-    // component S's post-streaming density (first read, kept in L2)
-    template <int S>
-    static __device__ __forceinline__ float density(const P3& q, unsigned long long pol) {
-        float r = ld_keep<poff<S, 0>()>(q.o, pol);
-        sfor<9>([&](auto K) {
-            constexpr int i = 2 * decltype(K)::value + 1;
-            r += ld_keep<poff<S, i>()>(src_plane<i>(q), pol) + ld_keep<poff<S, i + 1>()>(src_plane<i + 1>(q), pol);
-        });
-        return r;
-    }
-    static __device__ __forceinline__ void densities(const P3& q, unsigned long long pol, float& ra, float& rb) {
-        ra = density<0>(q, pol);
-        rb = density<1>(q, pol);
-    }
-    // the node's 38 pulled populations (second read, last use); rs: unused
-    // in float32 (the deviation forms return the node's rho* there)
-    static __device__ __forceinline__ void populations(const P3& q, float (&f)[2][19], float (&rs)[2]) {
-        rs[0] = rs[1] = 0.f;
-        sfor<19>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            f[0][i] = ld_last<poff<0, i>()>(src_plane<i>(q));
-            f[1][i] = ld_last<poff<1, i>()>(src_plane<i>(q));
-        });
-    }
-    // one read of the 38 pulled populations and the densities summed from
-    // them in the order of density() (the warp-specialised kernel)
-    static __device__ __forceinline__ void load_all(const P3& q, float (&f)[2][19], float (&rs)[2], float& ra,
-                                                    float& rb) {
-        populations(q, f, rs);
-        ra = f[0][0];
-        rb = f[1][0];
-#pragma unroll
-        for (int i = 1; i < 19; i += 2) {
-            ra += f[0][i] + f[0][i + 1];
-            rb += f[1][i] + f[1][i + 1];
-        }
-    }
-    template <int S, int I>
-    static __device__ __forceinline__ void store(Out o, float v) {
-        st_cs<4 * (S * 19 + I) * G::PITCH>(o, v);
-    }
-};
-
-// 16-bit deviation storage: per node the float4 block {rho*_A, rho*_B, f*_0A,
-// f*_0B} and the 18 words of deviation pairs {A, B}.  The plane pointers
-// point at the node's word slot (x0 + x) of its row block; the node's own
-// block lies a per-thread constant further (12 (x0 + x) bytes), and the word
-// of direction i at the immediate 4 (3 + i) pitch.
-template <int TX, typename T>
-struct RowIO<TX, Dev<T>> {
-    using G = RowGeo<TX, Dev<T>>;
-    struct P3 {
-        const char* m;
-        const char* o;
-        const char* p;
-        int blk;  // byte offset of the node's float4 block from o
-    };
-    struct Out {
-        unsigned* w;  // word slot of the node in the written plane
-        float4* b;    // the node's float4 block
-    };
-    static __device__ __forceinline__ const char* base(const Dev<T>* src, int x, int y) {
-        return reinterpret_cast<const char*>(src) + 2LL * (long long)(y + 1) * G::ROW + 4 * (G::X0 + x);
-    }
-    static __device__ __forceinline__ P3 planes(const char* b, const Layout& L, int p, int x) {
-        const long long pl = 2 * L.plane;
-        const char* o = b + (long long)(p + 1) * pl;
-        return {o - pl, o, o + pl, 12 * (G::X0 + x)};
-    }
-    static __device__ __forceinline__ Out out(Dev<T>* dst, const Layout& L, int x, int y, int z) {
-        char* o = reinterpret_cast<char*>(dst) + 2LL * ((long long)(z + 1) * L.plane + (long long)(y + 1) * G::ROW) +
-                  4 * (G::X0 + x);
-        return {reinterpret_cast<unsigned*>(o), reinterpret_cast<float4*>(o + 12 * (G::X0 + x))};
-    }
-    template <int I>
-    static constexpr int woff() {  // byte offset of the word of direction I pulled into the node
-        return 4 * (3 + I) * G::PITCH - 2 * cy_(I) * G::ROW - 4 * cx_(I);
-    }
-    template <int I>
-    static __device__ __forceinline__ const char* src_plane(const P3& q) {
-        return cz_(I) > 0 ? q.m : (cz_(I) < 0 ? q.p : q.o);
-    }
-    // sum_i (w_i rho* + d_i) + f*_0 = f*_0 + (1 - w_0) rho* + sum_i d_i, from
-    // the node's block o and its pulled words word(integral_constant<int, i>)
-    template <typename W>
-    static __device__ __forceinline__ void sum_words(const float4& o, W&& word, float& ra, float& rb) {
-        float da = 0.f, db = 0.f;
-        sfor<9>([&](auto K) {
-            constexpr int i = 2 * decltype(K)::value + 1;
-            const float2 u = dev_unpack2<T>(word(std::integral_constant<int, i>{}));
-            const float2 v = dev_unpack2<T>(word(std::integral_constant<int, i + 1>{}));
-            da += u.x + v.x;
-            db += u.y + v.y;
-        });
-        ra = o.z + (1.f - wgt<float>(0)) * o.x + da;
-        rb = o.w + (1.f - wgt<float>(0)) * o.y + db;
-    }
-    static __device__ __forceinline__ void densities(const P3& q, unsigned long long pol, float& ra, float& rb) {
-        const float4 o = ld_keep_f4(q.o + q.blk, pol);
-        sum_words(
-            o,
-            [&](auto I) {
-                constexpr int i = decltype(I)::value;
-                return ld_keep_u32<woff<i>()>(src_plane<i>(q), pol);
-            },
-            ra, rb);
-    }
-    // The collision's input in deviation form: f[s][0] the rest population,
-    // f[s][i >= 1] the pulled deviation d_i (the population is
-    // w_i rho*_s + d_i; collide_node folds w_i rho*_s into its constants),
-    // rs the node's rho* of both components.
-    static __device__ __forceinline__ void populations(const P3& q, float (&f)[2][19], float (&rs)[2]) {
-        const float4 o = ld_last_f4(q.o + q.blk);
-        f[0][0] = o.z;
-        f[1][0] = o.w;
-        rs[0] = o.x;
-        rs[1] = o.y;
-        sfor<18>([&](auto K) {
-            constexpr int i = decltype(K)::value + 1;
-            const float2 v = dev_unpack2<T>(ld_last_u32<woff<i>()>(src_plane<i>(q)));
-            f[0][i] = v.x;
-            f[1][i] = v.y;
-        });
-    }
-    // one read of the block and the 18 pulled words: the input of
-    // populations() and the densities of densities(), with their arithmetic
-    static __device__ __forceinline__ void load_all(const P3& q, float (&f)[2][19], float (&rs)[2], float& ra,
-                                                    float& rb) {
-        const float4 o = ld_last_f4(q.o + q.blk);
-        f[0][0] = o.z;
-        f[1][0] = o.w;
-        rs[0] = o.x;
-        rs[1] = o.y;
-        float da = 0.f, db = 0.f;
-        sfor<9>([&](auto K) {
-            constexpr int i = 2 * decltype(K)::value + 1;
-            const float2 u = dev_unpack2<T>(ld_last_u32<woff<i>()>(src_plane<i>(q)));
-            const float2 v = dev_unpack2<T>(ld_last_u32<woff<i + 1>()>(src_plane<i + 1>(q)));
-            da += u.x + v.x;
-            db += u.y + v.y;
-            f[0][i] = u.x;
-            f[1][i] = u.y;
-            f[0][i + 1] = v.x;
-            f[1][i + 1] = v.y;
-        });
-        ra = o.z + (1.f - wgt<float>(0)) * o.x + da;
-        rb = o.w + (1.f - wgt<float>(0)) * o.y + db;
-    }
-    template <int I>
-    static __device__ __forceinline__ void store_word(Out o, unsigned v) {
-        st_cs_u32<4 * (3 + I) * G::PITCH>(o.w, v);
-    }
-};
 
 // Outer-halo pulls of the staged variant, prefetched into shared memory one
 // march step ahead by asynchronous copies (each halo thread copies the
@@ -719,201 +424,21 @@ struct StagedLayout {
     static constexpr size_t bytes = halo_off + (HALO ? (size_t)HaloPrefetch<TX, ST>::BYTES : 0);
 };
 
-// Collision of one node from its 38 pulled populations f and the density
-// ring (rzm, rz0, rzp: this node's column in the slots of planes z - 1, z,
-// z + 1; row r of a slot is r * RW further): momentum (Eq. 6), Shan-Chen
-// force (Eq. 7), common velocity with the force shift, BGK relaxation to the
-// equilibrium of Eq. 8 (Eqs. 9, 10) -- or, with MRT (float32 storage), the
-// moment relaxation of the generic kernel -- and the store of the
-// post-collision state (float32 populations with the rest population closing
-// the mass balance, or 16-bit deviations).  Also accumulates the
-// centre-of-mass partials of the droplet phase and flags non-finite
-// densities.  Shared by the row kernels so that every variant computes
-// bit-identical states.
+// collide_core on the density ring of the row kernels (rzm, rz0, rzp: this
+// node's column in the slots of planes z - 1, z, z + 1; row r of a slot is r *
+// RW further).
 template <int TX, typename ST, bool MRT = false>
 __device__ __forceinline__ void collide_node(const float2* rzm, const float2* rz0, const float2* rzp,
                                              const float (&f)[2][19], const float (&rs)[2], const FastModel& m,
                                              typename RowIO<TX, ST>::Out out, float (&cm)[4], int& bad, float px,
                                              float py, float pz) {
-    using IO = RowIO<TX, ST>;
     constexpr int RW = TX + 2;
     // neighbour densities {A, B} at offset (dx, dy, dz)
     auto nb = [&](int dx, int dy, int dz) -> float2 {
         const float2* r = dz == 0 ? rz0 : (dz > 0 ? rzp : rzm);
         return r[(dy + 1) * RW + dx];
     };
-    const float2 rho2 = rz0[RW];
-    const float rho[2] = {rho2.x, rho2.y};
-    // momentum (Eq. 6), opposite pairs differenced first
-    float j[2][3];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        float jx = 0.f, jy = 0.f, jz = 0.f;
-#pragma unroll
-        for (int i = 1; i < 19; i += 2) {
-            const float d = f[s][i] - f[s][i + 1];
-            if (cx_(i)) jx += (float)cx_(i) * d;
-            if (cy_(i)) jy += (float)cy_(i) * d;
-            if (cz_(i)) jz += (float)cz_(i) * d;
-        }
-        j[s][0] = jx; j[s][1] = jy; j[s][2] = jz;
-    }
-    // Shan-Chen force (Eq. 7) sums sum_i w_i rho_s(x + c_i) c_i, neighbour
-    // pairs differenced first; the weight folds into the multiplier
-    float acc[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-#pragma unroll
-    for (int i = 1; i < 19; i += 2) {
-        const float2 np = nb(cx_(i), cy_(i), cz_(i)), nm = nb(-cx_(i), -cy_(i), -cz_(i));
-        const float dA = np.x - nm.x, dB = np.y - nm.y;
-        if (cx_(i)) { acc[0][0] += (wgt<float>(i) * cx_(i)) * dA; acc[1][0] += (wgt<float>(i) * cx_(i)) * dB; }
-        if (cy_(i)) { acc[0][1] += (wgt<float>(i) * cy_(i)) * dA; acc[1][1] += (wgt<float>(i) * cy_(i)) * dB; }
-        if (cz_(i)) { acc[0][2] += (wgt<float>(i) * cz_(i)) * dA; acc[1][2] += (wgt<float>(i) * cz_(i)) * dB; }
-    }
-    const float den = rho[0] * m.inv_tau[0] + rho[1] * m.inv_tau[1];
-    const float rden = __frcp_rn(den);
-    float up[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) up[a] = (j[0][a] * m.inv_tau[0] + j[1][a] * m.inv_tau[1]) * rden;
-    if (!(isfinite(rho[0]) && isfinite(rho[1]))) bad |= 1;
-    {
-        const float phi = __fdividef(rho[0] - rho[1], rho[0] + rho[1]);
-        const float w = fmaxf(phi, 0.f);
-        cm[0] += w;
-        cm[1] = fmaf(w, px, cm[1]);
-        cm[2] = fmaf(w, py, cm[2]);
-        cm[3] = fmaf(w, pz, cm[3]);
-    }
-    if constexpr (is_dev_t<ST>::value) {
-        // 16-bit deviations from w_i times the density of the node each
-        // population streams to (this CTA's density planes), the pair of
-        // components of one direction in one word
-        // f holds the pulled deviations (f_i = w_i rho*_s + d_i, rs = rho*):
-        // (1 - 1/tau) f_i = (1 - 1/tau) d_i + (1 - 1/tau) w_i rho*_s, whose
-        // second term joins the equilibrium's constant (W1 / W2 below), and
-        // the momentum's opposite-pair differences are those of the d_i
-        using T = decltype(dev_tag(ST{}));
-        float ux[2], uy[2], uz[2], base[2], e1[2], e2[2], W1[2], W2[2];
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            ux[s] = fmaf(m.sh[s], acc[1 - s][0], up[0]);
-            uy[s] = fmaf(m.sh[s], acc[1 - s][1], up[1]);
-            uz[s] = fmaf(m.sh[s], acc[1 - s][2], up[2]);
-            base[s] = 1.f - 1.5f * (ux[s] * ux[s] + uy[s] * uy[s] + uz[s] * uz[s]);
-            const float ir = m.inv_tau[s] * rho[s];
-            e1[s] = ir * wgt<float>(1);  // axis directions
-            e2[s] = ir * wgt<float>(7);  // edge directions
-            const float orr = m.omit[s] * rs[s];
-            W1[s] = orr * wgt<float>(1);
-            W2[s] = orr * wgt<float>(7);
-        }
-        float others[2] = {0.f, 0.f};
-        sfor<9>([&](auto K) {
-            constexpr int i = 2 * decltype(K)::value + 1;
-            // densities of the destinations x + c_i and x - c_i (read again
-            // from shared memory rather than held since the force)
-            const float2 np = nb(cx_(i), cy_(i), cz_(i)), nm = nb(-cx_(i), -cy_(i), -cz_(i));
-            float da[2], dbv[2];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const float cu = (float)cx_(i) * ux[s] + (float)cy_(i) * uy[s] + (float)cz_(i) * uz[s];
-                const float e = i < 7 ? e1[s] : e2[s];
-                const float ev = fmaf(e, fmaf(4.5f * cu, cu, base[s]), i < 7 ? W1[s] : W2[s]);
-                const float od = (3.f * e) * cu;
-                const float oa = fmaf(m.omit[s], f[s][i], ev + od);
-                const float ob = fmaf(m.omit[s], f[s][i + 1], ev - od);
-                // deviations from w_i times the destinations' densities
-                da[s] = fmaf(-wgt<float>(i), s ? np.y : np.x, oa);
-                dbv[s] = fmaf(-wgt<float>(i), s ? nm.y : nm.x, ob);
-            }
-            const unsigned wa = dev_pack2<T>(da[0], da[1]), wb = dev_pack2<T>(dbv[0], dbv[1]);
-            IO::template store_word<i>(out, wa);
-            IO::template store_word<i + 1>(out, wb);
-            // the values the readers will rebuild, for the mass balance
-            const float2 qa = dev_unpack2<T>(wa), qb = dev_unpack2<T>(wb);
-            others[0] += fmaf(wgt<float>(i), np.x, qa.x) + fmaf(wgt<float>(i), nm.x, qb.x);
-            others[1] += fmaf(wgt<float>(i), np.y, qa.y) + fmaf(wgt<float>(i), nm.y, qb.y);
-        });
-        st_cs_f4(out.b, make_float4(rho[0], rho[1], rho[0] - others[0], rho[1] - others[1]));
-    } else {
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const float ux = fmaf(m.sh[s], acc[1 - s][0], up[0]);
-            const float uy = fmaf(m.sh[s], acc[1 - s][1], up[1]);
-            const float uz = fmaf(m.sh[s], acc[1 - s][2], up[2]);
-            const float r = rho[s];
-            // moving populations; the rest population then closes the mass
-            // balance exactly (sum of outputs = rho), which keeps fp32
-            // rounding from drifting the interface
-            float others = 0.f;
-            if constexpr (MRT) {
-                // MRT: relax the moments of the deviation from equilibrium
-                // (d'Humieres basis; momentum and stress at 1/tau)
-                // as BGK plus the free moments' part (mrt_free); the
-                // equilibria are evaluated twice rather than held
-                const float base = 1.f - 1.5f * (ux * ux + uy * uy + uz * uz);
-                const float e1 = r * wgt<float>(1), e2 = r * wgt<float>(7), it = m.inv_tau[s];
-                float g[7] = {f[s][0] - (r * wgt<float>(0)) * base, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                float o[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                auto deviations = [&](auto I, float& dp, float& dm) {
-                    constexpr int i = decltype(I)::value;
-                    const float cu = (float)cx_(i) * ux + (float)cy_(i) * uy + (float)cz_(i) * uz;
-                    const float e = i < 7 ? e1 : e2;
-                    const float ev = e * fmaf(4.5f * cu, cu, base);
-                    const float od = (3.f * e) * cu;
-                    dp = f[s][i] - (ev + od);
-                    dm = f[s][i + 1] - (ev - od);
-                };
-                sfor<9>([&](auto K) {
-                    constexpr int i = 2 * decltype(K)::value + 1;
-                    float dp, dm;
-                    deviations(std::integral_constant<int, i>{}, dp, dm);
-                    mrt_gather<float>(i, dp, dm, g, o);
-                });
-                float ce[7], co[9];
-                mrt_free<float>(g, o, it, m.mrt, ce, co);
-                sfor<9>([&](auto K) {
-                    constexpr int i = 2 * decltype(K)::value + 1;
-                    float dp, dm;
-                    deviations(std::integral_constant<int, i>{}, dp, dm);
-                    const float e = ce[mrt_group(i)], d = mrt_odd<float>(i, co);
-                    const float oa = fmaf(-it, dp, f[s][i]) - (e + d);
-                    const float ob = fmaf(-it, dm, f[s][i + 1]) - (e - d);
-                    if (s == 0) {
-                        IO::template store<0, i>(out, oa);
-                        IO::template store<0, i + 1>(out, ob);
-                    } else {
-                        IO::template store<1, i>(out, oa);
-                        IO::template store<1, i + 1>(out, ob);
-                    }
-                    others += oa + ob;
-                });
-            } else {
-                const float base = 1.f - 1.5f * (ux * ux + uy * uy + uz * uz);
-                const float ir = m.inv_tau[s] * r;
-                const float e1 = ir * wgt<float>(1), e2 = ir * wgt<float>(7);
-                const float om = m.omit[s];
-                sfor<9>([&](auto K) {
-                    constexpr int i = 2 * decltype(K)::value + 1;
-                    const float cu = (float)cx_(i) * ux + (float)cy_(i) * uy + (float)cz_(i) * uz;
-                    const float e = i < 7 ? e1 : e2;
-                    const float ev = e * fmaf(4.5f * cu, cu, base);
-                    const float od = (3.f * e) * cu;
-                    const float oa = fmaf(om, f[s][i], ev + od);
-                    const float ob = fmaf(om, f[s][i + 1], ev - od);
-                    if (s == 0) {
-                        IO::template store<0, i>(out, oa);
-                        IO::template store<0, i + 1>(out, ob);
-                    } else {
-                        IO::template store<1, i>(out, oa);
-                        IO::template store<1, i + 1>(out, ob);
-                    }
-                    others += oa + ob;
-                });
-            }
-            if (s == 0) IO::template store<0, 0>(out, r - others);
-            else IO::template store<1, 0>(out, r - others);
-        }
-    }
+    collide_core<RowIO<TX, ST>, ST, MRT>(nb, rz0[RW], f, rs, m, out, cm, bad, px, py, pz);
 }
 
 // Outer-halo share of a CTA of the direct and staged kernels: the rows just

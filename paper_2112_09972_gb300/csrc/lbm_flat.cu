@@ -232,7 +232,7 @@ Shape flat_shape(const Layout& L, int num_sms) {
     long long zc = (per_plane * L.Lz + want - 1) / want;
     if (zc < 1) zc = 1;
     while ((L.Lz + zc - 1) / zc > 65535) ++zc;
-    sh.flat = 1;
+    sh.flat = kFlat64;
     sh.tx = L.Lx;
     sh.ty = L.Lx >= kFlatThreads ? 1 : kFlatThreads / L.Lx;
     sh.zchunk = (int)zc;

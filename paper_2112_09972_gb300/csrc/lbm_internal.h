@@ -103,7 +103,7 @@ struct Grad {
 // Launch shape of the stream-collide kernel.
 struct Shape {
     int rows;       // 1: the row-tiled cluster kernel (lbm_fast.cu), 0: the generic tile kernel
-    int flat;       // 1: the two-pass kernels (lbm_flat.cu), which need a density array
+    int flat;       // kFlat64, kFlatRows or kFlatAny: two-pass kernels, which need a density array
     int tx, ty;     // tile of the x-y plane per CTA
     int zchunk;     // z planes marched per CTA
     int variant;    // row kernel: kRowDirect, kRowStaged or kRowWs
@@ -111,6 +111,11 @@ struct Shape {
     int threads;
     size_t smem;
 };
+
+// Two-pass kernels: float64 (lbm_flat.cu), small boxes of the row-tiled widths
+// in float32 or 16-bit storage and float32 boxes of other extents
+// (lbm_flat32.cu).
+enum { kFlat64 = 1, kFlatRows = 2, kFlatAny = 3 };
 
 // Rows per thread-block cluster of the row kernels (lbm_fast.cu).
 constexpr int kRowClusterRows = 8;
@@ -148,6 +153,16 @@ long long flat_rho_bytes(const Layout& L);
 cudaError_t launch_flat_fill(void* rho, const Layout& L, const Model& m, cudaStream_t s);
 cudaError_t launch_flat(const void* src, void* dst, void* rho, const Layout& L, const Model& m, const Shape& sh,
                         CentreParts cp, int* d_err, cudaStream_t s);
+
+// ---- two-pass kernels (lbm_flat32.cu): fp32 or 16-bit deviations, ghost boundary ----
+Shape flat_rows_shape(const Shape& rows);
+Shape flat_any_shape(const Layout& L, int num_sms);
+long long flat32_rho_bytes(const Layout& L);
+cudaError_t launch_flat32_fill(void* rho, const Layout& L, const Model& m, cudaStream_t s);
+cudaError_t launch_flat_rows(int prec, const void* src, void* dst, void* rho, const Layout& L, const Model& m,
+                             const Shape& sh, CentreParts cp, int* d_err, cudaStream_t s);
+cudaError_t launch_flat_any(const void* src, void* dst, void* rho, const Layout& L, const Model& m, const Shape& sh,
+                            CentreParts cp, int* d_err, cudaStream_t s);
 
 // ---- row-tiled cluster kernel (lbm_fast.cu): fp32 or 16-bit deviations, ghost boundary,
 //      Lx in {32, 64, 128, 256}, Ly % 8 == 0 ----

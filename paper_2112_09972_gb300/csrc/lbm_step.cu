@@ -236,6 +236,11 @@ cudaError_t stream_collide_t(const void* src, void* dst, const Layout& L, const 
     return cudaGetLastError();
 }
 
+// Largest box of a row-tiled width on the two-pass kernels: their second read
+// of the populations has to come from L2.  Per step, two-pass against cluster
+// kernel: 64 x 40 x 23 fp32 13.8 us (39.1), 64^3 fp32 30.8 (37.2) and bf16 26.6
+// (34.7), 256 x 32 x 32 fp32 24.4 (39.2); 128 x 64 x 64 fp32 50.1 (46.9).
+constexpr long long kFlatRowsNodes = 3 << 17;
 constexpr int kMaxThreadsF32 = 512;
 constexpr int kMaxThreadsF64 = 256;
 
@@ -312,9 +317,15 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
             sh.grid = dim3(1, L.Ly, (L.Lz + sh.zchunk - 1) / sh.zchunk);
             sh.threads = L.Lx;
             sh.smem = 0;
+            if (allow_flat && variant_req == 0 && zchunk_req <= 0 && (long long)L.Lx * L.Ly * L.Lz <= kFlatRowsNodes)
+                return flat_rows_shape(sh);
             return sh;
         }
     }
+    // float32 boxes of other extents: two-pass at every size (per step against
+    // the tile kernel: 37 x 29 x 23 12.7 us (33.7), 60 x 50 x 44 19.7 (32.8), 96^3
+    // 92.8 (117), 200 x 200 x 100 337 (464))
+    if (allow_flat && prec == kFP32 && !periodic && ty_req <= 0 && zchunk_req <= 0) return flat_any_shape(L, num_sms);
     const int cbytes = prec == kFP64 ? 8 : 4;  // compute type of the density ring
     const int maxt = prec == kFP64 ? kMaxThreadsF64 : kMaxThreadsF32;
     sh.tx = L.Lx <= maxt ? L.Lx : 128;
@@ -389,7 +400,9 @@ cudaError_t launch_centre(int prec, const void* f, const Layout& L, CentreParts 
 cudaError_t launch_stream_collide(int prec, const void* src, void* dst, const Layout& L, const Model& m,
                                   const Shape& sh, const Grad& A, void* rho, CentreParts cp, int* d_err,
                                   cudaStream_t s) {
-    if (sh.flat) return launch_flat(src, dst, rho, L, m, sh, cp, d_err, s);
+    if (sh.flat == kFlat64) return launch_flat(src, dst, rho, L, m, sh, cp, d_err, s);
+    if (sh.flat == kFlatRows) return launch_flat_rows(prec, src, dst, rho, L, m, sh, cp, d_err, s);
+    if (sh.flat == kFlatAny) return launch_flat_any(src, dst, rho, L, m, sh, cp, d_err, s);
     if (sh.rows) return launch_stream_collide_rows(prec, sh.variant, src, dst, L, m, A, sh.zchunk, cp, d_err, s);
     if (prec == kFP64) return stream_collide_t<double, double, kMaxThreadsF64>(src, dst, L, m, sh, cp, d_err, s);
     if (prec == kFP32) return stream_collide_t<float, float, kMaxThreadsF32>(src, dst, L, m, sh, cp, d_err, s);
