@@ -17,7 +17,7 @@
 //                  float32 accumulation) for the shapes k_gemm_tc does not
 //                  tile (M not a multiple of 128, N not of 32, K not of 64)
 //   k_transpose -- bfloat16 tile transpose (operands of the weight gradients)
-//   k_prep, k_loss_grad, k_colsum_*, k_splitsum, k_adam, k_weights, k_output,
+//   k_prep*, k_loss_grad, k_colsum_part, k_splitsum, k_update, k_weights, k_output,
 //   k_deform_from_m -- input normalisation, mean-square loss and its
 //                  gradient, bias gradients, the sum of split-K partial
 //                  weight gradients, Adam, bfloat16 weight copies,
@@ -42,6 +42,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_eigen.cuh"
+#include "lbm_pdl.cuh"
 
 namespace lbmgb_mlp {
 
@@ -69,6 +70,10 @@ struct GemmArgs {
     // Cf + z c_split.  k_len = 0: one slice.
     int k_len;
     long long c_split;
+    // bfloat16 outputs also transposed, Ct[n ldt + m] (NULL: not wanted): the
+    // operands of the weight gradients
+    bf16* Ct;
+    int ldt;
 };
 
 // The K slice of blockIdx.z (see GemmArgs::k_len).
@@ -103,6 +108,8 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], 
 __global__ void __launch_bounds__(kGemmThreads) k_gemm_nt(GemmArgs g) {
     __shared__ __align__(16) bf16 sA[2][BM][SROW];
     __shared__ __align__(16) bf16 sB[2][BN][SROW];
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     gemm_slice(g);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
@@ -186,9 +193,14 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_nt(GemmArgs g) {
                 switch (g.epi) {
                     case kStoreF32: g.Cf[o] = v; break;
                     case kBiasF32: g.Cf[o] = v + g.bias[n]; break;
-                    case kBiasReluBf16: g.Cb[o] = __float2bfloat16_rn(fmaxf(v + g.bias[n], 0.f)); break;
-                    default:
-                        g.Cb[o] = __float2bfloat16_rn(__bfloat162float(g.mask[(long long)m * g.ldm + n]) > 0.f ? v : 0.f);
+                    default: {
+                        const bf16 h = __float2bfloat16_rn(
+                            g.epi == kBiasReluBf16
+                                ? fmaxf(v + g.bias[n], 0.f)
+                                : (__bfloat162float(g.mask[(long long)m * g.ldm + n]) > 0.f ? v : 0.f));
+                        g.Cb[o] = h;
+                        if (g.Ct) g.Ct[(long long)n * g.ldt + m] = h;
+                    }
                 }
             }
 }
@@ -356,6 +368,14 @@ __device__ __forceinline__ void tc_store32(const GemmArgs& g, float* Cf, int m, 
             w[e] = *reinterpret_cast<const unsigned*>(&h);
         }
         dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
+        if (g.Ct) {  // the lanes of a warp hold consecutive rows: 64 bytes per column
+            unsigned short* ct = reinterpret_cast<unsigned short*>(g.Ct) + (long long)(n + 8 * q) * g.ldt + m;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                ct[(long long)(2 * e) * g.ldt] = (unsigned short)(w[e] & 0xFFFFu);
+                ct[(long long)(2 * e + 1) * g.ldt] = (unsigned short)(w[e] >> 16);
+            }
+        }
     }
 }
 
@@ -399,6 +419,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *tmem_slot;
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
 
     const int tiles_mn = sh.m_tiles * sh.n_tiles, tiles = tiles_mn * sh.slices;
     // K range of a tile: chunks [k0 / 64, k0 / 64 + nk)
@@ -660,6 +682,8 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *tmem_slot;
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
 
     const int mine = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // tiles of this CTA
     const int L = a.layers, nk0 = a.d0 / TC_K;
@@ -865,6 +889,8 @@ namespace {
 // Normalised input in bfloat16: xb[r, c] = (x[r, c] - mean[c]) scale[c].
 __global__ void k_prep(const float* __restrict__ x, long long n, int d0, const float* __restrict__ mean,
                        const float* __restrict__ scale, bf16* __restrict__ xb) {
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n * d0) return;
     const int c = (int)(e % d0);
@@ -875,6 +901,8 @@ __global__ void k_prep(const float* __restrict__ x, long long n, int d0, const f
 // two float4 loads, one 16-byte store.
 __global__ void k_prep8(const float4* __restrict__ x, long long n8, int d08, const float4* __restrict__ mean,
                         const float4* __restrict__ scale, uint4* __restrict__ xb) {
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n8) return;
     const int c = (int)(e % d08);
@@ -891,9 +919,34 @@ __global__ void k_prep8(const float4* __restrict__ x, long long n8, int d08, con
     xb[e] = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// k_prep with the transposed copy xt[c ldt + r] beside it (32 x 32 tiles
+// through shared memory; d0 is a multiple of 32).
+__global__ void k_prep_t(const float* __restrict__ x, int n, int d0, const float* __restrict__ mean,
+                         const float* __restrict__ scale, bf16* __restrict__ xb, bf16* __restrict__ xt, int ldt) {
+    __shared__ bf16 tile[32][33];
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
+    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    const int c = c0 + threadIdx.x;
+    const float mu = mean[c], sc = scale[c];
+    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+        const int r = r0 + k;
+        if (r >= n) break;
+        const bf16 b = __float2bfloat16_rn((x[(long long)r * d0 + c] - mu) * sc);
+        xb[(long long)r * d0 + c] = b;
+        tile[k][threadIdx.x] = b;
+    }
+    __syncthreads();
+    const int r = r0 + threadIdx.x;
+    for (int k = threadIdx.y; k < 32; k += blockDim.y)
+        if (r < n) xt[(long long)(c0 + k) * ldt + r] = tile[threadIdx.x][k];
+}
+
 // out[c, r] = in[r, c] for an R x C matrix (32 x 32 tiles through shared memory).
 __global__ void k_transpose(const bf16* __restrict__ in, int R, int C, int ldi, bf16* __restrict__ out, int ldo) {
     __shared__ bf16 tile[32][33];
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     for (int k = threadIdx.y; k < 32; k += blockDim.y) {
         const int r = r0 + k, c = c0 + threadIdx.x;
@@ -907,15 +960,22 @@ __global__ void k_transpose(const bf16* __restrict__ in, int R, int C, int ldi, 
 }
 
 // Output-layer gradient g = 2 (y_hat - t_hat) / (n dL) in bfloat16 (zero in
-// the padding columns dL .. ldg-1) and per-block partial sums of the squared
-// error (float64).
+// the padding columns dL .. ldg-1), its transposed copy gt[c n + r], and the
+// mean squared error: per-block partial sums (float64), which the last block
+// to finish adds in a fixed order (thread t takes partials t, t + 256, ...,
+// then a tree over threads), so the result does not depend on scheduling.
 constexpr int kLossThreads = 256;
 __global__ void __launch_bounds__(kLossThreads) k_loss_grad(const float* __restrict__ yhat, int ldy,
                                                             const float* __restrict__ tgt, int n, int dL, int ldg,
                                                             const float* __restrict__ ymean,
                                                             const float* __restrict__ yscale, bf16* __restrict__ g,
-                                                            double* __restrict__ parts) {
-    __shared__ double red[kLossThreads / 32];
+                                                            bf16* __restrict__ gt, double* __restrict__ parts,
+                                                            unsigned* __restrict__ counter, double count,
+                                                            double* __restrict__ loss) {
+    __shared__ double red[kLossThreads];
+    __shared__ unsigned last;
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;  // n ldg <= 2^22 x 32
     double sq = 0.0;
     if (e < n * ldg) {
@@ -927,7 +987,9 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_grad(const float* __restr
             sq = (double)d * (double)d;
             gv = 2.f * d / (float)((long long)n * dL);
         }
-        g[e] = __float2bfloat16_rn(gv);
+        const bf16 h = __float2bfloat16_rn(gv);
+        g[e] = h;
+        if (gt) gt[(long long)c * n + r] = h;
     }
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_down_sync(0xffffffffu, sq, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
@@ -936,60 +998,73 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_grad(const float* __restr
         double s = 0.0;
         for (int w = 0; w < kLossThreads / 32; ++w) s += red[w];
         parts[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1 ? 1u : 0u;
     }
-}
-
-// Sum of the partials divided by count: the mean loss.  A fixed summation
-// order (thread t takes partials t, t + 256, ..., then a tree over threads),
-// so the result does not depend on scheduling.
-constexpr int kLossFinalThreads = 256;
-__global__ void __launch_bounds__(kLossFinalThreads) k_loss_final(const double* __restrict__ parts, int nparts,
-                                                                  double count, double* __restrict__ out) {
-    __shared__ double red[kLossFinalThreads];
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     double s = 0.0;
-    for (int b = threadIdx.x; b < nparts; b += kLossFinalThreads) s += parts[b];
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += kLossThreads) s += __ldcg(parts + b);
     red[threadIdx.x] = s;
     __syncthreads();
-    for (int o = kLossFinalThreads / 2; o > 0; o >>= 1) {
+    for (int o = kLossThreads / 2; o > 0; o >>= 1) {
         if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = red[0] / count;
+    if (threadIdx.x == 0) {
+        *loss = red[0] / count;
+        *counter = 0u;
+    }
 }
 
-// Bias gradient db[c] = sum_r g[r, c] of a bfloat16 [n, C] matrix, in two
-// passes with a fixed order: block (x, s) sums rows [s rows, (s + 1) rows)
-// of 32 columns (8 row phases, then the phases in order) into parts[s, c];
-// k_colsum_final adds the slices in order.
+// What the update of one layer reads and writes: the float32 gradient of its
+// weights as S slices at ws (S = 1: complete in the gradient array), the
+// bias gradient as cs_n partial column sums at cs, and the bfloat16 copies.
+constexpr int kMaxLayers = 16;
+struct LayerTable {
+    struct Layer {
+        long long offW, count, ws, cs;  // offsets in the parameter, workspace and column-sum arrays
+        int S, dout, din;
+        const bf16* G;
+        bf16 *Wb, *WTb;
+    } l[kMaxLayers];
+    int layers, cs_n;
+    long long nparam;
+};
+
+// Bias gradients db[c] = sum_r G_l[r, c] of every layer (blockIdx.z), first
+// pass: block (x, s) sums rows [s rows, (s + 1) rows) of 32 columns (8 row
+// phases, then the phases in order) into parts[cs_l + s dout + c]; the update
+// adds the slices in order.
 constexpr int kColSlices = 128;
-__global__ void __launch_bounds__(256) k_colsum_part(const bf16* __restrict__ g, int n, int C, int ldg, int rows,
+__global__ void __launch_bounds__(256) k_colsum_part(const __grid_constant__ LayerTable tb, int n, int rows,
                                                      float* __restrict__ parts) {
     __shared__ float red[8][33];
-    const int c = blockIdx.x * 32 + threadIdx.x;
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
+    const LayerTable::Layer& q = tb.l[blockIdx.z];
+    const int C = q.dout, c = blockIdx.x * 32 + threadIdx.x;
+    if (blockIdx.x * 32 >= C) return;
+    const bf16* g = q.G;
     const int r0 = blockIdx.y * rows, r1 = min(n, r0 + rows);
     float s = 0.f;
     if (c < C)
-        for (int r = r0 + threadIdx.y; r < r1; r += 8) s += __bfloat162float(g[(long long)r * ldg + c]);
+        for (int r = r0 + threadIdx.y; r < r1; r += 8) s += __bfloat162float(g[(long long)r * C + c]);
     red[threadIdx.y][threadIdx.x] = s;
     __syncthreads();
     if (threadIdx.y == 0 && c < C) {
         float t = red[0][threadIdx.x];
         for (int k = 1; k < 8; ++k) t += red[k][threadIdx.x];
-        parts[(long long)blockIdx.y * C + c] = t;
+        parts[q.cs + (long long)blockIdx.y * C + c] = t;
     }
-}
-
-__global__ void k_colsum_final(const float* __restrict__ parts, int S, int C, float* __restrict__ db) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    float s = 0.f;
-    for (int z = 0; z < S; ++z) s += parts[(long long)z * C + c];
-    db[c] = s;
 }
 
 // out[e] = sum over the S K slices of ws[z count + e], in slice order.
 constexpr int kMaxSplit = 32;
 __global__ void k_splitsum(const float* __restrict__ ws, int S, long long count, float* __restrict__ out) {
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= count) return;
     float s = ws[e];
@@ -997,18 +1072,53 @@ __global__ void k_splitsum(const float* __restrict__ ws, int S, long long count,
     out[e] = s;
 }
 
-// Adam on float32 parameters (bias-corrected moments).
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
-                       float c2) {
+// The gradient of every parameter from its partial sums, in slice order, and
+// with ADAM the step itself on the float32 parameters (bias-corrected
+// moments) and the refreshed bfloat16 weight copies W and W^T; without ADAM
+// the gradients go to g.  One launch in place of a slice sum, a column sum
+// and a weight copy per layer and the Adam step.
+template <bool ADAM>
+__global__ void __launch_bounds__(256) k_update(const __grid_constant__ LayerTable tb, const float* __restrict__ ws,
+                                                const float* __restrict__ cs, float* __restrict__ g,
+                                                float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
+                                                float lr, float b1, float b2, float eps, float c1, float c2) {
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const float ge = g[e];
+    if (e >= tb.nparam) return;
+    int l = 0;
+    while (l + 1 < tb.layers && e >= tb.l[l + 1].offW) ++l;
+    const LayerTable::Layer& q = tb.l[l];
+    const long long k = e - q.offW;
+    float ge;
+    if (k < q.count) {
+        if (q.S > 1) {
+            ge = ws[q.ws + k];
+            for (int z = 1; z < q.S; ++z) ge += ws[q.ws + (long long)z * q.count + k];
+        } else {
+            ge = g[e];
+        }
+    } else {
+        const long long c = k - q.count;
+        ge = 0.f;
+        for (int z = 0; z < tb.cs_n; ++z) ge += cs[q.cs + (long long)z * q.dout + c];
+    }
+    if (!ADAM) {
+        g[e] = ge;
+        return;
+    }
     const float me = b1 * m[e] + (1.f - b1) * ge;
     const float ve = b2 * v[e] + (1.f - b2) * ge * ge;
     m[e] = me;
     v[e] = ve;
-    p[e] -= lr * (me / c1) / (sqrtf(ve / c2) + eps);
+    const float pe = p[e] - lr * (me / c1) / (sqrtf(ve / c2) + eps);
+    p[e] = pe;
+    if (k < q.count) {
+        const int r = (int)(k / q.din), c = (int)(k - (long long)r * q.din);
+        const bf16 b = __float2bfloat16_rn(pe);
+        q.Wb[k] = b;
+        q.WTb[(long long)c * q.dout + r] = b;
+    }
 }
 
 // bfloat16 copies of a float32 weight matrix W [R, C]: Wb = W and WTb = W^T.
@@ -1025,6 +1135,8 @@ __global__ void k_weights(const float* __restrict__ W, int R, int C, bf16* __res
 // Outputs in physical units: y[r, c] = y_hat[r, c] / scale[c] + mean[c].
 __global__ void k_output(const float* __restrict__ yhat, int ldy, long long n, int dL,
                          const float* __restrict__ mean, const float* __restrict__ scale, float* __restrict__ y) {
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n * dL) return;
     const long long r = e / dL;
@@ -1036,6 +1148,8 @@ __global__ void k_output(const float* __restrict__ yhat, int ldy, long long n, i
 // xz, yy, yz, zz): D = (sqrt(l1) - sqrt(l3)) / (sqrt(l1) + sqrt(l3)) of its
 // eigenvalues (D does not depend on the normalisation of M).
 __global__ void k_deform_from_m(const float* __restrict__ m6, long long n, double* __restrict__ D) {
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const float* q = m6 + 6 * r;
@@ -1068,15 +1182,23 @@ struct lbm_mlp {
     std::vector<bf16*> H;        // H[0] the normalised input, H[l] hidden layer l
     float* yhat;                 // [max_batch, dp_L]
     std::vector<bf16*> G;        // G[l] gradient with respect to z_l, [max_batch, dp_l]
-    bf16 *T1, *T2;               // transposes for the weight gradients
+    // operands of the weight gradients, the batch index contiguous: GT[q] of
+    // the gradients (two layers in flight), HT[l] of the activations (NULL
+    // where there was no room: they are then transposed into T2 in turn)
+    bf16* GT[2];
+    std::vector<bf16*> HT;
+    bf16* T2;
+    bool ht_tried;
     double *loss_parts, *loss;
-    int loss_blocks;
+    unsigned* loss_counter;
     double* h_loss;              // pinned
     int tensor_path;             // 0: tcgen05 where the shape allows, 1: mma.sync only
     int* d_err;                  // bit 1: a bounded tensor-core wait gave up
     int sms;                     // multiprocessors of the device
-    float* ws;                   // split-K partials, kMaxSplit x the largest weight matrix
-    float* cs_parts;             // column-sum partials, kColSlices x the widest layer
+    float* ws;                   // split-K partials, kMaxSplit x every weight matrix (ws_all) or the largest
+    bool ws_all;
+    float* cs_parts;             // column-sum partials, kColSlices x the sum of the widths
+    LayerTable table;            // the update's view of the layers
     bool fused;                  // k_mlp_forward takes this network's shapes
     FwArgs fw;                   // its weights' tensor maps and constants (rows and pointers set per call)
 };
@@ -1148,6 +1270,21 @@ int tc_bn(const lbm_mlp* c, const GemmArgs& a) {
     return ok ? bn : 0;
 }
 
+// Launch of a kernel whose prologue may overlap its predecessor's end
+// (every kernel of this file waits before its first global read).
+template <typename... P, typename... A>
+cudaError_t launch(lbm_mlp* c, void (*k)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute attr[1] = {lbmgb::pdl_attribute()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
+}
+
 cudaError_t launch_gemm(lbm_mlp* c, const GemmArgs& a, int slices) {
     const int bn = tc_bn(c, a);
     CUtensorMap ma, mb;
@@ -1155,12 +1292,10 @@ cudaError_t launch_gemm(lbm_mlp* c, const GemmArgs& a, int slices) {
         const TcShape sh{a.M / TC_M, a.N / bn, slices, bn};
         const long long tiles = (long long)sh.m_tiles * sh.n_tiles * slices;
         const int grid = (int)std::min<long long>(tiles, c->sms);  // persistent: one CTA per SM at most
-        k_gemm_tc<<<grid, kTcThreads, kTcSmem, c->stream>>>(ma, mb, a, sh, c->d_err);
-    } else {
-        const dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM, slices);
-        k_gemm_nt<<<grid, kGemmThreads, 0, c->stream>>>(a);
+        return launch(c, k_gemm_tc, dim3(grid), dim3(kTcThreads), kTcSmem, ma, mb, a, sh, c->d_err);
     }
-    return cudaGetLastError();
+    const dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM, slices);
+    return launch(c, k_gemm_nt, grid, dim3(kGemmThreads), 0, a);
 }
 
 GemmArgs gemm_args(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, int epi, const float* bias,
@@ -1168,21 +1303,24 @@ GemmArgs gemm_args(const bf16* A, int lda, const bf16* B, int ldb, int M, int N,
     GemmArgs a;
     a.A = A; a.B = B; a.lda = lda; a.ldb = ldb; a.M = M; a.N = N; a.K = K; a.epi = epi;
     a.bias = bias; a.mask = mask; a.ldm = ldm; a.Cf = Cf; a.Cb = Cb; a.ldc = ldc;
-    a.k_len = 0; a.c_split = 0;
+    a.k_len = 0; a.c_split = 0; a.Ct = nullptr; a.ldt = 0;
     return a;
 }
 
 cudaError_t gemm(lbm_mlp* c, const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, int epi,
-                 const float* bias, const bf16* mask, int ldm, float* Cf, bf16* Cb, int ldc) {
-    return launch_gemm(c, gemm_args(A, lda, B, ldb, M, N, K, epi, bias, mask, ldm, Cf, Cb, ldc), 1);
+                 const float* bias, const bf16* mask, int ldm, float* Cf, bf16* Cb, int ldc, bf16* Ct = nullptr) {
+    GemmArgs a = gemm_args(A, lda, B, ldb, M, N, K, epi, bias, mask, ldm, Cf, Cb, ldc);
+    a.Ct = Ct;
+    a.ldt = M;
+    return launch_gemm(c, a, 1);
 }
 
 // out [M, N] (row stride N) = A B^T for a long K (the batch of the weight
 // gradients): K is cut into slices so that there are about two tiles x
-// slices per SM, each slice at least 8 K chunks; the float32 partials go to the
-// workspace and k_splitsum adds them in slice order.
+// slices per SM, each slice at least 8 K chunks; the float32 partials go to ws.
+// *S: the slices, which the caller adds in order (1: out is complete).
 cudaError_t gemm_long_k(lbm_mlp* c, const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K,
-                        float* out) {
+                        float* out, float* ws, int* slices_out) {
     GemmArgs a = gemm_args(A, lda, B, ldb, M, N, K, kStoreF32, nullptr, nullptr, 0, out, nullptr, N);
     const int bn = tc_bn(c, a);
     const int unit = bn ? TC_K : BK;
@@ -1190,22 +1328,18 @@ cudaError_t gemm_long_k(lbm_mlp* c, const bf16* A, int lda, const bf16* B, int l
         bn ? (long long)(M / TC_M) * (N / bn) : (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
     long long S = std::max(1LL, 2LL * c->sms / tiles);
     S = std::min<long long>(std::min<long long>(S, kMaxSplit), std::max(1, K / (8 * unit)));
+    *slices_out = 1;
     if (S <= 1) return launch_gemm(c, a, 1);
     const int k_len = (int)(((K + S - 1) / S + unit - 1) / unit * unit);
-    const int slices = (K + k_len - 1) / k_len;
-    a.Cf = c->ws;
+    a.Cf = ws;
     a.k_len = k_len;
     a.c_split = (long long)M * N;
-    cudaError_t e = launch_gemm(c, a, slices);
-    if (e != cudaSuccess) return e;
-    k_splitsum<<<blocks_for(a.c_split, 256), 256, 0, c->stream>>>(c->ws, slices, a.c_split, out);
-    return cudaGetLastError();
+    *slices_out = (K + k_len - 1) / k_len;
+    return launch_gemm(c, a, *slices_out);
 }
 
 cudaError_t transpose(lbm_mlp* c, const bf16* in, int R, int C, int ldi, bf16* out, int ldo) {
-    const dim3 grid((C + 31) / 32, (R + 31) / 32), block(32, 8);
-    k_transpose<<<grid, block, 0, c->stream>>>(in, R, C, ldi, out, ldo);
-    return cudaGetLastError();
+    return launch(c, k_transpose, dim3((C + 31) / 32, (R + 31) / 32), dim3(32, 8), 0, in, R, C, ldi, out, ldo);
 }
 
 cudaError_t refresh_weights(lbm_mlp* c) {
@@ -1218,26 +1352,48 @@ cudaError_t refresh_weights(lbm_mlp* c) {
 }
 
 // Forward pass of n <= max_batch samples (inputs x on the device, float32
-// [n, d0]): activations into H, normalised outputs into yhat.
-cudaError_t forward(lbm_mlp* c, const float* x, int n) {
+// [n, d0]): activations into H (train: and transposed into HT), normalised
+// outputs into yhat.
+cudaError_t forward(lbm_mlp* c, const float* x, int n, bool train) {
     const int d0 = c->d[0];
-    if (aligned16(x)) {  // d0 is a multiple of 32
+    const bool ht = train && c->HT[0];
+    cudaError_t e;
+    if (ht) {
+        e = launch(c, k_prep_t, dim3(d0 / 32, (n + 31) / 32), dim3(32, 8), 0, x, n, d0, (const float*)c->x_mean,
+                   (const float*)c->x_scale, c->H[0], c->HT[0], n);
+    } else if (aligned16(x)) {  // d0 is a multiple of 32
         const long long n8 = (long long)n * d0 / 8;
-        k_prep8<<<blocks_for(n8, 256), 256, 0, c->stream>>>(reinterpret_cast<const float4*>(x), n8, d0 / 8,
-                                                            reinterpret_cast<const float4*>(c->x_mean),
-                                                            reinterpret_cast<const float4*>(c->x_scale),
-                                                            reinterpret_cast<uint4*>(c->H[0]));
+        e = launch(c, k_prep8, dim3(blocks_for(n8, 256)), dim3(256), 0, reinterpret_cast<const float4*>(x), n8, d0 / 8,
+                   reinterpret_cast<const float4*>(c->x_mean), reinterpret_cast<const float4*>(c->x_scale),
+                   reinterpret_cast<uint4*>(c->H[0]));
     } else {
-        k_prep<<<blocks_for((long long)n * d0, 256), 256, 0, c->stream>>>(x, n, d0, c->x_mean, c->x_scale, c->H[0]);
+        e = launch(c, k_prep, dim3(blocks_for((long long)n * d0, 256)), dim3(256), 0, x, (long long)n, d0,
+                   (const float*)c->x_mean, (const float*)c->x_scale, c->H[0]);
     }
-    cudaError_t e = cudaGetLastError();
     for (int l = 1; l <= c->L && e == cudaSuccess; ++l) {
         const bool last = l == c->L;
         e = gemm(c, c->H[l - 1], c->d[l - 1], c->Wb[l], c->d[l - 1], n, c->dp[l], c->d[l - 1],
                  last ? kBiasF32 : kBiasReluBf16, c->p + c->offb[l], nullptr, 0, last ? c->yhat : nullptr,
-                 last ? nullptr : c->H[l], c->dp[l]);
+                 last ? nullptr : c->H[l], c->dp[l], ht && !last ? c->HT[l] : nullptr);
     }
     return e;
+}
+
+// The transposed activations of training, allocated when it is first asked
+// for (all of them or none).
+void training_buffers(lbm_mlp* c) {
+    if (c->ht_tried) return;
+    c->ht_tried = true;
+    for (int l = 0; l < c->L; ++l)
+        if (cudaMalloc((void**)&c->HT[l], sizeof(bf16) * (size_t)c->max_batch * c->d[l]) != cudaSuccess) {
+            cudaGetLastError();
+            c->HT[l] = nullptr;
+            for (int k = 0; k < l; ++k) {
+                cudaFree(c->HT[k]);
+                c->HT[k] = nullptr;
+            }
+            return;
+        }
 }
 
 // k_mlp_forward's constants: input width a multiple of 64, two layers or more,
@@ -1284,42 +1440,56 @@ cudaError_t fused_forward(lbm_mlp* c, const float* x, float* y, int64_t rows) {
         a.tiles = (int)std::min<int64_t>(kMaxTiles, rows / TC_M - t0);
         a.x = x + t0 * TC_M * c->d[0];
         a.y = y + t0 * TC_M * c->d[c->L];
-        k_mlp_forward<<<std::min(a.tiles, c->sms), kFwThreads, kFwSmem, c->stream>>>(a);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch(c, k_mlp_forward, dim3(std::min(a.tiles, c->sms)), dim3(kFwThreads), kFwSmem, a);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-// Loss and parameter gradients of n samples (targets t on the device, float32 [n, dL]).
+// Loss and the partial sums of the parameter gradients of n samples (targets t
+// on the device, float32 [n, dL]); k_update adds them.
 cudaError_t backward(lbm_mlp* c, const float* t, int n) {
     const int L = c->L, dL = c->d[L], dLp = c->dp[L];
-    const long long ne = (long long)n * dLp;
-    const int nb = (int)blocks_for(ne, kLossThreads);
-    k_loss_grad<<<nb, kLossThreads, 0, c->stream>>>(c->yhat, dLp, t, n, dL, dLp, c->y_mean, c->y_scale, c->G[L],
-                                                    c->loss_parts);
-    k_loss_final<<<1, kLossFinalThreads, 0, c->stream>>>(c->loss_parts, nb, (double)n * dL, c->loss);
-    cudaError_t e = cudaGetLastError();
+    const int nb = (int)blocks_for((long long)n * dLp, kLossThreads);
+    cudaError_t e = launch(c, k_loss_grad, dim3(nb), dim3(kLossThreads), 0, (const float*)c->yhat, dLp, t, n, dL, dLp,
+                           (const float*)c->y_mean, (const float*)c->y_scale, c->G[L], c->GT[L & 1], c->loss_parts,
+                           c->loss_counter, (double)n * dL, c->loss);
+    const int S = (int)std::min<long long>(kColSlices, blocks_for(n, 256));
+    c->table.cs_n = S;
+    int widest = 0;
     for (int l = L; l >= 1 && e == cudaSuccess; --l) {
         const int dout = c->dp[l], din = c->d[l - 1];
+        LayerTable::Layer& q = c->table.l[l - 1];
+        widest = std::max(widest, dout);
         // dW_l = G_l^T H_{l-1}: operands with the batch index contiguous
-        e = transpose(c, c->G[l], n, dout, dout, c->T1, n);
-        if (e == cudaSuccess) e = transpose(c, c->H[l - 1], n, din, din, c->T2, n);
-        if (e == cudaSuccess) e = gemm_long_k(c, c->T1, n, c->T2, n, dout, din, n, c->g + c->offW[l]);
-        if (e == cudaSuccess) {
-            const int S = (int)std::min<long long>(kColSlices, blocks_for(n, 256));
-            const int rows = (n + S - 1) / S;
-            k_colsum_part<<<dim3((dout + 31) / 32, S), dim3(32, 8), 0, c->stream>>>(c->G[l], n, dout, dout, rows,
-                                                                                   c->cs_parts);
-            k_colsum_final<<<blocks_for(dout, 128), 128, 0, c->stream>>>(c->cs_parts, S, dout, c->g + c->offb[l]);
-            e = cudaGetLastError();
+        bf16* ht = c->HT[l - 1];
+        if (!ht) {
+            ht = c->T2;
+            e = transpose(c, c->H[l - 1], n, din, din, ht, n);
+        }
+        if (e == cudaSuccess)
+            e = gemm_long_k(c, c->GT[l & 1], n, ht, n, dout, din, n, c->g + c->offW[l], c->ws + q.ws, &q.S);
+        if (e == cudaSuccess && q.S > 1 && !c->ws_all) {  // the workspace is the next layer's too
+            e = launch(c, k_splitsum, dim3(blocks_for(q.count, 256)), dim3(256), 0, (const float*)c->ws, q.S, q.count,
+                       c->g + c->offW[l]);
+            q.S = 1;
         }
         // G_{l-1} = (G_l W_l) masked by h_{l-1} > 0
         if (l > 1 && e == cudaSuccess)
             e = gemm(c, c->G[l], dout, c->WTb[l], dout, n, din, dout, kMaskBf16, nullptr, c->H[l - 1], din, nullptr,
-                     c->G[l - 1], din);
+                     c->G[l - 1], din, c->GT[(l - 1) & 1]);
     }
+    if (e == cudaSuccess)
+        e = launch(c, k_colsum_part, dim3((widest + 31) / 32, S, L), dim3(32, 8), 0, c->table, n, (n + S - 1) / S,
+                   c->cs_parts);
     return e;
+}
+
+// Gradients into g (adam false), or one Adam step.
+cudaError_t update(lbm_mlp* c, bool adam, float lr, float c1, float c2) {
+    return launch(c, adam ? k_update<true> : k_update<false>, dim3(blocks_for(c->nparam, 256)), dim3(256), 0, c->table,
+                  (const float*)c->ws, (const float*)c->cs_parts, c->g, c->p, c->m, c->v, lr, 0.9f, 0.999f, 1e-8f, c1,
+                  c2);
 }
 
 }  // namespace
@@ -1392,6 +1562,7 @@ int lbm_mlp_create(lbm_mlp** out, int32_t nlayers, const int32_t* sizes, int32_t
     c->WTb.assign(nlayers + 1, nullptr);
     c->G.assign(nlayers + 1, nullptr);
     c->H.assign(nlayers, nullptr);
+    c->HT.assign(nlayers, nullptr);
     int widest = 0;
     for (int l = 0; l <= nlayers; ++l) widest = std::max(widest, c->dp[l]);
     for (int l = 1; l <= nlayers; ++l) {
@@ -1401,16 +1572,37 @@ int lbm_mlp_create(lbm_mlp** out, int32_t nlayers, const int32_t* sizes, int32_t
     }
     for (int l = 0; l < nlayers; ++l) alloc((void**)&c->H[l], sizeof(bf16) * (size_t)max_batch * c->d[l]);
     alloc((void**)&c->yhat, sizeof(float) * (size_t)max_batch * 32);
-    alloc((void**)&c->T1, sizeof(bf16) * (size_t)max_batch * widest);
+    for (int q = 0; q < 2; ++q) alloc((void**)&c->GT[q], sizeof(bf16) * (size_t)max_batch * widest);
     alloc((void**)&c->T2, sizeof(bf16) * (size_t)max_batch * widest);
-    c->loss_blocks = (int)blocks_for((long long)max_batch * 32, kLossThreads);
-    alloc((void**)&c->loss_parts, sizeof(double) * c->loss_blocks);
+    alloc((void**)&c->loss_parts, sizeof(double) * blocks_for((long long)max_batch * 32, kLossThreads));
+    alloc((void**)&c->loss_counter, sizeof(unsigned));
     alloc((void**)&c->loss, sizeof(double));
     alloc((void**)&c->d_err, sizeof(int));
-    long long largest = 0;
-    for (int l = 1; l <= nlayers; ++l) largest = std::max(largest, (long long)c->dp[l] * c->d[l - 1]);
-    alloc((void**)&c->ws, sizeof(float) * kMaxSplit * largest);
-    alloc((void**)&c->cs_parts, sizeof(float) * kColSlices * widest);
+    // the split-K partials of every layer up to 1 GB, else the largest layer's
+    long long largest = 0, all = 0, cols = 0;
+    c->table.layers = nlayers;
+    c->table.nparam = off;
+    for (int l = 1; l <= nlayers; ++l) {
+        LayerTable::Layer& q = c->table.l[l - 1];
+        q.offW = c->offW[l];
+        q.count = (long long)c->dp[l] * c->d[l - 1];
+        q.ws = kMaxSplit * all;
+        q.cs = kColSlices * cols;
+        q.S = 1;
+        q.dout = c->dp[l];
+        q.din = c->d[l - 1];
+        q.G = c->G[l];
+        q.Wb = c->Wb[l];
+        q.WTb = c->WTb[l];
+        largest = std::max(largest, q.count);
+        all += q.count;
+        cols += c->dp[l];
+    }
+    c->ws_all = all <= (1LL << 30) / (long long)(sizeof(float) * kMaxSplit);
+    if (!c->ws_all)
+        for (int l = 0; l < nlayers; ++l) c->table.l[l].ws = 0;
+    alloc((void**)&c->ws, sizeof(float) * kMaxSplit * (c->ws_all ? all : largest));
+    alloc((void**)&c->cs_parts, sizeof(float) * kColSlices * cols);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
     alloc((void**)&c->x_mean, sizeof(float) * c->d[0]);
     alloc((void**)&c->x_scale, sizeof(float) * c->d[0]);
@@ -1446,8 +1638,9 @@ void lbm_mlp_destroy(lbm_mlp* c) {
     for (bf16* q : c->WTb) cudaFree(q);
     for (bf16* q : c->G) cudaFree(q);
     for (bf16* q : c->H) cudaFree(q);
-    cudaFree(c->yhat); cudaFree(c->T1); cudaFree(c->T2);
-    cudaFree(c->loss_parts); cudaFree(c->loss); cudaFree(c->d_err); cudaFree(c->ws); cudaFree(c->cs_parts);
+    for (bf16* q : c->HT) cudaFree(q);
+    cudaFree(c->yhat); cudaFree(c->GT[0]); cudaFree(c->GT[1]); cudaFree(c->T2);
+    cudaFree(c->loss_parts); cudaFree(c->loss_counter); cudaFree(c->loss); cudaFree(c->d_err); cudaFree(c->ws); cudaFree(c->cs_parts);
     cudaFree(c->x_mean); cudaFree(c->x_scale); cudaFree(c->y_mean); cudaFree(c->y_scale);
     if (c->h_loss) cudaFreeHost(c->h_loss);
     if (c->own_stream) cudaStreamDestroy(c->stream);
@@ -1487,22 +1680,17 @@ namespace {
 // W_1 [d_1, d_0], b_1, W_2, b_2, ... (to_host: device -> host).
 int copy_params(lbm_mlp* c, float* dev, float* host, bool to_host) {
     cudaSetDevice(c->device);
-    long long h = 0;
-    for (int l = 1; l <= c->L; ++l) {
-        const size_t wbytes = sizeof(float) * (size_t)c->d[l] * c->d[l - 1];  // real rows are first
-        float* dw = dev + c->offW[l];
-        float* db = dev + c->offb[l];
-        if (to_host) {
-            MLP_TRY(cudaMemcpyAsync(host + h, dw, wbytes, cudaMemcpyDeviceToHost, c->stream));
-            h += (long long)c->d[l] * c->d[l - 1];
-            MLP_TRY(cudaMemcpyAsync(host + h, db, sizeof(float) * c->d[l], cudaMemcpyDeviceToHost, c->stream));
-        } else {
-            MLP_TRY(cudaMemcpyAsync(dw, host + h, wbytes, cudaMemcpyHostToDevice, c->stream));
-            h += (long long)c->d[l] * c->d[l - 1];
-            MLP_TRY(cudaMemcpyAsync(db, host + h, sizeof(float) * c->d[l], cudaMemcpyHostToDevice, c->stream));
-        }
-        h += c->d[l];
-    }
+    const cudaMemcpyKind kind = to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
+    auto copy = [&](long long at, float* h, long long n) {
+        return to_host ? cudaMemcpyAsync(h, dev + at, sizeof(float) * (size_t)n, kind, c->stream)
+                       : cudaMemcpyAsync(dev + at, h, sizeof(float) * (size_t)n, kind, c->stream);
+    };
+    // the layouts agree up to the last layer, whose rows are padded (real rows first)
+    const int L = c->L;
+    const long long head = c->offW[L], w = (long long)c->d[L] * c->d[L - 1];
+    if (head) MLP_TRY(copy(0, host, head));
+    MLP_TRY(copy(head, host + head, w));
+    MLP_TRY(copy(c->offb[L], host + head + w, c->d[L]));
     MLP_TRY(cudaStreamSynchronize(c->stream));
     return LBM_OK;
 }
@@ -1538,10 +1726,9 @@ int lbm_mlp_forward(lbm_mlp* c, const float* x, float* y, int64_t n) {
     MLP_TRY(fused_forward(c, x, y, rows));
     for (int64_t s = rows; s < n; s += c->max_batch) {
         const int k = (int)std::min<int64_t>(c->max_batch, n - s);
-        MLP_TRY(forward(c, x + s * d0, k));
-        k_output<<<blocks_for((long long)k * dL, 256), 256, 0, c->stream>>>(c->yhat, 32, k, dL, c->y_mean, c->y_scale,
-                                                                          y + s * dL);
-        MLP_TRY(cudaGetLastError());
+        MLP_TRY(forward(c, x + s * d0, k, false));
+        MLP_TRY(launch(c, k_output, dim3(blocks_for((long long)k * dL, 256)), dim3(256), 0, (const float*)c->yhat, 32,
+                       (long long)k, dL, (const float*)c->y_mean, (const float*)c->y_scale, y + s * dL));
     }
     return LBM_OK;
 }
@@ -1550,16 +1737,17 @@ int lbm_mlp_deformation(lbm_mlp* c, const float* x, int64_t n, float* m6, double
     if (!c || n < 0 || (n > 0 && (!x || !m6 || !D)) || c->d[c->L] != 6) return LBM_EINVAL;
     int st = lbm_mlp_forward(c, x, m6, n);
     if (st || n == 0) return st;  // no launch for an empty batch
-    k_deform_from_m<<<blocks_for(n, 128), 128, 0, c->stream>>>(m6, n, D);
-    MLP_TRY(cudaGetLastError());
+    MLP_TRY(launch(c, k_deform_from_m, dim3(blocks_for(n, 128)), dim3(128), 0, (const float*)m6, (long long)n, D));
     return LBM_OK;
 }
 
 int lbm_mlp_gradients(lbm_mlp* c, const float* x, const float* t, int64_t n, double* loss, float* grads) {
     if (!c || !x || !t || n < 32 || n > c->max_batch || n % 32 != 0) return LBM_EINVAL;
     cudaSetDevice(c->device);
-    MLP_TRY(forward(c, x, (int)n));
+    training_buffers(c);
+    MLP_TRY(forward(c, x, (int)n, true));
     MLP_TRY(backward(c, t, (int)n));
+    MLP_TRY(update(c, false, 0.f, 1.f, 1.f));
     MLP_TRY(cudaMemcpyAsync(c->h_loss, c->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     if (grads) {
         int st = copy_params(c, c->g, grads, true);
@@ -1573,15 +1761,13 @@ int lbm_mlp_gradients(lbm_mlp* c, const float* x, const float* t, int64_t n, dou
 int lbm_mlp_train_step(lbm_mlp* c, const float* x, const float* t, int64_t n, float lr, double* loss) {
     if (!c || !x || !t || n < 32 || n > c->max_batch || n % 32 != 0 || !(lr > 0.f)) return LBM_EINVAL;
     cudaSetDevice(c->device);
-    MLP_TRY(forward(c, x, (int)n));
+    training_buffers(c);
+    MLP_TRY(forward(c, x, (int)n, true));
     MLP_TRY(backward(c, t, (int)n));
     c->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - std::pow(b1, (float)c->step), c2 = 1.f - std::pow(b2, (float)c->step);
-    k_adam<<<blocks_for(c->nparam, 256), 256, 0, c->stream>>>(c->p, c->g, c->m, c->v, c->nparam, lr, b1, b2, 1e-8f,
-                                                             c1, c2);
-    MLP_TRY(cudaGetLastError());
-    MLP_TRY(refresh_weights(c));
+    MLP_TRY(update(c, true, lr, c1, c2));
     if (loss) {
         MLP_TRY(cudaMemcpyAsync(c->h_loss, c->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         MLP_TRY(cudaStreamSynchronize(c->stream));
