@@ -173,6 +173,38 @@ __device__ __forceinline__ void mrt_relax(const C (&f)[19], const C (&dev)[19], 
     }
 }
 
+template <typename C>
+__device__ __forceinline__ C mrt_rate(int k, C inv_tau, const C (&r)[5]) {
+    return (k == 0 || k == 3 || k == 5 || k == 7 || k == 9 || k == 11 || k == 13 || k == 14 || k == 15)
+               ? inv_tau
+               : (k == 1 ? r[0] : (k == 2 ? r[1] : ((k == 4 || k == 6 || k == 8) ? r[2] : ((k == 10 || k == 12) ? r[3] : r[4]))));
+}
+
+// out_i = f_i - sum_k M_ki s_k (M dev)_k / |M_k|^2 with dev = f - f_eq, moment
+// by moment.  16-bit storage keeps this order of operations: any other moves
+// its roundings, and with them a run's states, by whole 16-bit steps.
+template <typename C>
+__device__ __forceinline__ void mrt_relax_full(const C (&f)[19], const C (&dev)[19], C inv_tau, const C (&r)[5],
+                                          C (&out)[19]) {
+    C rel[19];
+#pragma unroll
+    for (int k = 0; k < 19; ++k) {
+        C mk = C(0);
+#pragma unroll
+        for (int i = 0; i < 19; ++i)
+            if (mrt_row(k, i) != 0) mk += C(mrt_row(k, i)) * dev[i];
+        rel[k] = mrt_rate<C>(k, inv_tau, r) * mk / C(mrt_norm(k));
+    }
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {
+        C back = C(0);
+#pragma unroll
+        for (int k = 0; k < 19; ++k)
+            if (mrt_row(k, i) != 0) back += C(mrt_row(k, i)) * rel[k];
+        out[i] = f[i] - back;
+    }
+}
+
 __device__ __forceinline__ int wrap(int a, int n) {
     a = a < 0 ? a + n : a;
     return a >= n ? a - n : a;

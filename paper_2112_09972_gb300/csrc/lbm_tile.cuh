@@ -220,7 +220,8 @@ __device__ __forceinline__ void tile_march(const S* __restrict__ src, S* __restr
                     C dv[19];
 #pragma unroll
                     for (int i = 0; i < 19; ++i) dv[i] = fc[s][i] - feq<C>(i, rho[s], ux, uy, uz, u2x);
-                    mrt_relax<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
+                    if constexpr (is_dev_t<S>::value) mrt_relax_full<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
+                    else mrt_relax<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
                 } else {
 #pragma unroll
                     for (int i = 1; i < 19; ++i) {
