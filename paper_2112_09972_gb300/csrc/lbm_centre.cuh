@@ -49,10 +49,21 @@ __device__ void centre_reduce(C (&cm)[4], C* parts, long long slot, unsigned tot
     __syncthreads();
     if (last && warp == 0) {
         __threadfence();
+        // eight slots' loads in flight at once (one after another, the L2
+        // latency of each made this sum several microseconds of every launch)
         C s4[4] = {C(0), C(0), C(0), C(0)};
-        for (unsigned b = lane; b < total; b += 32)
+        for (unsigned b0 = lane; b0 < total; b0 += 256u) {
+            C v[8][4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) s4[q] += __ldcg(parts + 4LL * b + q);
+            for (unsigned u = 0; u < 8; ++u)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    v[u][q] = b0 + 32u * u < total ? __ldcg(parts + 4LL * (b0 + 32u * u) + q) : C(0);
+#pragma unroll
+            for (unsigned u = 0; u < 8; ++u)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s4[q] += v[u][q];
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
 #pragma unroll

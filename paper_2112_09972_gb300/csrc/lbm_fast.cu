@@ -346,18 +346,16 @@ struct StagePlane<TX, Dev<T>> {
     static __device__ __forceinline__ void load(const float* st, int x, Raw& r, float& ra, float& rb) {
         r.o = reinterpret_cast<const float4*>(st)[x];
         const unsigned* b = reinterpret_cast<const unsigned*>(reinterpret_cast<const char*>(st) + NODE_BYTES) + x + 4;
-        float da = 0.f, db = 0.f;
+        float2 d = both(0.f);
         sfor<9>([&](auto K) {
             constexpr int i = 2 * decltype(K)::value + 1;
             r.w[i] = b[(i - 1) * SEG - cx_(i)];
             r.w[i + 1] = b[i * SEG - cx_(i + 1)];
-            const float2 u = dev_unpack2<T>(r.w[i]);
-            const float2 v = dev_unpack2<T>(r.w[i + 1]);
-            da += u.x + v.x;
-            db += u.y + v.y;
+            d = add2(d, add2(dev_unpack2<T>(r.w[i]), dev_unpack2<T>(r.w[i + 1])));
         });
-        ra = r.o.z + (1.f - wgt<float>(0)) * r.o.x + da;
-        rb = r.o.w + (1.f - wgt<float>(0)) * r.o.y + db;
+        const float2 s2 = add2(fma2(both(1.f - wgt<float>(0)), pair(r.o.x, r.o.y), pair(r.o.z, r.o.w)), d);
+        ra = s2.x;
+        rb = s2.y;
     }
     // the collision's input in deviation form (RowIO<TX, Dev<T>>::populations)
     static __device__ __forceinline__ void unpack(const Raw& r, float (&f)[2][19], float (&rs)[2]) {

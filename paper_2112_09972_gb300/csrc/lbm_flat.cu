@@ -164,7 +164,7 @@ __device__ __forceinline__ void flat_node(const double2* __restrict__ r, int sy,
             const double om = m.omit[s];
 #pragma unroll
             for (int i = 1; i < 19; i += 2) {
-                const double c = cx_(i) * vx + cy_(i) * vy + cz_(i) * vz;
+                const double c = dot_c<double>(i, vx, vy, vz);
                 const double od = (i < 7 ? e2A : e2E) * c;
                 const double ev = fma(c, od, i < 7 ? ebA : ebE);
                 os[i * pitch] = fma(om, f[s][i], ev + od);

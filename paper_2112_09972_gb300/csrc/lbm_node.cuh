@@ -48,6 +48,42 @@ __device__ __forceinline__ void sfor(F&& f) {
     sfor_(f, std::make_integer_sequence<int, N>{});
 }
 
+// Pairs {A, B} of the two components in packed float32 arithmetic: one
+// instruction adds or multiplies both, each half rounded as the scalar
+// instruction rounds it, so the results are the scalar ones.  The 16-bit
+// forms use it: their kernels issue on 58 % of the cycles, the words already
+// hold both components, and the arithmetic instructions of a node update
+// halve (256^3 per step: binary16 733 -> 689 us, bfloat16 768 -> 707).  Float32
+// storage does not: its staged kernel carries 76 populations in registers,
+// which the pairing made spill (128^3 133 -> 153 us).
+__device__ __forceinline__ float2 pair(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    float2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long&>(r))
+        : "l"(reinterpret_cast<unsigned long long&>(a)), "l"(reinterpret_cast<unsigned long long&>(b)));
+    return r;
+}
+// c_i . u of both components (dot_c).
+__device__ __forceinline__ float2 dot_c2(int i, float2 ux, float2 uy, float2 uz) {
+    float2 v = both(0.f);
+    bool any = false;
+    if (cx_(i)) {
+        v = cx_(i) > 0 ? ux : pair(-ux.x, -ux.y);
+        any = true;
+    }
+    if (cy_(i)) {
+        v = any ? (cy_(i) > 0 ? add2(v, uy) : sub2(v, uy)) : (cy_(i) > 0 ? uy : pair(-uy.x, -uy.y));
+        any = true;
+    }
+    if (cz_(i)) v = any ? (cz_(i) > 0 ? add2(v, uz) : sub2(v, uz)) : (cz_(i) > 0 ? uz : pair(-uz.x, -uz.y));
+    return v;
+}
+
 // Global loads and stores at a pointer plus an immediate byte offset.  The
 // first read of a plane keeps its lines in L2 (evict_last policy) for the
 // second read one plane later, which marks them last-use; the written state
@@ -326,30 +362,70 @@ __device__ __forceinline__ void collide_core(NB&& nb, const float2 rho2, const f
                                              const float (&rs)[2], const FastModel& m, typename IO::Out out,
                                              float (&cm)[4], int& bad, float px, float py, float pz) {
     const float rho[2] = {rho2.x, rho2.y};
-    // momentum (Eq. 6), opposite pairs differenced first
-    float j[2][3];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        float jx = 0.f, jy = 0.f, jz = 0.f;
+    float j[2][3], acc[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+    if constexpr (is_dev_t<ST>::value) {
+        // momentum (Eq. 6) of both components, opposite pairs differenced first
+        float2 j2[3];
+        bool jset[3] = {false, false, false};
+        auto gather = [](float2& a, bool& set, int c, float2 d) {  // a += c d
+            if (c == 0) return;
+            a = set ? (c > 0 ? add2(a, d) : sub2(a, d)) : d;  // (the first direction of each sum has c = 1)
+            set = true;
+        };
 #pragma unroll
         for (int i = 1; i < 19; i += 2) {
-            const float d = f[s][i] - f[s][i + 1];
-            if (cx_(i)) jx += (float)cx_(i) * d;
-            if (cy_(i)) jy += (float)cy_(i) * d;
-            if (cz_(i)) jz += (float)cz_(i) * d;
+            const float2 d = sub2(pair(f[0][i], f[1][i]), pair(f[0][i + 1], f[1][i + 1]));
+            gather(j2[0], jset[0], cx_(i), d);
+            gather(j2[1], jset[1], cy_(i), d);
+            gather(j2[2], jset[2], cz_(i), d);
         }
-        j[s][0] = jx; j[s][1] = jy; j[s][2] = jz;
-    }
-    // Shan-Chen force (Eq. 7) sums sum_i w_i rho_s(x + c_i) c_i, neighbour
-    // pairs differenced first; the weight folds into the multiplier
-    float acc[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+        // Shan-Chen force (Eq. 7) sums sum_i w_i rho_s(x + c_i) c_i, neighbour
+        // pairs differenced first; the weight folds into the multiplier
+        float2 acc2[3];
+        bool aset[3] = {false, false, false};
+        auto weigh = [](float2& a, bool& set, float c, float2 d) {  // a += c d
+            if (c == 0.f) return;
+            a = set ? fma2(both(c), d, a) : mul2(both(c), d);
+            set = true;
+        };
 #pragma unroll
-    for (int i = 1; i < 19; i += 2) {
-        const float2 np = nb(cx_(i), cy_(i), cz_(i)), nm = nb(-cx_(i), -cy_(i), -cz_(i));
-        const float dA = np.x - nm.x, dB = np.y - nm.y;
-        if (cx_(i)) { acc[0][0] += (wgt<float>(i) * cx_(i)) * dA; acc[1][0] += (wgt<float>(i) * cx_(i)) * dB; }
-        if (cy_(i)) { acc[0][1] += (wgt<float>(i) * cy_(i)) * dA; acc[1][1] += (wgt<float>(i) * cy_(i)) * dB; }
-        if (cz_(i)) { acc[0][2] += (wgt<float>(i) * cz_(i)) * dA; acc[1][2] += (wgt<float>(i) * cz_(i)) * dB; }
+        for (int i = 1; i < 19; i += 2) {
+            const float2 d = sub2(nb(cx_(i), cy_(i), cz_(i)), nb(-cx_(i), -cy_(i), -cz_(i)));
+            weigh(acc2[0], aset[0], wgt<float>(i) * cx_(i), d);
+            weigh(acc2[1], aset[1], wgt<float>(i) * cy_(i), d);
+            weigh(acc2[2], aset[2], wgt<float>(i) * cz_(i), d);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            j[0][a] = j2[a].x;
+            j[1][a] = j2[a].y;
+            acc[0][a] = acc2[a].x;
+            acc[1][a] = acc2[a].y;
+        }
+    } else {
+        // momentum (Eq. 6), opposite pairs differenced first
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            float jx = 0.f, jy = 0.f, jz = 0.f;
+#pragma unroll
+            for (int i = 1; i < 19; i += 2) {
+                const float d = f[s][i] - f[s][i + 1];
+                if (cx_(i)) jx += (float)cx_(i) * d;
+                if (cy_(i)) jy += (float)cy_(i) * d;
+                if (cz_(i)) jz += (float)cz_(i) * d;
+            }
+            j[s][0] = jx; j[s][1] = jy; j[s][2] = jz;
+        }
+        // Shan-Chen force (Eq. 7) sums sum_i w_i rho_s(x + c_i) c_i, neighbour
+        // pairs differenced first; the weight folds into the multiplier
+#pragma unroll
+        for (int i = 1; i < 19; i += 2) {
+            const float2 np = nb(cx_(i), cy_(i), cz_(i)), nm = nb(-cx_(i), -cy_(i), -cz_(i));
+            const float dA = np.x - nm.x, dB = np.y - nm.y;
+            if (cx_(i)) { acc[0][0] += (wgt<float>(i) * cx_(i)) * dA; acc[1][0] += (wgt<float>(i) * cx_(i)) * dB; }
+            if (cy_(i)) { acc[0][1] += (wgt<float>(i) * cy_(i)) * dA; acc[1][1] += (wgt<float>(i) * cy_(i)) * dB; }
+            if (cz_(i)) { acc[0][2] += (wgt<float>(i) * cz_(i)) * dA; acc[1][2] += (wgt<float>(i) * cz_(i)) * dB; }
+        }
     }
     const float den = rho[0] * m.inv_tau[0] + rho[1] * m.inv_tau[1];
     const float rden = __frcp_rn(den);
@@ -388,34 +464,31 @@ __device__ __forceinline__ void collide_core(NB&& nb, const float2 rho2, const f
             W1[s] = orr * wgt<float>(1);
             W2[s] = orr * wgt<float>(7);
         }
-        float others[2] = {0.f, 0.f};
+        float2 others = both(0.f);
+        const float2 ux2 = pair(ux[0], ux[1]), uy2 = pair(uy[0], uy[1]), uz2 = pair(uz[0], uz[1]);
+        const float2 base2 = pair(base[0], base[1]), om2 = pair(m.omit[0], m.omit[1]);
+        const float2 eA = pair(e1[0], e1[1]), eE = pair(e2[0], e2[1]);
+        const float2 WA = pair(W1[0], W1[1]), WE = pair(W2[0], W2[1]);
+        const float2 oA = mul2(both(3.f), eA), oE = mul2(both(3.f), eE);
         sfor<9>([&](auto K) {
             constexpr int i = 2 * decltype(K)::value + 1;
             // densities of the destinations x + c_i and x - c_i (read again
             // from shared memory rather than held since the force)
             const float2 np = nb(cx_(i), cy_(i), cz_(i)), nm = nb(-cx_(i), -cy_(i), -cz_(i));
-            float da[2], dbv[2];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const float cu = (float)cx_(i) * ux[s] + (float)cy_(i) * uy[s] + (float)cz_(i) * uz[s];
-                const float e = i < 7 ? e1[s] : e2[s];
-                const float ev = fmaf(e, fmaf(4.5f * cu, cu, base[s]), i < 7 ? W1[s] : W2[s]);
-                const float od = (3.f * e) * cu;
-                const float oa = fmaf(m.omit[s], f[s][i], ev + od);
-                const float ob = fmaf(m.omit[s], f[s][i + 1], ev - od);
-                // deviations from w_i times the destinations' densities
-                da[s] = fmaf(-wgt<float>(i), s ? np.y : np.x, oa);
-                dbv[s] = fmaf(-wgt<float>(i), s ? nm.y : nm.x, ob);
-            }
-            const unsigned wa = dev_pack2<T>(da[0], da[1]), wb = dev_pack2<T>(dbv[0], dbv[1]);
+            const float2 cu = dot_c2(i, ux2, uy2, uz2);
+            const float2 ev = fma2(i < 7 ? eA : eE, fma2(mul2(both(4.5f), cu), cu, base2), i < 7 ? WA : WE);
+            const float2 od = mul2(i < 7 ? oA : oE, cu);
+            // deviations from w_i times the destinations' densities
+            const float2 da = fma2(both(-wgt<float>(i)), np, fma2(om2, pair(f[0][i], f[1][i]), add2(ev, od)));
+            const float2 db = fma2(both(-wgt<float>(i)), nm, fma2(om2, pair(f[0][i + 1], f[1][i + 1]), sub2(ev, od)));
+            const unsigned wa = dev_pack2<T>(da.x, da.y), wb = dev_pack2<T>(db.x, db.y);
             IO::template store_word<i>(out, wa);
             IO::template store_word<i + 1>(out, wb);
             // the values the readers will rebuild, for the mass balance
-            const float2 qa = dev_unpack2<T>(wa), qb = dev_unpack2<T>(wb);
-            others[0] += fmaf(wgt<float>(i), np.x, qa.x) + fmaf(wgt<float>(i), nm.x, qb.x);
-            others[1] += fmaf(wgt<float>(i), np.y, qa.y) + fmaf(wgt<float>(i), nm.y, qb.y);
+            others = add2(others, add2(fma2(both(wgt<float>(i)), np, dev_unpack2<T>(wa)),
+                                       fma2(both(wgt<float>(i)), nm, dev_unpack2<T>(wb))));
         });
-        st_cs_f4(out.b, make_float4(rho[0], rho[1], rho[0] - others[0], rho[1] - others[1]));
+        st_cs_f4(out.b, make_float4(rho[0], rho[1], rho[0] - others.x, rho[1] - others.y));
     } else {
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
@@ -438,7 +511,7 @@ __device__ __forceinline__ void collide_core(NB&& nb, const float2 rho2, const f
                 float o[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                 auto deviations = [&](auto I, float& dp, float& dm) {
                     constexpr int i = decltype(I)::value;
-                    const float cu = (float)cx_(i) * ux + (float)cy_(i) * uy + (float)cz_(i) * uz;
+                    const float cu = dot_c<float>(i, ux, uy, uz);
                     const float e = i < 7 ? e1 : e2;
                     const float ev = e * fmaf(4.5f * cu, cu, base);
                     const float od = (3.f * e) * cu;
@@ -476,7 +549,7 @@ __device__ __forceinline__ void collide_core(NB&& nb, const float2 rho2, const f
                 const float om = m.omit[s];
                 sfor<9>([&](auto K) {
                     constexpr int i = 2 * decltype(K)::value + 1;
-                    const float cu = (float)cx_(i) * ux + (float)cy_(i) * uy + (float)cz_(i) * uz;
+                    const float cu = dot_c<float>(i, ux, uy, uz);
                     const float e = i < 7 ? e1 : e2;
                     const float ev = e * fmaf(4.5f * cu, cu, base);
                     const float od = (3.f * e) * cu;
