@@ -199,71 +199,40 @@ __device__ void block_sum(double (&v)[K], double* out) {
     }
 }
 
-// How k_moments and k_grad_phi walk the box: a warp takes 32 consecutive
-// nodes of an x-y plane (flattened, so that no width leaves lanes idle) and
-// marches one of `zparts` parts of the z extent; units of work are numbered
-// segment first.
-struct Columns {
-    int segs, zparts, zlen;
-};
-Columns columns(const Layout& L, long long warps) {
-    Columns c;
-    c.segs = (int)(((long long)L.Lx * L.Ly + 31) / 32);
-    long long zp = warps / c.segs;
-    zp = zp < 1 ? 1 : (zp > L.Lz ? L.Lz : zp);
-    c.zlen = (int)((L.Lz + zp - 1) / zp);
-    c.zparts = (L.Lz + c.zlen - 1) / c.zlen;
-    return c;
-}
-
 // Ten moments of w = max(phi, 0).  Few nodes have phi > 0 (a droplet of R =
-// L / 8 fills 0.8 % of its box), so only those run FP64 instructions: a
-// lane's x and y stay fixed along its march, its three sums {w, w z, w z^2}
-// give all ten moments at the end, and warps and CTAs without a droplet node
-// skip the FP64 reductions.  128^3 float32 on GB300: 180 us with ten FP64
-// sums per node and the reductions in every warp, bound by the FP64 pipe.
+// L / 8 fills 0.8 % of its box), so only those run FP64 instructions, and
+// warps and CTAs without one skip the FP64 reductions.  The CTAs walk the box
+// together in node order: DRAM then serves neighbouring rows at the same time
+// (a march of each warp along z read as many bytes at 45 % of its peak).
+// 128^3 float32 on GB300: 180 us with ten FP64 sums per node and the
+// reductions in every warp, bound by the FP64 pipe; 102 us marching.
 template <typename S>
-__global__ void __launch_bounds__(kRedThreads, 4) k_moments(const S* __restrict__ f, Layout L, Columns c,
-                                                         double* __restrict__ partials) {
+__global__ void __launch_bounds__(kRedThreads, 4) k_moments(const S* __restrict__ f, Layout L,
+                                                            double* __restrict__ partials) {
     __shared__ double part[kRedThreads / 32][10];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const double cx = 0.5 * (L.Lx - 1), cy = 0.5 * (L.Ly - 1), cz = 0.5 * (L.Lz - 1);
     double m[10];
 #pragma unroll
     for (int k = 0; k < 10; ++k) m[k] = 0.0;
-    bool some = false;
-    const long long units = (long long)c.segs * c.zparts;
-    const long long stride = (long long)gridDim.x * (kRedThreads / 32);
-    for (long long u = (long long)blockIdx.x * (kRedThreads / 32) + warp; u < units; u += stride) {
-        const int zp = (int)(u / c.segs), p = (int)(u - (long long)zp * c.segs) * 32 + lane;
-        const bool on = p < L.Lx * L.Ly;
-        const int y = on ? p / L.Lx : 0, x = on ? p - y * L.Lx : 0;
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        bool drop = false;
-        const int z1 = min((zp + 1) * c.zlen, L.Lz);
-        for (int z = zp * c.zlen; z < z1; ++z) {
-            if (!on) continue;
-            const RhoPair<S> r = node_rho_pair(f, L, x, y, z);
-            if (!r.droplet()) continue;
-            const double ra = r.a(), rb = r.b();
-            const double phi = (ra - rb) / (ra + rb);
-            if (phi > 0.0) {
-                const double pz = z - cz, wz = phi * pz;
-                s0 += phi;
-                s1 += wz;
-                s2 = fma(wz, pz, s2);
-                drop = true;
-            }
-        }
-        if (__any_sync(0xffffffffu, drop)) {
-            const double px = x - cx, py = y - cy, sx = s0 * px, sy = s0 * py;
-            m[0] += s0;
-            m[1] += sx; m[2] += sy; m[3] += s1;
-            m[4] = fma(sx, px, m[4]); m[5] = fma(sx, py, m[5]); m[6] = fma(s1, px, m[6]);
-            m[7] = fma(sy, py, m[7]); m[8] = fma(s1, py, m[8]); m[9] += s2;
-            some = true;
+    bool drop = false;
+    const long long N = (long long)L.Lx * L.Ly * L.Lz;
+    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
+        const int row = (int)(n / L.Lx), y = row % L.Ly, z = row / L.Ly, x = (int)(n - (long long)row * L.Lx);
+        const RhoPair<S> r = node_rho_pair(f, L, x, y, z);
+        if (!r.droplet()) continue;
+        const double ra = r.a(), rb = r.b();
+        const double w = (ra - rb) / (ra + rb);
+        if (w > 0.0) {
+            const double px = x - 0.5 * (L.Lx - 1), py = y - 0.5 * (L.Ly - 1), pz = z - 0.5 * (L.Lz - 1);
+            const double wx = w * px, wy = w * py, wz = w * pz;
+            m[0] += w;
+            m[1] += wx; m[2] += wy; m[3] += wz;
+            m[4] = fma(wx, px, m[4]); m[5] = fma(wx, py, m[5]); m[6] = fma(wx, pz, m[6]);
+            m[7] = fma(wy, py, m[7]); m[8] = fma(wy, pz, m[8]); m[9] = fma(wz, pz, m[9]);
+            drop = true;
         }
     }
+    const bool some = __any_sync(0xffffffffu, drop);
     if (some) {
 #pragma unroll
         for (int k = 0; k < 10; ++k) {
@@ -292,8 +261,13 @@ __global__ void __launch_bounds__(kMomentsFinalThreads) k_moments_final(const do
     __shared__ double sum[10];
     const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
     double a = 0.0;
-#pragma unroll 4
-    for (int b = lane; b < nblocks; b += 32) a += partials[10LL * b + k];
+    for (int b0 = lane; b0 < nblocks; b0 += 256) {  // eight loads in flight
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = b0 + 32 * u < nblocks ? partials[10LL * (b0 + 32 * u) + k] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a += v[u];
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
     if (lane == 0) sum[k] = a;
@@ -561,25 +535,88 @@ __global__ void k_cc_roots(Layout L, const int* __restrict__ label, const int* _
 
 // ---- surface-area deformation (Eq. 17) and mass reinjection ----
 
-// phi of every fluid node into phi[n] (n = (z Ly + y) Lx + x) and per-block
-// {sum phi, min phi, max phi}.  Bound by the FP64 pipe after the float32
-// density sums: the quotient is div64.
+// phi = (a - b) / (a + b) of a node, kept for the gradient pass: a double for
+// float64 storage; for the float32 and 16-bit forms an unevaluated float32
+// pair hi + lo good to 2^-44, a thousandth of what the stored populations'
+// own rounding leaves, so that phi, its sum and its gradient stay off the
+// FP64 pipe (which bounded both passes: 96 and 88 us at 128^3 float32).
+struct Pair {
+    float h, l;
+};
+__device__ __forceinline__ Pair two_sum(float a, float b) {  // Knuth: a + b = h + l exactly
+    const float h = a + b, bb = h - a;
+    return {h, (a - (h - bb)) + (b - bb)};
+}
+__device__ __forceinline__ Pair renorm(float h, float l) {  // |h| >= |l|
+    const float s = h + l;
+    return {s, l - (s - h)};
+}
+__device__ __forceinline__ double phi_value(double p) { return p; }
+__device__ __forceinline__ double phi_value(Pair p) { return (double)p.h + (double)p.l; }
+__device__ __forceinline__ bool phi_number(double p) { return p == p; }
+__device__ __forceinline__ bool phi_number(Pair p) { return p.h == p.h; }
+__device__ __forceinline__ bool phi_less(double a, double b) { return a < b; }
+__device__ __forceinline__ bool phi_less(Pair a, Pair b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
+
 template <typename S>
-__global__ void __launch_bounds__(kRedThreads) k_phi(const S* __restrict__ f, Layout L, double* __restrict__ phi,
+struct PhiOf {
+    using T = typename std::conditional<std::is_same<S, double>::value, double, Pair>::type;
+};
+__device__ __forceinline__ double node_phi(const RhoPair<double>& r) { return div64(r.ah - r.bh, r.ah + r.bh); }
+template <typename S>
+__device__ __forceinline__ Pair node_phi(const RhoPair<S>& r) {
+    Pair d = two_sum(r.ah, -r.bh), t = two_sum(r.ah, r.bh);
+    d.l += r.al - r.bl;
+    t.l += r.al + r.bl;
+    if (!(fabsf(t.h) > 1e-25f && fabsf(t.h) < 1e25f && fabsf(d.h) < 1e25f)) {
+        const double p = (r.a() - r.b()) / (r.a() + r.b());
+        return {(float)p, isfinite(p) ? (float)(p - (double)(float)p) : 0.f};
+    }
+    const float y = __frcp_rn(t.h), q = d.h * y;
+    const float e = fmaf(-q, t.h, d.h) + fmaf(-q, t.l, d.l);
+    return renorm(q, e * y);
+}
+
+// Sums of phi and of |grad phi|.
+struct Acc64 {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double v) { s += v; }
+    __device__ __forceinline__ double value() const { return s; }
+};
+struct AccPair {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(Pair v) {
+        two_sum_acc(h, l, v.h);
+        l += v.l;
+    }
+    __device__ __forceinline__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
+};
+template <typename T>
+using Acc = typename std::conditional<std::is_same<T, double>::value, Acc64, AccPair>::type;
+
+// phi of every fluid node into phi[n] (n = (z Ly + y) Lx + x) and per-block
+// {sum phi, min phi, max phi}.
+template <typename S>
+__global__ void __launch_bounds__(kRedThreads) k_phi(const S* __restrict__ f, Layout L,
+                                                     typename PhiOf<S>::T* __restrict__ phi,
                                                      double* __restrict__ partials) {
+    using T = typename PhiOf<S>::T;
     __shared__ double red[3][kRedThreads / 32];
     const long long N = (long long)L.Lx * L.Ly * L.Lz;
-    double sum = 0.0, lo = 1e300, hi = -1e300;
+    Acc<T> acc;
+    T tlo, thi;
+    bool seen = false;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
         const int row = (int)(n / L.Lx), y = row % L.Ly, z = row / L.Ly, x = (int)(n - (long long)row * L.Lx);
-        double ra, rb;
-        node_rho(f, L, x, y, z, ra, rb);
-        const double p = div64(ra - rb, ra + rb);
+        const T p = node_phi(node_rho_pair(f, L, x, y, z));
         phi[n] = p;
-        sum += p;
-        lo = fmin(lo, p);
-        hi = fmax(hi, p);
+        acc.add(p);
+        if (!phi_number(p)) continue;  // as fmin and fmax, the extremes pass over NaN
+        if (!seen || phi_less(p, tlo)) tlo = p;
+        if (!seen || phi_less(thi, p)) thi = p;
+        seen = true;
     }
+    double sum = acc.value(), lo = seen ? phi_value(tlo) : 1e300, hi = seen ? phi_value(thi) : -1e300;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int o = 16; o > 0; o >>= 1) {
         sum += __shfl_down_sync(0xffffffffu, sum, o);
@@ -610,13 +647,51 @@ __device__ __forceinline__ double sqrt64(double s) {
     r = fma(fma(-r, r, s), h, r);
     return fma(fma(-r, r, s), h, r);
 }
+// |g| from the differences of phi across a node.
+__device__ __forceinline__ double magnitude(double x1, double x0, double y1, double y0, double z1, double z0) {
+    const double gx = x1 - x0, gy = y1 - y0, gz = z1 - z0;
+    return sqrt64(fma(gx, gx, fma(gy, gy, gz * gz)));
+}
+__device__ __forceinline__ Pair magnitude(Pair x1, Pair x0, Pair y1, Pair y0, Pair z1, Pair z0) {
+    auto square = [](Pair a, Pair b) -> Pair {  // (a - b)^2
+        Pair d = two_sum(a.h, -b.h);
+        d.l += a.l - b.l;
+        const float p = d.h * d.h;
+        return {p, fmaf(2.f * d.h, d.l, fmaf(d.h, d.h, -p))};
+    };
+    const Pair a = square(x1, x0), b = square(y1, y0), c = square(z1, z0);
+    const Pair ab = two_sum(a.h, b.h), s = two_sum(ab.h, c.h);
+    const float lo = s.l + ab.l + (a.l + b.l + c.l);
+    // outside, |g| < 1e-15 or above any physical phi; infinities and NaN pass through
+    if (!(s.h > 1e-30f && s.h < 1e30f)) return {sqrtf(s.h), 0.f};
+    const float y = rsqrtf(s.h), r = s.h * y;
+    return renorm(r, 0.5f * y * (fmaf(-r, r, s.h) + lo));
+}
+
+// How k_grad_phi walks the box: a warp takes 32 consecutive
+// nodes of an x-y plane (flattened, so that no width leaves lanes idle) and
+// marches one of `zparts` parts of the z extent; units of work are numbered
+// segment first.
+struct Columns {
+    int segs, zparts, zlen;
+};
+Columns columns(const Layout& L, long long warps) {
+    Columns c;
+    c.segs = (int)(((long long)L.Lx * L.Ly + 31) / 32);
+    long long zp = warps / c.segs;
+    zp = zp < 1 ? 1 : (zp > L.Lz ? L.Lz : zp);
+    c.zlen = (int)((L.Lz + zp - 1) / zp);
+    c.zparts = (L.Lz + c.zlen - 1) / c.zlen;
+    return c;
+}
 
 // Per-block sum of |grad phi| (central differences) over interior nodes into
 // partials[4 b + 3]; a lane marches in z (Columns) and keeps the two planes
 // beside it in registers.
-__global__ void __launch_bounds__(kRedThreads) k_grad_phi(Layout L, Columns c, const double* __restrict__ phi,
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads) k_grad_phi(Layout L, Columns c, const T* __restrict__ phi,
                                                           double* __restrict__ partials) {
-    double v[1] = {0.0};
+    Acc<T> acc;
     const long long sy = L.Lx, sz = (long long)L.Lx * L.Ly;
     const long long units = (long long)c.segs * c.zparts;
     const long long stride = (long long)gridDim.x * (kRedThreads / 32);
@@ -626,17 +701,16 @@ __global__ void __launch_bounds__(kRedThreads) k_grad_phi(Layout L, Columns c, c
         if (x < 1 || x > L.Lx - 2 || y < 1 || y > L.Ly - 2) continue;
         const int z0 = max(zp * c.zlen, 1), z1 = min((zp + 1) * c.zlen, L.Lz - 1);
         if (z0 >= z1) continue;
-        const double* q = phi + (long long)z0 * sz + p;
-        double below = q[-sz], here = q[0];
+        const T* q = phi + (long long)z0 * sz + p;
+        T below = q[-sz], here = q[0];
         for (int z = z0; z < z1; ++z, q += sz) {
-            const double above = q[sz];
-            const double gx = q[1] - q[-1], gy = q[sy] - q[-sy], gz = above - below;
-            v[0] += sqrt64(fma(gx, gx, fma(gy, gy, gz * gz)));
+            const T above = q[sz];
+            acc.add(magnitude(q[1], q[-1], q[sy], q[-sy], above, below));
             below = here;
             here = above;
         }
     }
-    v[0] *= 0.5;
+    double v[1] = {0.5 * acc.value()};
     double out[1];
     block_sum<1>(v, out);
     if (threadIdx.x == 0) partials[4LL * blockIdx.x + 3] = out[0];
@@ -722,12 +796,10 @@ int moments_blocks(const Layout& L, int num_sms) {
 
 cudaError_t launch_moments(int prec, const void* f, const Layout& L, double* partials, int nblocks, double* result,
                            cudaStream_t s) {
-    const Columns c = columns(L, (long long)nblocks * (kRedThreads / 32));
-    if (prec == kFP64) k_moments<double><<<nblocks, kRedThreads, 0, s>>>((const double*)f, L, c, partials);
-    else if (prec == kFP32) k_moments<float><<<nblocks, kRedThreads, 0, s>>>((const float*)f, L, c, partials);
-    else if (prec == kFP16Dev)
-        k_moments<Dev<__half>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__half>*)f, L, c, partials);
-    else k_moments<Dev<__nv_bfloat16>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__nv_bfloat16>*)f, L, c, partials);
+    if (prec == kFP64) k_moments<double><<<nblocks, kRedThreads, 0, s>>>((const double*)f, L, partials);
+    else if (prec == kFP32) k_moments<float><<<nblocks, kRedThreads, 0, s>>>((const float*)f, L, partials);
+    else if (prec == kFP16Dev) k_moments<Dev<__half>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__half>*)f, L, partials);
+    else k_moments<Dev<__nv_bfloat16>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__nv_bfloat16>*)f, L, partials);
     k_moments_final<<<1, kMomentsFinalThreads, 0, s>>>(partials, nblocks, result);
     return cudaGetLastError();
 }
@@ -813,14 +885,19 @@ namespace lbmgb {
 
 // out[0..3] = {sum phi, min phi, max phi, sum |grad phi| over interior nodes};
 // scratch: N doubles (phi) and 4 nblocks doubles.
+template <typename S>
+void surface_stats_t(const S* f, const Layout& L, void* scratch, double* partials, int nblocks, cudaStream_t s) {
+    using T = typename PhiOf<S>::T;
+    const Columns c = columns(L, (long long)nblocks * (kRedThreads / 32));
+    k_phi<S><<<nblocks, kRedThreads, 0, s>>>(f, L, (T*)scratch, partials);
+    k_grad_phi<T><<<nblocks, kRedThreads, 0, s>>>(L, c, (const T*)scratch, partials);
+}
 cudaError_t launch_surface_stats(int prec, const void* f, const Layout& L, double* phi, double* partials, int nblocks,
                                  double* out, cudaStream_t s) {
-    if (prec == kFP64) k_phi<double><<<nblocks, kRedThreads, 0, s>>>((const double*)f, L, phi, partials);
-    else if (prec == kFP32) k_phi<float><<<nblocks, kRedThreads, 0, s>>>((const float*)f, L, phi, partials);
-    else if (prec == kFP16Dev) k_phi<Dev<__half>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__half>*)f, L, phi, partials);
-    else k_phi<Dev<__nv_bfloat16>><<<nblocks, kRedThreads, 0, s>>>((const Dev<__nv_bfloat16>*)f, L, phi, partials);
-    const Columns c = columns(L, (long long)nblocks * (kRedThreads / 32));
-    k_grad_phi<<<nblocks, kRedThreads, 0, s>>>(L, c, phi, partials);
+    if (prec == kFP64) surface_stats_t((const double*)f, L, phi, partials, nblocks, s);
+    else if (prec == kFP32) surface_stats_t((const float*)f, L, phi, partials, nblocks, s);
+    else if (prec == kFP16Dev) surface_stats_t((const Dev<__half>*)f, L, phi, partials, nblocks, s);
+    else surface_stats_t((const Dev<__nv_bfloat16>*)f, L, phi, partials, nblocks, s);
     k_phi_final<<<1, kRedThreads, 0, s>>>(partials, nblocks, out);
     return cudaGetLastError();
 }
