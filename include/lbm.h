@@ -352,8 +352,9 @@ typedef struct lbm_batch lbm_batch; /* opaque */
  * (each 4 .. 1024), R[k] its droplet radius (2 R <= min extent - 2).
  * visc, G as for lbm_create.  opts must ask for LBM_FP32 and the ghost
  * boundary and must give rho_lo > 0 (the ghost density of the droplet
- * component); rho_hi <= 0 means 1.  opts->z_chunk (0: 32 for the row kernel,
- * 16 for the tile march) sets the initial z planes per work item; opts->tile_y
+ * component); rho_hi <= 0 means 1.  opts->z_chunk (0: as few chunks as fill 60 %
+ * of the CTA slots for the row kernel, 16 planes for the tile march) sets the
+ * initial z planes per work item; opts->tile_y
  * > 0 keeps the tile march.  Each box starts, on first use, at the equilibrium
  * tanh droplet in the flow of its gradient at step 0.
  */

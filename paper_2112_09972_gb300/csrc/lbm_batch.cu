@@ -164,60 +164,44 @@ __global__ void __launch_bounds__(kBatchThreads)
 }
 
 // Ten moments of w = max(phi, 0) per box: blockIdx.y = box, partials
-// [box][block][10].  As k_moments of the single box: a warp takes 32
-// consecutive nodes of an x-y plane and a part of the z extent, only nodes
-// with phi > 0 run FP64 instructions (this GPU's FP64 pipe runs at 1/64 of the
-// float32 rate), and warps and CTAs without one skip the reductions.
-// Measured on 24 boxes of edges 40 to 64 (3.5 M nodes): 242 us with ten FP64
-// sums per node.
-__global__ void __launch_bounds__(256) k_batch_moments(const BatchBox* __restrict__ boxes, int parity,
-                                                       double* __restrict__ partials) {
+// [box][block][10].  As k_moments of the single box: the CTAs of a box walk it
+// in node order, only nodes with phi > 0 run FP64 instructions (this GPU's
+// FP64 pipe runs at 1/64 of the float32 rate), and warps and CTAs without one
+// skip the reductions.
+__global__ void __launch_bounds__(256, 4) k_batch_moments(const BatchBox* __restrict__ boxes, int parity,
+                                                          double* __restrict__ partials) {
     const BatchBox b = boxes[blockIdx.y];
     const Layout& L = b.L;
     const float* f = b.f[parity];
     __shared__ double part[8][10];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int area = L.Lx * L.Ly, segs = (area + 31) / 32, warps = gridDim.x * 8;
-    const int zp = max(1, min(warps / segs, L.Lz)), zlen = (L.Lz + zp - 1) / zp, zparts = (L.Lz + zlen - 1) / zlen;
-    const double cx = 0.5 * (L.Lx - 1), cy = 0.5 * (L.Ly - 1), cz = 0.5 * (L.Lz - 1);
     double m[10];
 #pragma unroll
     for (int k = 0; k < 10; ++k) m[k] = 0.0;
-    bool some = false;
-    for (int u = blockIdx.x * 8 + warp; u < segs * zparts; u += warps) {
-        const int q = u / segs, p = (u - q * segs) * 32 + lane;
-        const bool on = p < area;
-        const int y = on ? p / L.Lx : 0, x = on ? p - y * L.Lx : 0;
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        bool drop = false;
-        const int z1 = min((q + 1) * zlen, L.Lz);
-        for (int z = q * zlen; z < z1; ++z) {
-            if (!on) continue;
-            const long long base = L.at(0, 0, x, y, z);
-            float ra = 0.f, rb = 0.f;
+    bool drop = false;
+    const long long N = (long long)L.Lx * L.Ly * L.Lz;
+    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
+        const int row = (int)(n / L.Lx), y = row % L.Ly, z = row / L.Ly, x = (int)(n - (long long)row * L.Lx);
+        const long long base = L.at(0, 0, x, y, z);
+        float ra = 0.f, rb = 0.f;
 #pragma unroll
-            for (int i = 0; i < 19; ++i) {
-                ra += f[base + (long long)i * L.pitch];
-                rb += f[base + (long long)(19 + i) * L.pitch];
-            }
-            const float phi = (ra - rb) / (ra + rb);
-            if (phi > 0.f) {
-                const double w = (double)phi, pz = z - cz, wz = w * pz;
-                s0 += w;
-                s1 += wz;
-                s2 = fma(wz, pz, s2);
-                drop = true;
-            }
+        for (int i = 0; i < 19; ++i) {
+            ra += f[base + (long long)i * L.pitch];
+            rb += f[base + (long long)(19 + i) * L.pitch];
         }
-        if (__any_sync(0xffffffffu, drop)) {
-            const double px = x - cx, py = y - cy, sx = s0 * px, sy = s0 * py;
-            m[0] += s0;
-            m[1] += sx; m[2] += sy; m[3] += s1;
-            m[4] = fma(sx, px, m[4]); m[5] = fma(sx, py, m[5]); m[6] = fma(s1, px, m[6]);
-            m[7] = fma(sy, py, m[7]); m[8] = fma(s1, py, m[8]); m[9] += s2;
-            some = true;
+        const float phi = (ra - rb) / (ra + rb);
+        if (phi > 0.f) {
+            const double w = (double)phi;
+            const double px = x - 0.5 * (L.Lx - 1), py = y - 0.5 * (L.Ly - 1), pz = z - 0.5 * (L.Lz - 1);
+            const double wx = w * px, wy = w * py, wz = w * pz;
+            m[0] += w;
+            m[1] += wx; m[2] += wy; m[3] += wz;
+            m[4] = fma(wx, px, m[4]); m[5] = fma(wx, py, m[5]); m[6] = fma(wx, pz, m[6]);
+            m[7] = fma(wy, py, m[7]); m[8] = fma(wy, pz, m[8]); m[9] = fma(wz, pz, m[9]);
+            drop = true;
         }
     }
+    const bool some = __any_sync(0xffffffffu, drop);
     if (some) {
 #pragma unroll
         for (int k = 0; k < 10; ++k) {
@@ -435,7 +419,24 @@ int lbm_batch_create(lbm_batch** out, int32_t nbox, const int32_t* boxes, const 
         rows_total += boxes[3 * k + 1];
     }
     b->rows = b->rows && rows_total <= 65535;
-    b->zchunk = o.z_chunk > 0 ? o.z_chunk : (b->rows ? 32 : 16);
+    // Row kernel: as few z chunks (each reads two halo planes more than it
+    // writes) as still put CTAs on 60 % of the slots.  Measured per step at
+    // chunks of 16 / 32 / 64 planes: 4 boxes of edges 40 to 64 73 / 98 / 158 us, 16
+    // boxes 254 / 234 / 229, 128 boxes 1761 / 1611 / 1573.
+    b->zchunk = 16;
+    if (b->rows) {
+        const int resident = rows_batch_resident_ctas();
+        int lz = 1;
+        for (int k = 0; k < nbox; ++k) lz = std::max(lz, boxes[3 * k + 2]);
+        for (int c = 1;; ++c) {
+            b->zchunk = (lz + c - 1) / c;
+            long long ctas = 0;
+            for (int k = 0; k < nbox; ++k)
+                ctas += (long long)boxes[3 * k + 1] * ((boxes[3 * k + 2] + b->zchunk - 1) / b->zchunk);
+            if (10 * ctas >= 6LL * resident || b->zchunk <= 8) break;
+        }
+    }
+    if (o.z_chunk > 0) b->zchunk = o.z_chunk;
     b->boxes.resize(nbox);
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < nbox && e == cudaSuccess; ++k) {

@@ -277,18 +277,19 @@ template <int TX>
 struct StagePlane<TX, float> {
     static constexpr int SEG = TX + 8;
     static constexpr unsigned SMEM = 38u * SEG * 4u;                               // bytes of the image
-    static constexpr unsigned BYTES = 2u * (9u * 4u * TX + 10u * 4u * (TX + 4));  // bytes copied per plane
+    // bytes copied per plane of rows of width w (a multiple of 4)
+    static __host__ __device__ constexpr unsigned bytes(unsigned w) { return 2u * (9u * 4u * w + 10u * 4u * (w + 4u)); }
     struct Raw {
         float f[2][19];
     };
     static __device__ __forceinline__ void issue(const float* src, const Layout& L, int y, int p, unsigned dst,
-                                                 unsigned mbar, int lane) {
+                                                 unsigned mbar, int lane, unsigned w) {
         for (int a = lane; a < 38; a += 32) {
             const int s = a / 19, i = a - 19 * s;
             int cx, cy, cz;
             dir_rt(i, cx, cy, cz);
             const int lo = cx > 0 ? -4 : 0;
-            const unsigned len = cx != 0 ? 4u * (TX + 4) : 4u * TX;
+            const unsigned len = cx != 0 ? 4u * (w + 4u) : 4u * w;
             bulk_g2s(dst + 4u * (unsigned)(SEG * a + lo + 4), src + L.at(s, i, lo, y - cy, p - cz), len, mbar);
         }
     }
@@ -323,13 +324,15 @@ struct StagePlane<TX, Dev<T>> {
     static constexpr int SEG = TX + 8;  // words per deviation segment
     static constexpr unsigned NODE_BYTES = 16u * TX;
     static constexpr unsigned SMEM = NODE_BYTES + 18u * SEG * 4u;
-    static constexpr unsigned BYTES = NODE_BYTES + 8u * 4u * TX + 10u * 4u * (TX + 4);
+    static __host__ __device__ constexpr unsigned bytes(unsigned) {  // rows are TX wide
+        return NODE_BYTES + 8u * 4u * TX + 10u * 4u * (TX + 4);
+    }
     struct Raw {
         float4 o;
         unsigned w[19];  // w[i]: the word of direction i >= 1
     };
     static __device__ __forceinline__ void issue(const Dev<T>* src, const Layout& L, int y, int p, unsigned dst,
-                                                 unsigned mbar, int lane) {
+                                                 unsigned mbar, int lane, unsigned) {
         if (lane == 0) {
             bulk_g2s(dst, reinterpret_cast<const float4*>(src) + L.dev_node(0, y, p), NODE_BYTES, mbar);
         } else if (lane < 19) {
@@ -558,6 +561,9 @@ __global__ void __launch_bounds__(TX, MINB)
     const int rank = (int)cluster.block_rank();  // == blockIdx.y % CY for cluster dims (1, CY, 1)
     const MarchPlan<CY> plan(L, zchunk, alt);
     const bool xact = !BATCH || x < L.Lx;  // BATCH: a node of the box (not row padding)
+    // width of the copied rows: BATCH boxes leave their row padding out (idle
+    // nodes then read whatever the stage held, and use none of it)
+    const unsigned copy_w = BATCH ? (unsigned)((L.Lx + 3) & ~3) : (unsigned)TX;
 
     const unsigned ring_s = smem_u32(ring);
     const unsigned mbar_s = smem_u32(mbar);
@@ -648,11 +654,12 @@ __global__ void __launch_bounds__(TX, MINB)
             if (!plane_wanted(k)) return;
             const int st = (K0 + k) % NST;
             if (x == 0) {
-                mbar_expect_tx(smbar_s + 8u * st, SP::BYTES);
+                mbar_expect_tx(smbar_s + 8u * st, SP::bytes(copy_w));
                 pending |= 1u << st;
             }
             __syncwarp();
-            SP::issue(src, L, y, plane_of(k), stage_s + (unsigned)(st * SP::SMEM), smbar_s + 8u * st, x);
+            SP::issue(src, L, y, plane_of(k), stage_s + (unsigned)(st * SP::SMEM), smbar_s + 8u * st, x,
+                      copy_w);
         };
         auto stage_wait = [&](int k) {
             const int st = (K0 + k) % NST;
@@ -1094,9 +1101,9 @@ cudaError_t launch_rows(const void* src, void* dst, const Layout& L, const Model
                               RowsBatch{});
 }
 
-template <int TX, int CY, typename S, bool STAGED, bool MRT>
+template <int TX, int CY, typename S, bool STAGED, bool MRT, bool BATCH = false>
 int max_clusters() {
-    auto k = k_stream_collide_rows<TX, CY, row_min_blocks<TX, STAGED>(), S, STAGED, MRT>;
+    auto k = k_stream_collide_rows<TX, CY, row_min_blocks<TX, STAGED>(), S, STAGED, MRT, BATCH>;
     const size_t smem = row_smem<TX, CY, S, STAGED>();
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
@@ -1267,6 +1274,10 @@ bool rows_batch_applies(int Lx, int Ly, int Lz) {
 }
 
 size_t rows_batch_smem() { return rows_batch_bytes(); }
+
+int rows_batch_resident_ctas() {
+    return max_clusters<kRowsBatchWidth, kRowCluster, float, true, false, true>() * kRowCluster;
+}
 
 cudaError_t launch_rows_batch(const RowsBatch& rb, int groups, int max_chunks, int zchunk, const Model& m,
                               int* d_err, cudaStream_t s) {

@@ -209,6 +209,8 @@ bool rows_batch_applies(int Lx, int Ly, int Lz);
 // groups: total row groups (grid y / kRowClusterRows); max_chunks: grid z.
 cudaError_t launch_rows_batch(const RowsBatch& rb, int groups, int max_chunks, int zchunk, const Model& m,
                               int* d_err, cudaStream_t s);
+// CTAs of a batched launch that the device holds at once (0 if unknown).
+int rows_batch_resident_ctas();
 // Dynamic shared memory of a batched launch (bytes).
 size_t rows_batch_smem();
 
