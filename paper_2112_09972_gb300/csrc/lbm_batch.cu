@@ -81,7 +81,9 @@ __global__ void __launch_bounds__(256)
         yc = box_frame[4 * box + 1];
         zc = box_frame[4 * box + 2];
     }
-    ghost_node<float, float>(b.f[parity], b.L, g, xc, yc, zc, x, y, z, half, d_err);
+    with_face(face, [&](auto F) {
+        ghost_node<float, float, decltype(F)::value>(b.f[parity], b.L, g, xc, yc, zc, x, y, z, half, d_err);
+    });
 }
 
 __global__ void __launch_bounds__(kBatchThreads)

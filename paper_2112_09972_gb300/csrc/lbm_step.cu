@@ -149,10 +149,13 @@ __global__ void __launch_bounds__(256) k_ghost(S* __restrict__ f, Layout L, Ghos
     const int half = face < 2 ? (a & 1) : -1;
     int x, y, z;
     if (!shell_node(L, face, face < 2 ? a >> 1 : a, blockIdx.y * blockDim.y + threadIdx.y, x, y, z)) return;
-    if constexpr (is_dev_t<S>::value)
-        ghost_node_dev<decltype(dev_tag(S{})), C>(f, L, g, xc, yc, zc, x, y, z, half, d_err);
-    else
-        ghost_node<S, C>(f, L, g, xc, yc, zc, x, y, z, half, d_err);
+    with_face(face, [&](auto F) {
+        constexpr int FACE = decltype(F)::value;
+        if constexpr (is_dev_t<S>::value)
+            ghost_node_dev<decltype(dev_tag(S{})), C, FACE>(f, L, g, xc, yc, zc, x, y, z, half, d_err);
+        else
+            ghost_node<S, C, FACE>(f, L, g, xc, yc, zc, x, y, z, half, d_err);
+    });
 }
 
 template <typename S, typename C, bool PER, bool MRT, int MAXT>

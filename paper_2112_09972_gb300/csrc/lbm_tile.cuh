@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <cstring>
+#include <type_traits>
 
 #include "lbm_dev.cuh"
 #include "lbm_ghost.cuh"
@@ -298,7 +299,16 @@ __device__ __forceinline__ void store_sector_part(E* sector, int lane, E v, int 
 // such sector this thread writes (0 or 1, a pair of threads per node), or
 // -1 when the thread writes whole sectors alone; any other ghost value is
 // written by the thread with half <= 0.
-template <typename S, typename C>
+//
+// FACE (see shell_node) fixes the five directions that can stream into the
+// box from that face: a test of all eighteen against the box per node was
+// most of the ghost kernels' instructions.
+template <int FACE>
+__host__ __device__ __forceinline__ constexpr bool face_inward(int i) {
+    const int c = FACE < 2 ? cx_(i) : (FACE < 4 ? cy_(i) : cz_(i));
+    return c == (FACE & 1 ? -1 : 1);
+}
+template <typename S, typename C, int FACE>
 __device__ __forceinline__ void ghost_node(S* __restrict__ f, const Layout& L, const GhostParams<C>& g, C xc, C yc,
                                            C zc, int x, int y, int z, int half, int* __restrict__ d_err) {
     const GhostFlow<C> u = ghost_flow<C>(g, L, xc, yc, zc, x, y, z);
@@ -307,11 +317,12 @@ __device__ __forceinline__ void ghost_node(S* __restrict__ f, const Layout& L, c
     // row).  That sector is written whole -- the value and zero padding,
     // which nothing reads -- so that no partial sector is merged with DRAM.
     constexpr int SEC = 32 / (int)sizeof(S);
-    const bool whole = (x == -1 || x == L.Lx) && L.x0 == SEC && L.Lx % SEC == 0;
-    const int lane = x == -1 ? SEC - 1 : 0;  // the ghost's place in its sector
+    const bool whole = FACE < 2 && L.x0 == SEC && L.Lx % SEC == 0;
+    const int lane = FACE == 0 ? SEC - 1 : 0;  // the ghost's place in its sector
     bool any = false;
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
+        if (!face_inward<FACE>(i)) continue;
         const int xi = x + cx_(i), yi = y + cy_(i), zi = z + cz_(i);
         if (xi < 0 || xi >= L.Lx || yi < 0 || yi >= L.Ly || zi < 0 || zi >= L.Lz) continue;
         any = true;
@@ -330,7 +341,7 @@ __device__ __forceinline__ void ghost_node(S* __restrict__ f, const Layout& L, c
 // to (rho* of the state in f), both components of a direction in one 32-bit
 // word; x-face words that sit alone in sectors of row padding are written as
 // whole sectors (half as in ghost_node).
-template <typename T, typename C>
+template <typename T, typename C, int FACE>
 __device__ __forceinline__ void ghost_node_dev(Dev<T>* __restrict__ f, const Layout& L, const GhostParams<C>& gp,
                                                C xc, C yc, C zc, int x, int y, int z, int half,
                                                int* __restrict__ d_err) {
@@ -338,12 +349,13 @@ __device__ __forceinline__ void ghost_node_dev(Dev<T>* __restrict__ f, const Lay
     const float4* nb = reinterpret_cast<const float4*>(f);
     unsigned* w32 = reinterpret_cast<unsigned*>(f);
     // words of a row: x0 padding words, the Lx nodes, padding up to pitch
-    const bool whole = (x == -1 && L.x0 % 8 == 0) ||
-                       (x == L.Lx && (L.x0 + L.Lx) % 8 == 0 && L.pitch >= L.x0 + L.Lx + 8);
-    const int lane = x == -1 ? 7 : 0;  // the word's place in its sector
+    const bool whole = (FACE == 0 && L.x0 % 8 == 0) ||
+                       (FACE == 1 && (L.x0 + L.Lx) % 8 == 0 && L.pitch >= L.x0 + L.Lx + 8);
+    const int lane = FACE == 0 ? 7 : 0;  // the word's place in its sector
     bool any = false;
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
+        if (!face_inward<FACE>(i)) continue;
         const int xi = x + cx_(i), yi = y + cy_(i), zi = z + cz_(i);
         if (xi < 0 || xi >= L.Lx || yi < 0 || yi >= L.Ly || zi < 0 || zi >= L.Lz) continue;
         any = true;
@@ -376,6 +388,19 @@ __device__ __forceinline__ bool shell_node(const Layout& L, int face, int a, int
         z = face == 5 ? L.Lz : -1; x = a; y = b;
     }
     return true;
+}
+
+// fn(std::integral_constant<int, face>) for a face number uniform in the CTA.
+template <typename F>
+__device__ __forceinline__ void with_face(int face, F&& fn) {
+    switch (face) {
+        case 0: fn(std::integral_constant<int, 0>{}); break;
+        case 1: fn(std::integral_constant<int, 1>{}); break;
+        case 2: fn(std::integral_constant<int, 2>{}); break;
+        case 3: fn(std::integral_constant<int, 3>{}); break;
+        case 4: fn(std::integral_constant<int, 4>{}); break;
+        default: fn(std::integral_constant<int, 5>{});
+    }
 }
 
 }  // namespace
