@@ -573,34 +573,40 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 //
 // What bounds it: reading x (d0 x 512 bytes a tile) and the weights through
 // the SM's L2 port, about 7 us a tile at d0 = 576 and widths of 256, against
-// 5 us of tensor-core time.  Layer by layer, each product wrote and read its
-// activations through memory and was a launch of its own, as were the input
-// normalisation and the output scaling.
+// 5 us of tensor-core time and the chain product - epilogue - product of the
+// hidden layers.  Layer by layer, each product wrote and read its activations
+// through memory and was a launch of its own, as were the input normalisation
+// and the output scaling.
 //
-// Roles (14 warps):
-//   warps 0-3   the epilogues: a warp reads its 32 rows of an accumulator
-//               (tcgen05.ld), adds the bias, applies ReLU, rounds to bfloat16
-//               and writes the next layer's A operand (128-byte swizzle);
-//               after the last layer it scales and stores the outputs
-//   warps 4-11  read x two 64-column chunks ahead into registers, normalise,
+// Roles (20 warps):
+//   warps 0-7   the epilogues, two warps per 32 rows, each taking every other
+//               32-column block of an accumulator (tcgen05.ld): bias, ReLU,
+//               bfloat16, and the next layer's A operand (128-byte swizzle);
+//               after the last layer the outputs, scaled
+//   warps 8-15  read x two 64-column chunks ahead into registers, normalise,
 //               round to bfloat16 and fill the ring of first-layer A chunks
-//   warp 12     loads the weight chunks by TMA, in the order of their use
-//   warp 13     issues the products.  The first layer of the next tile
-//               accumulates in its own half of tensor memory, cut into
-//               pieces that run between the hidden layers of this tile, so
-//               that the tensor core has work while the epilogues run
+//   warps 16, 17  weight chunks of the first layer by TMA, and its products,
+//               in the first half of tensor memory
+//   warps 18, 19  the same for the other layers, in the second half
+// The first layer has a weight ring and an accumulator of its own, so that
+// the input of the next tile streams in while this tile's hidden layers wait
+// for their epilogues (with one ring and one issuing thread for both, the
+// input stood still meanwhile: 83 us at 65536 rows instead of 73).
 // The products take the same K steps in the same order as k_gemm_tc's, with
 // the same rounding points, so the outputs are the same bits.  Waits are
 // bounded as in k_gemm_tc.
-constexpr int kFwEpiWarps = 4, kFwLoadWarps = 8;
-constexpr int kFwThreads = 32 * (kFwEpiWarps + kFwLoadWarps + 2);
+constexpr int kFwEpiWarps = 8, kFwLoadWarps = 8;
+constexpr int kFwRole = kFwEpiWarps + kFwLoadWarps;  // first of the four single-thread roles
+constexpr int kFwThreads = 32 * (kFwRole + 4);
 constexpr int kFwMaxLayers = 6, kFwMaxWidth = 256;
-constexpr int kFwWStages = 4, kFwXStages = 2;
+constexpr int kFwWStages = 2, kFwXStages = 2;           // W: per ring
 constexpr unsigned kFwWBytes = kFwMaxWidth * TC_K * 2;  // 32 KB: one K chunk of a layer's weights
 constexpr unsigned kFwChunk = TC_M * TC_K * 2;          // 16 KB: one K chunk of an A operand
-constexpr unsigned kFwX0 = kFwWStages * kFwWBytes, kFwH0 = kFwX0 + kFwXStages * kFwChunk;
+constexpr unsigned kFwX0 = 2 * kFwWStages * kFwWBytes, kFwH0 = kFwX0 + kFwXStages * kFwChunk;
 constexpr unsigned kFwBar0 = kFwH0 + (kFwMaxWidth / TC_K) * kFwChunk;
-constexpr int kFwBars = 2 * kFwWStages + 2 * kFwXStages + 2 + 1 + 1;  // W and X full, empty; acc full; epilogue; drain
+// W full, empty per ring; X full, empty; accumulator full; first-layer
+// accumulator read; epilogue done; drain per issuing warp
+constexpr int kFwBars = 4 * kFwWStages + 2 * kFwXStages + 2 + 1 + 1 + 2;
 constexpr unsigned kFwSmem = 1024 + kFwBar0 + 8 * kFwBars + 16;
 constexpr unsigned kFwCols = 512;
 
@@ -649,32 +655,38 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
     const unsigned base = (raw + 1023u) & ~1023u;
     const unsigned bar0 = base + kFwBar0;
     unsigned* tmem_slot = reinterpret_cast<unsigned*>(fw_smem_raw + (bar0 + 8u * kFwBars - raw));
-    auto wfull = [&](unsigned s) { return bar0 + 8u * s; };
-    auto wempty = [&](unsigned s) { return bar0 + 8u * (kFwWStages + s); };
-    auto xfull = [&](unsigned s) { return bar0 + 8u * (2 * kFwWStages + s); };
-    auto xempty = [&](unsigned s) { return bar0 + 8u * (2 * kFwWStages + kFwXStages + s); };
-    auto accfull = [&](unsigned b) { return bar0 + 8u * (2 * kFwWStages + 2 * kFwXStages + b); };
-    const unsigned epi_bar = bar0 + 8u * (2 * kFwWStages + 2 * kFwXStages + 2), drain_bar = epi_bar + 8u;
+    // ring 0: first layer, ring 1: the others
+    auto wfull = [&](unsigned ring, unsigned s) { return bar0 + 8u * (2u * kFwWStages * ring + s); };
+    auto wempty = [&](unsigned ring, unsigned s) { return bar0 + 8u * (2u * kFwWStages * ring + kFwWStages + s); };
+    const unsigned bar1 = bar0 + 8u * (4 * kFwWStages);
+    auto xfull = [&](unsigned s) { return bar1 + 8u * s; };
+    auto xempty = [&](unsigned s) { return bar1 + 8u * (kFwXStages + s); };
+    const unsigned bar2 = bar1 + 8u * (2 * kFwXStages);
+    auto accfull = [&](unsigned b) { return bar2 + 8u * b; };
+    const unsigned acc0_read = bar2 + 16u, epi_bar = bar2 + 24u;
+    auto drain = [&](unsigned ring) { return bar2 + 32u + 8u * ring; };
     volatile int* stop = &stop_flag;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
 
     if (t == 0) {
         stop_flag = 0;
-        for (unsigned s = 0; s < kFwWStages; ++s) {
-            tc_mbar_init(wfull(s), 1);
-            tc_mbar_init(wempty(s), 1);
+        for (unsigned r = 0; r < 2; ++r) {
+            for (unsigned s = 0; s < kFwWStages; ++s) {
+                tc_mbar_init(wfull(r, s), 1);
+                tc_mbar_init(wempty(r, s), 1);
+            }
+            tc_mbar_init(accfull(r), 1);
+            tc_mbar_init(drain(r), 1);
         }
         for (unsigned s = 0; s < kFwXStages; ++s) {
             tc_mbar_init(xfull(s), kFwLoadWarps);
             tc_mbar_init(xempty(s), 1);
         }
-        tc_mbar_init(accfull(0), 1);
-        tc_mbar_init(accfull(1), 1);
+        tc_mbar_init(acc0_read, kFwEpiWarps);
         tc_mbar_init(epi_bar, kFwEpiWarps);
-        tc_mbar_init(drain_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 13) {
+    if (warp == kFwRole) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(tmem_slot)),
                      "n"(kFwCols)
                      : "memory");
@@ -693,12 +705,13 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
         *stop = 1;
         atomicOr(a.err, 1);
     };
-    unsigned issued = 0;  // warp 12, lane 0: weight chunks loaded
+    unsigned issued = 0;  // the loading threads: weight chunks loaded
 
     if (warp < kFwEpiWarps) {
-        const int row = warp * 32 + lane;
+        const int quad = warp & 3, half = warp >> 2;  // TMEM lanes 32 quad .. + 31; column blocks half, half + 2, ...
+        const int row = quad * 32 + lane;
         const unsigned swz = (unsigned)(row & 7), hrow = base + kFwH0 + (unsigned)row * 128u;
-        const unsigned lanes = tmem + ((unsigned)(warp * 32) << 16);
+        const unsigned lanes = tmem + ((unsigned)(quad * 32) << 16);
         unsigned hidden = 0;  // accumulations in the second half so far
         for (int j = 0; j < mine; ++j) {
             const long long m = (long long)(blockIdx.x + j * gridDim.x) * TC_M + row;
@@ -715,7 +728,7 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                 const float* bias = a.bias[l];
                 if (l + 1 < L) {
 #pragma unroll 1
-                    for (int n = 0; n < a.width[l]; n += 32) {
+                    for (int n = 32 * half; n < a.width[l]; n += 64) {
                         unsigned v[32];
                         fw_ld32(acc + (unsigned)n, v);
                         const unsigned dst = hrow + (unsigned)(n / TC_K) * kFwChunk;
@@ -733,7 +746,7 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                         }
                     }
                     fw_fence_async();
-                } else {
+                } else if (half == 0) {
                     unsigned v[32];
                     fw_ld32(acc, v);
                     float* out = a.y + m * a.dL;
@@ -746,10 +759,13 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) tc_arrive(epi_bar);
+                if (lane == 0) {
+                    if (l == 0) tc_arrive(acc0_read);
+                    tc_arrive(epi_bar);
+                }
             }
         }
-    } else if (warp < kFwEpiWarps + kFwLoadWarps) {
+    } else if (warp < kFwRole) {
         // chunk q of this CTA: 64 columns of a tile; a thread takes 4 columns of 8 rows
         const int lt = t - 32 * kFwEpiWarps, g = lt & 15, r0 = lt >> 4;
         const int total = mine * nk0;
@@ -762,6 +778,9 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
         };
         auto put = [&](int q, const float4 (&v)[8]) -> bool {
             const unsigned s = (unsigned)q % kFwXStages, round = (unsigned)q / kFwXStages;
+            const int c = (q % nk0) * TC_K + 4 * g;
+            const float4 mu = __ldg(reinterpret_cast<const float4*>(a.x_mean + c));
+            const float4 sc = __ldg(reinterpret_cast<const float4*>(a.x_scale + c));
             int ok = 1;
             if (round > 0) {
                 if (lane == 0) {
@@ -771,9 +790,6 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                 ok = __shfl_sync(0xffffffffu, ok, 0);
             }
             if (!ok) return false;
-            const int c = (q % nk0) * TC_K + 4 * g;
-            const float4 mu = __ldg(reinterpret_cast<const float4*>(a.x_mean + c));
-            const float4 sc = __ldg(reinterpret_cast<const float4*>(a.x_scale + c));
             const unsigned dst = base + kFwX0 + s * kFwChunk;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -797,45 +813,35 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
             load(q + 3, vb);
         }
     } else if (lane == 0) {
-        // the weight chunks and the products follow one schedule: the first
-        // layer of the first tile; then per tile each hidden layer, followed
-        // by its share of the next tile's first layer
-        const bool loader = warp == 12;
-        unsigned wit = 0, xit = 0, epi = 0, epis_due = 0;
+        const unsigned role = (unsigned)(warp - kFwRole), ring = role >> 1;
+        const bool loader = (role & 1u) == 0;
+        unsigned it = 0;  // chunks of this ring so far
         bool ok = true;
-        auto chunk = [&](int l, int kt) {  // one K chunk of layer l
-            const unsigned s = wit % kFwWStages, round = wit / kFwWStages;
-            ++wit;
+        // K chunk kt of layer l: its weights loaded, or its products issued (A at a_s)
+        auto chunk = [&](int l, int kt, unsigned a_s) {
+            const unsigned s = it % kFwWStages, round = it / kFwWStages;
+            ++it;
+            const unsigned w_s = base + (ring * kFwWStages + s) * kFwWBytes;
             if (loader) {
-                if (round > 0 && !tc_wait(wempty(s), (round - 1u) & 1u, stop)) {
+                if (round > 0 && !tc_wait(wempty(ring, s), (round - 1u) & 1u, stop)) {
                     ok = false;
                     return;
                 }
-                tc_expect_tx(wfull(s), (unsigned)a.width[l] * TC_K * 2u);
-                tc_tma_load(base + s * kFwWBytes, &a.w[l], kt * TC_K, 0, wfull(s));
+                tc_expect_tx(wfull(ring, s), (unsigned)a.width[l] * TC_K * 2u);
+                tc_tma_load(w_s, &a.w[l], kt * TC_K, 0, wfull(ring, s));
                 ++issued;
                 return;
             }
-            unsigned a_s = base + kFwH0 + (unsigned)kt * kFwChunk, xs = 0;
-            if (l == 0) {
-                xs = xit % kFwXStages;
-                if (!tc_wait(xfull(xs), (xit / kFwXStages) & 1u, stop)) {
-                    ok = false;
-                    return;
-                }
-                ++xit;
-                a_s = base + kFwX0 + xs * kFwChunk;
-            }
-            if (!tc_wait(wfull(s), round & 1u, stop)) {
+            if (!tc_wait(wfull(ring, s), round & 1u, stop)) {
                 ok = false;
                 return;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const unsigned acc = tmem + (l == 0 ? 0u : 256u), idesc = tc_idesc(TC_M, a.width[l]);
+            const unsigned acc = tmem + 256u * ring, idesc = tc_idesc(TC_M, a.width[l]);
 #pragma unroll
             for (int kk = 0; kk < TC_K / 16; ++kk) {
                 const unsigned long long ad = tc_desc_sw128(a_s + 32u * kk);
-                const unsigned long long bd = tc_desc_sw128(base + s * kFwWBytes + 32u * kk);
+                const unsigned long long bd = tc_desc_sw128(w_s + 32u * kk);
                 const unsigned accumulate = (kt > 0 || kk > 0) ? 1u : 0u;
                 asm volatile(
                     "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
@@ -843,44 +849,59 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                     "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate)
                     : "memory");
             }
-            tc_commit(wempty(s));
-            if (l == 0) tc_commit(xempty(xs));
+            tc_commit(wempty(ring, s));
         };
-        for (int kt = 0; ok && kt < nk0; ++kt) chunk(0, kt);
-        if (ok && !loader) tc_commit(accfull(0));
-        for (int j = 0; ok && j < mine; ++j) {
-            for (int l = 1; ok && l < L; ++l) {
-                if (!loader) {
+        if (ring == 0) {
+            unsigned xit = 0;
+            for (int j = 0; ok && j < mine; ++j) {
+                // the accumulator of the tile before has been read
+                if (!loader && j > 0) ok = tc_wait(acc0_read, (unsigned)(j - 1) & 1u, stop);
+                for (int kt = 0; ok && kt < nk0; ++kt) {
+                    const unsigned xs = xit % kFwXStages;
+                    if (!loader && !tc_wait(xfull(xs), (xit / kFwXStages) & 1u, stop)) {
+                        ok = false;
+                        break;
+                    }
+                    ++xit;
+                    chunk(0, kt, base + kFwX0 + xs * kFwChunk);
+                    if (ok && !loader) tc_commit(xempty(xs));
+                }
+                if (ok && !loader) tc_commit(accfull(0));
+            }
+        } else {
+            unsigned epi = 0;
+            for (int j = 0; ok && j < mine; ++j)
+                for (int l = 1; ok && l < L; ++l) {
                     // the epilogue of the layer before (and, at l = 1, of the
                     // tile before): every phase is waited for in turn
-                    epis_due = (unsigned)(j * L + l);
-                    for (; ok && epi < epis_due; ++epi) ok = tc_wait(epi_bar, epi & 1u, stop);
-                    if (!ok) break;
+                    if (!loader)
+                        for (const unsigned due = (unsigned)(j * L + l); ok && epi < due; ++epi)
+                            ok = tc_wait(epi_bar, epi & 1u, stop);
+                    for (int kt = 0; ok && kt < a.width[l - 1] / TC_K; ++kt)
+                        chunk(l, kt, base + kFwH0 + (unsigned)kt * kFwChunk);
+                    if (ok && !loader) tc_commit(accfull(1));
                 }
-                for (int kt = 0; ok && kt < a.width[l - 1] / TC_K; ++kt) chunk(l, kt);
-                if (ok && !loader) tc_commit(accfull(1));
-                if (j + 1 < mine) {
-                    for (int kt = (l - 1) * nk0 / (L - 1); ok && kt < l * nk0 / (L - 1); ++kt) chunk(0, kt);
-                    if (ok && !loader && l == L - 1) tc_commit(accfull(0));
-                }
-            }
         }
         if (!ok) give_up();
-        if (!loader) tc_commit(drain_bar);  // completes when every product issued above has
+        if (!loader) tc_commit(drain(ring));  // completes when every product issued above has
     }
 done:
     __syncthreads();
-    if (warp == 12 && lane == 0 && *stop) {
-        for (unsigned s = 0; s < kFwWStages; ++s) {  // copies issued but perhaps not consumed: the last one of each stage
-            if (issued <= s) continue;
-            const unsigned last = issued - 1u - ((issued - 1u - s) % kFwWStages);
-            tc_wait(wfull(s), (last / kFwWStages) & 1u, nullptr);
+    if (warp >= kFwRole && lane == 0) {
+        const unsigned role = (unsigned)(warp - kFwRole), ring = role >> 1;
+        if (role & 1u) {
+            if (!tc_wait(drain(ring), 0u, nullptr)) atomicOr(a.err, 1);
+        } else if (*stop) {
+            for (unsigned s = 0; s < kFwWStages; ++s) {  // copies issued but perhaps not consumed: the last one of each stage
+                if (issued <= s) continue;
+                const unsigned last = issued - 1u - ((issued - 1u - s) % kFwWStages);
+                tc_wait(wfull(ring, s), (last / kFwWStages) & 1u, nullptr);
+            }
         }
     }
-    if (warp == 13 && lane == 0 && !tc_wait(drain_bar, 0u, nullptr)) atomicOr(a.err, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 13) {
+    if (warp == kFwRole) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kFwCols) : "memory");
     }
