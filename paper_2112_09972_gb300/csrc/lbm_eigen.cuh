@@ -78,16 +78,56 @@ __device__ __noinline__ double deformation_jacobi(const double (&m)[6]) {
     return hi + lo > 0.0 ? (hi - lo) / (hi + lo) : 0.0;
 }
 
-// 1 / sqrt(a) and 1 / a in float64 from float32 seeds (a within float32's range).
+// 1 / sqrt(a) and 1 / a in float64 from float32 seeds (a within float32's
+// range): with e = 1 - a y^2 or 1 - a y of the seed y (1e-7), the series of
+// (1 - e)^-1/2 and (1 - e)^-1 to e^2 leaves e^3.
 __device__ __forceinline__ double rsqrt64(double a) {
-    double y = (double)rsqrtf((float)a);
-    y = fma(0.5 * y, fma(-a * y, y, 1.0), y);
-    return fma(0.5 * y, fma(-a * y, y, 1.0), y);
+    const double y = (double)rsqrtf((float)a), e = fma(-a * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 __device__ __forceinline__ double rcp64(double a) {
-    double y = (double)__frcp_rn((float)a);
-    y = fma(y, fma(-a, y, 1.0), y);
-    return fma(y, fma(-a, y, 1.0), y);
+    const double y = (double)__frcp_rn((float)a), e = fma(-a, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// One Newton step of x^3 - 3 x = r2 with a float32 slope.
+__device__ __forceinline__ double root_step(double x, double r2) {
+    const double xx = x * x;
+    return fma(-fma(x, xx - 3.0, -r2), (double)__frcp_rn(3.f * ((float)xx - 1.f)), x);
+}
+
+// Half the distance of the two close eigenvalues of the traceless symmetric
+// N = (a, n1, n2; n1, b, n4; n2, n4, c) whose third one is mu, |mu| about
+// twice theirs: N is projected on the plane normal to mu's eigenvector, so
+// the error is that of N's entries however close the two are, where a root of
+// the characteristic polynomial would lose half the digits.
+__device__ __forceinline__ double half_gap(double a, double b, double c, double n1, double n2, double n4, double mu) {
+    // N - mu is -+3 p (1 - v v^T): the smallest diagonal entry names v's
+    // largest component, which the permutation makes the third
+    const double da = fabs(a - mu), db = fabs(b - mu), dc = fabs(c - mu);
+    if (da < dc && da <= db) {
+        double t = a; a = c; c = t;
+        t = n1; n1 = n4; n4 = t;
+    } else if (db < dc) {
+        double t = b; b = c; c = t;
+        t = n1; n1 = n2; n2 = t;
+    }
+    const double ea = a - mu, eb = b - mu;
+    double x = fma(n1, n4, -n2 * eb), y = fma(n1, n2, -n4 * ea), z = fma(ea, eb, -n1 * n1);
+    const double iv = rsqrt64(fma(x, x, fma(y, y, z * z)));
+    x *= iv;
+    y *= iv;
+    z *= iv;  // positive: (3 p)^2 v_z^2
+    // orthonormal u, w normal to (x, y, z)
+    const double g = -rcp64(1.0 + z), h = x * y * g;
+    const double u0 = fma(x * x, g, 1.0), w1 = fma(y * y, g, 1.0);
+    const double nu0 = fma(a, u0, fma(n1, h, -n2 * x)), nu1 = fma(n1, u0, fma(b, h, -n4 * x)),
+                 nu2 = fma(n2, u0, fma(n4, h, -c * x));
+    const double nw0 = fma(a, h, fma(n1, w1, -n2 * y)), nw1 = fma(n1, h, fma(b, w1, -n4 * y)),
+                 nw2 = fma(n2, h, fma(n4, w1, -c * y));
+    const double uu = fma(u0, nu0, fma(h, nu1, -x * nu2)), ww = fma(h, nw0, fma(w1, nw1, -y * nw2));
+    const double uw = fma(h, nu0, fma(w1, nu1, -y * nu2)), d = 0.5 * (uu - ww);
+    return sqrt(fma(d, d, uw * uw));
 }
 
 // The same D for the conformation tensors of the surrogate and of the
@@ -95,41 +135,51 @@ __device__ __forceinline__ double rcp64(double a) {
 // kernels, so instead of Jacobi sweeps (about 300 FP64 instructions) the two
 // outer eigenvalues q + p x are the outer roots of x^3 - 3 x = 2 r (q the mean
 // eigenvalue, p^2 = |m - q|^2 / 6, 2 r = det((m - q) / p)): x = 2 cos(.) in
-// float32, then three Newton steps whose slope's reciprocal is float32,
-// about 90 FP64 instructions.  Near a double root (|r| within 1e-4 of 1: the
-// roots' error is then amplified above 1e-13), near a sphere, for eigenvalues
-// that are not well above zero and outside float32's range, Jacobi decides.
+// float32, then two Newton steps whose slope's reciprocal is float32 (1e-7 ->
+// 1e-13 -> rounding); and sqrt(l1), sqrt(l3) enter as their product alone,
+//   D = (l1 - l3) / (l1 + l3 + 2 sqrt(l1 l3)),
+// about 60 FP64 instructions.  m - q is formed from the differences of the
+// diagonal, which keeps its digits near a sphere.  Near a double root (r
+// within 1e-3 of +-1) the simple root and half_gap give the eigenvalues.
+// For a sphere (|m - q| below 1e-10 q), for eigenvalues that are not well
+// above zero and outside float32's range Jacobi decides.
 __device__ __forceinline__ double deformation_of(const double (&m)[6]) {
-    const double q = (m[0] + m[3] + m[5]) * (1.0 / 3.0);
-    const double a = m[0] - q, b = m[3] - q, c = m[5] - q;
+    const double third = 1.0 / 3.0, q = (m[0] + m[3] + m[5]) * third;
+    const double d0 = m[0] - m[3], d1 = m[3] - m[5];
+    const double a = fma(2.0, d0, d1) * third, b = (d1 - d0) * third, c = -a - b;
     const double off2 = fma(m[1], m[1], fma(m[2], m[2], m[4] * m[4]));
     const double p2 = fma(a, a, fma(b, b, fma(c, c, 2.0 * off2))) * (1.0 / 6.0);
     const float qf = (float)q, p2f = (float)p2;
-    if (qf > 1e-12f && qf < 1e12f && p2f > 1e-10f * qf * qf && p2f < 0.2f * qf * qf) {
+    if (qf > 1e-12f && qf < 1e12f && p2f > 1e-30f && p2f > 1e-20f * qf * qf && p2f < 0.2f * qf * qf) {
         const double ip = rsqrt64(p2);
         const double p = p2 * ip;
         // 2 r = det(m - q) / p^3
         const double det = fma(a, fma(b, c, -m[4] * m[4]),
                                fma(m[1], fma(m[4], m[2], -m[1] * c), m[2] * fma(m[1], m[4], -b * m[2])));
         const double r2 = det * ip * ip * ip;
-        const float rf = 0.5f * (float)r2;
-        if (fabsf(rf) < 1.f - 1e-4f) {
-            const float phi = acosf(rf) * (1.f / 3.f);
-            double x[2] = {(double)(2.f * cosf(phi)), (double)(2.f * cosf(phi + 2.0943951f))};
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-#pragma unroll
-                for (int it = 0; it < 3; ++it) {
-                    const double xx = x[e] * x[e];
-                    const double f = fma(x[e], xx - 3.0, -r2);
-                    const float slope = 3.f * ((float)xx - 1.f);
-                    x[e] = fma(-f, (double)__frcp_rn(slope), x[e]);
-                }
-            const double l1 = fma(p, x[0], q), l3 = fma(p, x[1], q);
-            if (l3 > 1e-3 * q) {
-                const double s1 = l1 * rsqrt64(l1), s3 = l3 * rsqrt64(l3);
-                return (s1 - s3) * rcp64(s1 + s3);
-            }
+        // r = cos 3 phi, from its distance to the nearer end
+        const float ef = fmaxf((float)fma(-0.5, fabs(r2), 1.0), 0.f);
+        double l1, l3;
+        if (ef > 1e-3f) {
+            const float th = (2.f / 3.f) * asinf(sqrtf(0.5f * ef));
+            const float phi = r2 >= 0.0 ? th : 1.04719755f - th;
+            const double x1 = (double)(2.f * cosf(phi)), x3 = (double)(2.f * cosf(phi + 2.0943951f));
+            l1 = p * root_step(root_step(x1, r2), r2);
+            l3 = p * root_step(root_step(x3, r2), r2);
+        } else {
+            // the root near +-2, from 2 - 2 (1 - |r|) / 9
+            const double x = copysign(2.0 - (2.0 / 9.0) * (double)ef, r2);
+            const double mu = p * root_step(root_step(x, r2), r2);
+            const double gap = half_gap(a, b, c, m[1], m[2], m[4], mu);
+            l1 = r2 >= 0.0 ? mu : fma(-0.5, mu, gap);
+            l3 = r2 >= 0.0 ? fma(-0.5, mu, -gap) : mu;
+        }
+        const double n = l1 - l3;
+        l1 += q;
+        l3 += q;
+        if (l3 > 1e-3 * q) {
+            const double g = l1 * l3;
+            return n * rcp64(fma(2.0 * g, rsqrt64(g), l1 + l3));
         }
     }
     return deformation_jacobi(m);

@@ -1170,8 +1170,13 @@ __global__ void k_output(const float* __restrict__ yhat, int ldy, long long n, i
 // D of Sec. 2, Eq. 4 from a predicted conformation tensor M (entries xx, xy,
 // xz, yy, yz, zz): D = (sqrt(l1) - sqrt(l3)) / (sqrt(l1) + sqrt(l3)) of its
 // eigenvalues (D does not depend on the normalisation of M).
+// The FP64 pipe bounds it; two warps to a CTA spread a batch evenly over the
+// SMs.  It is launched without programmatic overlap: CTAs that start beside a
+// persistent kernel all land on the few SMs which that one leaves free and
+// then run there one after the other (65536 rows: 69 us instead of 20; forward
+// and D together 141 -> 93 us in a row of calls).
+constexpr int kDeformThreads = 64;
 __global__ void k_deform_from_m(const float* __restrict__ m6, long long n, double* __restrict__ D) {
-    lbmgb::pdl_wait();
     lbmgb::pdl_trigger();
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
@@ -1765,7 +1770,8 @@ int lbm_mlp_deformation(lbm_mlp* c, const float* x, int64_t n, float* m6, double
     if (!c || n < 0 || (n > 0 && (!x || !m6 || !D)) || c->d[c->L] != 6) return LBM_EINVAL;
     int st = lbm_mlp_forward(c, x, m6, n);
     if (st || n == 0) return st;  // no launch for an empty batch
-    MLP_TRY(launch(c, k_deform_from_m, dim3(blocks_for(n, 128)), dim3(128), 0, (const float*)m6, (long long)n, D));
+    k_deform_from_m<<<blocks_for(n, kDeformThreads), kDeformThreads, 0, c->stream>>>(m6, n, D);
+    MLP_TRY(cudaGetLastError());
     return LBM_OK;
 }
 
