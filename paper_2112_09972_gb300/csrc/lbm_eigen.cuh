@@ -78,31 +78,50 @@ __device__ __noinline__ double deformation_jacobi(const double (&m)[6]) {
     return hi + lo > 0.0 ? (hi - lo) / (hi + lo) : 0.0;
 }
 
-// 1 / sqrt(a) and 1 / a in float64 from float32 seeds (a within float32's
-// range): with e = 1 - a y^2 or 1 - a y of the seed y (1e-7), the series of
+// float64 to float32 (truncated) and back by shifts, for magnitudes between
+// 2^-100 and 2^100: conversions to and from 64 bits run on the FP64 pipe, at
+// its rate of one warp instruction per 16 cycles and SM.
+__device__ __forceinline__ float narrow(double d) {
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    return __uint_as_float((hi & 0x80000000u) | __funnelshift_l(lo, (hi & 0x7fffffffu) - (896u << 20), 3));
+}
+__device__ __forceinline__ double widen(float f) {
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+// 1 / d from the reciprocal unit, to 23 bits.
+__device__ __forceinline__ float rcp_seed(float d) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
+    return y;
+}
+
+// 1 / sqrt(a) and 1 / a in float64 from float32 seeds (a within 2^+-100):
+// with e = 1 - a y^2 or 1 - a y of the seed y (1e-7), the series of
 // (1 - e)^-1/2 and (1 - e)^-1 to e^2 leaves e^3.
 __device__ __forceinline__ double rsqrt64(double a) {
-    const double y = (double)rsqrtf((float)a), e = fma(-a * y, y, 1.0);
+    const double y = widen(rsqrtf(narrow(a))), e = fma(-a * y, y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 __device__ __forceinline__ double rcp64(double a) {
-    const double y = (double)__frcp_rn((float)a), e = fma(-a, y, 1.0);
+    const double y = widen(rcp_seed(narrow(a))), e = fma(-a, y, 1.0);
     return fma(y, fma(e, e, e), y);
 }
 
-// One Newton step of x^3 - 3 x = r2 with a float32 slope.
+// One Newton step of x^3 - 3 x = r2 near an outer root (1 < |x|) with a
+// float32 slope.
 __device__ __forceinline__ double root_step(double x, double r2) {
     const double xx = x * x;
-    return fma(-fma(x, xx - 3.0, -r2), (double)__frcp_rn(3.f * ((float)xx - 1.f)), x);
+    return fma(-fma(x, xx - 3.0, -r2), widen(rcp_seed(3.f * (narrow(xx) - 1.f))), x);
 }
 
 // Half the distance of the two close eigenvalues of the traceless symmetric
-// N = (a, n1, n2; n1, b, n4; n2, n4, c) whose third one is mu, |mu| about
-// twice theirs: N is projected on the plane normal to mu's eigenvector, so
+// N = (a, n1, n2; n1, b, n4; n2, n4, c) whose third one is mu, close to 2 or
+// -2: N is projected on the plane normal to mu's eigenvector, so
 // the error is that of N's entries however close the two are, where a root of
 // the characteristic polynomial would lose half the digits.
 __device__ __forceinline__ double half_gap(double a, double b, double c, double n1, double n2, double n4, double mu) {
-    // N - mu is -+3 p (1 - v v^T): the smallest diagonal entry names v's
+    // N - mu is -+3 (1 - v v^T): the smallest diagonal entry names v's
     // largest component, which the permutation makes the third
     const double da = fabs(a - mu), db = fabs(b - mu), dc = fabs(c - mu);
     if (da < dc && da <= db) {
@@ -117,7 +136,7 @@ __device__ __forceinline__ double half_gap(double a, double b, double c, double 
     const double iv = rsqrt64(fma(x, x, fma(y, y, z * z)));
     x *= iv;
     y *= iv;
-    z *= iv;  // positive: (3 p)^2 v_z^2
+    z *= iv;  // positive: 9 v_z^2 before
     // orthonormal u, w normal to (x, y, z)
     const double g = -rcp64(1.0 + z), h = x * y * g;
     const double u0 = fma(x * x, g, 1.0), w1 = fma(y * y, g, 1.0);
@@ -163,14 +182,14 @@ __device__ __forceinline__ double deformation_of(const double (&m)[6]) {
         if (ef > 1e-3f) {
             const float th = (2.f / 3.f) * asinf(sqrtf(0.5f * ef));
             const float phi = r2 >= 0.0 ? th : 1.04719755f - th;
-            const double x1 = (double)(2.f * cosf(phi)), x3 = (double)(2.f * cosf(phi + 2.0943951f));
+            const double x1 = widen(2.f * cosf(phi)), x3 = widen(2.f * cosf(phi + 2.0943951f));
             l1 = p * root_step(root_step(x1, r2), r2);
             l3 = p * root_step(root_step(x3, r2), r2);
         } else {
             // the root near +-2, from 2 - 2 (1 - |r|) / 9
             const double x = copysign(2.0 - (2.0 / 9.0) * (double)ef, r2);
-            const double mu = p * root_step(root_step(x, r2), r2);
-            const double gap = half_gap(a, b, c, m[1], m[2], m[4], mu);
+            const double xs = root_step(root_step(x, r2), r2), mu = p * xs;
+            const double gap = p * half_gap(a * ip, b * ip, c * ip, m[1] * ip, m[2] * ip, m[4] * ip, xs);
             l1 = r2 >= 0.0 ? mu : fma(-0.5, mu, gap);
             l3 = r2 >= 0.0 ? fma(-0.5, mu, -gap) : mu;
         }

@@ -49,6 +49,8 @@ def test_fused_forward_is_the_layered_one(built, sizes, n):
 def _tensors():
     rng = np.random.default_rng(9)
     out = [np.diag([2.0, 1.0, 0.5]), np.eye(3), np.zeros((3, 3)), np.diag([1.0, -1.0, 3.0]), 1e-6 * np.diag([3.0, 2, 1])]
+    # the simple eigenvalue along each axis, the largest and the smallest one
+    out += [np.diag(np.roll([a, 1.0, b], k)) for k in range(3) for a, b in ((1.5, 1.0), (0.7, 1.0 + 1e-6))]
     for lam in ([1.2, 1.2, 0.7], [1.5, 0.8, 0.8], [1.2, 1.2 - 1e-5, 0.7], [1 + 1e-4, 1, 1 - 2e-4], [5.0, 1.0, 1e-4],
                 [1.1, 1.0, 0.9], [30.0, 20.0, 10.0], [1.0, 1e-3, 1e-5]):
         q, _ = np.linalg.qr(rng.normal(size=(3, 3)))
