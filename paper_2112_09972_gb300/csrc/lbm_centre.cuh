@@ -11,6 +11,44 @@
 namespace lbmgb {
 namespace {
 
+// The final sum by one warp: slots 0 .. total - 1 in order.
+template <typename C>
+__device__ void centre_total(const C* parts, unsigned total, unsigned* counter, double* sum8, float* frame) {
+    const int lane = threadIdx.x & 31;
+    __threadfence();
+    // eight slots' loads in flight at once (one after another, the L2
+    // latency of each made this sum several microseconds of every launch)
+    C s4[4] = {C(0), C(0), C(0), C(0)};
+    for (unsigned b0 = lane; b0 < total; b0 += 256u) {
+        C v[8][4];
+#pragma unroll
+        for (unsigned u = 0; u < 8; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[u][q] = b0 + 32u * u < total ? __ldcg(parts + 4LL * (b0 + 32u * u) + q) : C(0);
+#pragma unroll
+        for (unsigned u = 0; u < 8; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s4[q] += v[u][q];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s4[q] += __shfl_down_sync(0xffffffffu, s4[q], o);
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sum8[q] = (double)s4[q];
+        // frame origin x_c = sum w x / sum w (box centre when there is no droplet)
+        const bool have = s4[0] > C(0);
+        for (int q = 0; q < 3; ++q) {
+            const C xc = have ? s4[1 + q] / s4[0] : C(0);
+            sum8[4 + q] = (double)xc;
+            frame[q] = (float)xc;
+        }
+        *counter = 0u;
+    }
+}
+
 // Fixed-order reduction of centre partials by the last CTA to finish
 // (threadfence-reduction pattern); every thread of the CTA calls it.  C is
 // the reduction type (float32 for the float32 and 16-bit storage kernels, so
@@ -47,41 +85,7 @@ __device__ void centre_reduce(C (&cm)[4], C* parts, long long slot, unsigned tot
         }
     }
     __syncthreads();
-    if (last && warp == 0) {
-        __threadfence();
-        // eight slots' loads in flight at once (one after another, the L2
-        // latency of each made this sum several microseconds of every launch)
-        C s4[4] = {C(0), C(0), C(0), C(0)};
-        for (unsigned b0 = lane; b0 < total; b0 += 256u) {
-            C v[8][4];
-#pragma unroll
-            for (unsigned u = 0; u < 8; ++u)
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    v[u][q] = b0 + 32u * u < total ? __ldcg(parts + 4LL * (b0 + 32u * u) + q) : C(0);
-#pragma unroll
-            for (unsigned u = 0; u < 8; ++u)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) s4[q] += v[u][q];
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s4[q] += __shfl_down_sync(0xffffffffu, s4[q], o);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) sum8[q] = (double)s4[q];
-            // frame origin x_c = sum w x / sum w (box centre when there is no droplet)
-            const bool have = s4[0] > C(0);
-            for (int q = 0; q < 3; ++q) {
-                const C xc = have ? s4[1 + q] / s4[0] : C(0);
-                sum8[4 + q] = (double)xc;
-                frame[q] = (float)xc;
-            }
-            *counter = 0u;
-        }
-    }
+    if (last && warp == 0) centre_total(parts, total, counter, sum8, frame);
 }
 
 // The same over every CTA of the launch, in CTA order, into CentreParts.

@@ -8,10 +8,10 @@
 //       chunk of z planes one after another, about 3 us a plane whatever the
 //       box, so a box too small to fill the chip waits for that chain (10
 //       planes at 64^3).  Here all planes of a chunk run at once; the second
-//       read of the populations comes from L2, which such a box fits.  A CTA
-//       has the row and the z chunk of a CTA of the cluster kernel, sums each
-//       node's droplet indicator in that kernel's order and shares its node
-//       arithmetic (collide_core), so both store bit-identical states.
+//       read of the populations comes from L2, which such a box fits.  The
+//       centre is summed from the densities in the cluster kernel's order and
+//       the node arithmetic is shared (collide_core), so both store
+//       bit-identical states.
 //   k_any_rho / k_any_collide -- float32 boxes of any other extents, in place
 //       of the tile kernel, whose tiles sum their halo's densities again
 //       (about as many nodes as the tile has) and march in z.
@@ -19,6 +19,8 @@
 // Density array: [Lz + 2][Ly + 2][Lx + 2] of {rho_A, rho_B}, its halo holding
 // the ghost densities.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "lbm_centre.cuh"
 #include "lbm_internal.h"
@@ -79,44 +81,109 @@ __global__ void __launch_bounds__(TX * row_rho_rows<TX>()) k_row_rho(const ST* _
     rho[g.at(x, y, z)] = make_float2(ra, rb);
 }
 
-// Grid and z chunks of the cluster kernel (1, Ly, chunks); TX x ZL threads,
-// plane k of the chunk's march on z lane k mod ZL.
-template <int TX, typename ST, bool MRT>
-__global__ void __launch_bounds__(512) k_row_collide(const ST* __restrict__ src, ST* __restrict__ dst, Layout L,
-                                                     FastModel m, const float2* __restrict__ rho, RhoGeo g,
-                                                     int zchunk, CentreParts cp, int* __restrict__ d_err) {
-    using IO = RowIO<TX, ST>;
-    extern __shared__ float wk[];  // [zchunk][TX] droplet indicators, in march order
-    __shared__ float red[4 * 16];
-    pdl_wait();
-    const int x = threadIdx.x % TX, zl = threadIdx.x / TX, ZL = blockDim.x / TX, y = blockIdx.y;
-    const int zc0 = blockIdx.z * zchunk, zc1 = min(zc0 + zchunk, L.Lz), n = zc1 - zc0;
-    const bool down = blockIdx.z & 1;  // odd chunks march down, as the cluster kernel's do
-    const float px = (float)x - 0.5f * (float)(L.Lx - 1), py = (float)y - 0.5f * (float)(L.Ly - 1);
-    int bad = 0;
-    for (int k = zl; k < n; k += ZL) {
-        const int z = down ? zc1 - 1 - k : zc0 + k;
-        float f[2][19], rs[2], cw[4] = {0.f, 0.f, 0.f, 0.f};
-        IO::populations(node_planes<TX, ST>(src, L, x, y, z), f, rs);
-        const float2* r = rho + g.at(x, y, z);
-        collide_core<IO, ST, MRT>(RhoNb{r, g.nx, g.nx * g.ny}, __ldg(r), f, rs, m, IO::out(dst, L, x, y, z), cw, bad,
-                                  px, py, (float)z - 0.5f * (float)(L.Lz - 1));
-        wk[k * TX + x] = cw[0];
+// Centre-of-mass partials of `units` pieces of the box by the `ctas` CTAs of a
+// launch that this is the cta-th of, from the density pass's array, one warp
+// to a unit.  unit(u, cm) leaves the sums of unit u in its lane 0.  The CTAs
+// that collide then hold nothing back for a reduction and end when their
+// nodes are stored; these few run beside the last of them.
+template <typename U>
+__device__ void centre_units(U&& unit, int units, int cta, int ctas, CentreParts cp) {
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, warps = blockDim.x / 32;
+    __shared__ unsigned last;
+    float* parts = reinterpret_cast<float*>(cp.p);
+    for (int u = cta * warps + warp; u < units; u += ctas * warps) {
+        float cm[4] = {0.f, 0.f, 0.f, 0.f};
+        unit(u, cm);
+        if (lane == 0)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) parts[4LL * u + q] = cm[q];
     }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(cp.counter, 1u) == (unsigned)ctas - 1u ? 1u : 0u;
+    }
+    __syncthreads();
+    if (last && warp == 0) centre_total<float>(parts, (unsigned)units, cp.counter, cp.sum, cp.frame);
+}
+__device__ __forceinline__ float warp_total(float a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    return a;
+}
+// the droplet indicator of collide_core
+__device__ __forceinline__ float indicator(float2 r) { return fmaxf(__fdividef(r.x - r.y, r.x + r.y), 0.f); }
+
+// The sums of the cluster kernel's CTA (y, chunk), in its order: thread x over
+// the planes of its march, then the warps' shuffles.
+template <int TX>
+__device__ __forceinline__ void row_unit(const float2* __restrict__ rho, const RhoGeo& g, const Layout& L, int y,
+                                         int chunk, int zchunk, float (&cm)[4]) {
+    const int lane = threadIdx.x % 32;
+    const int zc0 = chunk * zchunk, zc1 = min(zc0 + zchunk, L.Lz), n = zc1 - zc0;
+    const bool down = chunk & 1;  // odd chunks march down
+    const float py = (float)y - 0.5f * (float)(L.Ly - 1);
+    float s[TX / 32][4] = {};
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+        const int z = down ? zc1 - 1 - k : zc0 + k;
+        const float pz = (float)z - 0.5f * (float)(L.Lz - 1);
+#pragma unroll
+        for (int h = 0; h < TX / 32; ++h) {
+            const float w = indicator(__ldg(rho + g.at(32 * h + lane, y, z)));
+            const float px = (float)(32 * h + lane) - 0.5f * (float)(L.Lx - 1);
+            s[h][0] += w;
+            s[h][1] = fmaf(w, px, s[h][1]);
+            s[h][2] = fmaf(w, py, s[h][2]);
+            s[h][3] = fmaf(w, pz, s[h][3]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float a = 0.f;
+#pragma unroll
+        for (int h = 0; h < TX / 32; ++h) {
+            const float t = __shfl_sync(0xffffffffu, warp_total(s[h][q]), 0);
+            if (lane == h) a = t;
+        }
+        cm[q] = warp_total(a);
+    }
+}
+
+// One node per thread; the last CTAs of the grid sum the centre.  Registers
+// allow 512 threads to an SM, held as CTAs of 128 (256 for the widest rows),
+// so that 64^3 is 3.4 rounds of small CTAs.  (With 512 threads over the planes
+// of a z chunk and their sums at the end it was four waves, each as long as
+// its slowest warp and the reduction: 64^3 bf16 25.3 -> 18.9 us per step, fp32
+// 30.8 -> 24.9, 32^3 fp32 11.4 -> 10.4.)
+template <int TX>
+constexpr int row_collide_rows() {
+    return TX >= 128 ? 1 : 128 / TX;
+}
+template <int TX, typename ST, bool MRT>
+__global__ void __launch_bounds__(TX * row_collide_rows<TX>(), 512 / (TX * row_collide_rows<TX>()))
+    k_row_collide(const ST* __restrict__ src, ST* __restrict__ dst, Layout L, FastModel m,
+                  const float2* __restrict__ rho, RhoGeo g, int colliders, int zchunk, int units, CentreParts cp,
+                  int* __restrict__ d_err) {
+    using IO = RowIO<TX, ST>;
+    constexpr int R = row_collide_rows<TX>();
+    pdl_wait();
+    if ((int)blockIdx.x >= colliders) {
+        pdl_trigger();
+        centre_units([&](int u, float (&cm)[4]) { row_unit<TX>(rho, g, L, u % L.Ly, u / L.Ly, zchunk, cm); }, units,
+                     (int)blockIdx.x - colliders, (int)gridDim.x - colliders, cp);
+        return;
+    }
+    const int per_plane = L.Ly / R, z = blockIdx.x / per_plane;
+    const int x = threadIdx.x % TX, y = (blockIdx.x - z * per_plane) * R + threadIdx.x / TX;
+    int bad = 0;
+    float f[2][19], rs[2], cm[4] = {0.f, 0.f, 0.f, 0.f};
+    IO::populations(node_planes<TX, ST>(src, L, x, y, z), f, rs);
+    const float2* r = rho + g.at(x, y, z);
+    collide_core<IO, ST, MRT>(RhoNb{r, g.nx, g.nx * g.ny}, __ldg(r), f, rs, m, IO::out(dst, L, x, y, z), cm, bad, 0.f,
+                              0.f, 0.f);
     pdl_trigger();
     if (bad) atomicOr(d_err, bad);
-    __syncthreads();
-    // the sums of the cluster kernel's thread x, in its order
-    float cm[4] = {0.f, 0.f, 0.f, 0.f};
-    if (zl == 0)
-        for (int k = 0; k < n; ++k) {
-            const float w = wk[k * TX + x], pz = (float)(down ? zc1 - 1 - k : zc0 + k) - 0.5f * (float)(L.Lz - 1);
-            cm[0] += w;
-            cm[1] = fmaf(w, px, cm[1]);
-            cm[2] = fmaf(w, py, cm[2]);
-            cm[3] = fmaf(w, pz, cm[3]);
-        }
-    centre_epilogue(cm, cp, red);
 }
 
 template <int TX, typename ST, bool MRT>
@@ -132,11 +199,12 @@ cudaError_t launch_row_t(const void* src, void* dst, void* rho, const Layout& L,
     const RhoGeo g = rho_geo(L);
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_row_rho<TX, ST>, (const ST*)src, L, (float2*)rho, g);
     if (e != cudaSuccess) return e;
-    cfg.gridDim = sh.grid;
-    cfg.blockDim = dim3(sh.threads, 1, 1);
-    cfg.dynamicSmemBytes = sh.smem;
+    constexpr int threads = TX * row_collide_rows<TX>();
+    const int units = (int)(sh.grid.y * sh.grid.z), colliders = L.Ly / row_collide_rows<TX>() * L.Lz;
+    cfg.gridDim = dim3(colliders + (units + threads / 32 - 1) / (threads / 32), 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
     return cudaLaunchKernelEx(&cfg, k_row_collide<TX, ST, MRT>, (const ST*)src, (ST*)dst, L, fast_model(m),
-                              (const float2*)rho, g, sh.zchunk, cp, d_err);
+                              (const float2*)rho, g, colliders, sh.zchunk, units, cp, d_err);
 }
 
 template <int TX>
@@ -164,52 +232,67 @@ struct AnyIO {
 };
 
 constexpr int kAnyThreads = 128;
+constexpr int kAnyShares = 8;  // centre sums: shares of a plane's rows, a warp each, at most one per CTA of a plane
 __global__ void __launch_bounds__(kAnyThreads) k_any_rho(const float* __restrict__ src, Layout L,
-                                                         float2* __restrict__ rho, RhoGeo g, int zchunk) {
+                                                         float2* __restrict__ rho, RhoGeo g, int per_plane) {
     pdl_wait();
     pdl_trigger();
-    const int p = blockIdx.x * kAnyThreads + threadIdx.x;
+    const int z = blockIdx.x / per_plane, p = (blockIdx.x - z * per_plane) * kAnyThreads + threadIdx.x;
     if (p >= L.Lx * L.Ly) return;
     const int y = p / L.Lx, x = p - y * L.Lx;
     const Puller<float, float, false> P{src, L};
-    const int z1 = min(((int)blockIdx.y + 1) * zchunk, L.Lz);
-    for (int z = blockIdx.y * zchunk; z < z1; ++z) {
-        float f[2][19];
-        P.pull(x, y, z, f);
-        rho[g.at(x, y, z)] = make_float2(sum19<float>(f[0]), sum19<float>(f[1]));
+    float f[2][19];
+    P.pull(x, y, z, f);
+    rho[g.at(x, y, z)] = make_float2(sum19<float>(f[0]), sum19<float>(f[1]));
+}
+
+// The sums of one plane's share of rows, lanes over x.
+__device__ __forceinline__ void any_unit(const float2* __restrict__ rho, const RhoGeo& g, const Layout& L, int u,
+                                         int shares, float (&cm)[4]) {
+    const int lane = threadIdx.x % 32, z = u / shares, share = u - z * shares;
+    const float pz = (float)z - 0.5f * (float)(L.Lz - 1);
+    for (int y = share; y < L.Ly; y += shares) {
+        const float py = (float)y - 0.5f * (float)(L.Ly - 1);
+#pragma unroll 4
+        for (int x = lane; x < L.Lx; x += 32) {
+            const float w = indicator(__ldg(rho + g.at(x, y, z)));
+            cm[0] += w;
+            cm[1] = fmaf(w, (float)x - 0.5f * (float)(L.Lx - 1), cm[1]);
+            cm[2] = fmaf(w, py, cm[2]);
+            cm[3] = fmaf(w, pz, cm[3]);
+        }
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cm[q] = warp_total(cm[q]);
 }
 
 template <bool MRT>
 __global__ void __launch_bounds__(kAnyThreads, 5)
     k_any_collide(const float* __restrict__ src, float* __restrict__ dst, Layout L, FastModel m,
-                  const float2* __restrict__ rho, RhoGeo g, int zchunk, CentreParts cp, int* __restrict__ d_err) {
-    __shared__ float scratch[4 * (kAnyThreads / 32)];
+                  const float2* __restrict__ rho, RhoGeo g, int per_plane, int colliders, CentreParts cp,
+                  int* __restrict__ d_err) {
     pdl_wait();
-    const int p = blockIdx.x * kAnyThreads + threadIdx.x;
+    if ((int)blockIdx.x >= colliders) {
+        pdl_trigger();
+        const int shares = min(kAnyShares, per_plane);
+        centre_units([&](int u, float (&cm)[4]) { any_unit(rho, g, L, u, shares, cm); }, shares * L.Lz,
+                     (int)blockIdx.x - colliders, (int)gridDim.x - colliders, cp);
+        return;
+    }
+    const int z = blockIdx.x / per_plane, p = (blockIdx.x - z * per_plane) * kAnyThreads + threadIdx.x;
     const int y = p / L.Lx, x = p - y * L.Lx;
-    const Puller<float, float, false> P{src, L};
-    float cm[4] = {0.f, 0.f, 0.f, 0.f};
-    int bad = 0;
     if (p < L.Lx * L.Ly) {
-        const float px = (float)x - 0.5f * (float)(L.Lx - 1), py = (float)y - 0.5f * (float)(L.Ly - 1);
-        const int z1 = min(((int)blockIdx.y + 1) * zchunk, L.Lz);
-        for (int z = blockIdx.y * zchunk; z < z1; ++z) {
-            float f[2][19];
-            const float rs[2] = {0.f, 0.f};
-            P.pull(x, y, z, f);
-            const float2* r = rho + g.at(x, y, z);
-            collide_core<AnyIO, float, MRT>(RhoNb{r, g.nx, g.nx * g.ny}, __ldg(r), f, rs, m,
-                                            AnyIO::Out{dst + L.at(0, 0, x, y, z), L.pitch}, cm, bad, px, py,
-                                            (float)z - 0.5f * (float)(L.Lz - 1));
-        }
+        const Puller<float, float, false> P{src, L};
+        int bad = 0;
+        float f[2][19], cm[4] = {0.f, 0.f, 0.f, 0.f};
+        const float rs[2] = {0.f, 0.f};
+        P.pull(x, y, z, f);
+        const float2* r = rho + g.at(x, y, z);
+        collide_core<AnyIO, float, MRT>(RhoNb{r, g.nx, g.nx * g.ny}, __ldg(r), f, rs, m,
+                                        AnyIO::Out{dst + L.at(0, 0, x, y, z), L.pitch}, cm, bad, 0.f, 0.f, 0.f);
+        if (bad) atomicOr(d_err, bad);
     }
     pdl_trigger();
-    if (bad) atomicOr(d_err, bad);
-    const unsigned cta = blockIdx.y * gridDim.x + blockIdx.x, total = gridDim.x * gridDim.y;
-    const bool any = __syncthreads_or(cm[0] != 0.f) != 0;
-    centre_reduce_last<kAnyThreads>(cm, any, reinterpret_cast<float*>(cp.p), cta, total, cp.counter, cp.sum, cp.frame,
-                                    scratch);
 }
 
 }  // namespace
@@ -218,31 +301,25 @@ long long flat32_rho_bytes(const Layout& L) {
     return (long long)sizeof(float2) * (L.Lx + 2) * (L.Ly + 2) * (L.Lz + 2);
 }
 
-// The two-pass launch of a row-tiled shape: its grid and z chunks, with as
-// many planes of a chunk at once as 512 threads hold.
+// The two-pass launch of a row-tiled shape keeps its grid and z chunks, by
+// which the centre sums are ordered.
 Shape flat_rows_shape(const Shape& rows) {
     Shape sh = rows;
-    int zl = 512 / rows.tx;
-    if (zl > rows.zchunk) zl = rows.zchunk;
     sh.flat = kFlatRows;
-    sh.threads = zl * rows.tx;
-    sh.smem = sizeof(float) * (size_t)rows.zchunk * rows.tx;
+    sh.threads = rows.tx > 128 ? rows.tx : 128;
+    sh.smem = 0;
     return sh;
 }
 
-// Any float32 box: one node per thread; the z extent is cut so that the
-// launch has at most about 32 CTAs per SM (the last CTA sums their partials).
-Shape flat_any_shape(const Layout& L, int num_sms) {
+// Any float32 box: one node per thread.
+Shape flat_any_shape(const Layout& L) {
     Shape sh = {};
     const long long per_plane = ((long long)L.Lx * L.Ly + kAnyThreads - 1) / kAnyThreads;
-    const long long want = 32LL * (num_sms > 0 ? num_sms : 152);
-    long long zc = (per_plane * L.Lz + want - 1) / want;
-    if (zc < 1) zc = 1;
     sh.flat = kFlatAny;
     sh.tx = L.Lx;
     sh.ty = L.Lx >= kAnyThreads ? 1 : kAnyThreads / L.Lx;
-    sh.zchunk = (int)zc;
-    sh.grid = dim3((unsigned)per_plane, (unsigned)((L.Lz + zc - 1) / zc), 1);
+    sh.zchunk = 1;
+    sh.grid = dim3((unsigned)per_plane, (unsigned)L.Lz, 1);
     sh.threads = kAnyThreads;
     return sh;
 }
@@ -267,7 +344,8 @@ cudaError_t launch_flat_rows(int prec, const void* src, void* dst, void* rho, co
 cudaError_t launch_flat_any(const void* src, void* dst, void* rho, const Layout& L, const Model& m, const Shape& sh,
                             CentreParts cp, int* d_err, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = sh.grid;
+    const int per_plane = (int)sh.grid.x, colliders = (int)(sh.grid.x * sh.grid.y);
+    cfg.gridDim = dim3(colliders, 1, 1);
     cfg.blockDim = dim3(kAnyThreads, 1, 1);
     cfg.stream = s;
     cudaLaunchAttribute attr[1] = {pdl_attribute()};
@@ -275,10 +353,13 @@ cudaError_t launch_flat_any(const void* src, void* dst, void* rho, const Layout&
     cfg.numAttrs = 1;
     const RhoGeo g = rho_geo(L);
     const float* f = (const float*)src;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_any_rho, f, L, (float2*)rho, g, sh.zchunk);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_any_rho, f, L, (float2*)rho, g, per_plane);
     if (e != cudaSuccess) return e;
+    // centre sums: four units (a share of a plane's rows) to a CTA
+    const int units = std::min(kAnyShares, per_plane) * L.Lz;
+    cfg.gridDim = dim3(colliders + (units + kAnyThreads / 32 - 1) / (kAnyThreads / 32), 1, 1);
     return cudaLaunchKernelEx(&cfg, m.mrt ? k_any_collide<true> : k_any_collide<false>, f, (float*)dst, L,
-                              fast_model(m), (const float2*)rho, g, sh.zchunk, cp, d_err);
+                              fast_model(m), (const float2*)rho, g, per_plane, colliders, cp, d_err);
 }
 
 }  // namespace lbmgb

@@ -156,7 +156,7 @@ cudaError_t launch_flat(const void* src, void* dst, void* rho, const Layout& L, 
 
 // ---- two-pass kernels (lbm_flat32.cu): fp32 or 16-bit deviations, ghost boundary ----
 Shape flat_rows_shape(const Shape& rows);
-Shape flat_any_shape(const Layout& L, int num_sms);
+Shape flat_any_shape(const Layout& L);
 long long flat32_rho_bytes(const Layout& L);
 cudaError_t launch_flat32_fill(void* rho, const Layout& L, const Model& m, cudaStream_t s);
 cudaError_t launch_flat_rows(int prec, const void* src, void* dst, void* rho, const Layout& L, const Model& m,

@@ -241,8 +241,8 @@ cudaError_t stream_collide_t(const void* src, void* dst, const Layout& L, const 
 
 // Largest box of a row-tiled width on the two-pass kernels: their second read
 // of the populations has to come from L2.  Per step, two-pass against cluster
-// kernel: 64 x 40 x 23 fp32 13.8 us (39.1), 64^3 fp32 30.8 (37.2) and bf16 26.6
-// (34.7), 256 x 32 x 32 fp32 24.4 (39.2); 128 x 64 x 64 fp32 50.1 (46.9).
+// kernel: 64 x 40 x 23 fp32 11.6 us (37.2), 64^3 fp32 24.9 (37.2) and bf16 18.9
+// (33.0), 256 x 32 x 32 fp32 22.8 (37.3); 128 x 64 x 64 fp32 about 48 (45.7).
 constexpr long long kFlatRowsNodes = 3 << 17;
 constexpr int kMaxThreadsF32 = 512;
 constexpr int kMaxThreadsF64 = 256;
@@ -328,7 +328,7 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
     // float32 boxes of other extents: two-pass at every size (per step against
     // the tile kernel: 37 x 29 x 23 12.7 us (33.7), 60 x 50 x 44 19.7 (32.8), 96^3
     // 92.8 (117), 200 x 200 x 100 337 (464))
-    if (allow_flat && prec == kFP32 && !periodic && ty_req <= 0 && zchunk_req <= 0) return flat_any_shape(L, num_sms);
+    if (allow_flat && prec == kFP32 && !periodic && ty_req <= 0 && zchunk_req <= 0) return flat_any_shape(L);
     const int cbytes = prec == kFP64 ? 8 : 4;  // compute type of the density ring
     const int maxt = prec == kFP64 ? kMaxThreadsF64 : kMaxThreadsF32;
     sh.tx = L.Lx <= maxt ? L.Lx : 128;
