@@ -393,7 +393,8 @@ int lbm_step(lbm_ctx* c, int64_t n) {
                 cudaEventCreate(&b);
                 cudaEventRecord(a, c->stream);
             }
-            LBM_TRY(launch_ghost(c->prec, src, c->L, c->model, A, c->centre, c->d_err, c->stream));
+            if (c->shape.flat != kFlatRows)  // (their density pass writes the shell)
+                LBM_TRY(launch_ghost(c->prec, src, c->L, c->model, A, c->centre, c->d_err, c->stream));
             if (timed) {
                 cudaEventRecord(b, c->stream);
                 c->ev[1].push_back(a);

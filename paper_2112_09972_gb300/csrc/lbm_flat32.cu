@@ -4,14 +4,14 @@
 // lbm_flat.cu does for float64.  Two forms:
 //
 //   k_row_rho / k_row_collide -- the row-tiled widths (Lx = TX in {32, 64, 128,
-//       256}) for small boxes.  The cluster kernels (lbm_fast.cu) march a
-//       chunk of z planes one after another, about 3 us a plane whatever the
-//       box, so a box too small to fill the chip waits for that chain (10
-//       planes at 64^3).  Here all planes of a chunk run at once; the second
-//       read of the populations comes from L2, which such a box fits.  The
-//       centre is summed from the densities in the cluster kernel's order and
-//       the node arithmetic is shared (collide_core), so both store
-//       bit-identical states.
+//       256}) for small boxes; the density pass writes the ghost shell too.
+//       The cluster kernels (lbm_fast.cu) march a chunk of z planes one after
+//       another, about 3 us a plane whatever the box, so a box too small to
+//       fill the chip waits for that chain (10 planes at 64^3).  Here all
+//       planes run at once; the second read of the populations comes from
+//       L2, which such a box fits.  The centre is summed from the densities
+//       in the cluster kernel's order and the node arithmetic is shared
+//       (collide_core), so both store bit-identical states.
 //   k_any_rho / k_any_collide -- float32 boxes of any other extents, in place
 //       of the tile kernel, whose tiles sum their halo's densities again
 //       (about as many nodes as the tile has) and march in z.
@@ -63,21 +63,100 @@ __device__ __forceinline__ typename RowIO<TX, ST>::P3 node_planes(const ST* src,
     else return IO::planes(IO::base(src, x, y), L, z);
 }
 
+// The ghost populations that a row's nodes pull, written to the shell by the
+// warp that holds the nodes (every ghost population streams to one fluid
+// node, so none is written twice).  The partition of shell_node: x faces own
+// their edges, y faces theirs with z.  Arithmetic as ghost_node and
+// ghost_node_dev.
+template <typename ST>
+struct ShellWriter {
+    ST* f;
+    Layout L;
+    GhostParams<float> g;
+    float xc, yc, zc;
+    int* d_err;
+
+    __device__ __forceinline__ ShellWriter(ST* f_, const Layout& L_, const GhostParams<float>& g_,
+                                           const CentreParts& cp, int* err)
+        : f(f_), L(L_), g(g_), xc(0.f), yc(0.f), zc(0.f), d_err(err) {
+        if (g.frame) xc = cp.frame[0], yc = cp.frame[1], zc = cp.frame[2];
+    }
+    // direction i, weight w, from ghost node (x, y, z) into fluid node (xi, yi, zi); cu(u): c_i . u
+    template <typename CU>
+    __device__ __forceinline__ void put(int i, float w, int x, int y, int z, int xi, int yi, int zi, CU&& cu) const {
+        const GhostFlow<float> u = ghost_flow<float>(g, L, xc, yc, zc, x, y, z);
+        const float c = cu(u);
+        const float e[2] = {feq_of<float>(g.rho_b[0], w, c, u.u2x), feq_of<float>(g.rho_b[1], w, c, u.u2x)};
+        if constexpr (is_dev_t<ST>::value) {
+            using T = decltype(dev_tag(ST{}));
+            const float4 r = __ldg(reinterpret_cast<const float4*>(f) + L.dev_node(xi, yi, zi));
+            const unsigned short a = ghost_dev<T, float>(e[0], w, r.x), b = ghost_dev<T, float>(e[1], w, r.y);
+            reinterpret_cast<unsigned*>(f)[L.dev_word(i, x, y, z)] = (unsigned)a | ((unsigned)b << 16);
+        } else {
+            f[L.at(0, i, x, y, z)] = e[0];
+            f[L.at(1, i, x, y, z)] = e[1];
+        }
+        if (u.usq > g.mach2) atomicOr(d_err, 2);
+    }
+    // The k-th of the five directions into x plane 0 (sgn 1) or Lx - 1 (sgn
+    // -1) at (y, z): c = sgn (1, {0, 1, -1, 0, 0}[k], {0, 0, 0, 1, -1}[k]).
+    __device__ __forceinline__ void x_face(int k, int sgn, int y, int z) const {
+        const int cy = k == 1 ? sgn : (k == 2 ? -sgn : 0), cz = k == 3 ? sgn : (k == 4 ? -sgn : 0);
+        const int xi = sgn > 0 ? 0 : L.Lx - 1;
+        put((k == 0 ? 1 : 5 + 2 * k) + (sgn < 0), k == 0 ? wgt<float>(1) : wgt<float>(7), xi - sgn, y - cy, z - cz, xi,
+            y, z, [&](const GhostFlow<float>& u) {
+                const float b = k == 1 ? u.uy : (k == 2 ? -u.uy : (k == 3 ? u.uz : (k == 4 ? -u.uz : 0.f)));
+                const float c = u.ux + b;
+                return sgn > 0 ? c : -c;
+            });
+    }
+    template <int FACE>
+    __device__ __forceinline__ void yz_face(int x, int y, int z) const {
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            if (!face_inward<FACE>(i)) continue;
+            const int xs = x - cx_(i), ys = y - cy_(i), zs = z - cz_(i);
+            if (xs < 0 || xs >= L.Lx || (FACE >= 4 && (ys < 0 || ys >= L.Ly))) continue;
+            put(i, wgt<float>(i), xs, ys, zs, x, y, z,
+                [&](const GhostFlow<float>& u) { return dot_c<float>(i, u.ux, u.uy, u.uz); });
+        }
+    }
+    // All that the warp's 32 nodes of row (y, z) pull; its lanes read it after this.
+    __device__ __forceinline__ void row(int x, int y, int z) const {
+        const int lane = threadIdx.x & 31, x0 = x - lane;
+        if (lane < 5 ? x0 == 0 : (lane < 10 && x0 + 32 == L.Lx)) x_face(lane % 5, lane < 5 ? 1 : -1, y, z);
+        if (y == 0) yz_face<2>(x, y, z);
+        if (y == L.Ly - 1) yz_face<3>(x, y, z);
+        if (z == 0) yz_face<4>(x, y, z);
+        if (z == L.Lz - 1) yz_face<5>(x, y, z);
+        __syncwarp();
+    }
+};
+
 constexpr int kRowRhoThreads = 128;
 template <int TX>
 constexpr int row_rho_rows() {
     return TX >= kRowRhoThreads ? 1 : kRowRhoThreads / TX;
 }
+// Also writes the ghost populations that its nodes pull, which saves a launch
+// of the chain that a small box's step is (32^3 fp32 10.4 -> 9.4 us per step,
+// 64^3 24.9 -> 24.1, bf16 18.9 -> 17.7; the other two-pass kernels lost more registers to it than
+// the launch was worth: 37 x 29 x 23 fp32 11.7 -> 10.9 us, but 130^3 222 -> 242, and
+// in float64 32^3 41 -> 57).
 template <int TX, typename ST>
-__global__ void __launch_bounds__(TX * row_rho_rows<TX>()) k_row_rho(const ST* __restrict__ src, Layout L,
-                                                                     float2* __restrict__ rho, RhoGeo g) {
+__global__ void __launch_bounds__(TX * row_rho_rows<TX>())
+    k_row_rho(ST* src, Layout L, float2* __restrict__ rho, RhoGeo g, GhostParams<float> gp, CentreParts cp,
+              int* __restrict__ d_err) {
     pdl_wait();
     pdl_trigger();
     const int x = threadIdx.x % TX, y = blockIdx.x * row_rho_rows<TX>() + threadIdx.x / TX, z = blockIdx.y;
+    ShellWriter<ST>(src, L, gp, cp, d_err).row(x, y, z);
     unsigned long long pol;
     asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+    auto q = node_planes<TX, ST>(src, L, x, y, z);
+    asm volatile("" : "+l"(q.m), "+l"(q.o), "+l"(q.p)::"memory");  // the loads stay behind the ghost stores
     float ra, rb;
-    RowIO<TX, ST>::densities(node_planes<TX, ST>(src, L, x, y, z), pol, ra, rb);
+    RowIO<TX, ST>::template densities<false>(q, pol, ra, rb);
     rho[g.at(x, y, z)] = make_float2(ra, rb);
 }
 
@@ -187,8 +266,8 @@ __global__ void __launch_bounds__(TX * row_collide_rows<TX>(), 512 / (TX * row_c
 }
 
 template <int TX, typename ST, bool MRT>
-cudaError_t launch_row_t(const void* src, void* dst, void* rho, const Layout& L, const Model& m, const Shape& sh,
-                         CentreParts cp, int* d_err, cudaStream_t s) {
+cudaError_t launch_row_t(void* src, void* dst, void* rho, const Layout& L, const Model& m, const Grad& A,
+                         const Shape& sh, CentreParts cp, int* d_err, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1] = {pdl_attribute()};
     cfg.attrs = attr;
@@ -197,7 +276,8 @@ cudaError_t launch_row_t(const void* src, void* dst, void* rho, const Layout& L,
     cfg.gridDim = dim3(L.Ly / row_rho_rows<TX>(), L.Lz, 1);
     cfg.blockDim = dim3(TX * row_rho_rows<TX>(), 1, 1);
     const RhoGeo g = rho_geo(L);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_row_rho<TX, ST>, (const ST*)src, L, (float2*)rho, g);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_row_rho<TX, ST>, (ST*)src, L, (float2*)rho, g, ghost_params<float>(m, A.a),
+                                       cp, d_err);
     if (e != cudaSuccess) return e;
     constexpr int threads = TX * row_collide_rows<TX>();
     const int units = (int)(sh.grid.y * sh.grid.z), colliders = L.Ly / row_collide_rows<TX>() * L.Lz;
@@ -208,14 +288,14 @@ cudaError_t launch_row_t(const void* src, void* dst, void* rho, const Layout& L,
 }
 
 template <int TX>
-cudaError_t launch_row_w(int prec, const void* src, void* dst, void* rho, const Layout& L, const Model& m,
+cudaError_t launch_row_w(int prec, void* src, void* dst, void* rho, const Layout& L, const Model& m, const Grad& A,
                          const Shape& sh, CentreParts cp, int* d_err, cudaStream_t s) {
     if (prec == kFP32)
-        return m.mrt ? launch_row_t<TX, float, true>(src, dst, rho, L, m, sh, cp, d_err, s)
-                     : launch_row_t<TX, float, false>(src, dst, rho, L, m, sh, cp, d_err, s);
+        return m.mrt ? launch_row_t<TX, float, true>(src, dst, rho, L, m, A, sh, cp, d_err, s)
+                     : launch_row_t<TX, float, false>(src, dst, rho, L, m, A, sh, cp, d_err, s);
     if (m.mrt) return cudaErrorInvalidValue;
-    if (prec == kFP16Dev) return launch_row_t<TX, Dev<__half>, false>(src, dst, rho, L, m, sh, cp, d_err, s);
-    return launch_row_t<TX, Dev<__nv_bfloat16>, false>(src, dst, rho, L, m, sh, cp, d_err, s);
+    if (prec == kFP16Dev) return launch_row_t<TX, Dev<__half>, false>(src, dst, rho, L, m, A, sh, cp, d_err, s);
+    return launch_row_t<TX, Dev<__nv_bfloat16>, false>(src, dst, rho, L, m, A, sh, cp, d_err, s);
 }
 
 // ---- any extents, float32 ----
@@ -330,13 +410,13 @@ cudaError_t launch_flat32_fill(void* rho, const Layout& L, const Model& m, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_flat_rows(int prec, const void* src, void* dst, void* rho, const Layout& L, const Model& m,
-                             const Shape& sh, CentreParts cp, int* d_err, cudaStream_t s) {
+cudaError_t launch_flat_rows(int prec, void* src, void* dst, void* rho, const Layout& L, const Model& m,
+                             const Grad& A, const Shape& sh, CentreParts cp, int* d_err, cudaStream_t s) {
     switch (L.Lx) {
-        case 32: return launch_row_w<32>(prec, src, dst, rho, L, m, sh, cp, d_err, s);
-        case 64: return launch_row_w<64>(prec, src, dst, rho, L, m, sh, cp, d_err, s);
-        case 128: return launch_row_w<128>(prec, src, dst, rho, L, m, sh, cp, d_err, s);
-        case 256: return launch_row_w<256>(prec, src, dst, rho, L, m, sh, cp, d_err, s);
+        case 32: return launch_row_w<32>(prec, src, dst, rho, L, m, A, sh, cp, d_err, s);
+        case 64: return launch_row_w<64>(prec, src, dst, rho, L, m, A, sh, cp, d_err, s);
+        case 128: return launch_row_w<128>(prec, src, dst, rho, L, m, A, sh, cp, d_err, s);
+        case 256: return launch_row_w<256>(prec, src, dst, rho, L, m, A, sh, cp, d_err, s);
         default: return cudaErrorInvalidValue;
     }
 }

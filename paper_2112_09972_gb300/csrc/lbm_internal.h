@@ -137,10 +137,10 @@ cudaError_t launch_init(int prec, void* f, const Layout& L, double R, double xi,
                         Grad A0, cudaStream_t s);
 cudaError_t launch_ghost(int prec, void* f, const Layout& L, const Model& m, Grad A, CentreParts cp, int* d_err,
                          cudaStream_t s);
-// A: the boundary gradient of this step (the kernels read the ghost shell
-// written by launch_ghost; A is passed for kernels that may compute it).
-// rho: the density array of the two-pass kernels (sh.flat).
-cudaError_t launch_stream_collide(int prec, const void* src, void* dst, const Layout& L, const Model& m,
+// A: the boundary gradient of this step.  The two-pass row kernels (sh.flat
+// kFlatRows) write src's ghost shell themselves; the others read the one of
+// launch_ghost.  rho: the density array of the two-pass kernels (sh.flat).
+cudaError_t launch_stream_collide(int prec, void* src, void* dst, const Layout& L, const Model& m,
                                   const Shape& sh, const Grad& A, void* rho, CentreParts cp, int* d_err,
                                   cudaStream_t s);
 // Centre-of-mass partials of the stored populations f (cp.n CTAs, grid-stride).
@@ -159,8 +159,8 @@ Shape flat_rows_shape(const Shape& rows);
 Shape flat_any_shape(const Layout& L);
 long long flat32_rho_bytes(const Layout& L);
 cudaError_t launch_flat32_fill(void* rho, const Layout& L, const Model& m, cudaStream_t s);
-cudaError_t launch_flat_rows(int prec, const void* src, void* dst, void* rho, const Layout& L, const Model& m,
-                             const Shape& sh, CentreParts cp, int* d_err, cudaStream_t s);
+cudaError_t launch_flat_rows(int prec, void* src, void* dst, void* rho, const Layout& L, const Model& m,
+                             const Grad& A, const Shape& sh, CentreParts cp, int* d_err, cudaStream_t s);
 cudaError_t launch_flat_any(const void* src, void* dst, void* rho, const Layout& L, const Model& m, const Shape& sh,
                             CentreParts cp, int* d_err, cudaStream_t s);
 

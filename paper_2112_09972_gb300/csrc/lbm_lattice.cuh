@@ -47,11 +47,16 @@ __device__ __forceinline__ C dot_c(int i, C ux, C uy, C uz) {
     return v;
 }
 
+// Eq. 8 for weight w and cu = c_i . u.
+template <typename C>
+__device__ __forceinline__ C feq_of(C rho, C w, C cu, C u2x) {
+    return rho * w * (C(1) + C(3) * cu + C(4.5) * cu * cu - u2x);
+}
+
 // Eq. 8 with u2x = 1.5 |u|^2 precomputed.
 template <typename C>
 __device__ __forceinline__ C feq(int i, C rho, C ux, C uy, C uz, C u2x) {
-    const C cu = dot_c<C>(i, ux, uy, uz);
-    return rho * wgt<C>(i) * (C(1) + C(3) * cu + C(4.5) * cu * cu - u2x);
+    return feq_of<C>(rho, wgt<C>(i), dot_c<C>(i, ux, uy, uz), u2x);
 }
 
 // MRT collision: row k of the D3Q19 moment basis of d'Humieres et al. (2002)

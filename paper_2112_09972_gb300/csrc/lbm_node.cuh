@@ -89,10 +89,11 @@ __device__ __forceinline__ float2 dot_c2(int i, float2 ux, float2 uy, float2 uz)
 // second read one plane later, which marks them last-use; the written state
 // is streamed out.  The populations read are never written by the kernel, so
 // the loads may be scheduled freely.
-template <int OFF>
+template <int OFF, bool NC = true>
 __device__ __forceinline__ float ld_keep(const void* p, unsigned long long pol) {
     float v;
-    asm("ld.global.nc.L2::cache_hint.f32 %0, [%1+%3], %2;" : "=f"(v) : "l"(p), "l"(pol), "n"(OFF));
+    if constexpr (!NC) asm("ld.global.L2::cache_hint.f32 %0, [%1+%3], %2;" : "=f"(v) : "l"(p), "l"(pol), "n"(OFF));
+    else asm("ld.global.nc.L2::cache_hint.f32 %0, [%1+%3], %2;" : "=f"(v) : "l"(p), "l"(pol), "n"(OFF));
     return v;
 }
 template <int OFF>
@@ -101,10 +102,11 @@ __device__ __forceinline__ float ld_last(const void* p) {
     asm("ld.global.lu.f32 %0, [%1+%2];" : "=f"(v) : "l"(p), "n"(OFF));
     return v;
 }
-template <int OFF>
+template <int OFF, bool NC = true>
 __device__ __forceinline__ unsigned ld_keep_u32(const void* p, unsigned long long pol) {
     unsigned v;
-    asm("ld.global.nc.L2::cache_hint.b32 %0, [%1+%3], %2;" : "=r"(v) : "l"(p), "l"(pol), "n"(OFF));
+    if constexpr (!NC) asm("ld.global.L2::cache_hint.b32 %0, [%1+%3], %2;" : "=r"(v) : "l"(p), "l"(pol), "n"(OFF));
+    else asm("ld.global.nc.L2::cache_hint.b32 %0, [%1+%3], %2;" : "=r"(v) : "l"(p), "l"(pol), "n"(OFF));
     return v;
 }
 template <int OFF>
@@ -194,18 +196,21 @@ struct RowIO<TX, float> {
         return cz_(I) > 0 ? q.m : (cz_(I) < 0 ? q.p : q.o);
     }
     // component S's post-streaming density (first read, kept in L2)
-    template <int S>
+    template <int S, bool NC = true>
     static __device__ __forceinline__ float density(const P3& q, unsigned long long pol) {
-        float r = ld_keep<poff<S, 0>()>(q.o, pol);
+        float r = ld_keep<poff<S, 0>(), NC>(q.o, pol);
         sfor<9>([&](auto K) {
             constexpr int i = 2 * decltype(K)::value + 1;
-            r += ld_keep<poff<S, i>()>(src_plane<i>(q), pol) + ld_keep<poff<S, i + 1>()>(src_plane<i + 1>(q), pol);
+            r += ld_keep<poff<S, i>(), NC>(src_plane<i>(q), pol) +
+                 ld_keep<poff<S, i + 1>(), NC>(src_plane<i + 1>(q), pol);
         });
         return r;
     }
+    // NC false: the calling warp may have written what it reads
+    template <bool NC = true>
     static __device__ __forceinline__ void densities(const P3& q, unsigned long long pol, float& ra, float& rb) {
-        ra = density<0>(q, pol);
-        rb = density<1>(q, pol);
+        ra = density<0, NC>(q, pol);
+        rb = density<1, NC>(q, pol);
     }
     // the node's 38 pulled populations (second read, last use); rs: unused
     // in float32 (the deviation forms return the node's rho* there)
@@ -290,13 +295,14 @@ struct RowIO<TX, Dev<T>> {
         ra = o.z + (1.f - wgt<float>(0)) * o.x + da;
         rb = o.w + (1.f - wgt<float>(0)) * o.y + db;
     }
+    template <bool NC = true>
     static __device__ __forceinline__ void densities(const P3& q, unsigned long long pol, float& ra, float& rb) {
         const float4 o = ld_keep_f4(q.o + q.blk, pol);
         sum_words(
             o,
             [&](auto I) {
                 constexpr int i = decltype(I)::value;
-                return ld_keep_u32<woff<i>()>(src_plane<i>(q), pol);
+                return ld_keep_u32<woff<i>(), NC>(src_plane<i>(q), pol);
             },
             ra, rb);
     }

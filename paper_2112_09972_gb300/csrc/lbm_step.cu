@@ -241,8 +241,8 @@ cudaError_t stream_collide_t(const void* src, void* dst, const Layout& L, const 
 
 // Largest box of a row-tiled width on the two-pass kernels: their second read
 // of the populations has to come from L2.  Per step, two-pass against cluster
-// kernel: 64 x 40 x 23 fp32 11.6 us (37.2), 64^3 fp32 24.9 (37.2) and bf16 18.9
-// (33.0), 256 x 32 x 32 fp32 22.8 (37.3); 128 x 64 x 64 fp32 about 48 (45.7).
+// kernel: 64 x 40 x 23 fp32 10.3 us (37.2), 64^3 fp32 24.1 (35.9) and bf16 17.7
+// (33.0), 256 x 32 x 32 fp32 21.1 (37.3); 64 x 96 x 96 fp32 58.3 (55.1).
 constexpr long long kFlatRowsNodes = 3 << 17;
 constexpr int kMaxThreadsF32 = 512;
 constexpr int kMaxThreadsF64 = 256;
@@ -400,11 +400,11 @@ cudaError_t launch_centre(int prec, const void* f, const Layout& L, CentreParts 
     return cudaGetLastError();
 }
 
-cudaError_t launch_stream_collide(int prec, const void* src, void* dst, const Layout& L, const Model& m,
+cudaError_t launch_stream_collide(int prec, void* src, void* dst, const Layout& L, const Model& m,
                                   const Shape& sh, const Grad& A, void* rho, CentreParts cp, int* d_err,
                                   cudaStream_t s) {
     if (sh.flat == kFlat64) return launch_flat(src, dst, rho, L, m, sh, cp, d_err, s);
-    if (sh.flat == kFlatRows) return launch_flat_rows(prec, src, dst, rho, L, m, sh, cp, d_err, s);
+    if (sh.flat == kFlatRows) return launch_flat_rows(prec, src, dst, rho, L, m, A, sh, cp, d_err, s);
     if (sh.flat == kFlatAny) return launch_flat_any(src, dst, rho, L, m, sh, cp, d_err, s);
     if (sh.rows) return launch_stream_collide_rows(prec, sh.variant, src, dst, L, m, A, sh.zchunk, cp, d_err, s);
     if (prec == kFP64) return stream_collide_t<double, double, kMaxThreadsF64>(src, dst, L, m, sh, cp, d_err, s);
