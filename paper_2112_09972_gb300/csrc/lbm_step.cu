@@ -239,11 +239,15 @@ cudaError_t stream_collide_t(const void* src, void* dst, const Layout& L, const 
     return cudaGetLastError();
 }
 
-// Largest box of a row-tiled width on the two-pass kernels: their second read
-// of the populations has to come from L2.  Per step, two-pass against cluster
-// kernel: 64 x 40 x 23 fp32 10.3 us (37.2), 64^3 fp32 24.1 (35.9) and bf16 17.7
-// (33.0), 256 x 32 x 32 fp32 21.1 (37.3); 64 x 96 x 96 fp32 58.3 (55.1).
-constexpr long long kFlatRowsNodes = 3 << 17;
+// Largest box of a row-tiled width on the two-pass kernels, whose second read
+// of the populations has to come from L2, half as much of it in 16-bit
+// storage; and the cluster kernel that MRT takes is the slower one (its
+// direct variant).  Per step, two-pass against cluster kernel: fp32 64^3 24.1 us
+// (35.9), 128 x 64 x 64 44.1 (45.5), 64 x 96 x 96 58.3 (55.1); bf16 64^3 17.7
+// (33.0), 64 x 96 x 96 38.5 (46.5), 128 x 64 x 96 44.6 (49.2), 128 x 96 x 96 68.7
+// (64.0); MRT 64^3 24.1 (38.5), 128 x 64 x 64 44.9 (53.6), 128 x 64 x 96 71.6
+// (73.3), 128 x 96 x 96 105.5 (98.6).
+long long flat_rows_nodes(int prec, int mrt) { return prec == kFP32 && !mrt ? 1LL << 19 : 3LL << 18; }
 constexpr int kMaxThreadsF32 = 512;
 constexpr int kMaxThreadsF64 = 256;
 
@@ -320,7 +324,7 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
             sh.grid = dim3(1, L.Ly, (L.Lz + sh.zchunk - 1) / sh.zchunk);
             sh.threads = L.Lx;
             sh.smem = 0;
-            if (allow_flat && variant_req == 0 && zchunk_req <= 0 && (long long)L.Lx * L.Ly * L.Lz <= kFlatRowsNodes)
+            if (allow_flat && variant_req == 0 && zchunk_req <= 0 && (long long)L.Lx * L.Ly * L.Lz <= flat_rows_nodes(prec, mrt))
                 return flat_rows_shape(sh);
             return sh;
         }

@@ -49,6 +49,16 @@ def test_rows_two_pass_bit_identical(built, box, precision):
     assert np.array_equal(a[1], b[1])
 
 
+# the collision that alone keeps float32 boxes of 2^19 to 3 * 2^18 nodes on two passes
+@pytest.mark.parametrize("box", [(32, 32, 32), (64, 96, 96), (256, 8, 37)])
+def test_rows_two_pass_mrt(built, box):
+    start, a = _run(box, "fp32", 10, mrt=True)
+    _, b = _run(box, "fp32", 10, variant=1, mrt=True, start=start)
+    assert a[2] == 4 and b[2] == 1
+    assert np.array_equal(a[0], b[0])
+    assert np.array_equal(a[1], b[1])
+
+
 @pytest.mark.parametrize("mrt", [None, True])
 @pytest.mark.parametrize("box", [(4, 4, 4), (37, 29, 23), (128, 5, 9), (129, 7, 6), (260, 33, 5), (16, 12, 150)])
 def test_any_extents_two_pass(built, box, mrt):
