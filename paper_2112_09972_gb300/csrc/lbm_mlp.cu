@@ -38,6 +38,7 @@
 #include <cmath>
 #include <new>
 #include <random>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/lbm.h"
@@ -379,9 +380,90 @@ __device__ __forceinline__ void tc_store32(const GemmArgs& g, float* Cf, int m, 
     }
 }
 
+// What the update of one layer reads and writes: the float32 gradient of its
+// weights as S slices at ws (S = 1: complete in the gradient array), the
+// bias gradient as cs_n partial column sums at cs, and the bfloat16 copies.
+constexpr int kMaxLayers = 16;
+struct LayerTable {
+    struct Layer {
+        long long offW, count, ws, cs;  // offsets in the parameter, workspace and column-sum arrays
+        int S, dout, din;
+        const bf16* G;
+        bf16 *Wb, *WTb;
+    } l[kMaxLayers];
+    int layers, cs_n;
+    long long nparam;
+};
+
+// Bias gradients db[c] = sum_r G_l[r, c] of every layer, first pass: a block
+// sums rows [s rows, (s + 1) rows) of 32 columns (8 row
+// phases, then the phases in order) into parts[cs_l + s dout + c]; the update
+// adds the slices in order.
+constexpr int kColSlices = 128;
+struct ColSums {
+    LayerTable tb;
+    int n, rows, blocks, slices;  // rows to a slice; blocks of 32 columns of the widest layer
+    float* parts;
+};
+// Block b of blocks x slices x layers, by the CTA's first 256 threads.
+__device__ __forceinline__ void colsum_block(const ColSums& S, int b) {
+    __shared__ float red[8][33];
+    const int bx = b % S.blocks, slice = b / S.blocks % S.slices;
+    const LayerTable::Layer& q = S.tb.l[b / (S.blocks * S.slices)];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int C = q.dout, c = bx * 32 + tx;
+    if (bx * 32 >= C) return;
+    const bf16* g = q.G;
+    const int r0 = slice * S.rows, r1 = min(S.n, r0 + S.rows);
+    float s = 0.f;
+    if (c < C && ty < 8)
+        for (int r = r0 + ty; r < r1; r += 8) s += __bfloat162float(g[(long long)r * C + c]);
+    if (ty < 8) red[ty][tx] = s;
+    __syncthreads();
+    if (ty == 0 && c < C) {
+        float t = red[0][tx];
+        for (int k = 1; k < 8; ++k) t += red[k][tx];
+        S.parts[q.cs + (long long)slice * C + c] = t;
+    }
+}
+__global__ void __launch_bounds__(256) k_colsum_part(const __grid_constant__ ColSums S) {
+    lbmgb::pdl_wait();
+    lbmgb::pdl_trigger();
+    colsum_block(S, blockIdx.x);
+}
+
+// One product, or two that depend on nothing of each other (the first on the
+// CTAs below `first`, the second on the others): the gradient of a layer's
+// input and of its weights share a launch, which is what bounds small batches
+// (a training step at batch 512: 76 -> 66 us).
+struct TcLaunch {
+    CUtensorMap a[2], b[2];
+    GemmArgs g[2];
+    TcShape sh[2];
+    int first;
+};
+
+// SUMS: the CTAs after the product's sum columns (the last product of a
+// backward pass and the bias gradients).
+struct NoSums {};
+template <bool SUMS>
 __global__ void __launch_bounds__(kTcThreads, 1)
-    k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs g,
-              TcShape sh, int* __restrict__ err) {
+    k_gemm_tc(const __grid_constant__ TcLaunch P, const __grid_constant__ std::conditional_t<SUMS, ColSums, NoSums> S,
+              int* __restrict__ err) {
+    if constexpr (SUMS) {
+        if ((int)blockIdx.x >= P.first) {
+            lbmgb::pdl_wait();
+            lbmgb::pdl_trigger();
+            colsum_block(S, (int)blockIdx.x - P.first);
+            return;
+        }
+    }
+    const int which = (int)blockIdx.x < P.first ? 0 : 1;
+    const CUtensorMap &tmA = P.a[which], &tmB = P.b[which];
+    const GemmArgs& g = P.g[which];
+    const TcShape sh = P.sh[which];
+    const int cta = which ? (int)blockIdx.x - P.first : (int)blockIdx.x;
+    const int ctas = which ? (int)gridDim.x - P.first : P.first;
     extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
     __shared__ int stop_flag;
     const unsigned raw = tc_smem(tc_smem_raw);
@@ -441,7 +523,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (lane == 0) {
             const unsigned bytes = kTcTileA + (unsigned)sh.bn * TC_K * 2u;
             bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < tiles && !*stop; tile += gridDim.x) {
+            for (int tile = cta; ok && tile < tiles && !*stop; tile += ctas) {
                 const int r = tile % tiles_mn, m0 = (r / sh.n_tiles) * TC_M, n0 = (r % sh.n_tiles) * sh.bn;
                 int k0, nk;
                 tile_k(tile, k0, nk);
@@ -466,7 +548,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const unsigned idesc = tc_idesc(TC_M, sh.bn);
             unsigned it = 0, tc = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < tiles && !*stop; tile += gridDim.x) {
+            for (int tile = cta; ok && tile < tiles && !*stop; tile += ctas) {
                 int k0, nk;
                 tile_k(tile, k0, nk);
                 const int buf = (int)(tc & 1u);
@@ -510,7 +592,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int q = warp & 3;             // a warp reads TMEM lanes 32 (warp % 4) .. + 31
         const int first = ((warp - 2) >> 2) * 32;  // and column blocks first, first + 64, ...
         unsigned tc = 0;
-        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++tc) {
+        for (int tile = cta; tile < tiles; tile += ctas, ++tc) {
             const int buf = (int)(tc & 1u);
             int okw = 1;
             if (lane == 0) okw = tc_wait(accf_bar(buf), (tc >> 1) & 1u, stop) ? 1 : 0;
@@ -1041,48 +1123,6 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_grad(const float* __restr
     }
 }
 
-// What the update of one layer reads and writes: the float32 gradient of its
-// weights as S slices at ws (S = 1: complete in the gradient array), the
-// bias gradient as cs_n partial column sums at cs, and the bfloat16 copies.
-constexpr int kMaxLayers = 16;
-struct LayerTable {
-    struct Layer {
-        long long offW, count, ws, cs;  // offsets in the parameter, workspace and column-sum arrays
-        int S, dout, din;
-        const bf16* G;
-        bf16 *Wb, *WTb;
-    } l[kMaxLayers];
-    int layers, cs_n;
-    long long nparam;
-};
-
-// Bias gradients db[c] = sum_r G_l[r, c] of every layer (blockIdx.z), first
-// pass: block (x, s) sums rows [s rows, (s + 1) rows) of 32 columns (8 row
-// phases, then the phases in order) into parts[cs_l + s dout + c]; the update
-// adds the slices in order.
-constexpr int kColSlices = 128;
-__global__ void __launch_bounds__(256) k_colsum_part(const __grid_constant__ LayerTable tb, int n, int rows,
-                                                     float* __restrict__ parts) {
-    __shared__ float red[8][33];
-    lbmgb::pdl_wait();
-    lbmgb::pdl_trigger();
-    const LayerTable::Layer& q = tb.l[blockIdx.z];
-    const int C = q.dout, c = blockIdx.x * 32 + threadIdx.x;
-    if (blockIdx.x * 32 >= C) return;
-    const bf16* g = q.G;
-    const int r0 = blockIdx.y * rows, r1 = min(n, r0 + rows);
-    float s = 0.f;
-    if (c < C)
-        for (int r = r0 + threadIdx.y; r < r1; r += 8) s += __bfloat162float(g[(long long)r * C + c]);
-    red[threadIdx.y][threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.y == 0 && c < C) {
-        float t = red[0][threadIdx.x];
-        for (int k = 1; k < 8; ++k) t += red[k][threadIdx.x];
-        parts[q.cs + (long long)blockIdx.y * C + c] = t;
-    }
-}
-
 // out[e] = sum over the S K slices of ws[z count + e], in slice order.
 constexpr int kMaxSplit = 32;
 __global__ void k_splitsum(const float* __restrict__ ws, int S, long long count, float* __restrict__ out) {
@@ -1313,22 +1353,62 @@ cudaError_t launch(lbm_mlp* c, void (*k)(P...), dim3 grid, dim3 block, size_t sm
     return cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
 }
 
-cudaError_t launch_gemm(lbm_mlp* c, const GemmArgs& a, int slices) {
+// Fills slot k of a k_gemm_tc launch on `sms` SMs with this product; its CTAs, or 0 if it is one for k_gemm_nt.
+int tc_plan(lbm_mlp* c, const GemmArgs& a, int slices, int sms, TcLaunch& P, int k) {
     int bn = tc_bn(c, a);
     // narrower tiles while they still find idle SMs: a tile's K loop and
     // epilogue are a serial chain, which half the columns shorten, and every
     // output keeps its sum (ten training steps at batch 512: 968 -> 804 us;
     // with all SMs taken a narrow tile would only reload A)
-    while (bn > 32 && 2LL * (a.M / TC_M) * (a.N / bn) * slices <= c->sms) bn /= 2;
-    CUtensorMap ma, mb;
-    if (bn && tc_map(&ma, a.A, a.M, a.K, a.lda, TC_M) && tc_map(&mb, a.B, a.N, a.K, a.ldb, bn)) {
-        const TcShape sh{a.M / TC_M, a.N / bn, slices, bn};
-        const long long tiles = (long long)sh.m_tiles * sh.n_tiles * slices;
-        const int grid = (int)std::min<long long>(tiles, c->sms);  // persistent: one CTA per SM at most
-        return launch(c, k_gemm_tc, dim3(grid), dim3(kTcThreads), kTcSmem, ma, mb, a, sh, c->d_err);
+    while (bn > 32 && 2LL * (a.M / TC_M) * (a.N / bn) * slices <= sms) bn /= 2;
+    if (!bn || !tc_map(&P.a[k], a.A, a.M, a.K, a.lda, TC_M) || !tc_map(&P.b[k], a.B, a.N, a.K, a.ldb, bn)) return 0;
+    P.g[k] = a;
+    P.sh[k] = TcShape{a.M / TC_M, a.N / bn, slices, bn};
+    const long long tiles = (long long)P.sh[k].m_tiles * P.sh[k].n_tiles * slices;
+    return (int)std::min<long long>(tiles, c->sms);  // persistent: one CTA per SM at most
+}
+
+cudaError_t launch_gemm(lbm_mlp* c, const GemmArgs& a, int slices) {
+    TcLaunch P;
+    if (const int n = tc_plan(c, a, slices, c->sms, P, 0)) {
+        P.a[1] = P.a[0], P.b[1] = P.b[0], P.g[1] = P.g[0], P.sh[1] = P.sh[0];
+        P.first = n;
+        return launch(c, k_gemm_tc<false>, dim3(n), dim3(kTcThreads), kTcSmem, P, NoSums{}, c->d_err);
     }
     const dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM, slices);
     return launch(c, k_gemm_nt, grid, dim3(kGemmThreads), 0, a);
+}
+
+// Two products of which neither reads what the other writes, in one launch
+// while both find SMs of their own, half of the chip each (a training step at
+// batch 512 76 -> 66 us, 1024 76.7 -> 70.6, 2048 82.7 -> 81.4; without that rule
+// 2048 took 88).
+cudaError_t launch_gemm_pair(lbm_mlp* c, const GemmArgs& a0, int slices0, const GemmArgs& a1, int slices1) {
+    TcLaunch P;
+    const int n0 = tc_plan(c, a0, slices0, c->sms / 2, P, 0);
+    const int n1 = n0 ? tc_plan(c, a1, slices1, c->sms / 2, P, 1) : 0;
+    if (n1 && n0 + n1 <= c->sms) {
+        P.first = n0;
+        return launch(c, k_gemm_tc<false>, dim3(n0 + n1), dim3(kTcThreads), kTcSmem, P, NoSums{}, c->d_err);
+    }
+    const cudaError_t e = launch_gemm(c, a0, slices0);
+    return e == cudaSuccess ? launch_gemm(c, a1, slices1) : e;
+}
+
+// A product and the column sums, in one launch while both find SMs of their
+// own (a CTA of k_gemm_tc takes one whole, whatever it does): a training step
+// at batch 512 66 -> 63.5 us.
+cudaError_t launch_gemm_sums(lbm_mlp* c, const GemmArgs& a, int slices, const ColSums& S) {
+    const int blocks = S.blocks * S.slices * S.tb.layers;
+    TcLaunch P;
+    const int n = tc_plan(c, a, slices, c->sms, P, 0);
+    if (n && n + blocks <= c->sms) {
+        P.a[1] = P.a[0], P.b[1] = P.b[0], P.g[1] = P.g[0], P.sh[1] = P.sh[0];
+        P.first = n;
+        return launch(c, k_gemm_tc<true>, dim3(n + blocks), dim3(kTcThreads), kTcSmem, P, S, c->d_err);
+    }
+    const cudaError_t e = launch_gemm(c, a, slices);
+    return e == cudaSuccess ? launch(c, k_colsum_part, dim3(blocks), dim3(256), 0, S) : e;
 }
 
 GemmArgs gemm_args(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, int epi, const float* bias,
@@ -1351,24 +1431,22 @@ cudaError_t gemm(lbm_mlp* c, const bf16* A, int lda, const bf16* B, int ldb, int
 // out [M, N] (row stride N) = A B^T for a long K (the batch of the weight
 // gradients): K is cut into slices so that there are about two tiles x
 // slices per SM, each slice at least 8 K chunks; the float32 partials go to ws.
-// *S: the slices, which the caller adds in order (1: out is complete).
-cudaError_t gemm_long_k(lbm_mlp* c, const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K,
-                        float* out, float* ws, int* slices_out) {
-    GemmArgs a = gemm_args(A, lda, B, ldb, M, N, K, kStoreF32, nullptr, nullptr, 0, out, nullptr, N);
+// Returns the slices, which the caller adds in order (1: out is complete).
+int long_k(const lbm_mlp* c, const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, float* out, float* ws,
+           GemmArgs& a) {
+    a = gemm_args(A, lda, B, ldb, M, N, K, kStoreF32, nullptr, nullptr, 0, out, nullptr, N);
     const int bn = tc_bn(c, a);
     const int unit = bn ? TC_K : BK;
     const long long tiles =
         bn ? (long long)(M / TC_M) * (N / bn) : (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
     long long S = std::max(1LL, 2LL * c->sms / tiles);
     S = std::min<long long>(std::min<long long>(S, kMaxSplit), std::max(1, K / (8 * unit)));
-    *slices_out = 1;
-    if (S <= 1) return launch_gemm(c, a, 1);
+    if (S <= 1) return 1;
     const int k_len = (int)(((K + S - 1) / S + unit - 1) / unit * unit);
     a.Cf = ws;
     a.k_len = k_len;
     a.c_split = (long long)M * N;
-    *slices_out = (K + k_len - 1) / k_len;
-    return launch_gemm(c, a, *slices_out);
+    return (K + k_len - 1) / k_len;
 }
 
 cudaError_t transpose(lbm_mlp* c, const bf16* in, int R, int C, int ldi, bf16* out, int ldo) {
@@ -1500,21 +1578,31 @@ cudaError_t backward(lbm_mlp* c, const float* t, int n) {
             ht = c->T2;
             e = transpose(c, c->H[l - 1], n, din, din, ht, n);
         }
-        if (e == cudaSuccess)
-            e = gemm_long_k(c, c->GT[l & 1], n, ht, n, dout, din, n, c->g + c->offW[l], c->ws + q.ws, &q.S);
+        if (e != cudaSuccess) break;
+        GemmArgs dw;
+        q.S = long_k(c, c->GT[l & 1], n, ht, n, dout, din, n, c->g + c->offW[l], c->ws + q.ws, dw);
+        if (l > 1) {  // beside G_{l-1} = (G_l W_l) masked by h_{l-1} > 0
+            GemmArgs a = gemm_args(c->G[l], dout, c->WTb[l], dout, n, din, dout, kMaskBf16, nullptr, c->H[l - 1], din,
+                                   nullptr, c->G[l - 1], din);
+            a.Ct = c->GT[(l - 1) & 1];
+            a.ldt = n;
+            e = launch_gemm_pair(c, a, 1, dw, q.S);
+        } else {  // beside the bias gradients
+            ColSums cs;
+            cs.tb = c->table;
+            cs.n = n;
+            cs.rows = (n + S - 1) / S;
+            cs.blocks = (widest + 31) / 32;
+            cs.slices = S;
+            cs.parts = c->cs_parts;
+            e = launch_gemm_sums(c, dw, q.S, cs);
+        }
         if (e == cudaSuccess && q.S > 1 && !c->ws_all) {  // the workspace is the next layer's too
             e = launch(c, k_splitsum, dim3(blocks_for(q.count, 256)), dim3(256), 0, (const float*)c->ws, q.S, q.count,
                        c->g + c->offW[l]);
             q.S = 1;
         }
-        // G_{l-1} = (G_l W_l) masked by h_{l-1} > 0
-        if (l > 1 && e == cudaSuccess)
-            e = gemm(c, c->G[l], dout, c->WTb[l], dout, n, din, dout, kMaskBf16, nullptr, c->H[l - 1], din, nullptr,
-                     c->G[l - 1], din, c->GT[(l - 1) & 1]);
     }
-    if (e == cudaSuccess)
-        e = launch(c, k_colsum_part, dim3((widest + 31) / 32, S, L), dim3(32, 8), 0, c->table, n, (n + S - 1) / S,
-                   c->cs_parts);
     return e;
 }
 
@@ -1559,7 +1647,8 @@ int lbm_mlp_create(lbm_mlp** out, int32_t nlayers, const int32_t* sizes, int32_t
         c->own_stream = true;
     }
     // dynamic shared memory of the tensor-core GEMM above the 48 KB default
-    if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_gemm_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gemm_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem) != cudaSuccess) {
         if (c->own_stream) cudaStreamDestroy(c->stream);
         delete c;
         return LBM_ECUDA;

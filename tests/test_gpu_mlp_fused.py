@@ -80,3 +80,28 @@ def test_deformation_of_special_tensors(built):
         ref = np.where(s1 + s3 > 0, (s1 - s3) / np.where(s1 + s3 > 0, s1 + s3, 1), 0.0)
         assert np.max(np.abs(D.cpu().numpy() - ref)) <= 1e-12
     net.close()
+
+
+# both gradients of a layer and the bias sums in one launch each (512), two products but sums apart (2048), and with
+# an output layer that one 32-column tile holds
+@pytest.mark.parametrize("sizes,n", [((576, 256, 256, 256, 6), 512), ((576, 256, 256, 256, 6), 2048), ((64, 128, 6), 256)])
+def test_grouped_training_products(built, sizes, n):
+    """Against mma.sync, whose products run one launch each.  Both round to
+    bfloat16 at the same points and lie within 2e-2 (relative L2) of the
+    float64 model that does, so within 4e-2 of each other."""
+    net = MLP(sizes, max_batch=n, seed=11)
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    x, t = (torch.randn((n, k), device="cuda", generator=gen) for k in (sizes[0], sizes[-1]))
+    torch.cuda.synchronize()
+    loss, g = {}, {}
+    for path in (0, 1):
+        net.set_tensor_path(path)
+        loss[path], g[path] = net.gradients(x, t)
+    assert abs(loss[0] - loss[1]) <= 2e-3 * loss[1]
+    o = 0
+    for a, b in zip(sizes[:-1], sizes[1:]):
+        for k in (a * b, b):
+            assert np.linalg.norm(g[0][o:o + k] - g[1][o:o + k]) <= 4e-2 * np.linalg.norm(g[1][o:o + k]), (a, b, k)
+            o += k
+    assert o == g[0].size
+    net.close()
