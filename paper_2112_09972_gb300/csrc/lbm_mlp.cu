@@ -269,14 +269,17 @@ __device__ __forceinline__ void tc_mbar_init(unsigned mbar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(count) : "memory");
 }
 
+// Suspended for up to kTcNapNs or until the phase completes: a thread that
+// polls takes issue slots from the warps that work.
+constexpr unsigned kTcNapNs = 20000;
 __device__ __forceinline__ bool tc_mbar_try_wait(unsigned mbar, unsigned parity) {
     unsigned ok;
     asm volatile(
         "{\n .reg .pred p;\n"
-        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
         " selp.u32 %0, 1, 0, p;\n}"
         : "=r"(ok)
-        : "r"(mbar), "r"(parity)
+        : "r"(mbar), "r"(parity), "r"(kTcNapNs)
         : "memory");
     return ok != 0u;
 }
@@ -653,10 +656,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // its accumulators in tensor memory, so global memory sees the float32 input
 // once and the outputs once; the weights come from L2 for every tile.
 //
-// What bounds it: reading x (d0 x 512 bytes a tile) and the weights through
-// the SM's L2 port, about 7 us a tile at d0 = 576 and widths of 256, against
-// 5 us of tensor-core time and the chain product - epilogue - product of the
-// hidden layers.  Layer by layer, each product wrote and read its activations
+// What bounds it: the chain product - epilogue - product of a tile's layers,
+// about 15 us at d0 = 576 and widths of 256, against 5 us of tensor-core time
+// and 7 us for x (d0 x 512 bytes a tile) and the weights through the SM's L2
+// port (sharing the weights of two CTAs by multicast changed nothing).  So
+// the biases are loaded ahead of their use and waiting threads sleep: 65536
+// rows 73 -> 66.5 us.  Layer by layer, each product wrote and read its activations
 // through memory and was a launch of its own, as were the input normalisation
 // and the output scaling.
 //
@@ -716,6 +721,15 @@ __device__ __forceinline__ void fw_ld32(unsigned addr, unsigned (&v)[32]) {
           "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
         : "r"(addr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// The input, read once: not through L1, which holds little beside 225 KB of
+// shared memory and has the biases.
+__device__ __forceinline__ float4 fw_ld_input(const float* p) {
+    float4 v;
+    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p));
+    return v;
 }
 __device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);  // .x at the lower address
@@ -795,10 +809,25 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
         const unsigned swz = (unsigned)(row & 7), hrow = base + kFwH0 + (unsigned)row * 128u;
         const unsigned lanes = tmem + ((unsigned)(quad * 32) << 16);
         unsigned hidden = 0;  // accumulations in the second half so far
+        for (int l = 0; l < L; ++l)  // the biases into L1: a miss in an epilogue is part of the chain
+            if (t * 32 < a.width[l]) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.bias[l] + t * 32));
+        // bias, scale and mean of output `lane`
+        const bool has = lane < a.dL;
+        const float ob = has ? __ldg(a.bias[L - 1] + lane) : 0.f, os = has ? __ldg(a.y_scale + lane) : 1.f;
+        const float om = has ? __ldg(a.y_mean + lane) : 0.f;
+        // The biases of a block are on their way while the block before is
+        // worked on (or its product awaited): loaded where they are added,
+        // between the stores, their latency was most of an epilogue.
+        float4 bb[8];
+        auto load_bias = [&](int l, int n) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) bb[q] = __ldg(reinterpret_cast<const float4*>(a.bias[l] + n) + q);
+        };
         for (int j = 0; j < mine; ++j) {
             const long long m = (long long)(blockIdx.x + j * gridDim.x) * TC_M + row;
             for (int l = 0; l < L; ++l) {
                 int ok = 1;
+                if (l + 1 < L && 32 * half < a.width[l]) load_bias(l, 32 * half);
                 if (lane == 0) {
                     ok = l == 0 ? tc_wait(accfull(0), (unsigned)j & 1u, stop) : tc_wait(accfull(1), hidden & 1u, stop);
                     if (!ok) give_up();
@@ -807,25 +836,25 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                 if (!__shfl_sync(0xffffffffu, ok, 0)) goto done;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const unsigned acc = lanes + (l == 0 ? 0u : 256u);
-                const float* bias = a.bias[l];
                 if (l + 1 < L) {
 #pragma unroll 1
                     for (int n = 32 * half; n < a.width[l]; n += 64) {
-                        unsigned v[32];
+                        unsigned v[32], w[16];
                         fw_ld32(acc + (unsigned)n, v);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float f[4] = {__uint_as_float(v[4 * q]) + bb[q].x, __uint_as_float(v[4 * q + 1]) + bb[q].y,
+                                                __uint_as_float(v[4 * q + 2]) + bb[q].z,
+                                                __uint_as_float(v[4 * q + 3]) + bb[q].w};
+                            w[2 * q] = pack_bf16(fmaxf(f[0], 0.f), fmaxf(f[1], 0.f));
+                            w[2 * q + 1] = pack_bf16(fmaxf(f[2], 0.f), fmaxf(f[3], 0.f));
+                        }
+                        if (n + 64 < a.width[l]) load_bias(l, n + 64);
                         const unsigned dst = hrow + (unsigned)(n / TC_K) * kFwChunk;
                         const unsigned c0 = (unsigned)(n % TC_K) / 8u;  // 16-byte column of the 128-byte row
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float4 b0 = __ldg(reinterpret_cast<const float4*>(bias + n) + 2 * q);
-                            const float4 b1 = __ldg(reinterpret_cast<const float4*>(bias + n) + 2 * q + 1);
-                            const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-                            float f[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) f[e] = fmaxf(__uint_as_float(v[8 * q + e]) + bb[e], 0.f);
-                            st_shared16(dst + (((c0 + q) ^ swz) << 4), pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]),
-                                        pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
-                        }
+                        for (int q = 0; q < 4; ++q)
+                            st_shared16(dst + (((c0 + q) ^ swz) << 4), w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
                     }
                     fw_fence_async();
                 } else if (half == 0) {
@@ -835,8 +864,8 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
 #pragma unroll
                     for (int c = 0; c < 32; ++c)
                         if (c < a.dL) {
-                            const float yh = __uint_as_float(v[c]) + __ldg(bias + c);
-                            out[c] = yh / __ldg(a.y_scale + c) + __ldg(a.y_mean + c);
+                            const float yh = __uint_as_float(v[c]) + __shfl_sync(0xffffffffu, ob, c);
+                            out[c] = yh / __shfl_sync(0xffffffffu, os, c) + __shfl_sync(0xffffffffu, om, c);
                         }
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -856,7 +885,7 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
             const int j = q / nk0, c = q - j * nk0;
             const float* p = a.x + ((long long)(blockIdx.x + j * gridDim.x) * TC_M + r0) * a.d0 + c * TC_K + 4 * g;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = __ldcs(reinterpret_cast<const float4*>(p + (long long)(16 * i) * a.d0));
+            for (int i = 0; i < 8; ++i) v[i] = fw_ld_input(p + (long long)(16 * i) * a.d0);
         };
         auto put = [&](int q, const float4 (&v)[8]) -> bool {
             const unsigned s = (unsigned)q % kFwXStages, round = (unsigned)q / kFwXStages;
