@@ -660,8 +660,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // about 15 us at d0 = 576 and widths of 256, against 5 us of tensor-core time
 // and 7 us for x (d0 x 512 bytes a tile) and the weights through the SM's L2
 // port (sharing the weights of two CTAs by multicast changed nothing).  So
-// the biases are loaded ahead of their use and waiting threads sleep: 65536
-// rows 73 -> 66.5 us.  Layer by layer, each product wrote and read its activations
+// the biases wait in shared memory and waiting threads sleep: 65536 rows 73 ->
+// 64.6 us.  Layer by layer, each product wrote and read its activations
 // through memory and was a launch of its own, as were the input normalisation
 // and the output scaling.
 //
@@ -693,8 +693,10 @@ constexpr unsigned kFwX0 = 2 * kFwWStages * kFwWBytes, kFwH0 = kFwX0 + kFwXStage
 constexpr unsigned kFwBar0 = kFwH0 + (kFwMaxWidth / TC_K) * kFwChunk;
 // W full, empty per ring; X full, empty; accumulator full; first-layer
 // accumulator read; epilogue done; drain per issuing warp
-constexpr int kFwBars = 4 * kFwWStages + 2 * kFwXStages + 2 + 1 + 1 + 2;
-constexpr unsigned kFwSmem = 1024 + kFwBar0 + 8 * kFwBars + 16;
+constexpr int kFwBars = 4 * kFwWStages + 2 * kFwXStages + 2 + 1 + 1 + 2 + 1;
+// after the barriers the tensor memory's address and the stop flag, then two layers' biases
+constexpr unsigned kFwBias0 = kFwBar0 + 8 * kFwBars + 8;
+constexpr unsigned kFwSmem = kFwBias0 + 2 * kFwMaxWidth * 4;
 constexpr unsigned kFwCols = 512;
 
 struct FwArgs {
@@ -746,11 +748,16 @@ __device__ __forceinline__ void fw_fence_async() { asm volatile("fence.proxy.asy
 
 __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_constant__ FwArgs a) {
     extern __shared__ __align__(1024) unsigned char fw_smem_raw[];
-    __shared__ int stop_flag;
-    const unsigned raw = tc_smem(fw_smem_raw);
-    const unsigned base = (raw + 1023u) & ~1023u;
+    // no room is left to move up to the swizzle atoms' alignment, which the array has
+    const unsigned base = tc_smem(fw_smem_raw);
+    if (base & 1023u) {
+        if (threadIdx.x == 0) atomicOr(a.err, 1);
+        return;
+    }
     const unsigned bar0 = base + kFwBar0;
-    unsigned* tmem_slot = reinterpret_cast<unsigned*>(fw_smem_raw + (bar0 + 8u * kFwBars - raw));
+    unsigned* tmem_slot = reinterpret_cast<unsigned*>(fw_smem_raw + kFwBar0 + 8 * kFwBars);
+    int& stop_flag = *reinterpret_cast<int*>(tmem_slot + 1);
+    float* biases = reinterpret_cast<float*>(fw_smem_raw + kFwBias0);
     // ring 0: first layer, ring 1: the others
     auto wfull = [&](unsigned ring, unsigned s) { return bar0 + 8u * (2u * kFwWStages * ring + s); };
     auto wempty = [&](unsigned ring, unsigned s) { return bar0 + 8u * (2u * kFwWStages * ring + kFwWStages + s); };
@@ -761,6 +768,7 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
     auto accfull = [&](unsigned b) { return bar2 + 8u * b; };
     const unsigned acc0_read = bar2 + 16u, epi_bar = bar2 + 24u;
     auto drain = [&](unsigned ring) { return bar2 + 32u + 8u * ring; };
+    const unsigned bias_bar = bar2 + 48u;
     volatile int* stop = &stop_flag;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
 
@@ -780,6 +788,7 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
         }
         tc_mbar_init(acc0_read, kFwEpiWarps);
         tc_mbar_init(epi_bar, kFwEpiWarps);
+        tc_mbar_init(bias_bar, kFwEpiWarps);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kFwRole) {
@@ -809,27 +818,31 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
         const unsigned swz = (unsigned)(row & 7), hrow = base + kFwH0 + (unsigned)row * 128u;
         const unsigned lanes = tmem + ((unsigned)(quad * 32) << 16);
         unsigned hidden = 0;  // accumulations in the second half so far
-        for (int l = 0; l < L; ++l)  // the biases into L1: a miss in an epilogue is part of the chain
-            if (t * 32 < a.width[l]) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.bias[l] + t * 32));
         // bias, scale and mean of output `lane`
         const bool has = lane < a.dL;
         const float ob = has ? __ldg(a.bias[L - 1] + lane) : 0.f, os = has ? __ldg(a.y_scale + lane) : 1.f;
         const float om = has ? __ldg(a.y_mean + lane) : 0.f;
-        // The biases of a block are on their way while the block before is
-        // worked on (or its product awaited): loaded where they are added,
-        // between the stores, their latency was most of an epilogue.
-        float4 bb[8];
-        auto load_bias = [&](int l, int n) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) bb[q] = __ldg(reinterpret_cast<const float4*>(a.bias[l] + n) + q);
+        // The biases of epilogue e (counted over the tiles) lie in half e & 1 of
+        // `biases`: every thread loads one of the next epilogue's, stores it
+        // when it is done with this one and arrives at bias_bar, so they are
+        // there before the product is.  (Loaded from global memory where they
+        // are added, their latency was most of an epilogue.)
+        auto hidden_bias = [&](int l) { return l + 1 < L && t < a.width[l] ? __ldg(a.bias[l] + t) : 0.f; };
+        auto hand_over = [&](unsigned e, float v) {
+            biases[(e & 1u) * kFwMaxWidth + t] = v;
+            __syncwarp();
+            if (lane == 0) tc_arrive(bias_bar);
         };
+        hand_over(0u, hidden_bias(0));
+        unsigned e = 0;
         for (int j = 0; j < mine; ++j) {
             const long long m = (long long)(blockIdx.x + j * gridDim.x) * TC_M + row;
-            for (int l = 0; l < L; ++l) {
+            for (int l = 0; l < L; ++l, ++e) {
                 int ok = 1;
-                if (l + 1 < L && 32 * half < a.width[l]) load_bias(l, 32 * half);
+                const float next = hidden_bias(l + 1 < L ? l + 1 : 0);
                 if (lane == 0) {
                     ok = l == 0 ? tc_wait(accfull(0), (unsigned)j & 1u, stop) : tc_wait(accfull(1), hidden & 1u, stop);
+                    ok = ok && tc_wait(bias_bar, e & 1u, stop);
                     if (!ok) give_up();
                 }
                 if (l > 0) ++hidden;
@@ -839,17 +852,17 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                 if (l + 1 < L) {
 #pragma unroll 1
                     for (int n = 32 * half; n < a.width[l]; n += 64) {
+                        const float4* bb = reinterpret_cast<const float4*>(biases + (e & 1u) * kFwMaxWidth + n);
                         unsigned v[32], w[16];
                         fw_ld32(acc + (unsigned)n, v);
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
-                            const float f[4] = {__uint_as_float(v[4 * q]) + bb[q].x, __uint_as_float(v[4 * q + 1]) + bb[q].y,
-                                                __uint_as_float(v[4 * q + 2]) + bb[q].z,
-                                                __uint_as_float(v[4 * q + 3]) + bb[q].w};
+                            const float4 b = bb[q];
+                            const float f[4] = {__uint_as_float(v[4 * q]) + b.x, __uint_as_float(v[4 * q + 1]) + b.y,
+                                                __uint_as_float(v[4 * q + 2]) + b.z, __uint_as_float(v[4 * q + 3]) + b.w};
                             w[2 * q] = pack_bf16(fmaxf(f[0], 0.f), fmaxf(f[1], 0.f));
                             w[2 * q + 1] = pack_bf16(fmaxf(f[2], 0.f), fmaxf(f[3], 0.f));
                         }
-                        if (n + 64 < a.width[l]) load_bias(l, n + 64);
                         const unsigned dst = hrow + (unsigned)(n / TC_K) * kFwChunk;
                         const unsigned c0 = (unsigned)(n % TC_K) / 8u;  // 16-byte column of the 128-byte row
 #pragma unroll
@@ -874,6 +887,7 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                     if (l == 0) tc_arrive(acc0_read);
                     tc_arrive(epi_bar);
                 }
+                hand_over(e + 1u, next);
             }
         }
     } else if (warp < kFwRole) {
