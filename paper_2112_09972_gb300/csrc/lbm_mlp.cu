@@ -1538,16 +1538,20 @@ cudaError_t forward(lbm_mlp* c, const float* x, int n, bool train) {
 void training_buffers(lbm_mlp* c) {
     if (c->ht_tried) return;
     c->ht_tried = true;
-    for (int l = 0; l < c->L; ++l)
-        if (cudaMalloc((void**)&c->HT[l], sizeof(bf16) * (size_t)c->max_batch * c->d[l]) != cudaSuccess) {
-            cudaGetLastError();
+    // (a capture that this call may be part of does not see the allocations)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    bool all = true;
+    for (int l = 0; l < c->L && all; ++l)
+        all = cudaMalloc((void**)&c->HT[l], sizeof(bf16) * (size_t)c->max_batch * c->d[l]) == cudaSuccess;
+    if (!all) {
+        cudaGetLastError();
+        for (int l = 0; l < c->L; ++l) {
+            cudaFree(c->HT[l]);  // (the failed one is null)
             c->HT[l] = nullptr;
-            for (int k = 0; k < l; ++k) {
-                cudaFree(c->HT[k]);
-                c->HT[k] = nullptr;
-            }
-            return;
         }
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 // k_mlp_forward's constants: input width a multiple of 64, two layers or more,

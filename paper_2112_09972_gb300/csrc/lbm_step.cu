@@ -330,8 +330,8 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
         }
     }
     // float32 boxes of other extents: two-pass at every size (per step against
-    // the tile kernel: 37 x 29 x 23 12.7 us (33.7), 60 x 50 x 44 19.7 (32.8), 96^3
-    // 92.8 (117), 200 x 200 x 100 337 (464))
+    // the tile kernel: 37 x 29 x 23 11.7 us (34.5), 60 x 50 x 44 19.2 (31.1), 96^3
+    // 92.4 (116), 130^3 222 (327), 200 x 200 x 100 346 (460))
     if (allow_flat && prec == kFP32 && !periodic && ty_req <= 0 && zchunk_req <= 0) return flat_any_shape(L);
     const int cbytes = prec == kFP64 ? 8 : 4;  // compute type of the density ring
     const int maxt = prec == kFP64 ? kMaxThreadsF64 : kMaxThreadsF32;
