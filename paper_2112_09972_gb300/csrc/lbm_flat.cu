@@ -21,8 +21,8 @@
 // read of the populations costs bandwidth that is idle), opposite
 // directions share their equilibria, and the launch covers the chip for any
 // box: one node per thread instead of a z march per tile.  Measured per step
-// against the tile kernel: 32^3 44.8 us (178), 64^3 207 us (365), 128^3 1557 us
-// (3174), 37 x 29 x 23 37 us (160); float64 storage therefore takes these
+// against the tile kernel: 32^3 43 us (178), 64^3 200 us (365), 128^3 1466 us
+// (3174), 37 x 29 x 23 36 us (160); float64 storage therefore takes these
 // kernels at every size.
 #include <cuda_runtime.h>
 

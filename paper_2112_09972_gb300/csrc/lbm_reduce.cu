@@ -205,7 +205,8 @@ __device__ void block_sum(double (&v)[K], double* out) {
 // together in node order: DRAM then serves neighbouring rows at the same time
 // (a march of each warp along z read as many bytes at 45 % of its peak).
 // 128^3 float32 on GB300: 180 us with ten FP64 sums per node and the
-// reductions in every warp, bound by the FP64 pipe; 102 us marching.
+// reductions in every warp, bound by the FP64 pipe; 102 us marching; 67 us now
+// (0.70 of the measured copy rate, waiting for its loads).
 template <typename S>
 __global__ void __launch_bounds__(kRedThreads, 4) k_moments(const S* __restrict__ f, Layout L,
                                                             double* __restrict__ partials) {
@@ -539,7 +540,8 @@ __global__ void k_cc_roots(Layout L, const int* __restrict__ label, const int* _
 // float64 storage; for the float32 and 16-bit forms an unevaluated float32
 // pair hi + lo good to 2^-44, a thousandth of what the stored populations'
 // own rounding leaves, so that phi, its sum and its gradient stay off the
-// FP64 pipe (which bounded both passes: 96 and 88 us at 128^3 float32).
+// FP64 pipe (which bounded both passes: 96 and 88 us at 128^3 float32; 67 and
+// 16 us now).
 struct Pair {
     float h, l;
 };
