@@ -21,11 +21,12 @@
 // read of the populations costs bandwidth that is idle), opposite
 // directions share their equilibria, and the launch covers the chip for any
 // box: one node per thread instead of a z march per tile.  Measured per step
-// against the tile kernel: 32^3 43 us (178), 64^3 200 us (365), 128^3 1466 us
+// against the tile kernel: 32^3 42 us (178), 64^3 195 us (365), 128^3 1433 us
 // (3174), 37 x 29 x 23 36 us (160); float64 storage therefore takes these
 // kernels at every size.
 #include <cuda_runtime.h>
 
+#include "lbm_eigen.cuh"
 #include "lbm_internal.h"
 #include "lbm_lattice.cuh"
 #include "lbm_pdl.cuh"
@@ -111,29 +112,43 @@ __device__ __forceinline__ void flat_node(const double2* __restrict__ r, int sy,
     double j[2][3];
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-        double jx = 0.0, jy = 0.0, jz = 0.0;
+        double v[3];
+        bool set[3] = {false, false, false};
+        auto gather = [&](int a, int c, double d) {  // v[a] += c d
+            if (c == 0) return;
+            v[a] = set[a] ? (c > 0 ? v[a] + d : v[a] - d) : d;  // (the first direction of each sum has c = 1)
+            set[a] = true;
+        };
 #pragma unroll
         for (int i = 1; i < 19; i += 2) {
             const double d = f[s][i] - f[s][i + 1];
-            if (cx_(i)) jx = cx_(i) > 0 ? jx + d : jx - d;
-            if (cy_(i)) jy = cy_(i) > 0 ? jy + d : jy - d;
-            if (cz_(i)) jz = cz_(i) > 0 ? jz + d : jz - d;
+            gather(0, cx_(i), d);
+            gather(1, cy_(i), d);
+            gather(2, cz_(i), d);
         }
-        j[s][0] = jx; j[s][1] = jy; j[s][2] = jz;
+        j[s][0] = v[0]; j[s][1] = v[1]; j[s][2] = v[2];
     }
     // Shan-Chen force sums (Eq. 7) in units of the edge weight 1/36
-    double acc[2][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
+    double acc[2][3];
 #pragma unroll
     for (int i = 1; i < 19; i += 2) {
         const int off = cz_(i) * sz + cy_(i) * sy + cx_(i);
         const double2 a = r[off], b = r[-off];
-        const double dA = i < 7 ? 2.0 * (a.x - b.x) : a.x - b.x, dB = i < 7 ? 2.0 * (a.y - b.y) : a.y - b.y;
+        const double dA = a.x - b.x, dB = a.y - b.y;
+        if (i < 7) {  // axis directions come first, one per sum, with weight 2
+            acc[0][i / 2] = dA + dA;
+            acc[1][i / 2] = dB + dB;
+            continue;
+        }
         if (cx_(i)) { acc[0][0] += cx_(i) > 0 ? dA : -dA; acc[1][0] += cx_(i) > 0 ? dB : -dB; }
         if (cy_(i)) { acc[0][1] += cy_(i) > 0 ? dA : -dA; acc[1][1] += cy_(i) > 0 ? dB : -dB; }
         if (cz_(i)) { acc[0][2] += cz_(i) > 0 ? dA : -dA; acc[1][2] += cz_(i) > 0 ? dB : -dB; }
     }
     rho = *r;
-    const double rden = 1.0 / (rho.x * m.inv_tau[0] + rho.y * m.inv_tau[1]);
+    const double den = rho.x * m.inv_tau[0] + rho.y * m.inv_tau[1];
+    // (rcp64 between 2^-100 and 2^100)
+    const double rden =
+        (unsigned)__double2hiint(den) - (923u << 20) < (200u << 20) ? rcp64(den) : 1.0 / den;
     double up[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) up[a] = (j[0][a] * m.inv_tau[0] + j[1][a] * m.inv_tau[1]) * rden;
