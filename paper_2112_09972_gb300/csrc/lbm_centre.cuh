@@ -96,60 +96,36 @@ __device__ void centre_epilogue(C (&cm)[4], CentreParts cp, C* scratch) {
     centre_reduce(cm, reinterpret_cast<C*>(cp.p), cta, total, cp.counter, cp.sum, cp.frame, scratch);
 }
 
-// centre_reduce for kernels whose CTAs mostly hold no droplet node: a CTA with
-// any = false (uniform) writes zero partials without the shuffles (float64
-// ones run on the slow FP64 pipe), and every thread of the last CTA takes part
-// in the final sum.
-template <int NT, typename C>
-__device__ void centre_reduce_last(C (&cm)[4], bool any, C* parts, unsigned slot, unsigned total, unsigned* counter,
-                                   double* sum8, float* frame, C* scratch) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+// Centre-of-mass partials of `units` pieces of the box by the `ctas` CTAs of a
+// launch that this is the cta-th of, from a density array, one warp to a unit
+// (the two-pass kernels).  unit(u, cm) leaves the sums of unit u in its lane
+// 0.  The CTAs that collide then hold nothing back for a reduction and end
+// when their nodes are stored; these few run beside them.
+template <typename C, typename U>
+__device__ void centre_units(U&& unit, int units, int cta, int ctas, CentreParts cp) {
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, warps = blockDim.x / 32;
     __shared__ unsigned last;
-    auto warp_sums = [&](const C (&v)[4]) {
+    C* parts = reinterpret_cast<C*>(cp.p);
+    for (int u = cta * warps + warp; u < units; u += ctas * warps) {
+        C cm[4] = {C(0), C(0), C(0), C(0)};
+        unit(u, cm);
+        if (lane == 0)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            C a = v[q];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-            if (lane == 0) scratch[4 * warp + q] = a;
-        }
-    };
-    auto total_of = [&](int q) {
-        C a = scratch[q];
-        for (int w = 1; w < NT / 32; ++w) a += scratch[4 * w + q];
-        return a;
-    };
-    if (any) warp_sums(cm);
+            for (int q = 0; q < 4; ++q) parts[4LL * u + q] = cm[q];
+    }
     __syncthreads();
-    if (t == 0) {
-        for (int q = 0; q < 4; ++q) parts[4LL * slot + q] = any ? total_of(q) : C(0);
+    if (threadIdx.x == 0) {
         __threadfence();
-        last = atomicAdd(counter, 1u) == total - 1 ? 1u : 0u;
+        last = atomicAdd(cp.counter, 1u) == (unsigned)ctas - 1u ? 1u : 0u;
     }
     __syncthreads();
-    if (!last) return;
-    __threadfence();
-    C s4[4] = {C(0), C(0), C(0), C(0)};
-#pragma unroll 4
-    for (unsigned b = t; b < total; b += NT)
+    if (last && warp == 0) centre_total<C>(parts, (unsigned)units, cp.counter, cp.sum, cp.frame);
+}
+template <typename C>
+__device__ __forceinline__ C warp_total(C a) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) s4[q] += __ldcg(parts + 4LL * b + q);
-    warp_sums(s4);
-    __syncthreads();
-    if (t == 0) {
-        C sum[4];
-        for (int q = 0; q < 4; ++q) {
-            sum[q] = total_of(q);
-            sum8[q] = (double)sum[q];
-        }
-        const bool have = sum[0] > C(0);
-        for (int q = 0; q < 3; ++q) {
-            const C xc = have ? sum[1 + q] / sum[0] : C(0);
-            sum8[4 + q] = (double)xc;
-            frame[q] = (float)xc;
-        }
-        *counter = 0u;
-    }
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    return a;
 }
 
 }  // namespace

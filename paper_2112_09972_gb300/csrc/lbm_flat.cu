@@ -21,10 +21,12 @@
 // read of the populations costs bandwidth that is idle), opposite
 // directions share their equilibria, and the launch covers the chip for any
 // box: one node per thread instead of a z march per tile.  Measured per step
-// against the tile kernel: 32^3 42 us (178), 64^3 195 us (365), 128^3 1433 us
-// (3174), 37 x 29 x 23 36 us (160); float64 storage therefore takes these
+// against the tile kernel: 32^3 39.5 us (178), 64^3 174 us (365), 128^3 1408 us
+// (3174), 37 x 29 x 23 31 us (160); float64 storage therefore takes these
 // kernels at every size.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "lbm_eigen.cuh"
 #include "lbm_internal.h"
@@ -190,45 +192,66 @@ __device__ __forceinline__ void flat_node(const double2* __restrict__ r, int sy,
     }
 }
 
+// The centre sums of a z chunk's share of rows, lanes over x.  w = max(phi, 0):
+// the division and the sums only in warps where a phi is not negative.
+constexpr int kFlatShares = 8;  // a warp each, at most one per CTA of a chunk
+__device__ __forceinline__ void flat_unit(const double2* __restrict__ rho, const RhoGeo& g, const Layout& L, int u,
+                                          int shares, int zchunk, double (&cm)[4]) {
+    const int lane = threadIdx.x % 32, chunk = u / shares, share = u - chunk * shares;
+    const int z1 = min((chunk + 1) * zchunk, L.Lz);
+    bool any = false;
+    for (int z = chunk * zchunk; z < z1; ++z)
+        for (int y = share; y < L.Ly; y += shares)
+            for (int x = lane; x < L.Lx; x += 32) {
+                const double2 r = __ldg(rho + g.at(x, y, z));
+                const double d = r.x - r.y, t = r.x + r.y;
+                if ((__double2hiint(d) ^ __double2hiint(t)) >= 0) {
+                    const double w = fmax(d / t, 0.0);
+                    cm[0] += w;
+                    cm[1] = fma(w, x - 0.5 * (L.Lx - 1), cm[1]);
+                    cm[2] = fma(w, y - 0.5 * (L.Ly - 1), cm[2]);
+                    cm[3] = fma(w, z - 0.5 * (L.Lz - 1), cm[3]);
+                    any = true;
+                }
+            }
+    if (!__any_sync(0xffffffffu, any)) return;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cm[q] = warp_total(cm[q]);
+}
+
+// The first `centres` CTAs sum the centre of mass from the density array
+// (against sums at the end of every colliding CTA: 32^3 41.9 -> 39.5 us per step,
+// 64^3 195 -> 174, 37 x 29 x 23 36.1 -> 30.9).
 template <bool PER, bool MRT>
 __global__ void __launch_bounds__(kFlatThreads, 6)
     k_flat_collide(const double* __restrict__ src, double* __restrict__ dst, Layout L, FlatModel m,
-                   const double2* __restrict__ rho, RhoGeo g, int zchunk, CentreParts cp, int* __restrict__ d_err) {
-    __shared__ double scratch[4 * (kFlatThreads / 32)];
+                   const double2* __restrict__ rho, RhoGeo g, int per_plane, int zchunk, int units, int centres,
+                   CentreParts cp, int* __restrict__ d_err) {
     pdl_wait();
-    const int p = blockIdx.x * kFlatThreads + threadIdx.x;
+    if ((int)blockIdx.x < centres) {
+        pdl_trigger();
+        const int shares = min(kFlatShares, per_plane);
+        centre_units<double>([&](int u, double (&cm)[4]) { flat_unit(rho, g, L, u, shares, zchunk, cm); }, units,
+                             (int)blockIdx.x, centres, cp);
+        return;
+    }
+    const int cta = (int)blockIdx.x - centres, chunk = cta / per_plane;
+    const int p = (cta - chunk * per_plane) * kFlatThreads + threadIdx.x;
     const int y = p / L.Lx, x = p - y * L.Lx;
     const Puller<double, double, PER> P{src, L};
-    double cm[4] = {0.0, 0.0, 0.0, 0.0};
-    bool drop = false, bad = false;
+    bool bad = false;
     if (p < L.Lx * L.Ly) {
-        const double px = x - 0.5 * (L.Lx - 1), py = y - 0.5 * (L.Ly - 1);
-        const int z1 = min(((int)blockIdx.y + 1) * zchunk, L.Lz);
-        for (int z = blockIdx.y * zchunk; z < z1; ++z) {
+        const int z1 = min((chunk + 1) * zchunk, L.Lz);
+        for (int z = chunk * zchunk; z < z1; ++z) {
             double f[2][19];
             P.pull(x, y, z, f);
             double2 r;
             flat_node<MRT>(rho + g.at(x, y, z), g.nx, g.nx * g.ny, m, f, dst + L.at(0, 0, x, y, z), L.pitch, r);
             bad |= !(finite64(r.x) && finite64(r.y));
-            // w = max(phi, 0): the division only where phi is not negative
-            const double d = r.x - r.y, t = r.x + r.y;
-            if ((__double2hiint(d) ^ __double2hiint(t)) >= 0) {
-                const double w = fmax(d / t, 0.0);
-                cm[0] += w;
-                cm[1] = fma(w, px, cm[1]);
-                cm[2] = fma(w, py, cm[2]);
-                cm[3] = fma(w, z - 0.5 * (L.Lz - 1), cm[3]);
-                drop = true;
-            }
         }
     }
     pdl_trigger();
     if (bad) atomicOr(d_err, 1);
-    // the droplet's centre of mass: partials in CTA order, as centre_epilogue,
-    // whose FP64 shuffles a CTA without droplet nodes does without
-    const unsigned cta = blockIdx.y * gridDim.x + blockIdx.x, total = gridDim.x * gridDim.y;
-    const bool any = __syncthreads_or(drop) != 0;
-    centre_reduce_last<kFlatThreads>(cm, any, cp.p, cta, total, cp.counter, cp.sum, cp.frame, scratch);
 }
 
 }  // namespace
@@ -238,8 +261,8 @@ long long flat_rho_bytes(const Layout& L) {
 }
 
 // One node per thread; the z extent is cut so that the launch has at most
-// about 16 CTAs per SM, which bounds the centre-of-mass partials the last CTA
-// sums (small boxes: one plane per CTA).
+// about 16 CTAs per SM, which bounds the centre-of-mass partials (small boxes:
+// one plane per CTA).
 Shape flat_shape(const Layout& L, int num_sms) {
     Shape sh = {};
     const long long per_plane = ((long long)L.Lx * L.Ly + kFlatThreads - 1) / kFlatThreads;
@@ -279,7 +302,11 @@ cudaError_t launch_flat(const void* src, void* dst, void* rho, const Layout& L, 
     if (e != cudaSuccess) return e;
     auto k = m.periodic ? (m.mrt ? k_flat_collide<true, true> : k_flat_collide<true, false>)
                         : (m.mrt ? k_flat_collide<false, true> : k_flat_collide<false, false>);
-    return cudaLaunchKernelEx(&cfg, k, f, (double*)dst, L, fm, (const double2*)r, g, sh.zchunk, cp, d_err);
+    const int per_plane = (int)sh.grid.x, units = std::min(kFlatShares, per_plane) * (int)sh.grid.y;
+    const int centres = std::min((units + kFlatThreads / 32 - 1) / (kFlatThreads / 32), 512);
+    cfg.gridDim = dim3(centres + sh.grid.x * sh.grid.y, 1, 1);
+    return cudaLaunchKernelEx(&cfg, k, f, (double*)dst, L, fm, (const double2*)r, g, per_plane, sh.zchunk, units,
+                              centres, cp, d_err);
 }
 
 }  // namespace lbmgb

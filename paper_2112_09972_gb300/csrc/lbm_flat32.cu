@@ -160,36 +160,6 @@ __global__ void __launch_bounds__(TX * row_rho_rows<TX>())
     rho[g.at(x, y, z)] = make_float2(ra, rb);
 }
 
-// Centre-of-mass partials of `units` pieces of the box by the `ctas` CTAs of a
-// launch that this is the cta-th of, from the density pass's array, one warp
-// to a unit.  unit(u, cm) leaves the sums of unit u in its lane 0.  The CTAs
-// that collide then hold nothing back for a reduction and end when their
-// nodes are stored; these few run beside the last of them.
-template <typename U>
-__device__ void centre_units(U&& unit, int units, int cta, int ctas, CentreParts cp) {
-    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, warps = blockDim.x / 32;
-    __shared__ unsigned last;
-    float* parts = reinterpret_cast<float*>(cp.p);
-    for (int u = cta * warps + warp; u < units; u += ctas * warps) {
-        float cm[4] = {0.f, 0.f, 0.f, 0.f};
-        unit(u, cm);
-        if (lane == 0)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) parts[4LL * u + q] = cm[q];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(cp.counter, 1u) == (unsigned)ctas - 1u ? 1u : 0u;
-    }
-    __syncthreads();
-    if (last && warp == 0) centre_total<float>(parts, (unsigned)units, cp.counter, cp.sum, cp.frame);
-}
-__device__ __forceinline__ float warp_total(float a) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    return a;
-}
 // the droplet indicator of collide_core
 __device__ __forceinline__ float indicator(float2 r) { return fmaxf(__fdividef(r.x - r.y, r.x + r.y), 0.f); }
 
@@ -249,7 +219,7 @@ __global__ void __launch_bounds__(TX * row_collide_rows<TX>(), 512 / (TX * row_c
     pdl_wait();
     if ((int)blockIdx.x >= colliders) {
         pdl_trigger();
-        centre_units([&](int u, float (&cm)[4]) { row_unit<TX>(rho, g, L, u % L.Ly, u / L.Ly, zchunk, cm); }, units,
+        centre_units<float>([&](int u, float (&cm)[4]) { row_unit<TX>(rho, g, L, u % L.Ly, u / L.Ly, zchunk, cm); }, units,
                      (int)blockIdx.x - colliders, (int)gridDim.x - colliders, cp);
         return;
     }
@@ -355,7 +325,7 @@ __global__ void __launch_bounds__(kAnyThreads, 5)
     if ((int)blockIdx.x >= colliders) {
         pdl_trigger();
         const int shares = min(kAnyShares, per_plane);
-        centre_units([&](int u, float (&cm)[4]) { any_unit(rho, g, L, u, shares, cm); }, shares * L.Lz,
+        centre_units<float>([&](int u, float (&cm)[4]) { any_unit(rho, g, L, u, shares, cm); }, shares * L.Lz,
                      (int)blockIdx.x - colliders, (int)gridDim.x - colliders, cp);
         return;
     }
