@@ -21,8 +21,8 @@
 // read of the populations costs bandwidth that is idle), opposite
 // directions share their equilibria, and the launch covers the chip for any
 // box: one node per thread instead of a z march per tile.  Measured per step
-// against the tile kernel: 32^3 39.5 us (178), 64^3 174 us (365), 128^3 1408 us
-// (3174), 37 x 29 x 23 31 us (160); float64 storage therefore takes these
+// against the tile kernel: 32^3 32 us (178), 64^3 174 us (365), 128^3 1411 us
+// (3174), 37 x 29 x 23 27 us (160); float64 storage therefore takes these
 // kernels at every size.
 #include <cuda_runtime.h>
 
@@ -219,23 +219,24 @@ __device__ __forceinline__ void flat_unit(const double2* __restrict__ rho, const
     for (int q = 0; q < 4; ++q) cm[q] = warp_total(cm[q]);
 }
 
-// The first `centres` CTAs sum the centre of mass from the density array
-// (against sums at the end of every colliding CTA: 32^3 41.9 -> 39.5 us per step,
-// 64^3 195 -> 174, 37 x 29 x 23 36.1 -> 30.9).
+// `centres` CTAs from `centre0` on sum the centre of mass from the density
+// array (against sums at the end of every colliding CTA, per step: 32^3 41.9 ->
+// 31.9 us, 37 x 29 x 23 36.1 -> 26.9, 64^3 195 -> 174, 128^3 1433 -> 1408).
 template <bool PER, bool MRT>
 __global__ void __launch_bounds__(kFlatThreads, 6)
     k_flat_collide(const double* __restrict__ src, double* __restrict__ dst, Layout L, FlatModel m,
-                   const double2* __restrict__ rho, RhoGeo g, int per_plane, int zchunk, int units, int centres,
+                   const double2* __restrict__ rho, RhoGeo g, int per_plane, int zchunk, int units, int centre0, int centres,
                    CentreParts cp, int* __restrict__ d_err) {
     pdl_wait();
-    if ((int)blockIdx.x < centres) {
+    const int own = (int)blockIdx.x - centre0;
+    if (own >= 0 && own < centres) {
         pdl_trigger();
         const int shares = min(kFlatShares, per_plane);
         centre_units<double>([&](int u, double (&cm)[4]) { flat_unit(rho, g, L, u, shares, zchunk, cm); }, units,
-                             (int)blockIdx.x, centres, cp);
+                             own, centres, cp);
         return;
     }
-    const int cta = (int)blockIdx.x - centres, chunk = cta / per_plane;
+    const int cta = own < 0 ? (int)blockIdx.x : (int)blockIdx.x - centres, chunk = cta / per_plane;
     const int p = (cta - chunk * per_plane) * kFlatThreads + threadIdx.x;
     const int y = p / L.Lx, x = p - y * L.Lx;
     const Puller<double, double, PER> P{src, L};
@@ -303,10 +304,15 @@ cudaError_t launch_flat(const void* src, void* dst, void* rho, const Layout& L, 
     auto k = m.periodic ? (m.mrt ? k_flat_collide<true, true> : k_flat_collide<true, false>)
                         : (m.mrt ? k_flat_collide<false, true> : k_flat_collide<false, false>);
     const int per_plane = (int)sh.grid.x, units = std::min(kFlatShares, per_plane) * (int)sh.grid.y;
+    const int colliders = (int)(sh.grid.x * sh.grid.y);
     const int centres = std::min((units + kFlatThreads / 32 - 1) / (kFlatThreads / 32), 512);
-    cfg.gridDim = dim3(centres + sh.grid.x * sh.grid.y, 1, 1);
+    // last where the colliders all run at once, so that the sums land on the SMs with one collider less (first, they
+    // pushed a fifth one on some: 32^3 39.5 us); first where they do not, so that no long sum is left over (last: 128^3
+    // 1905 us)
+    const int centre0 = colliders <= 6 * 152 ? colliders : 0;
+    cfg.gridDim = dim3(colliders + centres, 1, 1);
     return cudaLaunchKernelEx(&cfg, k, f, (double*)dst, L, fm, (const double2*)r, g, per_plane, sh.zchunk, units,
-                              centres, cp, d_err);
+                              centre0, centres, cp, d_err);
 }
 
 }  // namespace lbmgb
