@@ -14,7 +14,9 @@
 //       (collide_core), so both store bit-identical states.
 //   k_any_rho / k_any_collide -- float32 boxes of any other extents, in place
 //       of the tile kernel, whose tiles sum their halo's densities again
-//       (about as many nodes as the tile has) and march in z.
+//       (about as many nodes as the tile has) and march in z.  The node
+//       arithmetic (tile_collide) and the order of the centre's sums are the
+//       tile kernel's, so both store bit-identical states here too.
 //
 // Density array: [Lz + 2][Ly + 2][Lx + 2] of {rho_A, rho_B}, its halo holding
 // the ghost densities.
@@ -141,8 +143,8 @@ constexpr int row_rho_rows() {
 // Also writes the ghost populations that its nodes pull, which saves a launch
 // of the chain that a small box's step is (32^3 fp32 10.4 -> 9.4 us per step,
 // 64^3 24.9 -> 24.1, bf16 18.9 -> 17.7; the other two-pass kernels lost more registers to it than
-// the launch was worth: 37 x 29 x 23 fp32 11.7 -> 10.9 us, but 130^3 222 -> 242, and
-// in float64 32^3 41 -> 57).
+// the launch was worth: tried in them, it took 37 x 29 x 23 fp32 from 11.7 to 10.9
+// us, but 130^3 from 222 to 242, and float64 32^3 from 41 to 57).
 template <int TX, typename ST>
 __global__ void __launch_bounds__(TX * row_rho_rows<TX>())
     k_row_rho(ST* src, Layout L, float2* __restrict__ rho, RhoGeo g, GhostParams<float> gp, CentreParts cp,
@@ -270,19 +272,11 @@ cudaError_t launch_row_w(int prec, void* src, void* dst, void* rho, const Layout
 
 // ---- any extents, float32 ----
 
-struct AnyIO {
-    struct Out {
-        float* p;
-        int pitch;
-    };
-    template <int S, int I>
-    static __device__ __forceinline__ void store(Out o, float v) {
-        __stcs(o.p + (S * 19 + I) * o.pitch, v);
-    }
-};
-
 constexpr int kAnyThreads = 128;
-constexpr int kAnyShares = 8;  // centre sums: shares of a plane's rows, a warp each, at most one per CTA of a plane
+constexpr int kAnyPerSM = 5;  // resident CTAs of the collision pass
+int any_per_plane(const Layout& L) { return (L.Lx * L.Ly + kAnyThreads - 1) / kAnyThreads; }
+int any_colliders(const Layout& L) { return any_per_plane(L) * L.Lz; }
+constexpr int kAnyTileWarps = 16;  // warps of the tile kernel's largest CTA
 __global__ void __launch_bounds__(kAnyThreads) k_any_rho(const float* __restrict__ src, Layout L,
                                                          float2* __restrict__ rho, RhoGeo g, int per_plane) {
     pdl_wait();
@@ -296,51 +290,122 @@ __global__ void __launch_bounds__(kAnyThreads) k_any_rho(const float* __restrict
     rho[g.at(x, y, z)] = make_float2(sum19<float>(f[0]), sum19<float>(f[1]));
 }
 
-// The sums of one plane's share of rows, lanes over x.
-__device__ __forceinline__ void any_unit(const float2* __restrict__ rho, const RhoGeo& g, const Layout& L, int u,
-                                         int shares, float (&cm)[4]) {
-    const int lane = threadIdx.x % 32, z = u / shares, share = u - z * shares;
-    const float pz = (float)z - 0.5f * (float)(L.Lz - 1);
-    for (int y = share; y < L.Ly; y += shares) {
-        const float py = (float)y - 0.5f * (float)(L.Ly - 1);
-#pragma unroll 4
-        for (int x = lane; x < L.Lx; x += 32) {
-            const float w = indicator(__ldg(rho + g.at(x, y, z)));
-            cm[0] += w;
-            cm[1] = fmaf(w, (float)x - 0.5f * (float)(L.Lx - 1), cm[1]);
-            cm[2] = fmaf(w, py, cm[2]);
-            cm[3] = fmaf(w, pz, cm[3]);
+// The tile kernel's launch for this box: tiles of tx x ty nodes, z chunks.
+struct AnyTiles {
+    int tx, ty, zchunk, nx, ny, ctas;  // nx, ny: tiles along x and y
+};
+
+// Centre of mass from the density array: one CTA for each CTA of the tile
+// kernel, its sums in that kernel's order -- thread t of the tile over the
+// planes of its march, the warps' shuffles, the shuffle over warps, and the
+// CTAs in order at the end (centre_reduce).  In small boxes this chain is the
+// longest of the launch, and its loads are what it waits for: sixteen of a
+// lane's in flight instead of one 37 x 29 x 23 13.4 -> 10.6 us per step, 60 x 50 x
+// 44 16.8 -> 14.6.
+__device__ void any_centre(const float2* __restrict__ rho, const RhoGeo& g, const Layout& L, const AnyTiles& a, int u,
+                           const CentreParts& cp) {
+    __shared__ float sums[kAnyTileWarps][4];
+    __shared__ unsigned last;
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int chunk = u / (a.nx * a.ny), tile = u - chunk * (a.nx * a.ny);
+    const int x0 = tile % a.nx * a.tx, y0 = tile / a.nx * a.ty;
+    const int z0 = chunk * a.zchunk, z1 = min(z0 + a.zchunk, L.Lz);
+    const int threads = a.tx * a.ty, warps = (threads + 31) / 32;
+    float* parts = reinterpret_cast<float*>(cp.p);
+    // warp w takes the tile's warps w, w + 4, ... side by side, so that their loads are in flight together
+    constexpr int H = kAnyTileWarps / (kAnyThreads / 32);
+    float cm[H][4] = {}, px[H], py[H];
+    const float2* r[H];
+    bool in[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+        const int t = 32 * (warp + k * (kAnyThreads / 32)) + lane, x = x0 + t % a.tx, y = y0 + t / a.tx;
+        in[k] = t < threads && x < L.Lx && y < L.Ly;
+        px[k] = (float)x - 0.5f * (float)(L.Lx - 1);
+        py[k] = (float)y - 0.5f * (float)(L.Ly - 1);
+        r[k] = rho + (in[k] ? g.at(x, y, z0) : 0);
+    }
+    const int sz = g.nx * g.ny;
+    constexpr int U = 4;  // planes read before the first of them is summed
+    for (int zu = z0; zu < z1; zu += U) {
+        float2 v[U][H];
+#pragma unroll
+        for (int i = 0; i < U; ++i)
+#pragma unroll
+            for (int k = 0; k < H; ++k) v[i][k] = __ldg(r[k] + (long long)(min(zu + i, z1 - 1) - z0) * sz);
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const float pz = (float)(zu + i) - 0.5f * (float)(L.Lz - 1);
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                const float rk[2] = {v[i][k].x, v[i][k].y};
+                // (a droplet's nodes: elsewhere w = 0 and the sums stay as they are)
+                if (in[k] && zu + i < z1 && (rk[0] > rk[1]) == (rk[0] + rk[1] > 0.f))
+                    droplet_sums<float>(rk, px[k], py[k], pz, cm[k]);
+            }
         }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) cm[q] = warp_total(cm[q]);
+    for (int k = 0; k < H; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float s = warp_total(cm[k][q]);
+            if (lane == 0) sums[warp + k * (kAnyThreads / 32)][q] = s;
+        }
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float s = warp_total(lane < warps ? sums[lane][q] : 0.f);
+            if (lane == 0) parts[4LL * u + q] = s;
+        }
+        if (lane == 0) {
+            __threadfence();
+            last = atomicAdd(cp.counter, 1u) == (unsigned)a.ctas - 1u ? 1u : 0u;
+        }
+        __syncwarp();
+        if (last) centre_total<float>(parts, (unsigned)a.ctas, cp.counter, cp.sum, cp.frame);
+    }
 }
 
+// a.ctas CTAs from `centre0` on sum the centre, the others take a node a thread.
 template <bool MRT>
-__global__ void __launch_bounds__(kAnyThreads, 5)
-    k_any_collide(const float* __restrict__ src, float* __restrict__ dst, Layout L, FastModel m,
-                  const float2* __restrict__ rho, RhoGeo g, int per_plane, int colliders, CentreParts cp,
+__global__ void __launch_bounds__(kAnyThreads, kAnyPerSM)
+    k_any_collide(const float* __restrict__ src, float* __restrict__ dst, Layout L, ModelC<float> m,
+                  const float2* __restrict__ rho, RhoGeo g, int per_plane, AnyTiles a, int centre0, CentreParts cp,
                   int* __restrict__ d_err) {
     pdl_wait();
-    if ((int)blockIdx.x >= colliders) {
+    const int own = (int)blockIdx.x - centre0;
+    if (own >= 0 && own < a.ctas) {
         pdl_trigger();
-        const int shares = min(kAnyShares, per_plane);
-        centre_units<float>([&](int u, float (&cm)[4]) { any_unit(rho, g, L, u, shares, cm); }, shares * L.Lz,
-                     (int)blockIdx.x - colliders, (int)gridDim.x - colliders, cp);
+        any_centre(rho, g, L, a, own, cp);
         return;
     }
-    const int z = blockIdx.x / per_plane, p = (blockIdx.x - z * per_plane) * kAnyThreads + threadIdx.x;
+    const int cta = own < 0 ? (int)blockIdx.x : (int)blockIdx.x - a.ctas;
+    const int z = cta / per_plane, p = (cta - z * per_plane) * kAnyThreads + threadIdx.x;
     const int y = p / L.Lx, x = p - y * L.Lx;
     if (p < L.Lx * L.Ly) {
         const Puller<float, float, false> P{src, L};
-        int bad = 0;
-        float f[2][19], cm[4] = {0.f, 0.f, 0.f, 0.f};
-        const float rs[2] = {0.f, 0.f};
+        float f[2][19];
         P.pull(x, y, z, f);
-        const float2* r = rho + g.at(x, y, z);
-        collide_core<AnyIO, float, MRT>(RhoNb{r, g.nx, g.nx * g.ny}, __ldg(r), f, rs, m,
-                                        AnyIO::Out{dst + L.at(0, 0, x, y, z), L.pitch}, cm, bad, 0.f, 0.f, 0.f);
-        if (bad) atomicOr(d_err, bad);
+        const RhoNb near{rho + g.at(x, y, z), g.nx, g.nx * g.ny};
+        const float2 own2 = near(0, 0, 0);
+        const float r[2] = {own2.x, own2.y};
+        float* o = dst + L.at(0, 0, x, y, z);
+        auto nb = [&](int s, int dx, int dy, int dz) {
+            const float2 v = near(dx, dy, dz);
+            return s ? v.y : v.x;
+        };
+        tile_collide<float, MRT, false>(f, r, m, nb, [&](int s, const float (&out)[19]) {
+            float others = 0.f;  // the rest population closes the mass balance
+#pragma unroll
+            for (int i = 1; i < 19; ++i) {
+                __stcs(o + (19 * s + i) * L.pitch, out[i]);
+                others += out[i];
+            }
+            __stcs(o + 19 * s * L.pitch, r[s] - others);
+        });
+        if (!(isfinite(r[0]) && isfinite(r[1]))) atomicOr(d_err, 1);
     }
     pdl_trigger();
 }
@@ -361,16 +426,15 @@ Shape flat_rows_shape(const Shape& rows) {
     return sh;
 }
 
-// Any float32 box: one node per thread.
-Shape flat_any_shape(const Layout& L) {
-    Shape sh = {};
-    const long long per_plane = ((long long)L.Lx * L.Ly + kAnyThreads - 1) / kAnyThreads;
+// Any float32 box: one node per thread.  Keeps the tile kernel's shape, by
+// which the centre sums are ordered.  Their CTAs come first where the grid
+// takes more than one wave, so that none is left over at its end (per step,
+// first against last: 60 x 50 x 44 17.0 us and 19.2, 130^3 206 and 240; 37 x 29 x
+// 23, one wave, 13.9 and 13.8).
+Shape flat_any_shape(const Layout& L, const Shape& tile, int num_sms) {
+    Shape sh = tile;
     sh.flat = kFlatAny;
-    sh.tx = L.Lx;
-    sh.ty = L.Lx >= kAnyThreads ? 1 : kAnyThreads / L.Lx;
-    sh.zchunk = 1;
-    sh.grid = dim3((unsigned)per_plane, (unsigned)L.Lz, 1);
-    sh.threads = kAnyThreads;
+    sh.centre_first = any_colliders(L) > kAnyPerSM * (num_sms > 0 ? num_sms : 152);
     return sh;
 }
 
@@ -394,7 +458,7 @@ cudaError_t launch_flat_rows(int prec, void* src, void* dst, void* rho, const La
 cudaError_t launch_flat_any(const void* src, void* dst, void* rho, const Layout& L, const Model& m, const Shape& sh,
                             CentreParts cp, int* d_err, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    const int per_plane = (int)sh.grid.x, colliders = (int)(sh.grid.x * sh.grid.y);
+    const int per_plane = any_per_plane(L), colliders = any_colliders(L);
     cfg.gridDim = dim3(colliders, 1, 1);
     cfg.blockDim = dim3(kAnyThreads, 1, 1);
     cfg.stream = s;
@@ -405,11 +469,12 @@ cudaError_t launch_flat_any(const void* src, void* dst, void* rho, const Layout&
     const float* f = (const float*)src;
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_any_rho, f, L, (float2*)rho, g, per_plane);
     if (e != cudaSuccess) return e;
-    // centre sums: four units (a share of a plane's rows) to a CTA
-    const int units = std::min(kAnyShares, per_plane) * L.Lz;
-    cfg.gridDim = dim3(colliders + (units + kAnyThreads / 32 - 1) / (kAnyThreads / 32), 1, 1);
+    const AnyTiles a = {sh.tx, sh.ty, sh.zchunk, (int)sh.grid.x, (int)sh.grid.y,
+                        (int)(sh.grid.x * sh.grid.y * sh.grid.z)};
+    cfg.gridDim = dim3(colliders + a.ctas, 1, 1);
     return cudaLaunchKernelEx(&cfg, m.mrt ? k_any_collide<true> : k_any_collide<false>, f, (float*)dst, L,
-                              fast_model(m), (const float2*)rho, g, per_plane, colliders, cp, d_err);
+                              model_c<float>(m), (const float2*)rho, g, per_plane, a,
+                              sh.centre_first ? 0 : colliders, cp, d_err);
 }
 
 }  // namespace lbmgb

@@ -103,6 +103,7 @@ struct Grad {
 // Launch shape of the stream-collide kernel.
 struct Shape {
     int rows;       // 1: the row-tiled cluster kernel (lbm_fast.cu), 0: the generic tile kernel
+    int centre_first;  // kFlatAny: the CTAs that sum the centre lead the grid
     int flat;       // kFlat64, kFlatRows or kFlatAny: two-pass kernels, which need a density array
     int tx, ty;     // tile of the x-y plane per CTA
     int zchunk;     // z planes marched per CTA
@@ -156,7 +157,7 @@ cudaError_t launch_flat(const void* src, void* dst, void* rho, const Layout& L, 
 
 // ---- two-pass kernels (lbm_flat32.cu): fp32 or 16-bit deviations, ghost boundary ----
 Shape flat_rows_shape(const Shape& rows);
-Shape flat_any_shape(const Layout& L);
+Shape flat_any_shape(const Layout& L, const Shape& tile, int num_sms);
 long long flat32_rho_bytes(const Layout& L);
 cudaError_t launch_flat32_fill(void* rho, const Layout& L, const Model& m, cudaStream_t s);
 cudaError_t launch_flat_rows(int prec, void* src, void* dst, void* rho, const Layout& L, const Model& m,

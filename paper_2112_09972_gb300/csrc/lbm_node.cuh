@@ -361,8 +361,8 @@ struct RowIO<TX, Dev<T>> {
 // post-collision state (float32 populations with the rest population closing
 // the mass balance, or 16-bit deviations).  Also accumulates the
 // centre-of-mass partials of the droplet phase and flags non-finite
-// densities.  Shared by the row kernels and the two-pass kernels so that
-// every variant computes bit-identical states.
+// densities.  Shared by the row kernels and the two-pass kernels of their
+// widths so that every variant computes bit-identical states.
 template <typename IO, typename ST, bool MRT, typename NB>
 __device__ __forceinline__ void collide_core(NB&& nb, const float2 rho2, const float (&f)[2][19],
                                              const float (&rs)[2], const FastModel& m, typename IO::Out out,

@@ -204,19 +204,6 @@ __global__ void __launch_bounds__(256) k_centre(const S* __restrict__ f, Layout 
     centre_epilogue(cm, cp, scratch);
 }
 
-template <typename C>
-ModelC<C> model_c(const Model& m) {
-    ModelC<C> r;
-    for (int s = 0; s < 2; ++s) {
-        r.tau[s] = (C)m.tau[s];
-        r.inv_tau[s] = (C)(1.0 / m.tau[s]);
-        r.rho_b[s] = (C)m.rho_b[s];
-    }
-    r.G = (C)m.G;
-    for (int k = 0; k < 5; ++k) r.mrt[k] = (C)m.mrt_rates[k];
-    return r;
-}
-
 template <typename S, typename C, bool PER, bool MRT, int MAXT>
 void stream_collide_launch(const void* src, void* dst, const Layout& L, const ModelC<C>& mc, const Shape& sh,
                            CentreParts cp, int* d_err, cudaStream_t s) {
@@ -278,6 +265,7 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
     Shape sh;
     sh.rows = 0;
     sh.flat = 0;
+    sh.centre_first = 0;
     sh.variant = kRowDirect;
     if (ty_req <= 0 && (!mrt || prec == kFP32) && rows_kernel_applies(L, prec, periodic)) {
         // One CTA per row.  MRT rows: direct loads only.  Automatic choice,
@@ -329,10 +317,6 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
             return sh;
         }
     }
-    // float32 boxes of other extents: two-pass at every size (per step against
-    // the tile kernel: 37 x 29 x 23 11.7 us (34.5), 60 x 50 x 44 19.2 (31.1), 96^3
-    // 92.4 (116), 130^3 222 (327), 200 x 200 x 100 346 (460))
-    if (allow_flat && prec == kFP32 && !periodic && ty_req <= 0 && zchunk_req <= 0) return flat_any_shape(L);
     const int cbytes = prec == kFP64 ? 8 : 4;  // compute type of the density ring
     const int maxt = prec == kFP64 ? kMaxThreadsF64 : kMaxThreadsF32;
     sh.tx = L.Lx <= maxt ? L.Lx : 128;
@@ -358,6 +342,10 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
     sh.smem = (size_t)4 * 2 * (sh.tx + 2) * (sh.ty + 2) * cbytes;
     const size_t red = (size_t)((sh.threads + 31) / 32) * 4 * sizeof(double);
     if (sh.smem < red) sh.smem = red;
+    // float32 boxes of other extents: two-pass at every size (per step against
+    // the tile kernel: 37 x 29 x 23 10.6 us (34.9), 60 x 50 x 44 14.6 (31.4), 96 x
+    // 96 x 95 78 (112), 130^3 212 (334), 200 x 200 x 100 309 (465))
+    if (allow_flat && prec == kFP32 && !periodic && ty_req <= 0 && zchunk_req <= 0) return flat_any_shape(L, sh, num_sms);
     return sh;
 }
 

@@ -24,6 +24,19 @@ struct ModelC {
     C mrt[5];  // MRT free rates s_e, s_eps, s_q, s_pi, s_m (used by MRT instantiations)
 };
 
+template <typename C>
+ModelC<C> model_c(const Model& m) {
+    ModelC<C> r;
+    for (int s = 0; s < 2; ++s) {
+        r.tau[s] = (C)m.tau[s];
+        r.inv_tau[s] = (C)(1.0 / m.tau[s]);
+        r.rho_b[s] = (C)m.rho_b[s];
+    }
+    r.G = (C)m.G;
+    for (int k = 0; k < 5; ++k) r.mrt[k] = (C)m.mrt_rates[k];
+    return r;
+}
+
 template <typename S, typename C, bool PER>
 struct Puller {
     const S* __restrict__ src;
@@ -103,6 +116,83 @@ struct Puller<Dev<T>, C, PER> {
 };
 
 
+// Droplet sums {sum w, sum w x, sum w y, sum w z} of a node, w = max(phi, 0);
+// they give the next step's frame origin.
+template <typename C>
+__device__ __forceinline__ void droplet_sums(const C (&rho)[2], C px, C py, C pz, C (&cm)[4]) {
+    const C phi = (rho[0] - rho[1]) / (rho[0] + rho[1]);
+    const C wphi = phi > C(0) ? phi : C(0);
+    cm[0] += wphi;
+    cm[1] += wphi * px;
+    cm[2] += wphi * py;
+    cm[3] += wphi * pz;
+}
+
+// Collision of one node from its pulled populations fc, its densities and its
+// neighbours' (nb(s, dx, dy, dz)): emit(s, out) takes component s's
+// post-collision moving populations out[1..18].  The tile march and the
+// two-pass kernels of float32 boxes (lbm_flat32.cu) share it, so that their
+// states agree bit for bit.
+template <typename C, bool MRT, bool Full, typename NB, typename Emit>
+__device__ __forceinline__ void tile_collide(const C (&fc)[2][19], const C (&rho)[2], const ModelC<C>& m, NB&& nb,
+                                             Emit&& emit) {
+    // momentum of each component (Eq. 6), opposite pairs first
+    C j[2][3];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        C jx = C(0), jy = C(0), jz = C(0);
+#pragma unroll
+        for (int i = 1; i < 19; i += 2) {
+            const C d = fc[s][i] - fc[s][i + 1];
+            if (cx_(i)) jx += C(cx_(i)) * d;
+            if (cy_(i)) jy += C(cy_(i)) * d;
+            if (cz_(i)) jz += C(cz_(i)) * d;
+        }
+        j[s][0] = jx; j[s][1] = jy; j[s][2] = jz;
+    }
+    // Shan-Chen force (Eq. 7): F^s = -G rho_s sum_i w_i rho_s'(x + c_i) c_i,
+    // with the neighbour pair x + c_i, x - c_i differenced first
+    C acc[2][3] = {{C(0), C(0), C(0)}, {C(0), C(0), C(0)}};
+#pragma unroll
+    for (int i = 1; i < 19; i += 2) {
+        const C da = wgt<C>(i) * (nb(0, cx_(i), cy_(i), cz_(i)) - nb(0, -cx_(i), -cy_(i), -cz_(i)));
+        const C db = wgt<C>(i) * (nb(1, cx_(i), cy_(i), cz_(i)) - nb(1, -cx_(i), -cy_(i), -cz_(i)));
+        if (cx_(i)) { acc[0][0] += C(cx_(i)) * da; acc[1][0] += C(cx_(i)) * db; }
+        if (cy_(i)) { acc[0][1] += C(cy_(i)) * da; acc[1][1] += C(cy_(i)) * db; }
+        if (cz_(i)) { acc[0][2] += C(cz_(i)) * da; acc[1][2] += C(cz_(i)) * db; }
+    }
+    // common velocity u' and per-component shifted velocity
+    const C den = rho[0] * m.inv_tau[0] + rho[1] * m.inv_tau[1];
+    C up[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) up[a] = (j[0][a] * m.inv_tau[0] + j[1][a] * m.inv_tau[1]) / den;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        // tau_s F^s / rho_s = -G tau_s * (the other component's sum)
+        const C sh = -m.G * m.tau[s];
+        const C ux = up[0] + sh * acc[1 - s][0];
+        const C uy = up[1] + sh * acc[1 - s][1];
+        const C uz = up[2] + sh * acc[1 - s][2];
+        const C u2x = C(1.5) * (ux * ux + uy * uy + uz * uz);
+        // post-collision populations: BGK, or MRT relaxation of the moments
+        C out[19];
+        if constexpr (MRT) {
+            C dv[19];
+#pragma unroll
+            for (int i = 0; i < 19; ++i) dv[i] = fc[s][i] - feq<C>(i, rho[s], ux, uy, uz, u2x);
+            if constexpr (Full) mrt_relax_full<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
+            else mrt_relax<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
+        } else {
+#pragma unroll
+            for (int i = 1; i < 19; ++i) {
+                const C f = fc[s][i];
+                out[i] = f - (f - feq<C>(i, rho[s], ux, uy, uz, u2x)) * m.inv_tau[s];
+            }
+        }
+        emit(s, out);
+    }
+}
+
 // One CTA's share of the stream-collide step: the TX x TY tile at (x0, y0)
 // of the x-y plane, marched over planes [zc0, zc1).  blockDim.x may exceed
 // TX * TY (the extra threads only help with the halo); every thread must
@@ -165,71 +255,13 @@ __device__ __forceinline__ void tile_march(const S* __restrict__ src, S* __restr
             P.pull(x, y, z, fc);
             const int s0 = (z - 1) & 3, s1 = z & 3, s2 = (z + 1) & 3;
             const C rho[2] = {R(s1, 0, tx, ty), R(s1, 1, tx, ty)};
-            // momentum of each component (Eq. 6), opposite pairs first
-            C j[2][3];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                C jx = C(0), jy = C(0), jz = C(0);
-#pragma unroll
-                for (int i = 1; i < 19; i += 2) {
-                    const C d = fc[s][i] - fc[s][i + 1];
-                    if (cx_(i)) jx += C(cx_(i)) * d;
-                    if (cy_(i)) jy += C(cy_(i)) * d;
-                    if (cz_(i)) jz += C(cz_(i)) * d;
-                }
-                j[s][0] = jx; j[s][1] = jy; j[s][2] = jz;
-            }
-            // Shan-Chen force (Eq. 7): F^s = -G rho_s sum_i w_i rho_s'(x + c_i) c_i,
-            // with the neighbour pair x + c_i, x - c_i differenced first
-            C acc[2][3] = {{C(0), C(0), C(0)}, {C(0), C(0), C(0)}};
-#pragma unroll
-            for (int i = 1; i < 19; i += 2) {
-                const int sp = cz_(i) == 0 ? s1 : (cz_(i) > 0 ? s2 : s0);
-                const int sm = cz_(i) == 0 ? s1 : (cz_(i) > 0 ? s0 : s2);
-                const C da = wgt<C>(i) * (R(sp, 0, tx + cx_(i), ty + cy_(i)) - R(sm, 0, tx - cx_(i), ty - cy_(i)));
-                const C db = wgt<C>(i) * (R(sp, 1, tx + cx_(i), ty + cy_(i)) - R(sm, 1, tx - cx_(i), ty - cy_(i)));
-                if (cx_(i)) { acc[0][0] += C(cx_(i)) * da; acc[1][0] += C(cx_(i)) * db; }
-                if (cy_(i)) { acc[0][1] += C(cy_(i)) * da; acc[1][1] += C(cy_(i)) * db; }
-                if (cz_(i)) { acc[0][2] += C(cz_(i)) * da; acc[1][2] += C(cz_(i)) * db; }
-            }
-            // common velocity u' and per-component shifted velocity
-            const C den = rho[0] * m.inv_tau[0] + rho[1] * m.inv_tau[1];
-            C up[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) up[a] = (j[0][a] * m.inv_tau[0] + j[1][a] * m.inv_tau[1]) / den;
             if (!(isfinite(rho[0]) && isfinite(rho[1]))) atomicOr(d_err, 1);
-            {
-                const C phi = (rho[0] - rho[1]) / (rho[0] + rho[1]);
-                const C wphi = phi > C(0) ? phi : C(0);
-                cm[0] += wphi;
-                cm[1] += wphi * pxc;
-                cm[2] += wphi * pyc;
-                cm[3] += wphi * (C(z) - C(0.5) * C(L.Lz - 1));
-            }
+            droplet_sums<C>(rho, pxc, pyc, C(z) - C(0.5) * C(L.Lz - 1), cm);
+            auto nb = [&](int s, int dx, int dy, int dz) -> C {
+                return R(dz == 0 ? s1 : (dz > 0 ? s2 : s0), s, tx + dx, ty + dy);
+            };
             C rest[2];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                // tau_s F^s / rho_s = -G tau_s * (the other component's sum)
-                const C sh = -m.G * m.tau[s];
-                const C ux = up[0] + sh * acc[1 - s][0];
-                const C uy = up[1] + sh * acc[1 - s][1];
-                const C uz = up[2] + sh * acc[1 - s][2];
-                const C u2x = C(1.5) * (ux * ux + uy * uy + uz * uz);
-                // post-collision populations: BGK, or MRT relaxation of the moments
-                C out[19];
-                if constexpr (MRT) {
-                    C dv[19];
-#pragma unroll
-                    for (int i = 0; i < 19; ++i) dv[i] = fc[s][i] - feq<C>(i, rho[s], ux, uy, uz, u2x);
-                    if constexpr (is_dev_t<S>::value) mrt_relax_full<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
-                    else mrt_relax<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
-                } else {
-#pragma unroll
-                    for (int i = 1; i < 19; ++i) {
-                        const C f = fc[s][i];
-                        out[i] = f - (f - feq<C>(i, rho[s], ux, uy, uz, u2x)) * m.inv_tau[s];
-                    }
-                }
+            tile_collide<C, MRT, is_dev_t<S>::value>(fc, rho, m, nb, [&](int s, const C (&out)[19]) {
                 // moving populations; the rest population then closes the
                 // mass balance exactly (sum of outputs = rho), which keeps
                 // fp32 rounding from drifting the interface
@@ -252,7 +284,7 @@ __device__ __forceinline__ void tile_march(const S* __restrict__ src, S* __restr
                     }
                 }
                 rest[s] = rho[s] - others;
-            }
+            });
             if constexpr (is_dev_t<S>::value) {
                 reinterpret_cast<float4*>(dst)[L.dev_node(x, y, z)] =
                     make_float4((float)rho[0], (float)rho[1], (float)rest[0], (float)rest[1]);
