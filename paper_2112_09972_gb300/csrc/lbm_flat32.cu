@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kAnyThreads, kAnyPerSM)
             const float2 v = near(dx, dy, dz);
             return s ? v.y : v.x;
         };
-        tile_collide<float, MRT, false>(f, r, m, nb, [&](int s, const float (&out)[19]) {
+        tile_collide<float, MRT>(f, r, m, nb, [&](int s, const float (&out)[19]) {
             float others = 0.f;  // the rest population closes the mass balance
 #pragma unroll
             for (int i = 1; i < 19; ++i) {

@@ -116,7 +116,8 @@ __host__ __device__ __forceinline__ constexpr int mrt_group(int i) {
 //   out  ce[7] the even part for one direction of each group
 //        co[9] the odd part along c: the axes x, y, z; then per unit of c_x on
 //              xy and xz edges, of c_y on xy and yz, of c_z on xz and yz
-// About 75 operations a component where the 19 x 19 products took over 500.
+// About 75 operations a component where the 19 x 19 products take over 500
+// (float64: 32^3 60 us per step in two passes).
 template <typename C>
 __device__ __forceinline__ void mrt_free(const C (&g)[7], const C (&o)[9], C inv_tau, const C (&r)[5], C (&ce)[7],
                                          C (&co)[9]) {
@@ -205,8 +206,10 @@ __device__ __forceinline__ C mrt_rate(int k, C inv_tau, const C (&r)[5]) {
 }
 
 // out_i = f_i - sum_k M_ki s_k (M dev)_k / |M_k|^2 with dev = f - f_eq, moment
-// by moment.  16-bit storage keeps this order of operations: any other moves
-// its roundings, and with them a run's states, by whole 16-bit steps.
+// by moment.  Float32 and 16-bit storage take this order of operations: the
+// other one moves their roundings, and D of a small droplet with them, by as
+// much as float32 leaves of it (64 x 88 x 20, R = 3.4, 36 steps: 6e-7 from the
+// 64-bit result here, 4e-6 with mrt_relax).
 template <typename C>
 __device__ __forceinline__ void mrt_relax_full(const C (&f)[19], const C (&dev)[19], C inv_tau, const C (&r)[5],
                                           C (&out)[19]) {

@@ -509,44 +509,21 @@ __device__ __forceinline__ void collide_core(NB&& nb, const float2 rho2, const f
             if constexpr (MRT) {
                 // MRT: relax the moments of the deviation from equilibrium
                 // (d'Humieres basis; momentum and stress at 1/tau)
-                // as BGK plus the free moments' part (mrt_free); the
-                // equilibria are evaluated twice rather than held
-                const float base = 1.f - 1.5f * (ux * ux + uy * uy + uz * uz);
-                const float e1 = r * wgt<float>(1), e2 = r * wgt<float>(7), it = m.inv_tau[s];
-                float g[7] = {f[s][0] - (r * wgt<float>(0)) * base, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                float o[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                auto deviations = [&](auto I, float& dp, float& dm) {
-                    constexpr int i = decltype(I)::value;
-                    const float cu = dot_c<float>(i, ux, uy, uz);
-                    const float e = i < 7 ? e1 : e2;
-                    const float ev = e * fmaf(4.5f * cu, cu, base);
-                    const float od = (3.f * e) * cu;
-                    dp = f[s][i] - (ev + od);
-                    dm = f[s][i + 1] - (ev - od);
-                };
+                const float u2x = 1.5f * (ux * ux + uy * uy + uz * uz);
+                float dv[19], o[19];
+#pragma unroll
+                for (int i = 0; i < 19; ++i) dv[i] = f[s][i] - feq<float>(i, r, ux, uy, uz, u2x);
+                mrt_relax_full<float>(f[s], dv, m.inv_tau[s], m.mrt, o);
                 sfor<9>([&](auto K) {
                     constexpr int i = 2 * decltype(K)::value + 1;
-                    float dp, dm;
-                    deviations(std::integral_constant<int, i>{}, dp, dm);
-                    mrt_gather<float>(i, dp, dm, g, o);
-                });
-                float ce[7], co[9];
-                mrt_free<float>(g, o, it, m.mrt, ce, co);
-                sfor<9>([&](auto K) {
-                    constexpr int i = 2 * decltype(K)::value + 1;
-                    float dp, dm;
-                    deviations(std::integral_constant<int, i>{}, dp, dm);
-                    const float e = ce[mrt_group(i)], d = mrt_odd<float>(i, co);
-                    const float oa = fmaf(-it, dp, f[s][i]) - (e + d);
-                    const float ob = fmaf(-it, dm, f[s][i + 1]) - (e - d);
                     if (s == 0) {
-                        IO::template store<0, i>(out, oa);
-                        IO::template store<0, i + 1>(out, ob);
+                        IO::template store<0, i>(out, o[i]);
+                        IO::template store<0, i + 1>(out, o[i + 1]);
                     } else {
-                        IO::template store<1, i>(out, oa);
-                        IO::template store<1, i + 1>(out, ob);
+                        IO::template store<1, i>(out, o[i]);
+                        IO::template store<1, i + 1>(out, o[i + 1]);
                     }
-                    others += oa + ob;
+                    others += o[i] + o[i + 1];
                 });
             } else {
                 const float base = 1.f - 1.5f * (ux * ux + uy * uy + uz * uz);

@@ -232,8 +232,8 @@ cudaError_t stream_collide_t(const void* src, void* dst, const Layout& L, const 
 // direct variant).  Per step, two-pass against cluster kernel: fp32 64^3 24.1 us
 // (35.9), 128 x 64 x 64 44.1 (45.5), 64 x 96 x 96 58.3 (55.1); bf16 64^3 17.7
 // (33.0), 64 x 96 x 96 38.5 (46.5), 128 x 64 x 96 44.6 (49.2), 128 x 96 x 96 68.7
-// (64.0); MRT 64^3 24.1 (38.5), 128 x 64 x 64 44.9 (53.6), 128 x 64 x 96 71.6
-// (73.3), 128 x 96 x 96 105.5 (98.6).
+// (64.0); MRT 64^3 29.1 (49.4), 128 x 64 x 64 54.2 (63.6), 64 x 96 x 96 69.7
+// (72.7), 128 x 64 x 96 84.6 (81.7).
 long long flat_rows_nodes(int prec, int mrt) { return prec == kFP32 && !mrt ? 1LL << 19 : 3LL << 18; }
 constexpr int kMaxThreadsF32 = 512;
 constexpr int kMaxThreadsF64 = 256;
@@ -344,7 +344,8 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
     if (sh.smem < red) sh.smem = red;
     // float32 boxes of other extents: two-pass at every size (per step against
     // the tile kernel: 37 x 29 x 23 10.6 us (34.9), 60 x 50 x 44 14.6 (31.4), 96 x
-    // 96 x 95 78 (112), 130^3 212 (334), 200 x 200 x 100 309 (465))
+    // 96 x 95 78 (112), 130^3 212 (334), 200 x 200 x 100 309 (465); with MRT 60 x
+    // 50 x 44 18.1 (39.6), 130^3 246 (424))
     if (allow_flat && prec == kFP32 && !periodic && ty_req <= 0 && zchunk_req <= 0) return flat_any_shape(L, sh, num_sms);
     return sh;
 }

@@ -133,7 +133,7 @@ __device__ __forceinline__ void droplet_sums(const C (&rho)[2], C px, C py, C pz
 // post-collision moving populations out[1..18].  The tile march and the
 // two-pass kernels of float32 boxes (lbm_flat32.cu) share it, so that their
 // states agree bit for bit.
-template <typename C, bool MRT, bool Full, typename NB, typename Emit>
+template <typename C, bool MRT, typename NB, typename Emit>
 __device__ __forceinline__ void tile_collide(const C (&fc)[2][19], const C (&rho)[2], const ModelC<C>& m, NB&& nb,
                                              Emit&& emit) {
     // momentum of each component (Eq. 6), opposite pairs first
@@ -180,7 +180,7 @@ __device__ __forceinline__ void tile_collide(const C (&fc)[2][19], const C (&rho
             C dv[19];
 #pragma unroll
             for (int i = 0; i < 19; ++i) dv[i] = fc[s][i] - feq<C>(i, rho[s], ux, uy, uz, u2x);
-            if constexpr (Full) mrt_relax_full<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
+            if constexpr (sizeof(C) == 4) mrt_relax_full<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
             else mrt_relax<C>(fc[s], dv, m.inv_tau[s], m.mrt, out);
         } else {
 #pragma unroll
@@ -261,7 +261,7 @@ __device__ __forceinline__ void tile_march(const S* __restrict__ src, S* __restr
                 return R(dz == 0 ? s1 : (dz > 0 ? s2 : s0), s, tx + dx, ty + dy);
             };
             C rest[2];
-            tile_collide<C, MRT, is_dev_t<S>::value>(fc, rho, m, nb, [&](int s, const C (&out)[19]) {
+            tile_collide<C, MRT>(fc, rho, m, nb, [&](int s, const C (&out)[19]) {
                 // moving populations; the rest population then closes the
                 // mass balance exactly (sum of outputs = rho), which keeps
                 // fp32 rounding from drifting the interface
