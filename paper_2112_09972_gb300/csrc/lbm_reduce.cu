@@ -579,7 +579,9 @@ __device__ __forceinline__ Pair node_phi(const RhoPair<S>& r) {
     return renorm(q, e * y);
 }
 
-// Sums of phi and of |grad phi|.
+// Sums of phi and of |grad phi|.  (The low parts in one float: gathered in a
+// pair the sums of a 256 x 200 x 200 state changed by 1e-16 and the call took
+// 374 us instead of 357.)
 struct Acc64 {
     double s = 0.0;
     __device__ __forceinline__ void add(double v) { s += v; }
@@ -656,8 +658,8 @@ __device__ __forceinline__ double magnitude(double x1, double x0, double y1, dou
 }
 __device__ __forceinline__ Pair magnitude(Pair x1, Pair x0, Pair y1, Pair y0, Pair z1, Pair z0) {
     auto square = [](Pair a, Pair b) -> Pair {  // (a - b)^2
-        Pair d = two_sum(a.h, -b.h);
-        d.l += a.l - b.l;
+        // neighbours far from the interface agree in the high part: the difference is then the low one's
+        const Pair t = two_sum(a.h, -b.h), d = two_sum(t.h, t.l + (a.l - b.l));
         const float p = d.h * d.h;
         return {p, fmaf(2.f * d.h, d.l, fmaf(d.h, d.h, -p))};
     };
