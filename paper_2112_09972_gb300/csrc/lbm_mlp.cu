@@ -885,7 +885,7 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
                 __syncwarp();
                 if (lane == 0) {
                     if (l == 0) tc_arrive(acc0_read);
-                    tc_arrive(epi_bar);
+                    if (l + 1 < L) tc_arrive(epi_bar);
                 }
                 hand_over(e + 1u, next);
             }
@@ -997,11 +997,13 @@ __global__ void __launch_bounds__(kFwThreads, 1) k_mlp_forward(const __grid_cons
             unsigned epi = 0;
             for (int j = 0; ok && j < mine; ++j)
                 for (int l = 1; ok && l < L; ++l) {
-                    // the epilogue of the layer before (and, at l = 1, of the
-                    // tile before): every phase is waited for in turn
-                    if (!loader)
-                        for (const unsigned due = (unsigned)(j * L + l); ok && epi < due; ++epi)
-                            ok = tc_wait(epi_bar, epi & 1u, stop);
+                    // The epilogue of the layer before (at l = 1 the first
+                    // layer's, by warps that have read this accumulator of the
+                    // tile before by then).  The last layer's does not arrive
+                    // here: each phase then needs products that this thread
+                    // issues after it has seen the phase before, so no two of
+                    // them can complete between its looks at one parity bit.
+                    if (!loader && (ok = tc_wait(epi_bar, epi & 1u, stop))) ++epi;
                     for (int kt = 0; ok && kt < a.width[l - 1] / TC_K; ++kt)
                         chunk(l, kt, base + kFwH0 + (unsigned)kt * kFwChunk);
                     if (ok && !loader) tc_commit(accfull(1));
