@@ -284,24 +284,12 @@ int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[
     c->prec = o.precision;
     c->elem = elem_bytes_of(c->prec);
     c->L = make_layout(box[0], box[1], box[2], c->prec);
-    c->shape = choose_shape(c->L, c->prec, o.bc == LBM_BC_PERIODIC_TEST, c->model.mrt, o.tile_y, o.z_chunk,
-                            o.row_variant, c->num_sms, true);
-    if (c->shape.flat && cudaMalloc(&c->rho, rho_bytes(c)) != cudaSuccess) {
-        cudaGetLastError();  // no room for the density array: the tile kernel needs none
-        c->rho = nullptr;
-        c->shape = choose_shape(c->L, c->prec, o.bc == LBM_BC_PERIODIC_TEST, c->model.mrt, o.tile_y, o.z_chunk,
-                                o.row_variant, c->num_sms, false);
-    }
     c->cur = 0;
     c->stream = (cudaStream_t)o.cuda_stream;
     c->own_stream = false;
     int st = LBM_OK;
     if (!c->stream) {
-        if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) {
-            cudaFree(c->rho);
-            delete c;
-            return LBM_ECUDA;
-        }
+        if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) { delete c; return LBM_ECUDA; }
         c->own_stream = true;
     }
     c->red_blocks = std::max(moments_blocks(c->L, c->num_sms), 1);
@@ -310,17 +298,31 @@ int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[
     if (e == cudaSuccess) e = cudaMalloc(&c->f[1], bytes);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&c->d_partials, sizeof(double) * 10 * c->red_blocks);
-    c->centre.n = (int)(c->shape.grid.x * c->shape.grid.y * c->shape.grid.z);
-    // partials, the 8 sums, the counter (16 bytes), the float32 frame origin (16 bytes)
-    const size_t centre_bytes = sizeof(double) * (4 * (size_t)c->centre.n + 8) + 32;
-    if (e == cudaSuccess) e = cudaMalloc(&c->centre.p, centre_bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_result, sizeof(double) * 32);
+    // last what depends on the launch shape: a two-pass shape only where its
+    // density array fits beside everything else (the other kernels need none)
+    size_t centre_bytes = 0;
+    for (bool flat = true; e == cudaSuccess; flat = false) {
+        c->shape = choose_shape(c->L, c->prec, o.bc == LBM_BC_PERIODIC_TEST, c->model.mrt, o.tile_y, o.z_chunk,
+                                o.row_variant, c->num_sms, flat);
+        c->centre.n = (int)(c->shape.grid.x * c->shape.grid.y * c->shape.grid.z);
+        // partials, the 8 sums, the counter (16 bytes), the float32 frame origin (16 bytes)
+        centre_bytes = sizeof(double) * (4 * (size_t)c->centre.n + 8) + 32;
+        e = cudaMalloc(&c->centre.p, centre_bytes);
+        if (e == cudaSuccess && c->shape.flat) e = cudaMalloc(&c->rho, rho_bytes(c));
+        if (e != cudaErrorMemoryAllocation || !c->shape.flat) break;
+        cudaGetLastError();
+        cudaFree(c->centre.p);
+        c->centre.p = nullptr;
+        c->rho = nullptr;
+        e = cudaSuccess;
+    }
     if (e == cudaSuccess) {
         c->centre.sum = c->centre.p + 4 * c->centre.n;
         c->centre.counter = (unsigned*)(c->centre.sum + 8);
         c->centre.frame = (float*)(c->centre.sum + 10);
         e = cudaMemsetAsync(c->centre.p, 0, centre_bytes, c->stream);
     }
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_result, sizeof(double) * 32);
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_result, sizeof(double) * 32);
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_err, sizeof(int));
     // Zero both buffers once: ghost entries that no direction reads stay defined.
