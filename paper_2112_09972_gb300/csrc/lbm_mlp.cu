@@ -1298,7 +1298,8 @@ struct lbm_mlp {
     float* yhat;                 // [max_batch, dp_L]
     std::vector<bf16*> G;        // G[l] gradient with respect to z_l, [max_batch, dp_l]
     // operands of the weight gradients, the batch index contiguous: GT[q] of
-    // the gradients (two layers in flight), HT[l] of the activations (NULL
+    // the gradients (two layers in flight; one buffer twice where there was
+    // no room for the second), HT[l] of the activations (NULL
     // where there was no room: they are then transposed into T2 in turn)
     bf16* GT[2];
     std::vector<bf16*> HT;
@@ -1312,7 +1313,8 @@ struct lbm_mlp {
     int sms;                     // multiprocessors of the device
     float* ws;                   // split-K partials, kMaxSplit x every weight matrix (ws_all) or the largest
     bool ws_all;
-    float* cs_parts;             // column-sum partials, kColSlices x the sum of the widths
+    float* cs_parts;             // column-sum partials, cs_slices x the sum of the widths
+    int cs_slices;
     LayerTable table;            // the update's view of the layers
     bool fused;                  // k_mlp_forward takes this network's shapes
     FwArgs fw;                   // its weights' tensor maps and constants (rows and pointers set per call)
@@ -1616,7 +1618,7 @@ cudaError_t backward(lbm_mlp* c, const float* t, int n) {
     cudaError_t e = launch(c, k_loss_grad, dim3(nb), dim3(kLossThreads), 0, (const float*)c->yhat, dLp, t, n, dL, dLp,
                            (const float*)c->y_mean, (const float*)c->y_scale, c->G[L], c->GT[L & 1], c->loss_parts,
                            c->loss_counter, (double)n * dL, c->loss);
-    const int S = (int)std::min<long long>(kColSlices, blocks_for(n, 256));
+    const int S = (int)std::min<long long>(c->cs_slices, blocks_for(n, 256));
     c->table.cs_n = S;
     int widest = 0;
     for (int l = L; l >= 1 && e == cudaSuccess; --l) {
@@ -1637,7 +1639,12 @@ cudaError_t backward(lbm_mlp* c, const float* t, int n) {
                                    nullptr, c->G[l - 1], din);
             a.Ct = c->GT[(l - 1) & 1];
             a.ldt = n;
-            e = launch_gemm_pair(c, a, 1, dw, q.S);
+            if (c->GT[0] != c->GT[1]) {
+                e = launch_gemm_pair(c, a, 1, dw, q.S);
+            } else {  // a overwrites what dw reads
+                e = launch_gemm(c, dw, q.S);
+                if (e == cudaSuccess) e = launch_gemm(c, a, 1);
+            }
         } else {  // beside the bias gradients
             ColSums cs;
             cs.tb = c->table;
@@ -1745,13 +1752,12 @@ int lbm_mlp_create(lbm_mlp** out, int32_t nlayers, const int32_t* sizes, int32_t
     }
     for (int l = 0; l < nlayers; ++l) alloc((void**)&c->H[l], sizeof(bf16) * (size_t)max_batch * c->d[l]);
     alloc((void**)&c->yhat, sizeof(float) * (size_t)max_batch * 32);
-    for (int q = 0; q < 2; ++q) alloc((void**)&c->GT[q], sizeof(bf16) * (size_t)max_batch * widest);
+    alloc((void**)&c->GT[0], sizeof(bf16) * (size_t)max_batch * widest);
     alloc((void**)&c->T2, sizeof(bf16) * (size_t)max_batch * widest);
     alloc((void**)&c->loss_parts, sizeof(double) * blocks_for((long long)max_batch * 32, kLossThreads));
     alloc((void**)&c->loss_counter, sizeof(unsigned));
     alloc((void**)&c->loss, sizeof(double));
     alloc((void**)&c->d_err, sizeof(int));
-    // the split-K partials of every layer up to 1 GB, else the largest layer's
     long long largest = 0, all = 0, cols = 0;
     c->table.layers = nlayers;
     c->table.nparam = off;
@@ -1760,7 +1766,7 @@ int lbm_mlp_create(lbm_mlp** out, int32_t nlayers, const int32_t* sizes, int32_t
         q.offW = c->offW[l];
         q.count = (long long)c->dp[l] * c->d[l - 1];
         q.ws = kMaxSplit * all;
-        q.cs = kColSlices * cols;
+        q.cs = cols;
         q.S = 1;
         q.dout = c->dp[l];
         q.din = c->d[l - 1];
@@ -1771,16 +1777,42 @@ int lbm_mlp_create(lbm_mlp** out, int32_t nlayers, const int32_t* sizes, int32_t
         all += q.count;
         cols += c->dp[l];
     }
-    c->ws_all = all <= (1LL << 30) / (long long)(sizeof(float) * kMaxSplit);
-    if (!c->ws_all)
-        for (int l = 0; l < nlayers; ++l) c->table.l[l].ws = 0;
-    alloc((void**)&c->ws, sizeof(float) * kMaxSplit * (c->ws_all ? all : largest));
-    alloc((void**)&c->cs_parts, sizeof(float) * kColSlices * cols);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
     alloc((void**)&c->x_mean, sizeof(float) * c->d[0]);
     alloc((void**)&c->x_scale, sizeof(float) * c->d[0]);
     alloc((void**)&c->y_mean, sizeof(float) * 32);
     alloc((void**)&c->y_scale, sizeof(float) * 32);
+    // What the launches need: column-sum partials as large as one layer's in
+    // kColSlices slices, split-K partials of the largest layer, which the layers take in turn
+    c->cs_slices = kColSlices / nlayers;
+    c->ws_all = false;
+    alloc((void**)&c->cs_parts, sizeof(float) * c->cs_slices * cols);
+    alloc((void**)&c->ws, sizeof(float) * kMaxSplit * largest);
+    // What makes them fewer, where there is room beside all that: column-sum
+    // partials of all slices, split-K partials of every layer up to 1 GB, and
+    // a second transposed gradient, so that a layer's two products run together
+    auto larger = [&](float*& ptr, size_t bytes) -> bool {
+        void* q = nullptr;
+        if (e != cudaSuccess) return false;
+        if (cudaMalloc(&q, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        cudaFree(ptr);
+        ptr = (float*)q;
+        return true;
+    };
+    if (larger(c->cs_parts, sizeof(float) * kColSlices * cols)) c->cs_slices = kColSlices;
+    if (all <= (1LL << 30) / (long long)(sizeof(float) * kMaxSplit))
+        c->ws_all = larger(c->ws, sizeof(float) * kMaxSplit * all);
+    if (e == cudaSuccess && cudaMalloc((void**)&c->GT[1], sizeof(bf16) * (size_t)max_batch * widest) != cudaSuccess) {
+        cudaGetLastError();
+        c->GT[1] = c->GT[0];
+    }
+    for (int l = 0; l < nlayers; ++l) {
+        c->table.l[l].cs *= c->cs_slices;
+        if (!c->ws_all) c->table.l[l].ws = 0;
+    }
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_loss, sizeof(double));
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->p, init.data(), sizeof(float) * off, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) {
@@ -1812,7 +1844,7 @@ void lbm_mlp_destroy(lbm_mlp* c) {
     for (bf16* q : c->G) cudaFree(q);
     for (bf16* q : c->H) cudaFree(q);
     for (bf16* q : c->HT) cudaFree(q);
-    cudaFree(c->yhat); cudaFree(c->GT[0]); cudaFree(c->GT[1]); cudaFree(c->T2);
+    cudaFree(c->yhat); cudaFree(c->GT[0]); cudaFree(c->GT[1] != c->GT[0] ? c->GT[1] : nullptr); cudaFree(c->T2);
     cudaFree(c->loss_parts); cudaFree(c->loss_counter); cudaFree(c->loss); cudaFree(c->d_err); cudaFree(c->ws); cudaFree(c->cs_parts);
     cudaFree(c->x_mean); cudaFree(c->x_scale); cudaFree(c->y_mean); cudaFree(c->y_scale);
     if (c->h_loss) cudaFreeHost(c->h_loss);

@@ -1,14 +1,14 @@
-"""A box that fits only without the memory that its faster kernels would take.
+"""Contexts that fit only without the memory that faster launches would take.
 
-A ballast leaves what the kernels need and a little more, less than the density array of the two-pass kernels.  The box is
-created all the same, on the kernel that does without.
+A ballast leaves what the kernels need and a little more, less than the density array of the two-pass kernels or the
+second gradient buffer of the surrogate.  Both contexts are created all the same, on the kernels that do without.
 """
 
 import numpy as np
 import pytest
 
 from paper_2112_09972_gb300 import workloads
-from paper_2112_09972_gb300.lbm import DropletLBM
+from paper_2112_09972_gb300.lbm import MLP, DropletLBM
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -58,3 +58,33 @@ def test_box_without_room_for_its_densities(built):
     assert np.max(np.abs(g.populations() - h.populations())) <= 1e-13
     g.close()
     h.close()
+
+
+def test_surrogate_without_room_for_grouped_launches(built):
+    sizes, batch, n = (576, 256, 256, 256, 6), 1 << 20, 512
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    x, t = torch.randn((n, 576), device="cuda", generator=gen), torch.randn((n, 6), device="cuda", generator=gen)
+    torch.cuda.synchronize()
+
+    def train(net):
+        grads = net.gradients(x, t)[1]
+        for _ in range(3):
+            net.train_step(x, t, 1e-3)
+        out = grads, net.get_params()
+        net.close()
+        return out
+
+    ref = train(MLP(sizes, max_batch=batch, seed=3))
+    # bfloat16: hidden gradients and output gradients, input and hidden activations, one transposed gradient and one
+    # transposed activation of the widest layer; the outputs in float32; weights and partial sums below 100 MB.
+    # A second transposed gradient would take 1152 MB more, the transposed activations 2688 MB.
+    need = 2 * batch * (3 * 256 + 32 + 576 + 3 * 256 + 2 * 576) + 4 * batch * 32
+    held = _ballast(need + 500 * MB)
+    try:
+        net = MLP(sizes, max_batch=batch, seed=3)
+        got = train(net)
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    for a, b in zip(ref, got):
+        assert np.array_equal(a, b)
