@@ -13,16 +13,16 @@
 //
 // What bounds it.  This GPU's FP64 pipe issues one warp instruction per 16
 // cycles and SM, so a float64 node update is bound by its FP64 instructions,
-// not by memory: at 128^3 the 608 bytes of a node take 94 ns per 512 nodes of
-// copy bandwidth and 300 FP64 instructions five times that.  The marched tile
+// not by memory: the 608 bytes of 512 nodes take 46 ns at the measured copy
+// bandwidth, their 340 FP64 instructions a node 290 ns (128^3: 379 ns measured).  The marched tile
 // kernel sums every density about twice (the tile's halo, and the planes
 // before and after each z chunk) and evaluates each equilibrium on its own,
 // 560 instructions per node.  Here each density is summed once (the second
 // read of the populations costs bandwidth that is idle), opposite
 // directions share their equilibria, and the launch covers the chip for any
 // box: one node per thread instead of a z march per tile.  Measured per step
-// against the tile kernel: 32^3 32 us (178), 64^3 174 us (365), 128^3 1411 us
-// (3174), 37 x 29 x 23 27 us (160); float64 storage therefore takes these
+// against the tile kernel: 32^3 34 us (178), 64^3 191 us (365), 128^3 1551 us
+// (3174), 37 x 29 x 23 29 us (160); float64 storage therefore takes these
 // kernels at every size.
 #include <cuda_runtime.h>
 
@@ -161,6 +161,7 @@ __device__ __forceinline__ void flat_node(const double2* __restrict__ r, int sy,
         const double uy = fma(m.sh[s], acc[1 - s][1], up[1]);
         const double uz = fma(m.sh[s], acc[1 - s][2], up[2]);
         double* os = o + (long long)(19 * s) * pitch;
+        double others = 0.0;
         if constexpr (MRT) {
             const double u2x = 1.5 * (ux * ux + uy * uy + uz * uz);
             double dv[19], out[19];
@@ -168,7 +169,11 @@ __device__ __forceinline__ void flat_node(const double2* __restrict__ r, int sy,
             for (int i = 0; i < 19; ++i) dv[i] = f[s][i] - feq<double>(i, rs, ux, uy, uz, u2x);
             mrt_relax<double>(f[s], dv, m.inv_tau[s], m.mrt, out);
 #pragma unroll
-            for (int i = 0; i < 19; ++i) os[i * pitch] = out[i];
+            for (int i = 1; i < 19; i += 2) {
+                os[i * pitch] = out[i];
+                os[(i + 1) * pitch] = out[i + 1];
+                others += out[i] + out[i + 1];
+            }
         } else {
             // with v = 1.5 u and c = c_i . v, the even and odd parts of
             // f_eq / tau of a pair are e base + c (2 e c) and 2 e c
@@ -184,11 +189,16 @@ __device__ __forceinline__ void flat_node(const double2* __restrict__ r, int sy,
                 const double c = dot_c<double>(i, vx, vy, vz);
                 const double od = (i < 7 ? e2A : e2E) * c;
                 const double ev = fma(c, od, i < 7 ? ebA : ebE);
-                os[i * pitch] = fma(om, f[s][i], ev + od);
-                os[(i + 1) * pitch] = fma(om, f[s][i + 1], ev - od);
+                const double oa = fma(om, f[s][i], ev + od), ob = fma(om, f[s][i + 1], ev - od);
+                os[i * pitch] = oa;
+                os[(i + 1) * pitch] = ob;
+                others += oa + ob;
             }
-            os[0] = fma(om, f[s][0], ib * (1.0 / 3.0));
         }
+        // the rest population closes the mass balance exactly (sum of outputs
+        // = rho), as the tile kernel's does: the sum's 36 additions a node
+        // took 64^3 from 174 to 191 us per step
+        os[0] = rs - others;
     }
 }
 
