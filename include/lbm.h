@@ -266,8 +266,8 @@ int lbm_get_step(lbm_ctx* ctx, int64_t* step);
 
 /*
  * Checkpoint: lbm_save writes the parameters, the step counter, the gradient
- * table and the populations (float64; the raw device buffer for 16-bit
- * deviation storage) with a 64-bit FNV-1a checksum;
+ * table and the populations (float64; for 16-bit deviation storage the raw
+ * device layout, zeros outside the box) with a 64-bit FNV-1a checksum;
  * lbm_load restores them into a context created with the same box, precision
  * and boundary mode (LBM_EINVAL otherwise, LBM_EIO for a missing, short or
  * corrupt file).  A resumed run is bit-identical to an uninterrupted one.

@@ -325,7 +325,10 @@ int lbm_create(lbm_ctx** out, const int32_t box[3], double R, const double visc[
     }
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_result, sizeof(double) * 32);
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_err, sizeof(int));
-    // Zero both buffers once: ghost entries that no direction reads stay defined.
+    // Zero both buffers once: every entry is defined.  The observables use the
+    // buffer of the next step's state as scratch, so entries that no kernel
+    // writes -- row padding, ghosts that no direction reads -- can hold any
+    // bits later; nothing computes with them.
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[0], 0, bytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, bytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
@@ -609,6 +612,28 @@ int lbm_get_step(lbm_ctx* c, int64_t* step) {
     return LBM_OK;
 }
 
+// Zeros in the padding and ghost entries of a raw buffer of deviation storage
+// (the next step writes its ghosts anew): equal states give equal files,
+// whatever an observable or an earlier step left there.
+static void only_fluid(const Layout& L, uint16_t* raw) {
+    const long long head = L.x0, tail = L.pitch - L.x0 - L.Lx;
+    for (int z = 0; z < L.nz; ++z)
+        for (int y = 0; y < L.ny; ++y) {
+            uint16_t* row = raw + z * L.plane + y * L.row;
+            if (z == 0 || z == L.nz - 1 || y == 0 || y == L.ny - 1) {
+                memset(row, 0, sizeof(uint16_t) * (size_t)L.row);
+                continue;
+            }
+            // the row of 16-byte node blocks, then the 18 rows of 4-byte words
+            for (int i = 0; i < 19; ++i) {
+                const long long unit = i ? 2 : 8;  // 2-byte units per entry
+                uint16_t* p = row + (i ? (6 + 2 * i) * (long long)L.pitch : 0);
+                memset(p, 0, sizeof(uint16_t) * (size_t)(unit * head));
+                memset(p + unit * (head + L.Lx), 0, sizeof(uint16_t) * (size_t)(unit * tail));
+            }
+        }
+}
+
 int lbm_save(lbm_ctx* c, const char* path) {
     if (!c || !path) return LBM_EINVAL;
     const size_t E = ckpt_pop_words(c);
@@ -620,6 +645,7 @@ int lbm_save(lbm_ctx* c, const char* path) {
         LBM_TRY(cudaMemcpyAsync(pop.data(), c->f[c->cur], (size_t)c->L.total * c->elem, cudaMemcpyDeviceToHost,
                                 c->stream));
         if ((st = sync_and_check(c))) return st;
+        only_fluid(c->L, reinterpret_cast<uint16_t*>(pop.data()));
     } else if ((st = lbm_get_populations(c, pop.data()))) {
         return st;
     }
