@@ -742,16 +742,17 @@ int lbm_load(lbm_ctx* c, const char* path) {
     } else if ((st = lbm_set_populations(c, pop.data()))) {
         return st;
     }
-    // restore the saved frame origin partials when the launch shape matches
-    // (otherwise the ones just recomputed from the populations stay)
+    // the saved frame origin, whatever launch shape the file's partials are of
+    // (the one just recomputed from the populations differs by its rounding);
+    // the partials themselves when the shape matches
+    const double* sums = cparts.data() + 4 * (size_t)h.ncentre;
+    if (h.ncentre == c->centre.n)
+        LBM_TRY(cudaMemcpyAsync(c->centre.p, cparts.data(), sizeof(double) * 4 * (size_t)h.ncentre,
+                                cudaMemcpyHostToDevice, c->stream));
+    LBM_TRY(cudaMemcpyAsync(c->centre.sum, sums, sizeof(double) * 8, cudaMemcpyHostToDevice, c->stream));
     float fr[3];  // the frame origin's float32 copy, as the reduction writes it (alive until the sync below)
-    if (h.ncentre == c->centre.n) {
-        LBM_TRY(cudaMemcpyAsync(c->centre.p, cparts.data(), sizeof(double) * cparts.size(), cudaMemcpyHostToDevice,
-                                c->stream));
-        const size_t o = (size_t)4 * c->centre.n + 4;
-        for (int q = 0; q < 3; ++q) fr[q] = (float)cparts[o + q];
-        LBM_TRY(cudaMemcpyAsync(c->centre.frame, fr, sizeof(fr), cudaMemcpyHostToDevice, c->stream));
-    }
+    for (int q = 0; q < 3; ++q) fr[q] = (float)sums[4 + q];
+    LBM_TRY(cudaMemcpyAsync(c->centre.frame, fr, sizeof(fr), cudaMemcpyHostToDevice, c->stream));
     c->step = h.step;
     LBM_TRY(cudaStreamSynchronize(c->stream));
     return LBM_OK;
