@@ -1197,12 +1197,9 @@ cudaError_t ws_for(bool query, const void* src, void* dst, const Layout& L, cons
 template <int TX, typename S>
 cudaError_t rows_variant(int variant, bool query, const void* src, void* dst, const Layout& L, const Model& m,
                          int zchunk, CentreParts cp, int* d_err, cudaStream_t s, int* resident) {
-    if (m.mrt) {  // MRT: float32 storage, direct or staged
-        if constexpr (std::is_same<S, float>::value) {
-            if (variant == kRowStaged)
-                return rows_for<TX, S, true, true>(query, src, dst, L, m, zchunk, cp, d_err, s, resident);
+    if (m.mrt) {  // MRT: float32 storage, direct loads only
+        if constexpr (std::is_same<S, float>::value)
             return rows_for<TX, S, false, true>(query, src, dst, L, m, zchunk, cp, d_err, s, resident);
-        }
         return cudaErrorInvalidValue;
     }
     if (variant == kRowWs) return ws_for<TX, kRowCluster, S>(query, src, dst, L, m, zchunk, cp, d_err, s, resident);
