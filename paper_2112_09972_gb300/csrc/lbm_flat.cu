@@ -37,6 +37,7 @@
 namespace lbmgb {
 namespace {
 
+constexpr int kFlatPerSM = 6;     // resident CTAs of the collision pass
 constexpr int kFlatThreads = 64;  // two warps: CTAs spread evenly over the SMs, whose FP64 pipes are the bound
 
 // The padded density array: node (x, y, z) at ((z + 1) ny + y + 1) nx + x + 1.
@@ -233,7 +234,7 @@ __device__ __forceinline__ void flat_unit(const double2* __restrict__ rho, const
 // array (against sums at the end of every colliding CTA, per step: 32^3 41.9 ->
 // 31.9 us, 37 x 29 x 23 36.1 -> 26.9, 64^3 195 -> 174, 128^3 1433 -> 1408).
 template <bool PER, bool MRT>
-__global__ void __launch_bounds__(kFlatThreads, 6)
+__global__ void __launch_bounds__(kFlatThreads, kFlatPerSM)
     k_flat_collide(const double* __restrict__ src, double* __restrict__ dst, Layout L, FlatModel m,
                    const double2* __restrict__ rho, RhoGeo g, int per_plane, int zchunk, int units, int centre0, int centres,
                    CentreParts cp, int* __restrict__ d_err) {
@@ -282,6 +283,10 @@ Shape flat_shape(const Layout& L, int num_sms) {
     if (zc < 1) zc = 1;
     while ((L.Lz + zc - 1) / zc > 65535) ++zc;
     sh.flat = kFlat64;
+    // last where the colliders all run at once, so that the sums land on the SMs with one collider less (first, they
+    // pushed a fifth one on some: 32^3 39.5 us against 31.5); first where they do not, so that no long sum is left over
+    // (last: 128^3 1905 us against 1411)
+    sh.centre_first = per_plane * ((L.Lz + zc - 1) / zc) > kFlatPerSM * (num_sms > 0 ? num_sms : 152);
     sh.tx = L.Lx;
     sh.ty = L.Lx >= kFlatThreads ? 1 : kFlatThreads / L.Lx;
     sh.zchunk = (int)zc;
@@ -316,10 +321,7 @@ cudaError_t launch_flat(const void* src, void* dst, void* rho, const Layout& L, 
     const int per_plane = (int)sh.grid.x, units = std::min(kFlatShares, per_plane) * (int)sh.grid.y;
     const int colliders = (int)(sh.grid.x * sh.grid.y);
     const int centres = std::min((units + kFlatThreads / 32 - 1) / (kFlatThreads / 32), 512);
-    // last where the colliders all run at once, so that the sums land on the SMs with one collider less (first, they
-    // pushed a fifth one on some: 32^3 39.5 us); first where they do not, so that no long sum is left over (last: 128^3
-    // 1905 us)
-    const int centre0 = colliders <= 6 * 152 ? colliders : 0;
+    const int centre0 = sh.centre_first ? 0 : colliders;
     cfg.gridDim = dim3(colliders + centres, 1, 1);
     return cudaLaunchKernelEx(&cfg, k, f, (double*)dst, L, fm, (const double2*)r, g, per_plane, sh.zchunk, units,
                               centre0, centres, cp, d_err);

@@ -103,7 +103,7 @@ struct Grad {
 // Launch shape of the stream-collide kernel.
 struct Shape {
     int rows;       // 1: the row-tiled cluster kernel (lbm_fast.cu), 0: the generic tile kernel
-    int centre_first;  // kFlatAny: the CTAs that sum the centre lead the grid
+    int centre_first;  // kFlat64, kFlatAny: the CTAs that sum the centre lead the grid
     int flat;       // kFlat64, kFlatRows or kFlatAny: two-pass kernels, which need a density array
     int tx, ty;     // tile of the x-y plane per CTA
     int zchunk;     // z planes marched per CTA
