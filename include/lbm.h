@@ -296,9 +296,12 @@ int lbm_launch_shape(lbm_ctx* ctx, int32_t* tile_y, int32_t* z_chunk, int32_t* c
  * k_stream_collide_rows; 3 loader and collider threads, k_stream_collide_ws),
  * or 4 a density and a collision pass without a march, which these take
  * unless opts->tile_y, z_chunk or (second) row_variant is set: float64 storage
- * (k_flat_rho, k_flat_collide); boxes of a row-tiled shape up to 524288 nodes (786432 in 16-bit storage or with MRT)
+ * (k_flat_rho, k_flat_collide); boxes of a row-tiled shape up to 524288 nodes
+ * (float32; 393216 at 32-wide rows), 786432 (16-bit storage, and MRT at 32- and
+ * 256-wide rows) or 589824 (MRT at 64- and 128-wide rows)
  * (k_row_rho, k_row_collide; the cluster kernel's states bit for bit); float32
- * boxes of other shapes with the ghost boundary (k_any_rho, k_any_collide).
+ * boxes of other shapes with the ghost boundary (k_any_rho, k_any_collide; the
+ * tile kernel's states bit for bit).
  * LBM_EINVAL for a NULL context or pointer. */
 int lbm_launch_variant(lbm_ctx* ctx, int32_t* variant);
 

@@ -229,12 +229,19 @@ cudaError_t stream_collide_t(const void* src, void* dst, const Layout& L, const 
 // Largest box of a row-tiled width on the two-pass kernels, whose second read
 // of the populations has to come from L2, half as much of it in 16-bit
 // storage; and the cluster kernel that MRT takes is the slower one (its
-// direct variant).  Per step, two-pass against cluster kernel: fp32 64^3 24.1 us
-// (35.9), 128 x 64 x 64 44.1 (45.5), 64 x 96 x 96 58.3 (55.1); bf16 64^3 17.7
-// (33.0), 64 x 96 x 96 38.5 (46.5), 128 x 64 x 96 44.6 (49.2), 128 x 96 x 96 68.7
-// (64.0); MRT 64^3 29.1 (49.4), 128 x 64 x 64 54.2 (63.6), 64 x 96 x 96 69.7
-// (72.7), 128 x 64 x 96 84.6 (81.7).
-long long flat_rows_nodes(int prec, int mrt) { return prec == kFP32 && !mrt ? 1LL << 19 : 3LL << 18; }
+// direct variant).  Per step, two-pass against cluster kernel, by width:
+//   fp32  32 x 128 x 96 44.5 us (47.2), 32 x 128 x 128 61.7 (57.1); 64^3 23.7
+//         (36.4), 64 x 96 x 96 58.3 (55.1); 128 x 64 x 64 43.9 (45.1); 256 x 32 x
+//         64 41.8 (44.8)
+//   bf16  32 x 192 x 128 63.5 (69.9), 64 x 128 x 96 51.1 (57.0), 128 x 64 x 96
+//         44.3 (48.9), 128 x 96 x 96 68.7 (64.0), 256 x 32 x 96 44.6 (46.7)
+//   MRT   32 x 192 x 128 104 (132), 256 x 32 x 96 83.9 (93.8); 64 x 96 x 96 69.7
+//         (72.7), 64 x 128 x 96 93.1 (92.6), 128 x 64 x 96 84.6 (81.7)
+long long flat_rows_nodes(const Layout& L, int prec, int mrt) {
+    if (prec == kFP32 && !mrt) return L.Lx == 32 ? 3LL << 17 : 1LL << 19;
+    if (mrt && (L.Lx == 64 || L.Lx == 128)) return 9LL << 16;
+    return 3LL << 18;
+}
 constexpr int kMaxThreadsF32 = 512;
 constexpr int kMaxThreadsF64 = 256;
 
@@ -312,7 +319,7 @@ Shape choose_shape(const Layout& L, int prec, int periodic, int mrt, int ty_req,
             sh.grid = dim3(1, L.Ly, (L.Lz + sh.zchunk - 1) / sh.zchunk);
             sh.threads = L.Lx;
             sh.smem = 0;
-            if (allow_flat && variant_req == 0 && zchunk_req <= 0 && (long long)L.Lx * L.Ly * L.Lz <= flat_rows_nodes(prec, mrt))
+            if (allow_flat && variant_req == 0 && zchunk_req <= 0 && (long long)L.Lx * L.Ly * L.Lz <= flat_rows_nodes(L, prec, mrt))
                 return flat_rows_shape(sh);
             return sh;
         }
