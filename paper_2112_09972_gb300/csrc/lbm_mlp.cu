@@ -1590,9 +1590,14 @@ void fused_setup(lbm_mlp* c) {
 
 // The leading rows of a forward pass that k_mlp_forward takes: those of the
 // chunks of max_batch rows whose products would all run on k_gemm_tc (whole
-// 128-row tiles), so that every row keeps its arithmetic.
-int64_t fused_rows(const lbm_mlp* c, const float* x, int64_t n) {
+// 128-row tiles), so that every row keeps its arithmetic.  None where y lies
+// in x: the chunks take such a call one after the other, each reading its
+// inputs before it writes its outputs, but the tiles of k_mlp_forward run in
+// no order.
+int64_t fused_rows(const lbm_mlp* c, const float* x, const float* y, int64_t n) {
     if (!c->fused || c->tensor_path != 0 || !aligned16(x) || c->max_batch % TC_M) return 0;
+    const uintptr_t a = (uintptr_t)x, b = (uintptr_t)y;
+    if (a < b + sizeof(float) * (uintptr_t)n * c->d[c->L] && b < a + sizeof(float) * (uintptr_t)n * c->d[0]) return 0;
     const int64_t tail = n % c->max_batch;
     return tail % TC_M ? n - tail : n;
 }
@@ -1927,7 +1932,7 @@ int lbm_mlp_forward(lbm_mlp* c, const float* x, float* y, int64_t n) {
     if (!c || n < 0 || (n > 0 && (!x || !y))) return LBM_EINVAL;
     cudaSetDevice(c->device);
     const int d0 = c->d[0], dL = c->d[c->L];
-    const int64_t rows = fused_rows(c, x, n);
+    const int64_t rows = fused_rows(c, x, y, n);
     MLP_TRY(fused_forward(c, x, y, rows));
     for (int64_t s = rows; s < n; s += c->max_batch) {
         const int k = (int)std::min<int64_t>(c->max_batch, n - s);
