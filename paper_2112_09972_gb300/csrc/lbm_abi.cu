@@ -536,7 +536,8 @@ int lbm_components(lbm_ctx* c, double threshold, int64_t min_nodes, int32_t* cou
                       c->stream));
     LBM_TRY(cudaMemcpyAsync(h, flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     LBM_TRY(cudaMemcpyAsync(h + 1, out, sizeof(long long) * kFirst, cudaMemcpyDeviceToHost, c->stream));
-    if ((st = sync_and_check(c))) return st;
+    st = sync_and_check(c);  // a latched condition is returned beside the result
+    if (st == LBM_ECUDA || st == LBM_ENOMEM) return st;
     int h_flags[2];
     memcpy(h_flags, h, sizeof(h_flags));
     if (h_flags[0]) return LBM_ETIMEOUT;
@@ -556,7 +557,7 @@ int lbm_components(lbm_ctx* c, double threshold, int64_t min_nodes, int32_t* cou
     std::sort(kept.begin(), kept.end(), [](long long a, long long b) { return a > b; });
     *count = (int32_t)kept.size();
     for (int32_t k = 0; k < max_sizes; ++k) sizes[k] = k < (int32_t)kept.size() ? kept[k] : 0;
-    return LBM_OK;
+    return st;
 }
 
 int lbm_surface_deformation(lbm_ctx* c, double* D_lbm, double* area, double* volume) {
