@@ -158,10 +158,45 @@ __device__ __forceinline__ Sym<C> axpy(const Sym<C>& m, C h, const Sym<C>& k) {
     return r;
 }
 
+// M between substeps: float32 keeps what the diagonal's sums round off.  The
+// diagonal lies near one, where a substep's rounding is 6e-8, and D of a nearly
+// spherical droplet is a small difference of its entries: hundreds of substeps
+// left 1e-6 of D, and as much by chance in one form of the arithmetic as
+// another.  (The other entries are as small as D, and so are their roundings.)
+template <typename C>
+struct State {
+    Sym<C> m;
+    C lo[3];
+    // m += h k, with k as rhs leaves it
+    __device__ __forceinline__ void add(C h, const Sym<C>& k) {
+        if constexpr (sizeof(C) == 4) {
+            const Sym<C> p = axpy(m, h, k);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int e = a == 0 ? 0 : 2 + a + (a == 2);  // xx, yy, zz
+                const C inc = fma(h, k.v[e], lo[a]), s = m.v[e] + inc;
+                lo[a] = inc - (s - m.v[e]);  // exact while |inc| <= |m|
+                m.v[e] = s;
+            }
+            m.v[1] = p.v[1], m.v[2] = p.v[2], m.v[4] = p.v[4];
+        } else {
+            m = axpy(m, h, k);
+        }
+    }
+    __device__ __forceinline__ void entries(double (&out)[6]) const {
+#pragma unroll
+        for (int e = 0; e < 6; ++e) out[e] = (double)m.v[e];
+        if constexpr (sizeof(C) == 4)
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                if (isfinite(lo[a])) out[a == 0 ? 0 : 2 + a + (a == 2)] += (double)lo[a];  // (not so where m overflowed)
+    }
+};
+
 // The substeps of one time step from M and the flow Fs at its start; false
 // where a quotient's denominator was out of range.
 template <bool Safe, typename C>
-__device__ __forceinline__ bool time_step(Sym<C>& M, Flow<C>& Fs, const C (&v0)[9], const C (&d)[9], C ca, C f2_0, C k,
+__device__ __forceinline__ bool time_step(State<C>& M, Flow<C>& Fs, const C (&v0)[9], const C (&d)[9], C ca, C f2_0, C k,
                                           C h, int substeps) {
     bool ok = true;
     const C k3 = C(3) * k;
@@ -171,35 +206,43 @@ __device__ __forceinline__ bool time_step(Sym<C>& M, Flow<C>& Fs, const C (&v0)[
         // A at the middle and end of the substep (linear in t)
         const Flow<C> Fm = flow_at<Safe, C>(v0, d, fma(q, h, C(0.5) * h), ca, f2_0, k, ok);
         q += C(1);
-        const Sym<C> k1 = rhs<Safe>(M, Fs, k3, ok);
-        const Sym<C> k2 = rhs<Safe>(axpy(M, C(0.5) * h, k1), Fm, k3, ok);
-        const Sym<C> kc = rhs<Safe>(axpy(M, C(0.5) * h, k2), Fm, k3, ok);
+        const Sym<C> k1 = rhs<Safe>(M.m, Fs, k3, ok);
+        const Sym<C> k2 = rhs<Safe>(axpy(M.m, C(0.5) * h, k1), Fm, k3, ok);
+        const Sym<C> kc = rhs<Safe>(axpy(M.m, C(0.5) * h, k2), Fm, k3, ok);
         Fs = flow_at<Safe, C>(v0, d, q * h, ca, f2_0, k, ok);
-        const Sym<C> k4 = rhs<Safe>(axpy(M, h, kc), Fs, k3, ok);
+        const Sym<C> k4 = rhs<Safe>(axpy(M.m, h, kc), Fs, k3, ok);
         Sym<C> sum;
 #pragma unroll
         for (int e = 0; e < 6; ++e) sum.v[e] = fma(C(2), k2.v[e] + kc.v[e], k1.v[e]) + k4.v[e];
-        M = axpy(M, h / C(6), sum);
+        M.add(h / C(6), sum);
     }
     return ok;
 }
 
 template <typename C>
-__device__ __forceinline__ double deformation(const Sym<C>& M) {
-    const double m[6] = {(double)M.v[0], (double)M.v[1], (double)M.v[2],
-                         (double)M.v[3], (double)M.v[4], (double)M.v[5]};
+__device__ __forceinline__ double deformation(const State<C>& M) {
+    double m[6];
+    M.entries(m);
     return lbmgb::deformation_of(m);
+}
+
+template <typename C>
+__device__ __forceinline__ void store_entries(const State<C>& M, double* out) {
+    double m[6];
+    M.entries(m);
+#pragma unroll
+    for (int e = 0; e < 6; ++e) out[e] = m[e];
 }
 
 // The substeps from row to row of A with the rows in gradient form: v0 is the
 // row before, v1 the row after.
 template <typename C>
-__device__ __forceinline__ void advance(Sym<C>& M, Flow<C>& Fs, C (&v0)[9], const C (&v1)[9], C ca, C f2_0, C kf, C h,
+__device__ __forceinline__ void advance(State<C>& M, Flow<C>& Fs, C (&v0)[9], const C (&v1)[9], C ca, C f2_0, C kf, C h,
                                         int substeps) {
     C d[9];
 #pragma unroll
     for (int j = 0; j < 9; ++j) d[j] = v1[j] - v0[j];
-    const Sym<C> M0 = M;
+    const State<C> M0 = M;
     const Flow<C> F0 = Fs;
     if (!time_step<false>(M, Fs, v0, d, ca, f2_0, kf, h, substeps)) {
         M = M0;
@@ -217,8 +260,8 @@ __device__ __forceinline__ Flow<C> first_flow(const C (&v0)[9], C ca, C f2_0, C 
     return ok ? F : flow_at<true, C>(v0, d, C(0), ca, f2_0, kf, ok);
 }
 template <typename C>
-__device__ __forceinline__ Sym<C> sphere() {
-    return {{C(1), C(0), C(0), C(1), C(0), C(1)}};
+__device__ __forceinline__ State<C> sphere() {
+    return {{{C(1), C(0), C(0), C(1), C(0), C(1)}}, {C(0), C(0), C(0)}};
 }
 
 // One warp per CTA, so that few trajectories still spread over the SMs: at
@@ -239,7 +282,7 @@ __global__ void __launch_bounds__(kMMThreads) k_mm_rk4(const double* __restrict_
                                                        double* __restrict__ D, double* __restrict__ Mout) {
     const long long k = (long long)blockIdx.x * kMMThreads + threadIdx.x;
     if (k >= n) return;
-    Sym<C> M = sphere<C>();
+    State<C> M = sphere<C>();
     D[k] = 0.0;
     const C h = C(1) / C(substeps);
     C a[9], v0[9];
@@ -269,9 +312,7 @@ __global__ void __launch_bounds__(kMMThreads) k_mm_rk4(const double* __restrict_
             D[++rec * n + k] = deformation(M);
         }
     }
-    if (Mout)
-#pragma unroll
-        for (int e = 0; e < 6; ++e) Mout[k * 6 + e] = (double)M.v[e];
+    if (Mout) store_entries(M, Mout + k * 6);
 }
 
 // The float32 form for no more trajectories than the chip has schedulers for
@@ -293,7 +334,7 @@ __global__ void __launch_bounds__(kMMThreads) k_mm_rk4(const double* __restrict_
 constexpr int kMMGroup = 4;  // integrating warps of a full CTA
 struct MMSlot {
     float row[9][32];
-    float m[6][32];
+    float m[9][32];  // M, then the diagonal's low parts
 };
 __device__ __forceinline__ void pair_sync(int id) {
     __syncwarp();
@@ -347,16 +388,18 @@ __global__ void __launch_bounds__(96 * kMMGroup) k_mm_rk4_served(const double* _
     } else if (role == 2) {
         if (live) D[k] = 0.0;
         for (long long rec = 1; rec <= records; ++rec) {
-            Sym<float> M;
+            State<float> M;
             pair_sync(m_full);
 #pragma unroll
-            for (int e = 0; e < 6; ++e) M.v[e] = q.m[e][lane];
+            for (int e = 0; e < 6; ++e) M.m.v[e] = q.m[e][lane];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) M.lo[a] = q.m[6 + a][lane];
             if (rec < records) pair_arrive(m_empty);
             const double def = deformation(M);
             if (live) D[rec * n + k] = def;
         }
     } else {
-        Sym<float> M = sphere<float>();
+        State<float> M = sphere<float>();
         const float h = 1.f / (float)substeps;
         float v0[9];
         pair_sync(row_full);
@@ -377,13 +420,13 @@ __global__ void __launch_bounds__(96 * kMMGroup) k_mm_rk4_served(const double* _
                 until = record_every;
                 if (rec++) pair_sync(m_empty);
 #pragma unroll
-                for (int e = 0; e < 6; ++e) q.m[e][lane] = M.v[e];
+                for (int e = 0; e < 6; ++e) q.m[e][lane] = M.m.v[e];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) q.m[6 + a][lane] = M.lo[a];
                 pair_arrive(m_full);
             }
         }
-        if (Mout && live)
-#pragma unroll
-            for (int e = 0; e < 6; ++e) Mout[k * 6 + e] = (double)M.v[e];
+        if (Mout && live) store_entries(M, Mout + k * 6);
     }
 }
 
