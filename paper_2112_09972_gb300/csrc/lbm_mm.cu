@@ -161,8 +161,10 @@ __device__ __forceinline__ Sym<C> axpy(const Sym<C>& m, C h, const Sym<C>& k) {
 // M between substeps: float32 keeps what the diagonal's sums round off.  The
 // diagonal lies near one, where a substep's rounding is 6e-8, and D of a nearly
 // spherical droplet is a small difference of its entries: hundreds of substeps
-// left 1e-6 of D, and as much by chance in one form of the arithmetic as
+// left 1e-6 of D, twice as much by chance in one form of the arithmetic as in
 // another.  (The other entries are as small as D, and so are their roundings.)
+// 16384 trajectories, 250 steps of 10 substeps: D 1.3e-6 -> 2.2e-7 from the
+// float64 integrator's, 653 -> 675 us.
 template <typename C>
 struct State {
     Sym<C> m;
@@ -322,7 +324,7 @@ __global__ void __launch_bounds__(kMMThreads) k_mm_rk4(const double* __restrict_
 // So two more warps serve each integrating one through shared memory: a
 // feeder that loads, converts and splits the rows of A two ahead, and a
 // recorder that turns M into D.  The arithmetic is that of k_mm_rk4.
-// 16384 trajectories, 250 steps of 10 substeps, 31 records: 655 us against 788
+// 16384 trajectories, 250 steps of 10 substeps, 31 records: 675 us; 655 against 788
 // without the serving warps (and 4908 with the stages as in the note above);
 // 500 us of it are the substeps, 400 cycles each for some 300 instructions.
 //
