@@ -14,8 +14,8 @@
 // What bounds it.  This GPU's FP64 pipe issues one warp instruction per 16
 // cycles and SM, so a float64 node update is bound by its FP64 instructions,
 // not by memory: the 608 bytes of 512 nodes take 46 ns at the measured copy
-// bandwidth, their 340 FP64 instructions a node 290 ns (128^3: 379 ns measured).  The marched tile
-// kernel sums every density about twice (the tile's halo, and the planes
+// bandwidth, their 340 FP64 instructions a node 290 ns (128^3: 379 ns
+// measured).  The marched tile kernel sums every density about twice (the tile's halo, and the planes
 // before and after each z chunk) and evaluates each equilibrium on its own,
 // 560 instructions per node.  Here each density is summed once (the second
 // read of the populations costs bandwidth that is idle), opposite
@@ -231,8 +231,9 @@ __device__ __forceinline__ void flat_unit(const double2* __restrict__ rho, const
 }
 
 // `centres` CTAs from `centre0` on sum the centre of mass from the density
-// array (against sums at the end of every colliding CTA, per step: 32^3 41.9 ->
-// 31.9 us, 37 x 29 x 23 36.1 -> 26.9, 64^3 195 -> 174, 128^3 1433 -> 1408).
+// array (against sums at the end of every colliding CTA, per step and before
+// the rest population closed the mass: 32^3 41.9 -> 31.9 us, 37 x 29 x 23 36.1 ->
+// 26.9, 64^3 195 -> 174, 128^3 1433 -> 1408).
 template <bool PER, bool MRT>
 __global__ void __launch_bounds__(kFlatThreads, kFlatPerSM)
     k_flat_collide(const double* __restrict__ src, double* __restrict__ dst, Layout L, FlatModel m,
